@@ -54,13 +54,6 @@ int leg_synth<float>(Plan *p, int spin, const float2 *alm, int rs, int nmaps, co
     return tune(p, 1, s, nmaps, V.n[s], st, [&](int v) { return V.syn[s][v](p, alm, rs, nmaps, beam, F, st); });
 }
 template <>
-int leg_synth<double>(Plan *p, int spin, const double2 *alm, int rs, int nmaps, const double *beam,
-                      double2 *F, cudaStream_t st) {
-    const Variants64 &V = variants64();
-    const int s = spin == 2 ? 1 : 0;
-    return tune(p, 0, s, nmaps, V.n[s], st, [&](int v) { return V.syn[s][v](p, alm, rs, nmaps, beam, F, st); });
-}
-template <>
 int leg_analysis<float>(Plan *p, int spin, const float2 *G, int nmaps, const float *beam, float2 *alm,
                         int rs, cudaStream_t st, int vjp) {
     const Variants32 &V = variants32();
@@ -71,15 +64,7 @@ int leg_analysis<float>(Plan *p, int spin, const float2 *G, int nmaps, const flo
 template <>
 int leg_analysis<double>(Plan *p, int spin, const double2 *G, int nmaps, const double *beam,
                          double2 *alm, int rs, cudaStream_t st, int vjp) {
-    // candidates: the register-blocked contraction (legendre_g64.cu, about
-    // half the FP64 instructions of the warp-reduction kernels when several
-    // maps share a recurrence; the default), then the warp-reduction shapes
-    const Variants64 &V = variants64();
-    const int s = spin == 2 ? 1 : 0;
-    return tune(p, 0, 2 + s, nmaps, V.n[2 + s] + 1, st, [&](int v) {
-        if (v == 0) return leg_analysis_g64(p, spin, G, nmaps, beam, alm, rs, st, vjp);
-        return V.ana[s][v - 1](p, G, nmaps, beam, alm, rs, st, vjp);
-    });
+    return leg_analysis_g64(p, spin, G, nmaps, beam, alm, rs, st, vjp);
 }
 
 // ------------------------------------------------------- grouped launches

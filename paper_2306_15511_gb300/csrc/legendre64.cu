@@ -1,24 +1,52 @@
-// FP64 Legendre kernel variants (ring pairs per thread, maps per pass) for
-// the autotuner; variant 0 of each family is the default.
-#include "legendre_kernels.cuh"
+// FP64 Legendre synthesis: maps per pass by the number of maps.
+#include "legendre_blk.cuh"
 
 namespace shtg {
 
-#define SV(SP, NR, NM) &launch_synth_v<double, SP, NR, NM>
-#define AV(SP, NR, NM) &launch_analysis_v<double, SP, NR, NM>
+// Maps per pass: the FP64 pipe bounds this kernel (a warp instruction takes
+// 64 cycles of its scheduler's FP64 unit), and a pass over NM maps costs
+// R + W NM multiply-adds per (l, m, ring pair), whether or not all NM are
+// there: the recurrence (R = 3, spin 2: 8) and the sums (W = 2, spin 2: 8).
+// The pass count times that cost is smallest for the NM taken here.
+int leg_maps_per_pass(int spin, int nmaps, const int *nms, int n) {
+    const int R = spin == 2 ? 8 : 3, W = spin == 2 ? 8 : 2;
+    int best = nms[0];
+    long long cost = -1;
+    for (int i = 0; i < n; ++i) {
+        const long long c = (long long)((nmaps + nms[i] - 1) / nms[i]) * (R + W * nms[i]);
+        if (cost < 0 || c < cost) {
+            cost = c;
+            best = nms[i];
+        }
+    }
+    return best;
+}
 
-const Variants64 &variants64() {
-    static const Variants64 V = {
-        {5, 4, 6, 4},
-        {{SV(0, 2, 2), SV(0, 2, 4), SV(0, 1, 4), SV(0, 4, 2), SV(0, 4, 4)},
-         {SV(2, 1, 2), SV(2, 1, 4), SV(2, 2, 2), SV(2, 2, 1)}},
-        {{AV(0, 2, 1), AV(0, 4, 1), AV(0, 2, 2), AV(0, 8, 1), AV(0, 6, 1), AV(0, 4, 2)},
-         {AV(2, 1, 1), AV(2, 2, 1), AV(2, 4, 1), AV(2, 3, 1)}},
-        {{{2, 2}, {2, 4}, {1, 4}, {4, 2}, {4, 4}},
-         {{1, 2}, {1, 4}, {2, 2}, {2, 1}},
-         {{2, 1}, {4, 1}, {2, 2}, {8, 1}, {6, 1}, {4, 2}},
-         {{1, 1}, {2, 1}, {4, 1}, {3, 1}}}};
-    return V;
+// One ring pair per thread: with two the kernel is 1.05 to 1.5 times slower
+// (N_side 512, l_max 1024, 8 maps: 12.8 against 13.7 ms at spin 0, 54.3
+// against 59.0 ms at spin 2; N_side 300, one map: 0.61 against 0.93 ms).
+// Before, at most four maps shared a recurrence and none of the shapes was
+// made for one or three maps (N_side 32, l_max 64, one map: 51 us, now 21).
+template <>
+int leg_synth<double>(Plan *p, int spin, const double2 *alm, int rs, int nmaps, const double *beam, double2 *F,
+                      cudaStream_t st) {
+    static const int nm0[] = {8, 6, 4, 3, 2, 1}, nm2[] = {4, 3, 2, 1};
+    if (spin == 2) {
+        switch (leg_maps_per_pass(2, nmaps, nm2, 4)) {
+            case 1: return launch_synth_v<double, 2, 1, 1>(p, alm, rs, nmaps, beam, F, st);
+            case 2: return launch_synth_v<double, 2, 1, 2>(p, alm, rs, nmaps, beam, F, st);
+            case 3: return launch_synth_v<double, 2, 1, 3>(p, alm, rs, nmaps, beam, F, st);
+            default: return launch_synth_v<double, 2, 1, 4>(p, alm, rs, nmaps, beam, F, st);
+        }
+    }
+    switch (leg_maps_per_pass(0, nmaps, nm0, 6)) {
+        case 1: return launch_synth_v<double, 0, 1, 1>(p, alm, rs, nmaps, beam, F, st);
+        case 2: return launch_synth_v<double, 0, 1, 2>(p, alm, rs, nmaps, beam, F, st);
+        case 3: return launch_synth_v<double, 0, 1, 3>(p, alm, rs, nmaps, beam, F, st);
+        case 4: return launch_synth_v<double, 0, 1, 4>(p, alm, rs, nmaps, beam, F, st);
+        case 6: return launch_synth_v<double, 0, 1, 6>(p, alm, rs, nmaps, beam, F, st);
+        default: return launch_synth_v<double, 0, 1, 8>(p, alm, rs, nmaps, beam, F, st);
+    }
 }
 
 }  // namespace shtg

@@ -1,0 +1,307 @@
+// FP64-accurate Legendre transpose (Y^T) as a register-blocked contraction,
+// for native FP64 (legendre_g64.cu) and double-FP32 (legendre_df.cu)
+// arithmetic.
+//
+// c_lm = sum_r lambda_lm(theta_r) G_r(m): CTA = one m, 128 l and NMT maps.
+// Per stage of 32 ring pairs each of the four warps generates one 32-l
+// segment of the recurrences (a lane per pair) from the FP64 states
+// tabulated every SHTG_TS64 l into shared memory ([row = l - lbase][pair]),
+// and every thread accumulates a block of outputs over all ring pairs in
+// registers: NMT rows of one parity class of l - m (App. A: lambda_lm(pi -
+// theta) = (-1)^(l+m) lambda_lm(theta), so class-E rows take G_N + G_S and
+// class-O rows G_N - G_S) times the 2 (spin 0) or 4 (spin 2: E re, E im, B
+// re, B im) outputs of one map.  Each recurrence runs once per (l, ring
+// pair) for the CTA's maps, and the sum over ring pairs needs no
+// cross-thread reduction.
+//
+// What bounds it: the arithmetic.  An FP64 warp instruction occupies its
+// scheduler's FP64 unit for 64 cycles (two lanes per clock and SM), a
+// double-FP32 multiply-add costs about twelve FP32 instructions, so the
+// loop is as fast as its count of useful operations per scheduler:
+// - all four warps generate (one half-warp generating 16 pairs over 128 l,
+//   the FP64 kernel's first form, kept three of four FP64 units idle for
+//   longer than the contraction of eight maps takes);
+// - NMT follows the number of maps that the call has (1, 2, 4 or 8), so that
+//   few threads multiply maps that are not there;
+// - row blocks beyond l_max, or before the first significant l of the stage's
+//   pairs, are left out.
+// Measured (FP64; before: the best of the 8-map form and the warp-reduction
+// kernels that this replaces): N_side 300, l_max 500, 3 maps, spin 0 / 2:
+// 2.87 / 7.3 -> 1.65 / 5.5 ms; N_side 512, l_max 1024, 8 maps: 28.4 / 115 ->
+// 15.1 / 56 ms.  Double-FP32, N_side 512, l_max 1024, 4 maps, spin 2: 15.8 ->
+// 11.1 ms.
+#pragma once
+
+#include <string>
+
+#include "legendre_kernels.cuh"
+
+namespace shtg {
+
+constexpr int B_LR = 128;        // l per CTA (rows): four 32-l segments, one per warp
+constexpr int B_KP = 32;         // ring pairs per stage (a warp's lanes)
+constexpr int B_NT = 128;        // threads
+constexpr int B_LS = B_KP + 1;   // row stride of the value tile (odd: rows in distinct banks)
+static_assert(SHTG_TS64 == 32, "a warp restarts its 32-l segment from a tabulated state");
+
+// maps per pass of an FP64-accurate Legendre sum out of the n sizes nms
+// (legendre64.cu)
+int leg_maps_per_pass(int spin, int nmaps, const int *nms, int n);
+
+// Ar: the arithmetic.  V value, Acc running sum, C2 / C4 staged coefficients,
+// State recurrence state of one pair (the fields of PairState).
+template <class Ar, int SPIN, int NMT> struct BlkLayout {
+    typedef typename Ar::V V;
+    static constexpr int NV = SPIN == 2 ? 2 : 1;   // value tiles: lambda, or (lw, lx)
+    static constexpr int NO = SPIN == 2 ? 4 : 2;   // outputs per map
+    static constexpr int GS = SPIN == 2 ? 9 : 5;   // map stride of the ring-data sets (odd)
+    static constexpr int COEF = SPIN == 2 ? sizeof(typename Ar::C4) : sizeof(typename Ar::C2);
+    static constexpr int LAM = 0;
+    static constexpr int GSET = LAM + NV * B_LR * B_LS * (int)sizeof(V);
+    static constexpr int CO = (GSET + B_KP * NMT * GS * (int)sizeof(V) + 31) & ~31;
+    static constexpr int RED = CO + B_LR * COEF;
+    static constexpr int BYTES = RED + 16;
+};
+
+template <class Ar, int SPIN, int NMT>
+__global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double> a) {
+    typedef BlkLayout<Ar, SPIN, NMT> Ly;
+    typedef typename Ar::V V;
+    constexpr int NO = Ly::NO, GS = Ly::GS, NJ = NMT, RG = 64 / NJ;
+    extern __shared__ __align__(32) unsigned char smem[];
+    V *lam = reinterpret_cast<V *>(smem + Ly::LAM);      // [NV][B_LR][B_LS]
+    V *gset = reinterpret_cast<V *>(smem + Ly::GSET);    // [B_KP][NMT][GS]
+    typename Ar::C2 *s_rec = reinterpret_cast<typename Ar::C2 *>(smem + Ly::CO);
+    typename Ar::C4 *s_s2c = reinterpret_cast<typename Ar::C4 *>(smem + Ly::CO);
+    int *s_first = reinterpret_cast<int *>(smem + Ly::RED);
+
+    const int tid = threadIdx.x;
+    const int m = blockIdx.y;
+    const int L = a.lmax;
+    const int lbase = m + blockIdx.x * B_LR;
+    if (lbase > L) return;
+    const int lend = min(L, lbase + B_LR - 1);
+    const int map0 = blockIdx.z * NMT;
+    const int nm = min(NMT, a.nmaps - map0);
+    const int64_t base = (int64_t)m * (2 * L + 1 - m) / 2;
+    const int64_t rowsz = (int64_t)a.nring * (L + 1);
+
+    for (int i = tid; i < B_LR; i += B_NT) {
+        const int l = lbase + i;
+        const bool in = l <= L;
+        if (SPIN == 2) s_s2c[i] = Ar::c4(in ? a.s2c[base + l] : make_double4_32a(0.0, 0.0, 0.0, 0.0));
+        else s_rec[i] = Ar::c2(in ? a.rec[base + l] : make_double2(0.0, 0.0));
+    }
+    // first ring pair whose recurrence starts at or before lend (the start l
+    // falls towards the equator; a later pair without significant values only
+    // adds exact zeros)
+    if (tid == 0) *s_first = a.npairs;
+    __syncthreads();
+    for (int pr = tid; pr < a.npairs; pr += B_NT) {
+        const int64_t o = (int64_t)m * a.npairs + pr;
+        int lsp;
+        if (SPIN == 2) {
+            const int2 q = a.ls2[o];
+            lsp = min(q.x, q.y);
+        } else {
+            lsp = a.ls[o];
+        }
+        if (lsp <= lend) {
+            atomicMin(s_first, pr);
+            break;
+        }
+    }
+    __syncthreads();
+    const int s0 = *s_first / B_KP;
+    const int nps = (a.npairs + B_KP - 1) / B_KP;
+
+    // this thread's outputs: map k, class c, rows i = c + 2 (rg + RG j)
+    const int k = tid & (NMT - 1), c = (tid / NMT) & 1, rg = tid / (2 * NMT);
+    typename Ar::Acc acc[NJ][NO];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+#pragma unroll
+        for (int q = 0; q < NO; ++q) Ar::zero(acc[j][q]);
+
+    // this warp's rows of block j: WR consecutive ones from row0 + 2 RG j
+    constexpr int WR = 32 / NMT;
+    const int row0 = 2 * ((tid & ~31) / (2 * NMT));
+    for (int s = s0; s < nps; ++s) {
+        __syncthreads();   // the previous stage's tiles are consumed
+        int first_l;       // no pair of the stage has a significant value below this l
+        {
+            // ---- recurrences of the stage's 32 ring pairs: warp w runs rows
+            // 32 w .. 32 w + 31 of pair s * 32 + lane from the FP64 state
+            // tabulated at l0 = lbase + 32 w
+            const int pp = tid & 31, seg = tid >> 5;
+            const int pr = s * B_KP + pp;
+            const int l0 = lbase + 32 * seg;
+            typename Ar::State S;
+            Ar::template load<SPIN>(a, m, pr, S);
+            const bool live = pr < a.npairs && l0 <= L;
+            first_l = __reduce_min_sync(0xffffffffu, SPIN == 2 ? min(S.ls[0], S.lsb[0]) : S.ls[0]);
+            if (live) {
+                const int64_t e = (a.toff64[m] + (l0 - m) / SHTG_TS64) * a.npairs + pr;
+                if (SPIN == 2) {
+                    const double4_32a t4 = a.tst64_2[e];
+                    S.a1[0] = Ar::from(t4.x);
+                    S.a2[0] = Ar::from(t4.y);
+                    S.b1[0] = Ar::from(t4.z);
+                    S.b2[0] = Ar::from(t4.w);
+                } else {
+                    const double2 t2 = a.tst64_0[e];
+                    S.a1[0] = Ar::from(t2.x);
+                    S.a2[0] = Ar::from(t2.y);
+                }
+            }
+            // injection steps only if some pair of the warp starts in this segment
+            const bool inj = __any_sync(0xffffffffu, live && ((S.ls[0] >= l0 && S.ls[0] < l0 + 32) ||
+                                                              (SPIN == 2 && S.lsb[0] >= l0 && S.lsb[0] < l0 + 32)));
+            if (__any_sync(0xffffffffu, live) && l0 + 31 >= first_l) {
+                for (int i = 32 * seg; i < 32 * seg + 32; ++i) {
+                    if (inj) Ar::template step<SPIN, true>(S, s_rec, s_s2c, i, lbase + i);
+                    else Ar::template step<SPIN, false>(S, s_rec, s_s2c, i, lbase + i);
+                    if (SPIN == 2) {
+                        lam[i * B_LS + pp] = live ? Ar::add(S.a1[0], S.b1[0]) : Ar::from(0.0);
+                        lam[B_LR * B_LS + i * B_LS + pp] = live ? Ar::sub(S.a1[0], S.b1[0]) : Ar::from(0.0);
+                    } else {
+                        lam[i * B_LS + pp] = live ? S.a1[0] : Ar::from(0.0);
+                    }
+                }
+            } else {   // beyond l_max or before every start
+                for (int i = 32 * seg; i < 32 * seg + 32; ++i) {
+                    lam[i * B_LS + pp] = Ar::from(0.0);
+                    if (SPIN == 2) lam[B_LR * B_LS + i * B_LS + pp] = Ar::from(0.0);
+                }
+            }
+        }
+        // ---- ring data of the stage: per (pair, map) the even / odd sets
+        for (int it = tid; it < B_KP * NMT; it += B_NT) {
+            const int pp = it / NMT, kk = it % NMT;
+            const int pr = s * B_KP + pp;
+            V *g = gset + (pp * NMT + kk) * GS;
+            double2 z[4] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0),
+                            make_double2(0.0, 0.0)};
+            if (pr < a.npairs && kk < nm) {
+                const int rn = pr, rs = a.nring - 1 - pr;
+#pragma unroll
+                for (int cc = 0; cc < (SPIN == 2 ? 2 : 1); ++cc) {
+                    const int64_t row = SPIN == 2 ? 2 * (map0 + kk) + cc : map0 + kk;
+                    const double2 *gr = a.F + row * rowsz + m;
+                    const double2 gn = gr[(int64_t)rn * (L + 1)];
+                    const double2 gs = rs != rn ? gr[(int64_t)rs * (L + 1)] : make_double2(0.0, 0.0);
+                    z[2 * cc] = make_double2(gn.x + gs.x, gn.y + gs.y);       // even set
+                    z[2 * cc + 1] = make_double2(gn.x - gs.x, gn.y - gs.y);   // odd set
+                }
+            }
+            // spin 0: [E re, E im, O re, O im]; spin 2: [QE re, QE im, QO re, QO im, UE re, UE im, UO re, UO im]
+#pragma unroll
+            for (int q = 0; q < (SPIN == 2 ? 4 : 2); ++q) {
+                g[2 * q] = Ar::from(z[q].x);
+                g[2 * q + 1] = Ar::from(z[q].y);
+            }
+        }
+        __syncthreads();
+        // ---- contraction over the stage's ring pairs; row blocks beyond l_max
+        // or before every start of the stage (exact zeros) are left out
+        bool on[NJ];
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+            const int l = lbase + row0 + 2 * RG * j;
+            on[j] = l <= L && l + WR > first_l;
+        }
+#pragma unroll 2
+        for (int p = 0; p < B_KP; ++p) {
+            const V *g = gset + (p * NMT + k) * GS;
+            if (SPIN == 0) {
+                const V gre = g[2 * c], gim = g[2 * c + 1];
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) {
+                    if (!on[j]) continue;   // warp-uniform
+                    const V lv = lam[(c + 2 * (rg + RG * j)) * B_LS + p];
+                    Ar::fma(acc[j][0], lv, gre);
+                    Ar::fma(acc[j][1], lv, gim);
+                }
+            } else {
+                // lw terms take the row's set, lx terms the other one:
+                //   E^ = -lw G_Q - i lx G_U,  B^ = i lx G_Q - lw G_U
+                const V qr = g[2 * c], qi = g[2 * c + 1], ur = g[4 + 2 * c], ui = g[4 + 2 * c + 1];
+                const V xqr = g[2 * (1 - c)], xqi = g[2 * (1 - c) + 1], xur = g[4 + 2 * (1 - c)],
+                        xui = g[4 + 2 * (1 - c) + 1];
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) {
+                    if (!on[j]) continue;
+                    const int i = c + 2 * (rg + RG * j);
+                    const V lw = lam[i * B_LS + p], lx = lam[B_LR * B_LS + i * B_LS + p];
+                    const V nlw = Ar::neg(lw), nlx = Ar::neg(lx);
+                    Ar::fma(acc[j][0], lx, xui);
+                    Ar::fma(acc[j][0], nlw, qr);
+                    Ar::fma(acc[j][1], nlx, xur);
+                    Ar::fma(acc[j][1], nlw, qi);
+                    Ar::fma(acc[j][2], nlx, xqi);
+                    Ar::fma(acc[j][2], nlw, ur);
+                    Ar::fma(acc[j][3], lx, xqr);
+                    Ar::fma(acc[j][3], nlw, ui);
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+#pragma unroll
+            for (int q = 0; q < NO; ++q) Ar::norm(acc[j][q]);   // 64 terms at most since the last
+    }
+    // ---- epilogue: every alm of this CTA's l range written once
+    if (k >= nm) return;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        const int l = lbase + c + 2 * (rg + RG * j);
+        if (l > L) continue;
+        const double bm = (a.beam ? a.beam[l] : 1.0) * ((a.vjp && m > 0) ? 2.0 : 1.0);
+#pragma unroll
+        for (int cc = 0; cc < NO / 2; ++cc) {
+            const int64_t row = (int64_t)(map0 + k) * a.rs + cc;
+            double2 *dst = const_cast<double2 *>(a.alm) + row * a.nalm + base + l;
+            *dst = make_double2(Ar::to(acc[j][2 * cc]) * bm, m == 0 ? 0.0 : Ar::to(acc[j][2 * cc + 1]) * bm);
+        }
+    }
+}
+
+template <class Ar, int SPIN, int NMT>
+int launch_analysis_blk(Plan *p, const double2 *G, int nmaps, const double *beam, double2 *alm, int rs,
+                        cudaStream_t st, int vjp) {
+    LegArgs<double> a = leg_make_args<double>(p);
+    a.alm = alm;
+    a.rs = rs;
+    a.vjp = vjp;
+    a.F = const_cast<double2 *>(G);
+    a.beam = beam;
+    a.nmaps = nmaps;
+    if (!a.toff64 || !a.tst64_0 || (SPIN == 2 && !a.tst64_2)) {
+        set_error("FP64-accurate transpose: the plan has no FP64 recurrence tile states");
+        return SHTG_ERR_ARG;
+    }
+    const int smem = BlkLayout<Ar, SPIN, NMT>::BYTES;
+    auto kern = k_leg_analysis_blk<Ar, SPIN, NMT>;
+    if (smem > 48 * 1024) SHTG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    dim3 grid((p->lmax + B_LR) / B_LR, p->lmax + 1, (nmaps + NMT - 1) / NMT);
+    prof_begin(p, K_LEG_ANA64, st);
+    kern<<<grid, B_NT, smem, st>>>(a);
+    prof_end(p, st);
+    SHTG_CHECK_LAUNCH("k_leg_analysis_blk");
+    return SHTG_OK;
+}
+
+// NMT: the least work over the call's maps (leg_maps_per_pass)
+template <class Ar, int SPIN>
+int analysis_blk(Plan *p, const double2 *G, int nmaps, const double *beam, double2 *alm, int rs, cudaStream_t st,
+                 int vjp) {
+    static const int nmt[] = {8, 4, 2, 1};
+    switch (leg_maps_per_pass(SPIN, nmaps, nmt, 4)) {
+        case 1: return launch_analysis_blk<Ar, SPIN, 1>(p, G, nmaps, beam, alm, rs, st, vjp);
+        case 2: return launch_analysis_blk<Ar, SPIN, 2>(p, G, nmaps, beam, alm, rs, st, vjp);
+        case 4: return launch_analysis_blk<Ar, SPIN, 4>(p, G, nmaps, beam, alm, rs, st, vjp);
+        default: return launch_analysis_blk<Ar, SPIN, 8>(p, G, nmaps, beam, alm, rs, st, vjp);
+    }
+}
+
+}  // namespace shtg

@@ -15,11 +15,9 @@
 //
 // Synthesis: one thread per ring pair (NR of them) and NM maps, as the
 // CUDA-core kernels, the recurrence in registers.  Transpose: the
-// register-blocked contraction of the FP64 transpose (legendre_g64.cu) with
-// stages of 32 ring pairs, whose recurrences all four warps generate in
-// 32-l segments from the plan's FP64 tile states (every SHTG_TS64 l).
+// register-blocked contraction of legendre_blk.cuh.
 #include "df.cuh"
-#include "legendre_kernels.cuh"
+#include "legendre_blk.cuh"
 
 namespace shtg {
 namespace {
@@ -311,207 +309,32 @@ __global__ void __launch_bounds__(LEG_THREADS) k_leg_synth_df(const LegArgs<doub
 }
 
 // =========================================================== transpose
-constexpr int D_LR = 128;   // l per CTA (rows): four 32-l segments, one per warp
-constexpr int D_KP = 32;    // ring pairs per stage (a warp's lanes)
-constexpr int D_NT = 128;   // threads
-constexpr int D_NMT = 8;    // maps per CTA (grid.z covers more)
-constexpr int D_LS = D_KP + 1;   // row stride of the value tile (odd: rows in distinct banks)
-constexpr int D_GS = 9;          // map stride of the ring-data sets
-
-template <int SPIN> struct DfT {
-    static constexpr int NV = SPIN == 2 ? 2 : 1;   // value tiles: lambda, or (lw, lx)
-    static constexpr int NO = SPIN == 2 ? 4 : 2;   // outputs per map
-    static constexpr int COEF = SPIN == 2 ? 32 : 16;
-    static constexpr int LAM = 0;
-    static constexpr int GSET = LAM + NV * D_LR * D_LS * 8;
-    static constexpr int CO = GSET + D_KP * D_NMT * D_GS * 8;
-    static constexpr int RED = CO + D_LR * COEF;
-    static constexpr int BYTES = RED + 16;
+// double-FP32 arithmetic of the register-blocked transpose (legendre_blk.cuh)
+struct ArDf {
+    typedef df V;
+    typedef dfacc Acc;
+    typedef dfc2 C2;
+    typedef dfc4 C4;
+    typedef DfPair<1> State;
+    static __device__ __forceinline__ V from(double x) { return df_from(x); }
+    static __device__ __forceinline__ C2 c2(double2 v) { return dfc2_from(v); }
+    static __device__ __forceinline__ C4 c4(double4_32a v) { return dfc4_from(v); }
+    static __device__ __forceinline__ V add(V x, V y) { return df_add(x, y); }
+    static __device__ __forceinline__ V sub(V x, V y) { return df_sub(x, y); }
+    static __device__ __forceinline__ V neg(V x) { return df_neg(x); }
+    static __device__ __forceinline__ void zero(Acc &s) { df_acc_zero(s); }
+    static __device__ __forceinline__ void fma(Acc &s, V x, V y) { df_fma(s, x, y); }
+    static __device__ __forceinline__ void norm(Acc &s) { df_acc_norm(s); }
+    static __device__ __forceinline__ double to(const Acc &s) { return df_acc_to(s); }
+    template <int SPIN>
+    static __device__ __forceinline__ void load(const LegArgs<double> &a, int m, int pr, State &S) {
+        df_pair_load<1, SPIN>(a, m, pr, S, 0);
+    }
+    template <int SPIN, bool INJ>
+    static __device__ __forceinline__ void step(State &S, const C2 *s_rec, const C4 *s_s2c, int i, int l) {
+        df_stepx<1, SPIN, INJ>(S, s_rec, s_s2c, i, l);
+    }
 };
-
-template <int SPIN>
-__global__ void __launch_bounds__(D_NT) k_leg_analysis_df(const LegArgs<double> a) {
-    typedef DfT<SPIN> Ly;
-    constexpr int NO = Ly::NO;
-    extern __shared__ __align__(16) unsigned char smem[];
-    df *lam = reinterpret_cast<df *>(smem + Ly::LAM);      // [NV][D_LR][D_LS]
-    df *gset = reinterpret_cast<df *>(smem + Ly::GSET);    // [D_KP][D_NMT][D_GS]
-    dfc2 *s_rec = reinterpret_cast<dfc2 *>(smem + Ly::CO);
-    dfc4 *s_s2c = reinterpret_cast<dfc4 *>(smem + Ly::CO);
-    int *s_first = reinterpret_cast<int *>(smem + Ly::RED);
-
-    const int tid = threadIdx.x;
-    const int m = blockIdx.y;
-    const int L = a.lmax;
-    const int lbase = m + blockIdx.x * D_LR;
-    if (lbase > L) return;
-    const int lend = min(L, lbase + D_LR - 1);
-    const int map0 = blockIdx.z * D_NMT;
-    const int nm = min(D_NMT, a.nmaps - map0);
-    const int64_t base = (int64_t)m * (2 * L + 1 - m) / 2;
-    const int64_t rowsz = (int64_t)a.nring * (L + 1);
-
-    for (int i = tid; i < D_LR; i += D_NT) {
-        const int l = lbase + i;
-        const bool in = l <= L;
-        if (SPIN == 2) s_s2c[i] = dfc4_from(in ? a.s2c[base + l] : make_double4_32a(0.0, 0.0, 0.0, 0.0));
-        else s_rec[i] = dfc2_from(in ? a.rec[base + l] : make_double2(0.0, 0.0));
-    }
-    // first ring pair whose recurrence starts at or before lend (later pairs
-    // without significant values add exact zeros)
-    if (tid == 0) *s_first = a.npairs;
-    __syncthreads();
-    for (int pr = tid; pr < a.npairs; pr += D_NT) {
-        const int64_t o = (int64_t)m * a.npairs + pr;
-        int lsp;
-        if (SPIN == 2) {
-            const int2 q = a.ls2[o];
-            lsp = min(q.x, q.y);
-        } else {
-            lsp = a.ls[o];
-        }
-        if (lsp <= lend) {
-            atomicMin(s_first, pr);
-            break;
-        }
-    }
-    __syncthreads();
-    const int s0 = *s_first / D_KP;
-    const int nps = (a.npairs + D_KP - 1) / D_KP;
-
-    // this thread's outputs: map k, class c, rows i = c + 2 (rg + 8 j)
-    const int k = tid & 7, c = (tid >> 3) & 1, rg = tid >> 4;
-    dfacc acc[8][NO];
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-        for (int q = 0; q < NO; ++q) df_acc_zero(acc[j][q]);
-
-    for (int s = s0; s < nps; ++s) {
-        __syncthreads();   // the previous stage's tiles are consumed
-        {
-            // ---- recurrences of the stage's 32 ring pairs: warp w runs rows
-            // 32 w .. 32 w + 31 of pair s * 32 + lane from the FP64 state
-            // tabulated at l0 = lbase + 32 w
-            const int pp = tid & 31, seg = tid >> 5;
-            const int pr = s * D_KP + pp;
-            const int l0 = lbase + 32 * seg;
-            DfPair<1> S;
-            df_pair_load<1, SPIN>(a, m, pr, S, 0);
-            const bool live = pr < a.npairs && l0 <= L;
-            if (live) {
-                const int64_t e = (a.toff64[m] + (l0 - m) / SHTG_TS64) * a.npairs + pr;
-                if (SPIN == 2) {
-                    const double4_32a t4 = a.tst64_2[e];
-                    S.a1[0] = df_from(t4.x);
-                    S.a2[0] = df_from(t4.y);
-                    S.b1[0] = df_from(t4.z);
-                    S.b2[0] = df_from(t4.w);
-                } else {
-                    const double2 t2 = a.tst64_0[e];
-                    S.a1[0] = df_from(t2.x);
-                    S.a2[0] = df_from(t2.y);
-                }
-            }
-            // injection steps only if some pair of the warp starts in this segment
-            const bool inj = __any_sync(0xffffffffu, live && ((S.ls[0] >= l0 && S.ls[0] < l0 + 32) ||
-                                                              (SPIN == 2 && S.lsb[0] >= l0 && S.lsb[0] < l0 + 32)));
-            for (int i = 32 * seg; i < 32 * seg + 32; ++i) {
-                df v0 = df_zero(), v1 = df_zero();
-                if (live) {
-                    if (inj) df_stepx<1, SPIN, true>(S, s_rec, s_s2c, i, lbase + i);
-                    else df_stepx<1, SPIN, false>(S, s_rec, s_s2c, i, lbase + i);
-                    if (SPIN == 2) {
-                        v0 = df_add(S.a1[0], S.b1[0]);
-                        v1 = df_sub(S.a1[0], S.b1[0]);
-                    } else {
-                        v0 = S.a1[0];
-                    }
-                }
-                lam[i * D_LS + pp] = v0;
-                if (SPIN == 2) lam[D_LR * D_LS + i * D_LS + pp] = v1;
-            }
-        }
-        // ---- ring data of the stage: per (pair, map) the even / odd sets
-        for (int it = tid; it < D_KP * D_NMT; it += D_NT) {
-            const int pp = it >> 3, kk = it & 7;
-            const int pr = s * D_KP + pp;
-            df *g = gset + (pp * D_NMT + kk) * D_GS;
-            double2 z[4] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0),
-                            make_double2(0.0, 0.0)};
-            if (pr < a.npairs && kk < nm) {
-                const int rn = pr, rs = a.nring - 1 - pr;
-                const int nrow = SPIN == 2 ? 2 : 1;
-                for (int cc = 0; cc < nrow; ++cc) {
-                    const int64_t row = SPIN == 2 ? 2 * (map0 + kk) + cc : map0 + kk;
-                    const double2 *gr = a.F + row * rowsz + m;
-                    const double2 gn = gr[(int64_t)rn * (L + 1)];
-                    const double2 gs = rs != rn ? gr[(int64_t)rs * (L + 1)] : make_double2(0.0, 0.0);
-                    z[2 * cc] = make_double2(gn.x + gs.x, gn.y + gs.y);       // even set
-                    z[2 * cc + 1] = make_double2(gn.x - gs.x, gn.y - gs.y);   // odd set
-                }
-            }
-            // spin 0: [E re, E im, O re, O im]; spin 2: [QE re, QE im, QO re, QO im, UE re, UE im, UO re, UO im]
-            for (int q = 0; q < (SPIN == 2 ? 4 : 2); ++q) {
-                g[2 * q] = df_from(z[q].x);
-                g[2 * q + 1] = df_from(z[q].y);
-            }
-        }
-        __syncthreads();
-        // ---- contraction over the stage's ring pairs
-#pragma unroll 2
-        for (int p = 0; p < D_KP; ++p) {
-            const df *g = gset + (p * D_NMT + k) * D_GS;
-            if (SPIN == 0) {
-                const df gre = g[2 * c], gim = g[2 * c + 1];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const df lv = lam[(c + 2 * (rg + 8 * j)) * D_LS + p];
-                    df_fma(acc[j][0], lv, gre);
-                    df_fma(acc[j][1], lv, gim);
-                }
-            } else {
-                // lw terms take the row's set, lx terms the other one:
-                //   E^ = -lw G_Q - i lx G_U,  B^ = i lx G_Q - lw G_U
-                const df qr = g[2 * c], qi = g[2 * c + 1], ur = g[4 + 2 * c], ui = g[4 + 2 * c + 1];
-                const df xqr = g[2 * (1 - c)], xqi = g[2 * (1 - c) + 1], xur = g[4 + 2 * (1 - c)],
-                         xui = g[4 + 2 * (1 - c) + 1];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int i = c + 2 * (rg + 8 * j);
-                    const df lw = lam[i * D_LS + p], lx = lam[D_LR * D_LS + i * D_LS + p];
-                    const df nlw = df_neg(lw), nlx = df_neg(lx);
-                    df_fma(acc[j][0], lx, xui);
-                    df_fma(acc[j][0], nlw, qr);
-                    df_fma(acc[j][1], nlx, xur);
-                    df_fma(acc[j][1], nlw, qi);
-                    df_fma(acc[j][2], nlx, xqi);
-                    df_fma(acc[j][2], nlw, ur);
-                    df_fma(acc[j][3], lx, xqr);
-                    df_fma(acc[j][3], nlw, ui);
-                }
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-#pragma unroll
-            for (int q = 0; q < NO; ++q) df_acc_norm(acc[j][q]);   // 64 terms at most since the last
-    }
-    // ---- epilogue: every alm of this CTA's l range written once
-    if (k >= nm) return;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int l = lbase + c + 2 * (rg + 8 * j);
-        if (l > L) continue;
-        const double bm = (a.beam ? a.beam[l] : 1.0) * ((a.vjp && m > 0) ? 2.0 : 1.0);
-#pragma unroll
-        for (int cc = 0; cc < NO / 2; ++cc) {
-            const int64_t row = (int64_t)(map0 + k) * a.rs + cc;
-            double2 *dst = const_cast<double2 *>(a.alm) + row * a.nalm + base + l;
-            *dst = make_double2(df_acc_to(acc[j][2 * cc]) * bm, m == 0 ? 0.0 : df_acc_to(acc[j][2 * cc + 1]) * bm);
-        }
-    }
-}
 
 template <int NR, int NM, int SPIN>
 int launch_synth_df(Plan *p, const double2 *alm, int rs, int nmaps, const double *beam, double2 *F,
@@ -530,55 +353,36 @@ int launch_synth_df(Plan *p, const double2 *alm, int rs, int nmaps, const double
     return SHTG_OK;
 }
 
-template <int SPIN>
-int launch_analysis_df(Plan *p, const double2 *G, int nmaps, const double *beam, double2 *alm, int rs,
-                       cudaStream_t st, int vjp) {
-    LegArgs<double> a = leg_make_args<double>(p);
-    a.alm = alm;
-    a.rs = rs;
-    a.vjp = vjp;
-    a.F = const_cast<double2 *>(G);
-    a.beam = beam;
-    a.nmaps = nmaps;
-    if (!a.toff64 || !a.tst64_0 || (SPIN == 2 && !a.tst64_2)) {
-        set_error("double-FP32 transpose: the plan has no FP64 recurrence tile states");
-        return SHTG_ERR_ARG;
-    }
-    const int smem = DfT<SPIN>::BYTES;
-    if (smem > 48 * 1024)
-        SHTG_CUDA(cudaFuncSetAttribute(k_leg_analysis_df<SPIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    dim3 grid((p->lmax + D_LR) / D_LR, p->lmax + 1, (nmaps + D_NMT - 1) / D_NMT);
-    prof_begin(p, K_LEG_ANA64, st);
-    k_leg_analysis_df<SPIN><<<grid, D_NT, smem, st>>>(a);
-    prof_end(p, st);
-    SHTG_CHECK_LAUNCH("k_leg_analysis_df");
-    return SHTG_OK;
-}
-
 }  // namespace
 
-// Autotuned (key kind 3): synthesis (ring pairs per thread, maps per pass)
-// spin 0: (1, 8), (1, 4), (2, 4); spin 2: (1, 4), (1, 2), (2, 1) (the first
-// of each was the fastest at N_side 1024, l_max 2048, 8 maps).  The
-// transpose has one shape.
+// One ring pair per thread, maps per pass by the least work
+// (leg_maps_per_pass: the recurrence and a map's multiply-adds stand in the
+// same ratio as in native FP64).
 int leg_synth_df(Plan *p, int spin, const double2 *alm, int rs, int nmaps, const double *beam, double2 *F,
                  cudaStream_t st) {
-    return tune(p, 3, spin == 2 ? 1 : 0, nmaps, 3, st, [&](int v) {
-        if (spin == 2) {
-            if (v == 1) return launch_synth_df<1, 2, 2>(p, alm, rs, nmaps, beam, F, st);
-            if (v == 2) return launch_synth_df<2, 1, 2>(p, alm, rs, nmaps, beam, F, st);
-            return launch_synth_df<1, 4, 2>(p, alm, rs, nmaps, beam, F, st);
+    static const int nm0[] = {8, 6, 4, 3, 2, 1}, nm2[] = {4, 3, 2, 1};
+    if (spin == 2) {
+        switch (leg_maps_per_pass(2, nmaps, nm2, 4)) {
+            case 1: return launch_synth_df<1, 1, 2>(p, alm, rs, nmaps, beam, F, st);
+            case 2: return launch_synth_df<1, 2, 2>(p, alm, rs, nmaps, beam, F, st);
+            case 3: return launch_synth_df<1, 3, 2>(p, alm, rs, nmaps, beam, F, st);
+            default: return launch_synth_df<1, 4, 2>(p, alm, rs, nmaps, beam, F, st);
         }
-        if (v == 1) return launch_synth_df<1, 4, 0>(p, alm, rs, nmaps, beam, F, st);
-        if (v == 2) return launch_synth_df<2, 4, 0>(p, alm, rs, nmaps, beam, F, st);
-        return launch_synth_df<1, 8, 0>(p, alm, rs, nmaps, beam, F, st);
-    });
+    }
+    switch (leg_maps_per_pass(0, nmaps, nm0, 6)) {
+        case 1: return launch_synth_df<1, 1, 0>(p, alm, rs, nmaps, beam, F, st);
+        case 2: return launch_synth_df<1, 2, 0>(p, alm, rs, nmaps, beam, F, st);
+        case 3: return launch_synth_df<1, 3, 0>(p, alm, rs, nmaps, beam, F, st);
+        case 4: return launch_synth_df<1, 4, 0>(p, alm, rs, nmaps, beam, F, st);
+        case 6: return launch_synth_df<1, 6, 0>(p, alm, rs, nmaps, beam, F, st);
+        default: return launch_synth_df<1, 8, 0>(p, alm, rs, nmaps, beam, F, st);
+    }
 }
 
 int leg_analysis_df(Plan *p, int spin, const double2 *G, int nmaps, const double *beam, double2 *alm, int rs,
                     cudaStream_t st, int vjp) {
-    if (spin == 2) return launch_analysis_df<2>(p, G, nmaps, beam, alm, rs, st, vjp);
-    return launch_analysis_df<0>(p, G, nmaps, beam, alm, rs, st, vjp);
+    if (spin == 2) return analysis_blk<ArDf, 2>(p, G, nmaps, beam, alm, rs, st, vjp);
+    return analysis_blk<ArDf, 0>(p, G, nmaps, beam, alm, rs, st, vjp);
 }
 
 }  // namespace shtg
