@@ -207,7 +207,8 @@ int shtg_plan_create(int geom, int nside_or_nring, int nphi_gauss, int lmax, int
         p->nring = nside_or_nring;
         p->nphi_gauss = nphi_gauss;
     }
-    if (cudaGetDevice(&p->device) != cudaSuccess) {
+    if (cudaGetDevice(&p->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&p->nsm, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
         cudaGetLastError();
         delete p;
         set_error("no CUDA device");

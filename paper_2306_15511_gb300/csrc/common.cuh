@@ -69,19 +69,6 @@ struct RingFFT {
     int64_t ph_off;     // shifted rings: offset of e^{i pi k / n}, k = 0 .. min(lmax, n - 1)
 };
 
-// Ring FFT launches (ringfft.cu): threads per CTA for a launch whose
-// longest buffer is 2^logm, and the butterflies per thread of the first
-// radix-R pass (R = 2, 4, 8; log2 M not a multiple of four) that the kernel
-// of that thread count is compiled for.  Launch buckets hold rings with
-// M = 2^logm (and M = 2^(logm - 1) for aliased direct rings); the bucket of
-// lengths <= 1024 runs 64 threads.
-__host__ __device__ constexpr int ring_threads(int logm) {
-    return logm >= 13 ? 512 : logm == 12 ? 256 : logm == 11 ? 128 : 64;
-}
-__host__ __device__ constexpr int ring_first_bpt(int R, int nt) {
-    return nt >= 512 ? (R == 2 ? 8 : 1) : nt == 256 ? 1 : nt == 128 ? (R == 2 ? 1 : 2) : (R == 8 ? 1 : 4);
-}
-
 // grouped launches (chains of several geometries): plans per launch
 #define SHTG_MAX_GROUPS 16
 
@@ -159,7 +146,7 @@ struct AzBlk {
 };
 
 struct Plan {
-    int device = 0;
+    int device = 0, nsm = 0;       // CUDA device and its SM count
     Prof prof;
     std::map<long long, int> tuned;   // autotuned kernel variant per (precision, family, nmaps)
     int geom = 0, nside = 0, nring = 0, npairs = 0, lmax = 0, max_batch = 0, flags = 0;
@@ -201,28 +188,29 @@ struct Plan {
     int fft_logmax = 0;
     RingFFT *d_rfft = nullptr;
     std::vector<RingFFT> h_rfft;
-    // two-level twiddle table for e^{-2 pi i t / Mmax}, t = th 2^tw_blo + tl:
-    // [lo: e^{-2 pi i tl / Mmax}, 2^tw_blo entries | hi: e^{-2 pi i th 2^tw_blo / Mmax}]
-    double2 *d_tw64 = nullptr;
-    float2 *d_tw32 = nullptr;
-    int tw_blo = 0, tw_nlo = 0, tw_nhi = 0;
     double2 *d_chirp64 = nullptr, *d_bfwd64 = nullptr, *d_binv64 = nullptr;
     float2 *d_chirp32 = nullptr, *d_bfwd32 = nullptr, *d_binv32 = nullptr;
-    // fixed-length launches (ringfft.cu): per-pass twiddles of the radix-16
-    // passes for M = 2^logm, at twf_off[logm] (logm = 10 .. 13)
-    double2 *d_twf64 = nullptr;
+    // pass twiddles of M = 2^logm at twr_off64 / twr_off32 [logm] (ring_twiddles, ringfft.cu)
+    double2 *d_twr64 = nullptr;
+    float2 *d_twr32 = nullptr;
+    int twr_off64[SHTG_FFT_LOGMAX + 1] = {}, twr_off32[SHTG_FFT_LOGMAX + 1] = {};
+    // FP32 radix-16 launches: pass twiddles for M = 2^logm, at twf_off[logm]
+    // (logm = 10 .. 13), and the two-level table for e^{-2 pi i t / Mmax}, t =
+    // th 2^tw_blo + tl: [lo: e^{-2 pi i tl / Mmax}, 2^tw_blo entries | hi:
+    // e^{-2 pi i th 2^tw_blo / Mmax}]
     float2 *d_twf32 = nullptr;
     int64_t twf_off[SHTG_FFT_LOGMAX + 1] = {};
+    float2 *d_tw32 = nullptr;
+    int tw_blo = 0, tw_nlo = 0, tw_nhi = 0;
     double2 *d_rph64 = nullptr;   // ring phase tables (RingFFT::ph_off)
     float2 *d_rph32 = nullptr;
-    size_t fft_smem64 = 0, fft_smem32 = 0;
     int *d_ring_groups = nullptr;    // ring pairs, ordered by launch bucket
     struct RingLaunch {
         int off, count;   // slice of d_ring_groups
         int logm;         // log2 of the bucket's buffer length (every member's M, and 2n if aliased)
         int alias;        // bucket holds rings with n < 2 lmax
         int chirp;        // longest Bluestein ring of the bucket (its chirp is staged in shared memory)
-        int fix;          // launches of 128 threads and more: log2 of every member's M (fixed-length passes); 0 = any
+        int fix;          // buckets above 1024: log2 of every member's M; 0 = any length up to 1024
     };
     std::vector<RingLaunch> ring_launch;
 
@@ -392,6 +380,8 @@ int leg_analysis_df(Plan *p, int spin, const double2 *G, int nmaps, const double
                     cudaStream_t st, int vjp);
 
 // ringfft.cu
+// pass twiddles of every transform length (FP32: up to 1024), and where each starts
+void ring_twiddles(std::vector<double2> &t64, int *off64, std::vector<float2> &t32, int *off32);
 // mode 0: F -> map (synthesis); mode 1: map -> G (adjoint, wmode 1 = quadrature weights);
 // mode 2: F -> N^-1 -> G (fused, in place allowed).
 template <typename T>

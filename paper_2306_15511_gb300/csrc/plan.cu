@@ -511,21 +511,18 @@ static int build_fft_tables(Plan *p) {
     p->tw_blo = (logmax + 1) / 2;
     p->tw_nlo = 1 << p->tw_blo;
     p->tw_nhi = 1 << (logmax - p->tw_blo);
-    std::vector<double2> tw64(p->tw_nlo + p->tw_nhi);
-    std::vector<float2> tw32(tw64.size());
+    std::vector<float2> tw32(p->tw_nlo + p->tw_nhi);
     for (int i = 0; i < p->tw_nlo + p->tw_nhi; ++i) {
         const int64_t t = i < p->tw_nlo ? i : (int64_t)(i - p->tw_nlo) << p->tw_blo;
         const double ang = -2.0 * PI * (double)t / (double)Mmax;
-        tw64[i] = make_double2(cos(ang), sin(ang));
         tw32[i] = make_float2((float)cos(ang), (float)sin(ang));
     }
-    // per-pass twiddles of the fixed-length FFT passes (ringfft.cu) for
-    // M = 2^10 .. 2^13: radix-16 pass p with NS = 2^(logm mod 4) 16^p > 1 holds
-    // e^{-2 pi i r k / (16 NS)} for r = 1 at k and r = 4 at NS + k, k < NS
-    std::vector<double2> twf64;
+    // pass twiddles of the FP32 radix-16 launches (ringfft.cu) for M = 2^10 ..
+    // 2^13: pass p with NS = 2^(logm mod 4) 16^p > 1 holds e^{-2 pi i r k /
+    // (16 NS)} for r = 1 at k and r = 4 at NS + k, k < NS
     std::vector<float2> twf32;
     for (int lg = 10; lg <= SHTG_FFT_LOGMAX; ++lg) {
-        p->twf_off[lg] = (int64_t)twf64.size();
+        p->twf_off[lg] = (int64_t)twf32.size();
         for (int ps = 0; ps < (lg >> 2); ++ps) {
             const int ns = (1 << (lg & 3)) << (4 * ps);
             if (ns == 1) continue;
@@ -533,11 +530,13 @@ static int build_fft_tables(Plan *p) {
                 for (int k = 0; k < ns; ++k) {
                     const int64_t t = ((int64_t)r * k) % (16 * (int64_t)ns);
                     const double ang = -2.0 * PI * (double)t / (16.0 * ns);
-                    twf64.push_back(make_double2(cos(ang), sin(ang)));
                     twf32.push_back(make_float2((float)cos(ang), (float)sin(ang)));
                 }
         }
     }
+    std::vector<double2> twr64;
+    std::vector<float2> twr32;
+    ring_twiddles(twr64, p->twr_off64, twr32, p->twr_off32);
     std::vector<double2> ch64(chirp_total), bf64(bhat_total), bi64(bhat_total);
     std::vector<float2> ch32(chirp_total), bf32(bhat_total), bi32(bhat_total);
     for (auto &kv : offs) {
@@ -605,13 +604,13 @@ static int build_fft_tables(Plan *p) {
     SHTG_TRY(upload(p->d_rph32, ph32));
     SHTG_TRY(dalloc(p, &p->d_rfft, R));
     SHTG_TRY(upload(p->d_rfft, p->h_rfft));
-    SHTG_TRY(dalloc(p, &p->d_twf64, twf64.size()));
+    SHTG_TRY(dalloc(p, &p->d_twr64, twr64.size()));
+    SHTG_TRY(dalloc(p, &p->d_twr32, twr32.size()));
     SHTG_TRY(dalloc(p, &p->d_twf32, twf32.size()));
-    SHTG_TRY(upload(p->d_twf64, twf64));
-    SHTG_TRY(upload(p->d_twf32, twf32));
-    SHTG_TRY(dalloc(p, &p->d_tw64, tw64.size()));
     SHTG_TRY(dalloc(p, &p->d_tw32, tw32.size()));
-    SHTG_TRY(upload(p->d_tw64, tw64));
+    SHTG_TRY(upload(p->d_twr64, twr64));
+    SHTG_TRY(upload(p->d_twr32, twr32));
+    SHTG_TRY(upload(p->d_twf32, twf32));
     SHTG_TRY(upload(p->d_tw32, tw32));
     SHTG_TRY(dalloc(p, &p->d_chirp64, ch64.size()));
     SHTG_TRY(dalloc(p, &p->d_chirp32, ch32.size()));
@@ -625,10 +624,7 @@ static int build_fft_tables(Plan *p) {
     SHTG_TRY(upload(p->d_binv64, bi64));
     SHTG_TRY(upload(p->d_bfwd32, bf32));
     SHTG_TRY(upload(p->d_binv32, bi32));
-    p->fft_smem64 = (size_t)Mmax * sizeof(double2);
-    p->fft_smem32 = (size_t)Mmax * sizeof(float2);
-    // Launch buckets by transform length, each launch with M / 16 threads
-    // (one radix-16 butterfly per thread): Bluestein rings by their M, direct
+    // Launch buckets by transform length: Bluestein rings by their M, direct
     // rings without aliasing (n >= 2 lmax) by n, aliased direct rings by 2n so
     // that the south ring's folded spectrum fits in buf[n, 2n); buckets of
     // length 1024 and below share one launch.  Buckets above 1024 are split
@@ -656,20 +652,18 @@ static int build_fft_tables(Plan *p) {
             g.fix = kv.first.second;
             g.alias = 0;
             g.chirp = 0;
-            const int nt = g.fix ? (1 << g.fix) / 16 : ring_threads(g.logm);
             for (int r : kv.second) {
                 const RingFFT &f = p->h_rfft[r];
                 groups.push_back(r);
                 if (f.n < 2 * p->lmax) g.alias = 1;
                 if (f.blue) g.chirp = std::max(g.chirp, f.n);
-                // the kernel's passes cover this ring: M / 16 butterflies per
-                // radix-16 pass, M / R in the first pass
-                const int M = 1 << f.logM, R = 1 << (f.logM & 3);
-                // launches of buckets above 1024 run the fixed-length passes
-                // of their members' one length, 2^logm or 2^(logm - 1)
+                // launches of buckets above 1024 run the passes of their
+                // members' one length, 2^logm or 2^(logm - 1)
+                const int M = 1 << f.logM;
                 const bool fix_ok = g.fix == 0 ? g.logm <= 10
                                                : (g.fix == f.logM && (f.logM == g.logm || f.logM == g.logm - 1));
-                const bool ok = fix_ok && M <= 16 * nt && (R == 1 || M / R <= nt * ring_first_bpt(R, nt)) &&
+                // (64-thread radix-16 launches: M <= 16 x 64)
+                const bool ok = fix_ok && M <= (1 << g.logm) &&
                                 (f.n >= 2 * p->lmax || 2 * (int64_t)f.n <= ((int64_t)1 << g.logm));
                 if (!ok) {
                     set_error("ring " + std::to_string(r) + ": transform length " + std::to_string(M) +
@@ -772,15 +766,15 @@ void plan_free(Plan *p) {
     void *ptrs[] = {p->d_nphi, p->d_ofs, p->d_wring, p->d_u64, p->d_u32, p->d_x64, p->d_is2_64,
                     p->d_x32, p->d_is2_32, p->d_lofidx, p->d_mofidx, p->d_rec64, p->d_rec32,
                     p->d_ls64, p->d_ls32, p->d_st64, p->d_st32, p->d_s2c64, p->d_s2c32,
-                    p->d_rfft, p->d_tw64, p->d_tw32, p->d_chirp64, p->d_bfwd64, p->d_binv64,
+                    p->d_rfft, p->d_chirp64, p->d_bfwd64, p->d_binv64,
                     p->d_chirp32, p->d_bfwd32, p->d_binv32, p->d_phase64, p->d_phase32,
                     p->d_map64, p->d_map32, p->d_ninv64, p->d_ninv32, p->d_minv64,
                     p->d_minv32, p->d_diagT, p->d_diagP, p->d_wpairT, p->d_wpairP,
                     p->d_ltab64, p->d_ltab32, p->d_scal, p->d_part, p->d_lsum, p->d_stage,
                     p->d_ls2_64, p->d_st2_64, p->d_ls2_32, p->d_st2_32, p->d_ring_groups, p->d_flag,
                     p->d_toff, p->d_tst0, p->d_tst2, p->d_isc64, p->d_rsc64, p->d_isc32,
-                    p->d_toff64, p->d_tst64_0, p->d_tst64_2, p->d_rph64, p->d_rph32, p->d_twf64,
-                    p->d_twf32, p->d_jtab, p->d_blk, p->d_blklam, p->d_blkw, p->d_blkoff,
+                    p->d_toff64, p->d_tst64_0, p->d_tst64_2, p->d_rph64, p->d_rph32, p->d_twr64, p->d_twr32,
+                    p->d_tw32, p->d_twf32, p->d_jtab, p->d_blk, p->d_blklam, p->d_blkw, p->d_blkoff,
                     p->d_blkflag};
     for (void *q : ptrs)
         if (q) cudaFree(q);

@@ -9,29 +9,49 @@
 // pass loads R elements per butterfly into registers, applies the twiddles,
 // does the radix-R DFT in registers and writes the R outputs to their sorted
 // places (Govindaraju et al. 2008, "High performance discrete Fourier
-// transforms on graphics processors", with one radix-2, -4 or -8 pass first,
-// where it needs no twiddles, and radix-16 passes after it).  The buffer is
-// padded by one element per 16 so that the
-// scattered writes of the early passes hit distinct banks.  Rings whose n is
+// transforms on graphics processors"; radix 8 in FP32, 4 in FP64, with one
+// radix-2 or -4 pass first where the length needs it).  The buffer is padded
+// by one element per 16 so that the scattered writes of the early passes hit
+// distinct banks.  Rings whose n is
 // not a power of two (HEALPix polar caps) use Bluestein's chirp convolution
 // with precomputed kernel spectra.  The fused variant applies N^-1 between
 // the inverse and the forward transform, so the pixel map never goes to
 // global memory inside an operator application.
 #include <algorithm>
+#include <cmath>
 #include <string>
+#include <vector>
 
 #include "common.cuh"
 
 namespace shtg {
 
-// Threads per CTA: M / 16 for the launch's longest transform M (every
-// radix-16 pass then has one butterfly per thread), at least 64; resident
-// CTAs per SM for a budget of 128 registers a thread in FP32 (the inlined
-// passes do not spill; the fixed-length launches, M = 16 NT: 64 registers,
-// so twice as many threads share an SM), 255 in FP64 up to 256 threads (the
-// FP64 passes spill at 128).
-template <typename T, int NT, int FIX> struct RingBlocks {
-    static constexpr int v = sizeof(T) == 8 ? (NT >= 256 ? 1 : 256 / NT) : (FIX > 0 ? 1024 : 512) / NT;
+// Radix of the passes and threads per CTA.  FP64: radix 4, M / 4 threads (1024
+// with two butterflies at M = 8192).  An FP64 warp instruction takes 64 cycles
+// of its scheduler's FP64 unit, so a ring's transform takes as long as its
+// busiest scheduler's FP64 instructions: radix-16 butterflies (272 FP64
+// instructions each, M / 16 of them, two of three twiddles computed) left a
+// short ring's work on one or two warps of an SM; radix-4 ones take 28 on four
+// times as many threads, spread over all four schedulers.  Fused stage of one
+// map at N_side 32: 104 -> 30 us; of 12 T, Q, U maps at N_side 128, l_max 256:
+// 1009 -> 584 us; synthesis of 8 maps at N_side 512, M = 4096: 1.85 -> 1.71
+// ms (near the FP64 pipe).  FP32 lengths up to 1024: radix 8, 128 threads
+// (latency bound: one radix-16 butterfly a pass on 64 threads took longer);
+// the same 12 maps at N_side 128: 80 -> 50 us.  Launches of lengths up to
+// 1024 run one kernel for all their lengths with the threads of the longest.
+template <typename T> struct RingRadix { static constexpr int LR = sizeof(T) == 8 ? 2 : 3; };
+template <typename T> __host__ __device__ constexpr int ring_nt(int logm) {
+    return logm <= 10 ? 1 << (10 - RingRadix<T>::LR)
+                      : (1 << (logm - RingRadix<T>::LR)) > 1024 ? 1024 : 1 << (logm - RingRadix<T>::LR);
+}
+// Which passes a launch runs: radix 4 / 8 as above (FP64; FP32 lengths up to
+// 1024 in the analysis and the fused stage), or FP32 radix 16 with M / 16
+// threads, of one length (FIX > 0) or (64 threads) of any length up to 1024.
+enum { RING_R48 = 0, RING_R16 = 1, RING_R16_ANY = 2 };
+template <typename T, int MODE, int FIX> struct RingCore {
+    static constexpr int kind = sizeof(T) == 8 ? RING_R48 : FIX > 0 ? RING_R16 : MODE == 0 ? RING_R16_ANY : RING_R48;
+    static constexpr int nt = kind == RING_R48 ? ring_nt<T>(FIX > 0 ? FIX : 10) : kind == RING_R16 ? (1 << FIX) / 16 : 64;
+    static constexpr int sm_threads = kind == RING_R16_ANY ? 512 : 1024;   // at 64 (R16_ANY: 128) registers
 };
 
 __device__ __forceinline__ int rpad(int i) { return i + (i >> 4); }
@@ -49,18 +69,201 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 }
 __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
 
-// v * e^{-+2 pi i k / 16} (minus sign: forward transform, plus: inverse); k is
-// a compile-time constant after unrolling, so the switch folds away
-template <bool INV, typename C>
+// ---------------------------------------------------------------------------
+// Radix-R DFTs in registers, forward (e^{-2 pi i r s / R}), natural order in
+// and out.
+template <typename C>
+__device__ __forceinline__ void dft2(C &a, C &b) {
+    const C t = a;
+    a = cadd(t, b);
+    b = csub(t, b);
+}
+template <typename C>
+__device__ __forceinline__ void dft4(C &x0, C &x1, C &x2, C &x3) {
+    const C t0 = cadd(x0, x2), t1 = csub(x0, x2), t2 = cadd(x1, x3);
+    const C d = csub(x1, x3);
+    const C t3 = C{d.y, -d.x};
+    x0 = cadd(t0, t2);
+    x2 = csub(t0, t2);
+    x1 = cadd(t1, t3);
+    x3 = csub(t1, t3);
+}
+template <int R, typename C> struct Dft;
+template <typename C> struct Dft<2, C> {
+    static __device__ __forceinline__ void run(C *v) { dft2(v[0], v[1]); }
+};
+template <typename C> struct Dft<4, C> {
+    static __device__ __forceinline__ void run(C *v) { dft4(v[0], v[1], v[2], v[3]); }
+};
+// r = 4 r1 + r2, s = s1 + 2 s2: four DFTs of length 2, twiddles w_8^(r2 s1),
+// two DFTs of length 4
+template <typename C> struct Dft<8, C> {
+    static __device__ __forceinline__ void run(C *v) {
+        typedef decltype(v[0].x) T;
+        const T h = T(0.70710678118654752440);
+        C y[4][2];
+#pragma unroll
+        for (int r2 = 0; r2 < 4; ++r2) {
+            y[r2][0] = v[r2];
+            y[r2][1] = v[4 + r2];
+            dft2(y[r2][0], y[r2][1]);
+        }
+        C t = y[1][1];
+        y[1][1] = C{h * (t.x + t.y), h * (t.y - t.x)};      // w_8
+        t = y[2][1];
+        y[2][1] = C{t.y, -t.x};                             // w_8^2
+        t = y[3][1];
+        y[3][1] = C{h * (t.y - t.x), -(h * (t.x + t.y))};   // w_8^3
+#pragma unroll
+        for (int s1 = 0; s1 < 2; ++s1) {
+            dft4(y[0][s1], y[1][s1], y[2][s1], y[3][s1]);
+#pragma unroll
+            for (int s2 = 0; s2 < 4; ++s2) v[s1 + 2 * s2] = y[s2][s1];
+        }
+    }
+};
+
+// Stockham FFT of length M = 2^LOGM, forward, unnormalized, natural order in
+// and out, in place in shared memory (all reads of a pass finish before its
+// writes).  Passes: NS = 1 with radix 2^(LOGM mod LR) where that is above one,
+// then radix 2^LR with NS growing by the radix.  Butterfly j of a pass (k = j
+// mod NS) takes x[j + r M / R], multiplies element r by w^r (w = e^{-2 pi i
+// k / (R NS)}), does a radix-R DFT and writes output s to (j - k) R + k + s NS.
+//
+// Twiddles of the passes with NS > 1 come from a table rounded once from
+// FP64 (ring_twiddles): FP64 holds w, w^2, w^3 at k, NS + k, 2 NS + k; FP32
+// holds w and w^4 and forms the others as products (at most three extra
+// roundings).  A warp's consecutive k read consecutive entries.
+//
+// Padded addresses: rpad(i) = i + i / 16.  Loads: rpad(j + r NB) is rpad(j) +
+// r (NB + NB / 16) where 16 divides NB = M / R.  Stores to o = d + r NS, d =
+// (j - k) R + k: NS >= 16: rpad(d) + r (NS + NS / 16); NS < 16 (NS divides 16,
+// k < NS): d + (d - k) / 16 + r NS + (r NS) / 16.
+template <int R, int LOGM, int NS, int NT, typename C>
+__device__ __forceinline__ void fft_pass(C *buf, const C *__restrict__ tw) {
+    constexpr int M = 1 << LOGM, NB = M / R, BPT = (NB + NT - 1) / NT;
+    C v[BPT][R];
+#pragma unroll
+    for (int b = 0; b < BPT; ++b) {
+        const int j = threadIdx.x + b * NT;
+        if (NB % NT == 0 || j < NB) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                v[b][r] = NB % 16 == 0 ? buf[rpad(j) + r * (NB + NB / 16)] : buf[rpad(j + r * NB)];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int b = 0; b < BPT; ++b) {
+        const int j = threadIdx.x + b * NT;
+        if (NB % NT == 0 || j < NB) {
+            const int k = j & (NS - 1);
+            if constexpr (NS > 1 && R == 4) {
+                v[b][1] = cmul(v[b][1], tw[k]);
+                v[b][2] = cmul(v[b][2], tw[NS + k]);
+                v[b][3] = cmul(v[b][3], tw[2 * NS + k]);
+            }
+            if constexpr (NS > 1 && R == 8) {
+                const C w1 = tw[k], w4 = tw[NS + k];
+                const C w2 = cmul(w1, w1), w3 = cmul(w2, w1);
+                v[b][1] = cmul(v[b][1], w1);
+                v[b][2] = cmul(v[b][2], w2);
+                v[b][3] = cmul(v[b][3], w3);
+                v[b][4] = cmul(v[b][4], w4);
+                v[b][5] = cmul(v[b][5], cmul(w4, w1));
+                v[b][6] = cmul(v[b][6], cmul(w4, w2));
+                v[b][7] = cmul(v[b][7], cmul(w4, w3));
+            }
+            Dft<R, C>::run(v[b]);
+            const int d = (j - k) * R + k;
+            const int bo = NS >= 16 ? d + (d >> 4) : d + ((d - k) >> 4);
+#pragma unroll
+            for (int r = 0; r < R; ++r) buf[bo + (NS >= 16 ? r * (NS + NS / 16) : r * NS + (r * NS) / 16)] = v[b][r];
+        }
+    }
+    __syncthreads();
+}
+// table entries of the passes of one length before the pass with this NS
+template <typename T> __host__ __device__ constexpr int ring_tw_off(int logm, int ns) {
+    constexpr int LR = RingRadix<T>::LR, PER = sizeof(T) == 8 ? 3 : 2;
+    int o = 0;
+    for (int q = 1 << (logm % LR); q < ns; q <<= LR)
+        if (q > 1) o += PER * q;
+    return o;
+}
+template <typename T> __host__ __device__ constexpr int ring_tw_len(int logm) {
+    return ring_tw_off<T>(logm, 1 << logm);
+}
+template <int LOGM, int NS, int NT, typename C>
+__device__ __forceinline__ void fft_passes(C *buf, const C *__restrict__ tw) {
+    typedef decltype(buf[0].x + buf[0].x) T;
+    constexpr int LR = RingRadix<T>::LR;
+    if constexpr (NS < (1 << LOGM)) {
+        fft_pass<(1 << LR), LOGM, NS, NT>(buf, tw + ring_tw_off<T>(LOGM, NS));
+        fft_passes<LOGM, (NS << LR), NT>(buf, tw);
+    }
+}
+template <int LOGM, int NT, typename C>
+__device__ __forceinline__ void fft_fixed(C *buf, const C *__restrict__ tw) {
+    typedef decltype(buf[0].x + buf[0].x) T;
+    constexpr int R0 = 1 << (LOGM % RingRadix<T>::LR);
+    if constexpr (R0 > 1) fft_pass<R0, LOGM, 1, NT>(buf, tw);
+    fft_passes<LOGM, R0, NT>(buf, tw);
+}
+// One of the lengths of a launch that holds several (FIX 0), as a function
+// of its own: inlined side by side, the ten lengths' addresses are all kept
+// in registers across the calls and spill (1.7 KB a thread).  The buffer is
+// passed as its offset in the dynamic shared memory (a pointer would lose
+// its address space).
+template <int LOGM, int NT, typename C>
+__device__ __noinline__ void fft_small(const int buf_off, const C *__restrict__ tw) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    fft_fixed<LOGM, NT>(reinterpret_cast<C *>(s_raw) + buf_off, tw);
+}
+// any length up to 1024 (FIX 0), or 2^FIX
+template <int FIX, int NT, typename C>
+__device__ __forceinline__ void fft_run(C *buf, const int buf_off, const int logM, const C *__restrict__ tw) {
+    if constexpr (FIX > 0) {
+        fft_fixed<FIX, NT>(buf, tw);
+    } else {
+        switch (logM) {
+            case 1: fft_small<1, NT>(buf_off, tw); break;
+            case 2: fft_small<2, NT>(buf_off, tw); break;
+            case 3: fft_small<3, NT>(buf_off, tw); break;
+            case 4: fft_small<4, NT>(buf_off, tw); break;
+            case 5: fft_small<5, NT>(buf_off, tw); break;
+            case 6: fft_small<6, NT>(buf_off, tw); break;
+            case 7: fft_small<7, NT>(buf_off, tw); break;
+            case 8: fft_small<8, NT>(buf_off, tw); break;
+            case 9: fft_small<9, NT>(buf_off, tw); break;
+            case 10: fft_small<10, NT>(buf_off, tw); break;
+            default: break;   // length 1
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// FP32 radix-16 passes (M / 16 threads): the long rings, where they move the
+// least shared memory per point (radix 8 with M / 8 threads was 3 % slower on
+// the whole transform of 8 Q/U maps at N_side 1024), and the synthesis of the
+// short ones, so that FP32 maps (and what is summed over them, such as the
+// log-posterior's value) keep their rounding.
+// butterflies per thread of the first radix-R pass of a launch with nt threads
+__host__ __device__ constexpr int ring_first_bpt(int R, int nt) {
+    return nt >= 512 ? (R == 2 ? 8 : 1) : nt == 256 ? 1 : nt == 128 ? (R == 2 ? 1 : 2) : (R == 8 ? 1 : 4);
+}
+// v * e^{-2 pi i k / 16}; k is a compile-time constant after unrolling, so the
+// switch folds away
+template <typename C>
 __device__ __forceinline__ C rot16(const C v, const int k) {
     typedef decltype(v.x) T;
     const T c1 = T(0.92387953251128675613), s1 = T(0.38268343236508977173), h = T(0.70710678118654752440);
     T c, s;   // cos, sin of k pi / 8
     switch (k & 15) {
         case 0: return v;
-        case 4: return INV ? C{-v.y, v.x} : C{v.y, -v.x};
+        case 4: return C{v.y, -v.x};
         case 8: return C{-v.x, -v.y};
-        case 12: return INV ? C{v.y, -v.x} : C{-v.y, v.x};
+        case 12: return C{-v.y, v.x};
         case 1: c = c1; s = s1; break;
         case 2: c = h; s = h; break;
         case 3: c = s1; s = c1; break;
@@ -74,58 +277,28 @@ __device__ __forceinline__ C rot16(const C v, const int k) {
         case 14: c = h; s = -h; break;
         default: c = c1; s = -s1; break;   // 15
     }
-    if (INV) return C{v.x * c - v.y * s, v.x * s + v.y * c};
     return C{v.x * c + v.y * s, v.y * c - v.x * s};
 }
 
-template <bool INV, typename C>
-__device__ __forceinline__ void dft2(C &a, C &b) {
-    const C t = a;
-    a = cadd(t, b);
-    b = csub(t, b);
-}
-
-// natural order in and out: X_s = sum_r x_r e^{-+2 pi i r s / 4}
-template <bool INV, typename C>
-__device__ __forceinline__ void dft4(C &x0, C &x1, C &x2, C &x3) {
-    const C t0 = cadd(x0, x2), t1 = csub(x0, x2), t2 = cadd(x1, x3);
-    const C d = csub(x1, x3);
-    const C t3 = INV ? C{-d.y, d.x} : C{d.y, -d.x};
-    x0 = cadd(t0, t2);
-    x2 = csub(t0, t2);
-    x1 = cadd(t1, t3);
-    x3 = csub(t1, t3);
-}
-
-// Composite radix-R DFT in registers, natural order in and out: with
-// r = N2 r1 + r2 and s = s1 + N1 s2, X_s = sum_r2 w_R^{r2 s1} w_N2^{r2 s2}
-// (sum_r1 x_r w_N1^{r1 s1}): N2 DFTs of length N1, twiddles, N1 DFTs of length N2.
-template <int R, bool INV, typename C> struct Dft;
-template <bool INV, typename C> struct Dft<2, INV, C> {
-    static __device__ __forceinline__ void run(C *v) { dft2<INV>(v[0], v[1]); }
-};
-template <bool INV, typename C> struct Dft<4, INV, C> {
-    static __device__ __forceinline__ void run(C *v) { dft4<INV>(v[0], v[1], v[2], v[3]); }
-};
-template <bool INV, typename C> struct Dft<8, INV, C> {   // N1 = 2, N2 = 4
+template <typename C> struct Dft8s {   // N1 = 2, N2 = 4
     static __device__ __forceinline__ void run(C *v) {
         C y[4][2];
 #pragma unroll
         for (int r2 = 0; r2 < 4; ++r2) {
             y[r2][0] = v[r2];
             y[r2][1] = v[4 + r2];
-            dft2<INV>(y[r2][0], y[r2][1]);
-            y[r2][1] = rot16<INV>(y[r2][1], 2 * r2);   // w_8^{r2} = w_16^{2 r2}
+            dft2(y[r2][0], y[r2][1]);
+            y[r2][1] = rot16(y[r2][1], 2 * r2);   // w_8^{r2} = w_16^{2 r2}
         }
 #pragma unroll
         for (int s1 = 0; s1 < 2; ++s1) {
-            dft4<INV>(y[0][s1], y[1][s1], y[2][s1], y[3][s1]);
+            dft4(y[0][s1], y[1][s1], y[2][s1], y[3][s1]);
 #pragma unroll
             for (int s2 = 0; s2 < 4; ++s2) v[s1 + 2 * s2] = y[s2][s1];
         }
     }
 };
-template <bool INV, typename C> struct Dft<16, INV, C> {   // N1 = N2 = 4
+template <typename C> struct Dft16s {   // N1 = N2 = 4
     static __device__ __forceinline__ void run(C *v) {
         C y[4][4];
 #pragma unroll
@@ -134,18 +307,24 @@ template <bool INV, typename C> struct Dft<16, INV, C> {   // N1 = N2 = 4
             y[r2][1] = v[4 + r2];
             y[r2][2] = v[8 + r2];
             y[r2][3] = v[12 + r2];
-            dft4<INV>(y[r2][0], y[r2][1], y[r2][2], y[r2][3]);
+            dft4(y[r2][0], y[r2][1], y[r2][2], y[r2][3]);
 #pragma unroll
-            for (int s1 = 1; s1 < 4; ++s1) y[r2][s1] = rot16<INV>(y[r2][s1], r2 * s1);
+            for (int s1 = 1; s1 < 4; ++s1) y[r2][s1] = rot16(y[r2][s1], r2 * s1);
         }
 #pragma unroll
         for (int s1 = 0; s1 < 4; ++s1) {
-            dft4<INV>(y[0][s1], y[1][s1], y[2][s1], y[3][s1]);
+            dft4(y[0][s1], y[1][s1], y[2][s1], y[3][s1]);
 #pragma unroll
             for (int s2 = 0; s2 < 4; ++s2) v[s1 + 4 * s2] = y[s2][s1];
         }
     }
 };
+
+template <int R, typename C> struct DftS;
+template <typename C> struct DftS<2, C> : Dft<2, C> {};
+template <typename C> struct DftS<4, C> : Dft<4, C> {};
+template <typename C> struct DftS<8, C> : Dft8s<C> {};
+template <typename C> struct DftS<16, C> : Dft16s<C> {};
 
 // Twiddles from the two-level table in shared memory: e^{-2 pi i t / Mmax}
 template <typename C> struct TwTab {
@@ -207,7 +386,7 @@ __device__ __forceinline__ void spass(C *buf, const int M, const int Ns, const T
                     v[b][r] = cmul(v[b][r], w);
                 }
             }
-            Dft<R, false, C>::run(v[b]);
+            DftS<R, C>::run(v[b]);
             const int d = (j - k) * R + k;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
@@ -226,7 +405,7 @@ __device__ __forceinline__ void spass(C *buf, const int M, const int Ns, const T
 // null) and conjugates when cj is set.  The inverse transform is
 // conj(DFT(conj x)): callers conjugate on the way in and out.  Passes: one
 // radix-8, -4 or -2 pass when log2 M is not a multiple of four, then radix
-// 16.  Each kernel calls it from one place, so it is inlined once.
+// 16.  One call site, inlined once.
 template <int NT, typename C>
 __device__ __forceinline__ void fft_stockham(C *buf, const int logM, const TwTab<C> tw,
                                           const C *__restrict__ post, const bool cj) {
@@ -255,8 +434,8 @@ __device__ __forceinline__ void fft_stockham(C *buf, const int logM, const TwTab
 }
 
 // ---------------------------------------------------------------------------
-// Fixed-length Stockham FFT (M = 2^LOGM known at compile time), used by the
-// launches of the long rings.  Same passes as fft_stockham (one radix-2, -4 or
+// FP32 fixed-length Stockham FFT (M = 2^LOGM known at compile time), used by
+// the launches of the long rings.  Same passes as fft_stockham (one radix-2, -4 or
 // -8 pass when log2 M is not a multiple of four, then radix-16 passes), but
 // every shared-memory address of a pass is a per-thread base plus a
 // compile-time offset, and the twiddles of each radix-16 pass come from a
@@ -281,7 +460,7 @@ __host__ __device__ constexpr int twf_pass_off(int logm, int p) {
 }
 
 // Radix-16 DFT in place with its outputs left transposed: X[s] ends at
-// v[4 (s mod 4) + s / 4] (the same 4 x 4 decomposition as Dft<16>: DFT-4 down
+// v[4 (s mod 4) + s / 4] (the same 4 x 4 decomposition as Dft16s: DFT-4 down
 // the columns r2, twiddles w16^(r2 s1), DFT-4 along the rows s1), so no second
 // array of 16 values is live; callers read the outputs through the
 // compile-time permutation dft16_at.
@@ -290,13 +469,13 @@ template <typename C>
 __device__ __forceinline__ void dft16_tp(C *v) {
 #pragma unroll
     for (int r2 = 0; r2 < 4; ++r2) {
-        dft4<false>(v[r2], v[r2 + 4], v[r2 + 8], v[r2 + 12]);
-        v[r2 + 4] = rot16<false>(v[r2 + 4], r2);
-        v[r2 + 8] = rot16<false>(v[r2 + 8], 2 * r2);
-        v[r2 + 12] = rot16<false>(v[r2 + 12], 3 * r2);
+        dft4(v[r2], v[r2 + 4], v[r2 + 8], v[r2 + 12]);
+        v[r2 + 4] = rot16(v[r2 + 4], r2);
+        v[r2 + 8] = rot16(v[r2 + 8], 2 * r2);
+        v[r2 + 12] = rot16(v[r2 + 12], 3 * r2);
     }
 #pragma unroll
-    for (int s1 = 0; s1 < 4; ++s1) dft4<false>(v[4 * s1], v[4 * s1 + 1], v[4 * s1 + 2], v[4 * s1 + 3]);
+    for (int s1 = 0; s1 < 4; ++s1) dft4(v[4 * s1], v[4 * s1 + 1], v[4 * s1 + 2], v[4 * s1 + 3]);
 }
 
 __host__ __device__ constexpr int twf_len(int logm) { return twf_pass_off(logm, logm >> 2); }
@@ -321,7 +500,7 @@ __device__ __forceinline__ void fpass_first(C *buf) {
     for (int b = 0; b < BPT; ++b) {
         const int j = threadIdx.x + b * NT;
         if (NB % NT == 0 || j < NB) {
-            Dft<R, false, C>::run(v[b]);
+            DftS<R, C>::run(v[b]);
             const int o0 = j * R;
             const int bo = o0 + (o0 >> 4);
 #pragma unroll
@@ -394,30 +573,40 @@ __device__ __forceinline__ void fft16_passes(C *buf, const C *__restrict__ tw) {
 
 // Length-2^LOGM forward DFT of buf in place (natural order in and out).
 template <int LOGM, int NT, typename C>
-__device__ __forceinline__ void fft_fixed(C *buf, const C *__restrict__ tw) {
+__device__ __forceinline__ void fft16_fixed(C *buf, const C *__restrict__ tw) {
     static_assert(LOGM >= 8, "fixed-length passes need M >= 256");
     constexpr int R0L = LOGM & 3;
     if constexpr (R0L != 0) fpass_first<(1 << R0L), LOGM, NT>(buf);
     fft16_passes<LOGM, NT, 0>(buf, tw);
 }
 
-// One transform direction with the fixed-length FFT (see transform_dir)
-// (the Bluestein spectrum multiply is a separate sweep over the buffer with
-// coalesced loads of the spectrum, so no pass keeps sixteen of them in flight)
-template <int LOGM, int NT, typename C>
-__device__ __forceinline__ void transform_dir_fixed(C *buf, const C *__restrict__ tw, const C *__restrict__ bh) {
-    constexpr int M = 1 << LOGM;
-    if (bh) {
-        fft_fixed<LOGM, NT>(buf, tw);
-#pragma unroll 4
-        for (int i = threadIdx.x; i < M; i += NT) {
-            C y = cmul(buf[rpad(i)], __ldg(bh + i));
-            y.y = -y.y;
-            buf[rpad(i)] = y;
-        }
-        __syncthreads();
+// One transform direction in place: a DFT for power-of-two rings (bh null), a
+// Bluestein convolution with kernel spectrum bh otherwise (buf then holds its
+// conjugate); one FFT call site.
+template <int KIND, int FIX, int NT, typename C>
+__device__ __forceinline__ void transform_dir(C *buf, const int buf_off, const int logM, const C *__restrict__ tw,
+                                              const TwTab<C> &tw2, const C *__restrict__ bh) {
+    const int nf = bh ? 2 : 1;
+    if constexpr (KIND == RING_R16_ANY) {
+        for (int k = 0; k < nf; ++k)
+            fft_stockham<NT>(buf, logM, tw2, k == 0 ? bh : nullptr, bh != nullptr && k == 0);
+        return;
     }
-    fft_fixed<LOGM, NT>(buf, tw);
+    const int M = 1 << logM;
+#pragma unroll 1
+    for (int k = 0; k < nf; ++k) {
+        if (k == 1) {
+#pragma unroll 4
+            for (int i = threadIdx.x; i < M; i += NT) {
+                C y = cmul(buf[rpad(i)], __ldg(bh + i));
+                y.y = -y.y;
+                buf[rpad(i)] = y;
+            }
+            __syncthreads();
+        }
+        if constexpr (KIND == RING_R16) fft16_fixed<(FIX > 0 ? FIX : 8), NT>(buf, tw);
+        else fft_run<FIX, NT>(buf, buf_off, logM, tw);
+    }
 }
 
 template <typename T> struct RingArgs {
@@ -427,11 +616,15 @@ template <typename T> struct RingArgs {
     const RingFFT *rf;
     const int64_t *ofs;
     const double *wring;
-    const C *tw;      // two-level twiddle table [lo | hi]
-    int tw_blo, tw_nlo, tw_nhi, logmax;
     const C *chirp, *bfwd, *binv;
     const C *rph;     // ring phase tables e^{i pi k / n}
-    const C *twf;     // fixed-length launches: pass twiddles for M = 2^FIX
+    // twiddles: RING_R48 pass tables of every length, those of M = 2^logM at
+    // tw_off[logM]; RING_R16 the pass table of M = 2^FIX; RING_R16_ANY the
+    // two-level table [lo | hi]
+    const C *tw;
+    int tw_off[SHTG_FFT_LOGMAX + 1];
+    int tw_blo, tw_nlo, logmax;   // RING_R16_ANY
+    int tw_len;       // entries staged in shared memory
     int mpg;          // maps per CTA: CTA (pair, y) handles maps [y mpg, min(nmaps, (y + 1) mpg))
     C *FG;            // [map][ring][m]
     T *map;           // [map][npix]
@@ -443,15 +636,6 @@ template <typename T> struct RingArgs {
     const int *pairs; // ring pairs handled by this launch (one CTA each)
 };
 
-// One transform direction in place: a DFT for power-of-two rings (bh null),
-// a Bluestein convolution with kernel spectrum bh otherwise (buf then holds
-// its conjugate).  One FFT call site.
-template <int NT, typename C>
-__device__ __forceinline__ void transform_dir(C *buf, const int logM, const TwTab<C> &tw, const C *__restrict__ bh) {
-    const int nf = bh ? 2 : 1;
-    for (int k = 0; k < nf; ++k) fft_stockham<NT>(buf, logM, tw, k == 0 ? bh : nullptr, bh != nullptr && k == 0);
-}
-
 // The transforms of one map: [fold or load] -> one (MODE 0, 1) or two
 // (MODE 2, with the N^-1 weighting between) transform directions -> [write
 // map or unfold].  A direction is one FFT (power-of-two rings) or, for
@@ -461,31 +645,20 @@ __device__ __forceinline__ void transform_dir(C *buf, const int logM, const TwTa
 // The work of one CTA: ring pair a.pairs[pidx], maps [y mpg, (y + 1) mpg).
 // Called by the plan's kernel (the block indices) and by the grouped kernel
 // (one work item of a list that spans several geometries).
-template <typename T, int MODE, int NT, int FIX>
+template <typename T, int MODE, int FIX>
 __device__ __forceinline__ void ring_cta(const RingArgs<T> &a, const int pidx, const int y) {
     typedef typename VT<T>::C C;
     extern __shared__ __align__(16) unsigned char s_raw[];
-    // FIX > 0: every ring of the launch has M = 2^FIX and the fixed-length
-    // passes run (twiddles from twf, no shared twiddle table)
+    // FIX > 0: every ring of the launch has M = 2^FIX
     constexpr bool fixed = FIX > 0;
-    // FP32 fixed-length launches stage their pass twiddles in shared memory
-    // (at most 1092 entries); FP64 ones read them through L1 (the FP64
-    // 8192-point buffer and chirp leave no room)
-    constexpr bool twf_smem = fixed && sizeof(T) == 4;
-    const int ntw = fixed ? (twf_smem ? twf_len(FIX > 0 ? FIX : 8) : 0) : a.tw_nlo + a.tw_nhi;
+    constexpr int KIND = RingCore<T, MODE, FIX>::kind, NT = RingCore<T, MODE, FIX>::nt;
+    // FP32 launches stage their twiddles in shared memory, FP64 ones read them
+    // through L1 (the FP64 8192-point buffer and chirp leave no room)
+    constexpr bool tw_smem = sizeof(T) == 4;
     C *s_tw = reinterpret_cast<C *>(s_raw);
-    C *buf = s_tw + ntw;
+    C *buf = s_tw + a.tw_len;
     C *s_chirp = buf + a.buf_len;          // this ring's chirp (Bluestein rings)
     C *scr_p = s_chirp + a.chirp_len;      // aliased fold: partial sums [north | south][NT] (generic launches)
-    const C *tw_src = fixed ? a.twf : a.tw;
-    for (int i = threadIdx.x; i < ntw; i += NT) s_tw[i] = tw_src[i];
-    const C *twf = twf_smem ? s_tw : a.twf;
-    TwTab<C> tw;
-    tw.lo = s_tw;
-    tw.hi = s_tw + a.tw_nlo;
-    tw.blo = a.tw_blo;
-    tw.logmax = a.logmax;
-    // (the first FFT pass starts after a barrier that follows the fill below)
 
     const int pr = a.pairs[pidx];
     const int rn = pr, rs = a.nring - 1 - pr;
@@ -493,6 +666,17 @@ __device__ __forceinline__ void ring_cta(const RingArgs<T> &a, const int pidx, c
     const RingFFT f = a.rf[rn];
     const int n = f.n, logM = f.logM, M = 1 << logM;
     const int L = a.lmax;
+    const C *tw = KIND == RING_R48 ? a.tw + a.tw_off[logM] : a.tw;
+    if (tw_smem) {
+        const int ntw = KIND == RING_R48 ? ring_tw_len<T>(logM) : a.tw_len;
+        for (int i = threadIdx.x; i < ntw; i += NT) s_tw[i] = tw[i];
+        tw = s_tw;
+    }
+    TwTab<C> tw2;   // RING_R16_ANY
+    tw2.lo = s_tw;
+    tw2.hi = s_tw + a.tw_nlo;
+    tw2.blo = a.tw_blo;
+    tw2.logmax = a.logmax;
     // the chirp is read up to five times per element and map: stage it once
     const C *chirp = a.chirp + f.chirp_off;
     if (f.blue) {
@@ -653,11 +837,7 @@ __device__ __forceinline__ void ring_cta(const RingArgs<T> &a, const int pidx, c
             // MODE 2, forward (e^{-2 pi i jk/n}) otherwise
             const bool fwd = MODE == 1 || dir == 1;
             const C *bh = f.blue ? (fwd ? a.bfwd : a.binv) + f.bhat_off : nullptr;
-            if constexpr (fixed) {
-                transform_dir_fixed<(fixed ? FIX : 8), NT>(buf, twf, bh);
-            } else {
-                transform_dir<NT>(buf, logM, tw, bh);
-            }
+            transform_dir<KIND, FIX, NT>(buf, a.tw_len, logM, tw, tw2, bh);
             if (MODE == 2 && dir == 0) {
                 // ---- N^-1 weighting (each thread rewrites the elements it reads)
                 const int comp = q < a.nT ? 0 : 1;
@@ -767,13 +947,14 @@ __device__ __forceinline__ void ring_cta(const RingArgs<T> &a, const int pidx, c
     }
 }
 
-template <typename T, int MODE, int NT, int FIX>
-__global__ void __launch_bounds__(NT, (RingBlocks<T, NT, FIX>::v)) k_ring(const RingArgs<T> a) {
-    ring_cta<T, MODE, NT, FIX>(a, blockIdx.x, blockIdx.y);
+template <typename T, int MODE, int FIX>
+__global__ void __launch_bounds__((RingCore<T, MODE, FIX>::nt), (RingCore<T, MODE, FIX>::sm_threads / RingCore<T, MODE, FIX>::nt))
+    k_ring(const RingArgs<T> a) {
+    ring_cta<T, MODE, FIX>(a, blockIdx.x, blockIdx.y);
 }
 
 // Grouped launch (chains of several geometries): one launch per
-// transform-length class (the template's NT and FIX) over the launch buckets
+// transform-length class (the template's FIX) over the launch buckets
 // of that class of every plan; entry e is one (plan, bucket) with its own
 // arguments, flat CTA i belongs to the entry with first[e] <= i <
 // first[e + 1] and runs ring pair i' % count[e], map group i' / count[e]
@@ -788,24 +969,20 @@ template <typename T> struct RingGroups {
     RingArgs<T> a[SHTG_RING_ENTRIES];
 };
 
-template <typename T, int MODE, int NT, int FIX>
-__global__ void __launch_bounds__(NT, (RingBlocks<T, NT, FIX>::v)) k_ring_grp(const __grid_constant__ RingGroups<T> G) {
+template <typename T, int MODE, int FIX>
+__global__ void __launch_bounds__((RingCore<T, MODE, FIX>::nt), (RingCore<T, MODE, FIX>::sm_threads / RingCore<T, MODE, FIX>::nt))
+    k_ring_grp(const __grid_constant__ RingGroups<T> G) {
     const int i = blockIdx.x;
     int e = 0;
     while (e + 1 < G.ne && i >= G.first[e + 1]) ++e;
     if (G.active[e] && *G.active[e] == 0) return;
     const int li = i - G.first[e];
-    ring_cta<T, MODE, NT, FIX>(G.a[e], li % G.count[e], li / G.count[e]);
+    ring_cta<T, MODE, FIX>(G.a[e], li % G.count[e], li / G.count[e]);
 }
-
-template <typename T> static const typename VT<T>::C *ring_twf(Plan *p);
-template <> const float2 *ring_twf<float>(Plan *p) { return p->d_twf32; }
-template <> const double2 *ring_twf<double>(Plan *p) { return p->d_twf64; }
 
 template <typename T> static RingArgs<T> ring_args(Plan *p);
 template <> RingArgs<float> ring_args<float>(Plan *p) {
     RingArgs<float> a{};
-    a.tw = p->d_tw32;
     a.chirp = p->d_chirp32;
     a.rph = p->d_rph32;
     a.bfwd = p->d_bfwd32;
@@ -814,7 +991,6 @@ template <> RingArgs<float> ring_args<float>(Plan *p) {
 }
 template <> RingArgs<double> ring_args<double>(Plan *p) {
     RingArgs<double> a{};
-    a.tw = p->d_tw64;
     a.chirp = p->d_chirp64;
     a.rph = p->d_rph64;
     a.bfwd = p->d_bfwd64;
@@ -822,29 +998,41 @@ template <> RingArgs<double> ring_args<double>(Plan *p) {
     return a;
 }
 
-template <typename T, int MODE, int NT, int FIX>
-static int launch_ring_nt(RingArgs<T> a, int ctas, size_t smem, cudaStream_t st) {
-    auto kern = k_ring<T, MODE, NT, FIX>;
-    if (smem > 48 * 1024) SHTG_CUDA(allow_max_smem(kern));
-    // The maps of a ring pair are split over grid.y when the pairs alone give
-    // fewer than four waves of resident CTAs (a CTA still handles at least
-    // two maps, so its chirp and twiddle staging stay amortized)
-    int dev = 0, nsm = 0, per = 0;
-    SHTG_CUDA(cudaGetDevice(&dev));
-    SHTG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    SHTG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, NT, smem));
-    const int want = 4 * nsm * (per > 0 ? per : 1);
-    int groups = (want + ctas - 1) / ctas;
-    groups = std::max(1, std::min(groups, (a.nmaps + 1) / 2));
-    a.mpg = (a.nmaps + groups - 1) / groups;
-    groups = (a.nmaps + a.mpg - 1) / a.mpg;
-    kern<<<dim3(ctas, groups), NT, smem, st>>>(a);
-    return SHTG_OK;
+template <typename T, typename C>
+static void ring_twiddles_t(int logmax, std::vector<C> &t, int *off) {
+    const double PI = 3.14159265358979323846;
+    constexpr int LR = RingRadix<T>::LR;
+    for (int lg = 0; lg <= logmax; ++lg) {
+        off[lg] = (int)t.size();
+        for (int ns = 1 << (lg % LR); ns < (1 << lg); ns <<= LR) {
+            if (ns == 1) continue;
+            for (int r = 1; r < (1 << LR); ++r) {
+                if (sizeof(T) == 4 && r != 1 && r != 4) continue;
+                for (int k = 0; k < ns; ++k) {
+                    const double ang = -2.0 * PI * (double)((int64_t)r * k) / ((double)(1 << LR) * ns);
+                    t.push_back(C{T(cos(ang)), T(sin(ang))});
+                }
+            }
+        }
+    }
+}
+void ring_twiddles(std::vector<double2> &t64, int *off64, std::vector<float2> &t32, int *off32) {
+    ring_twiddles_t<double>(SHTG_FFT_LOGMAX, t64, off64);
+    ring_twiddles_t<float>(10, t32, off32);
 }
 
-template <typename T, int MODE>
-static int launch_ring(Plan *p, RingArgs<T> a, cudaStream_t st) {
+template <typename T> static const typename VT<T>::C *ring_tab(Plan *p);
+template <> const float2 *ring_tab<float>(Plan *p) { return p->d_twr32; }
+template <> const double2 *ring_tab<double>(Plan *p) { return p->d_twr64; }
+
+// launch arguments and shared memory of one bucket of plan p.  Buckets above
+// 1024 hold rings of one transform length M = 2^FIX (FIX = g.fix: 2^logm, or
+// 2^(logm - 1) for aliased direct rings, whose buffer still holds 2^logm:
+// checked at plan creation).
+template <typename T, int MODE, int FIX>
+static void ring_bucket_args(Plan *p, const Plan::RingLaunch &g, RingArgs<T> &a, size_t &smem) {
     typedef typename VT<T>::C C;
+    typedef RingCore<T, MODE, FIX> Core;
     a.lmax = p->lmax;
     a.nring = p->nring;
     a.npairs = p->npairs;
@@ -855,7 +1043,53 @@ static int launch_ring(Plan *p, RingArgs<T> a, cudaStream_t st) {
     a.logmax = p->fft_logmax;
     a.tw_blo = p->tw_blo;
     a.tw_nlo = p->tw_nlo;
-    a.tw_nhi = p->tw_nhi;
+    const int M = 1 << g.logm;
+    a.buf_len = M + M / 16;
+    a.chirp_len = g.chirp;
+    a.tw_len = 0;
+    if constexpr (Core::kind == RING_R48) {
+        a.tw = ring_tab<T>(p);
+        for (int lg = 0; lg <= SHTG_FFT_LOGMAX; ++lg)
+            a.tw_off[lg] = sizeof(T) == 8 ? p->twr_off64[lg] : p->twr_off32[lg];
+        if (sizeof(T) == 4)   // room for the longest table of the launch
+            for (int lg = 0; lg <= 10; ++lg) a.tw_len = std::max(a.tw_len, ring_tw_len<T>(lg));
+    } else if constexpr (Core::kind == RING_R16) {
+        a.tw = p->d_twf32 + p->twf_off[FIX];
+        a.tw_len = twf_len(FIX);
+    } else {
+        a.tw = p->d_tw32;
+        a.tw_len = p->tw_nlo + p->tw_nhi;
+    }
+    // shared memory: twiddles, buffer, chirp, and the aliased fold's partial
+    // sums (FIX = 0 only: the other launches' rings have n > NT / 2, so they
+    // never split a residue's sum)
+    smem = sizeof(C) * ((size_t)a.tw_len + a.buf_len + a.chirp_len + ((g.alias && FIX == 0) ? 2 * Core::nt : 0));
+    a.pairs = p->d_ring_groups + g.off;
+}
+
+template <typename T, int MODE, int FIX>
+static int launch_ring_fix(Plan *p, const Plan::RingLaunch &g, RingArgs<T> a, cudaStream_t st) {
+    typedef RingCore<T, MODE, FIX> Core;
+    size_t smem = 0;
+    ring_bucket_args<T, MODE, FIX>(p, g, a, smem);
+    const int ctas = g.count;
+    auto kern = k_ring<T, MODE, FIX>;
+    if (smem > 48 * 1024) SHTG_CUDA(allow_max_smem(kern));
+    // The maps of a ring pair are split over grid.y when the pairs alone give
+    // fewer than four waves of resident CTAs (a CTA still handles at least
+    // two maps, so its chirp and twiddle staging stay amortized)
+    const int per = std::max(1, std::min(Core::sm_threads / Core::nt, smem ? (int)((227 * 1024) / (smem + 1024)) : 32));
+    const int want = 4 * p->nsm * per;
+    int groups = (want + ctas - 1) / ctas;
+    groups = std::max(1, std::min(groups, (a.nmaps + 1) / 2));
+    a.mpg = (a.nmaps + groups - 1) / groups;
+    groups = (a.nmaps + a.mpg - 1) / a.mpg;
+    kern<<<dim3(ctas, groups), Core::nt, smem, st>>>(a);
+    return SHTG_OK;
+}
+
+template <typename T, int MODE>
+static int launch_ring(Plan *p, RingArgs<T> a, cudaStream_t st) {
     // one launch per length bucket, each with the thread count and shared
     // memory of its longest transform.  The buckets touch disjoint ring
     // pairs, so all but the first run on the plan's side streams, forked from
@@ -874,30 +1108,13 @@ static int launch_ring(Plan *p, RingArgs<T> a, cudaStream_t st) {
             ls = p->ring_side[nside];
             SHTG_CUDA(cudaStreamWaitEvent(ls, p->ring_fork, 0));
         }
-        const int M = 1 << g.logm;
-        // launches of buckets above 1024 hold rings of one transform length
-        // M = 2^g.fix (2^logm, or 2^(logm - 1) for aliased direct rings, whose
-        // buffer still holds 2^logm: checked at plan creation) and run the
-        // fixed-length passes with M / 16 threads
-        const bool fix = g.fix > 0;
-        const int nt = fix ? (1 << g.fix) / 16 : ring_threads(g.logm);
-        a.buf_len = M + M / 16;
-        a.chirp_len = g.chirp;
-        a.twf = fix ? ring_twf<T>(p) + p->twf_off[g.fix] : nullptr;
-        // shared memory: twiddles (generic: two-level table; FP32 fixed: the
-        // pass tables), buffer, chirp, and the aliased fold's partial sums
-        // (generic launches only: a fixed launch's rings have n >= M / 2 >
-        // NT / 2, so they never split a residue's sum)
-        const size_t ntw = fix ? (sizeof(T) == 4 ? (size_t)twf_len(g.fix) : 0) : (size_t)p->tw_nlo + p->tw_nhi;
-        const size_t smem = sizeof(C) * (ntw + a.buf_len + a.chirp_len + ((g.alias && !fix) ? 2 * nt : 0));
-        a.pairs = p->d_ring_groups + g.off;
         int rc = SHTG_OK;
         switch (g.fix) {
-            case 10: rc = launch_ring_nt<T, MODE, 64, 10>(a, g.count, smem, ls); break;
-            case 11: rc = launch_ring_nt<T, MODE, 128, 11>(a, g.count, smem, ls); break;
-            case 12: rc = launch_ring_nt<T, MODE, 256, 12>(a, g.count, smem, ls); break;
-            case 13: rc = launch_ring_nt<T, MODE, 512, 13>(a, g.count, smem, ls); break;
-            default: rc = launch_ring_nt<T, MODE, 64, 0>(a, g.count, smem, ls); break;
+            case 10: rc = launch_ring_fix<T, MODE, 10>(p, g, a, ls); break;
+            case 11: rc = launch_ring_fix<T, MODE, 11>(p, g, a, ls); break;
+            case 12: rc = launch_ring_fix<T, MODE, 12>(p, g, a, ls); break;
+            case 13: rc = launch_ring_fix<T, MODE, 13>(p, g, a, ls); break;
+            default: rc = launch_ring_fix<T, MODE, 0>(p, g, a, ls); break;
         }
         if (rc != SHTG_OK) return rc;
         if (ls != st) {
@@ -912,37 +1129,60 @@ static int launch_ring(Plan *p, RingArgs<T> a, cudaStream_t st) {
     return SHTG_OK;
 }
 
-// launch arguments of one bucket of plan p (the fields launch_ring sets)
-template <typename T>
-static void ring_bucket_args(Plan *p, const Plan::RingLaunch &g, RingArgs<T> &a, size_t &smem) {
-    typedef typename VT<T>::C C;
-    a.lmax = p->lmax;
-    a.nring = p->nring;
-    a.npairs = p->npairs;
-    a.npix = p->npix;
-    a.rf = p->d_rfft;
-    a.ofs = p->d_ofs;
-    a.wring = p->d_wring;
-    a.logmax = p->fft_logmax;
-    a.tw_blo = p->tw_blo;
-    a.tw_nlo = p->tw_nlo;
-    a.tw_nhi = p->tw_nhi;
-    const int M = 1 << g.logm;
-    const bool fix = g.fix > 0;
-    const int nt = fix ? (1 << g.fix) / 16 : ring_threads(g.logm);
-    a.buf_len = M + M / 16;
-    a.chirp_len = g.chirp;
-    a.twf = fix ? ring_twf<T>(p) + p->twf_off[g.fix] : nullptr;
-    const size_t ntw = fix ? (sizeof(T) == 4 ? (size_t)twf_len(g.fix) : 0) : (size_t)p->tw_nlo + p->tw_nhi;
-    smem = sizeof(C) * (ntw + a.buf_len + a.chirp_len + ((g.alias && !fix) ? 2 * nt : 0));
-    a.pairs = p->d_ring_groups + g.off;
-}
-
-template <typename T, int MODE, int NT, int FIX>
-static int launch_ring_grp(RingGroups<T> &G, size_t smem, int64_t total, cudaStream_t st) {
-    auto kern = k_ring_grp<T, MODE, NT, FIX>;
+// the buckets of one transform-length class (FIX; 0: lengths up to 1024) of
+// every plan as one launch; nl counts the launches made
+template <typename T, int FIX>
+static int ring_grp_class(int ng, Plan *const *ps, typename VT<T>::C *const *FG, const int *nmaps, const int *nT,
+                          const T *const *ninv, const int *const *active, cudaStream_t st, int &nl) {
+    typedef RingCore<T, 2, FIX> Core;
+    RingGroups<T> G{};
+    size_t smem = 0;
+    int npair = 0;
+    for (int g = 0; g < ng; ++g)
+        for (const Plan::RingLaunch &b : ps[g]->ring_launch)
+            if (b.fix == FIX && b.count > 0) {
+                if (G.ne == SHTG_RING_ENTRIES) {
+                    set_error("grouped ring launch: more than " + std::to_string(SHTG_RING_ENTRIES) +
+                              " launch buckets of one length");
+                    return SHTG_ERR_ARG;
+                }
+                RingArgs<T> a = ring_args<T>(ps[g]);
+                size_t sm = 0;
+                ring_bucket_args<T, 2, FIX>(ps[g], b, a, sm);
+                a.FG = FG[g];
+                a.nmaps = nmaps[g];
+                a.nT = nT[g];
+                a.ninv = ninv[g];
+                smem = std::max(smem, sm);
+                G.a[G.ne] = a;
+                G.count[G.ne] = b.count;
+                G.active[G.ne] = active ? active[g] : nullptr;
+                G.ne += 1;
+                npair += b.count;
+            }
+    if (G.ne == 0) return SHTG_OK;
+    // maps per CTA as in the plan's launches: enough CTAs for about four
+    // waves, at least two maps per CTA
+    const int want = 4 * ps[0]->nsm * std::max(1, Core::sm_threads / Core::nt);
+    int64_t total = 0;
+    for (int e = 0; e < G.ne; ++e) {
+        RingArgs<T> &a = G.a[e];
+        int groups = (want + npair - 1) / npair;
+        groups = std::max(1, std::min(groups, (a.nmaps + 1) / 2));
+        a.mpg = (a.nmaps + groups - 1) / groups;
+        groups = (a.nmaps + a.mpg - 1) / a.mpg;
+        G.first[e] = (int)total;
+        total += (int64_t)G.count[e] * groups;
+        if (total > 0x7fffffff) {
+            set_error("grouped ring launch: too many CTAs");
+            return SHTG_ERR_ARG;
+        }
+    }
+    G.first[G.ne] = (int)total;
+    auto kern = k_ring_grp<T, 2, FIX>;
     if (smem > 48 * 1024) SHTG_CUDA(allow_max_smem(kern));
-    kern<<<(unsigned)total, NT, smem, st>>>(G);
+    kern<<<(unsigned)total, Core::nt, smem, st>>>(G);
+    ++nl;
     return SHTG_OK;
 }
 
@@ -954,70 +1194,13 @@ int ring_fused_grp(int ng, Plan *const *ps, typename VT<T>::C *const *FG, const 
         return SHTG_ERR_ARG;
     }
     Plan *acct = ps[0];
-    int dev = 0, nsm = 0;
-    SHTG_CUDA(cudaGetDevice(&dev));
-    SHTG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     prof_begin(acct, sizeof(T) == 8 ? K_RING64 : K_RING32, st);
     int nl = 0;
-    // classes by FIX (0: the generic passes of the buckets <= 1024, 64 threads)
-    for (int fix : {13, 12, 11, 10, 0}) {
-        RingGroups<T> G{};
-        size_t smem = 0;
-        int npair = 0;
-        for (int g = 0; g < ng; ++g)
-            for (const Plan::RingLaunch &b : ps[g]->ring_launch)
-                if (b.fix == fix && b.count > 0) {
-                    if (G.ne == SHTG_RING_ENTRIES) {
-                        set_error("grouped ring launch: more than " + std::to_string(SHTG_RING_ENTRIES) +
-                                  " launch buckets of one length");
-                        return SHTG_ERR_ARG;
-                    }
-                    RingArgs<T> a = ring_args<T>(ps[g]);
-                    size_t sm = 0;
-                    ring_bucket_args<T>(ps[g], b, a, sm);
-                    a.FG = FG[g];
-                    a.nmaps = nmaps[g];
-                    a.nT = nT[g];
-                    a.ninv = ninv[g];
-                    smem = std::max(smem, sm);
-                    G.a[G.ne] = a;
-                    G.count[G.ne] = b.count;
-                    G.active[G.ne] = active ? active[g] : nullptr;
-                    G.ne += 1;
-                    npair += b.count;
-                }
-        if (G.ne == 0) continue;
-        // maps per CTA as in the plan's launches: enough CTAs for about four
-        // waves, at least two maps per CTA
-        const int nt = fix ? (1 << fix) / 16 : 64;
-        const int per = std::max(1, (sizeof(T) == 4 ? (fix > 0 ? 1024 : 512) : 256) / nt);
-        const int want = 4 * nsm * per;
-        int64_t total = 0;
-        for (int e = 0; e < G.ne; ++e) {
-            RingArgs<T> &a = G.a[e];
-            int groups = (want + npair - 1) / npair;
-            groups = std::max(1, std::min(groups, (a.nmaps + 1) / 2));
-            a.mpg = (a.nmaps + groups - 1) / groups;
-            groups = (a.nmaps + a.mpg - 1) / a.mpg;
-            G.first[e] = (int)total;
-            total += (int64_t)G.count[e] * groups;
-            if (total > 0x7fffffff) {
-                set_error("grouped ring launch: too many CTAs");
-                return SHTG_ERR_ARG;
-            }
-        }
-        G.first[G.ne] = (int)total;
-        int rc = SHTG_OK;
-        switch (fix) {
-            case 10: rc = launch_ring_grp<T, 2, 64, 10>(G, smem, total, st); break;
-            case 11: rc = launch_ring_grp<T, 2, 128, 11>(G, smem, total, st); break;
-            case 12: rc = launch_ring_grp<T, 2, 256, 12>(G, smem, total, st); break;
-            case 13: rc = launch_ring_grp<T, 2, 512, 13>(G, smem, total, st); break;
-            default: rc = launch_ring_grp<T, 2, 64, 0>(G, smem, total, st); break;
-        }
-        if (rc != SHTG_OK) return rc;
-        ++nl;
-    }
+    SHTG_TRY((ring_grp_class<T, 13>(ng, ps, FG, nmaps, nT, ninv, active, st, nl)));
+    SHTG_TRY((ring_grp_class<T, 12>(ng, ps, FG, nmaps, nT, ninv, active, st, nl)));
+    SHTG_TRY((ring_grp_class<T, 11>(ng, ps, FG, nmaps, nT, ninv, active, st, nl)));
+    SHTG_TRY((ring_grp_class<T, 10>(ng, ps, FG, nmaps, nT, ninv, active, st, nl)));
+    SHTG_TRY((ring_grp_class<T, 0>(ng, ps, FG, nmaps, nT, ninv, active, st, nl)));
     prof_end(acct, st, nl);
     SHTG_CHECK_LAUNCH("k_ring_grp");
     return SHTG_OK;
