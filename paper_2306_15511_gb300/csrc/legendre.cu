@@ -49,17 +49,14 @@ template <> LegArgs<double> leg_make_args<double>(Plan *p) {
 template <>
 int leg_synth<float>(Plan *p, int spin, const float2 *alm, int rs, int nmaps, const float *beam,
                      float2 *F, cudaStream_t st) {
-    const Variants32 &V = variants32();
-    const int s = spin == 2 ? 1 : 0;
-    return tune(p, 1, s, nmaps, V.n[s], st, [&](int v) { return V.syn[s][v](p, alm, rs, nmaps, beam, F, st); });
+    return tune(p, 1, spin == 2 ? 1 : 0, nmaps, leg_synth32_count(spin, nmaps), st,
+                [&](int v) { return leg_synth32_shape(p, spin, v, alm, rs, nmaps, beam, F, st); });
 }
 template <>
 int leg_analysis<float>(Plan *p, int spin, const float2 *G, int nmaps, const float *beam, float2 *alm,
                         int rs, cudaStream_t st, int vjp) {
-    const Variants32 &V = variants32();
-    const int s = spin == 2 ? 1 : 0;
-    return tune(p, 1, 2 + s, nmaps, V.n[2 + s], st,
-                [&](int v) { return V.ana[s][v](p, G, nmaps, beam, alm, rs, st, vjp); });
+    return tune(p, 1, spin == 2 ? 3 : 2, nmaps, leg_analysis32_count(spin, nmaps), st,
+                [&](int v) { return leg_analysis32_shape(p, spin, v, G, nmaps, beam, alm, rs, st, vjp); });
 }
 template <>
 int leg_analysis<double>(Plan *p, int spin, const double2 *G, int nmaps, const double *beam,

@@ -163,6 +163,10 @@ struct PairState {
 };
 
 // Load the per-pair geometry and start states; returns the warp's l range.
+// A warp's 32 NR pairs are consecutive: their starts lie close together, so
+// the loop over l begins late for a polar warp and few of its steps inject a
+// start (with the pairs of a thread 128 apart, every warp spanned all
+// latitudes and injected over most of its l range).
 template <typename T, int NR, int SPIN>
 __device__ __forceinline__ void load_pairs(const LegArgs<T> &a, int bx, int m, PairState<T, NR> &S,
                                            int &warp_lo, int &warp_hi) {
@@ -170,7 +174,7 @@ __device__ __forceinline__ void load_pairs(const LegArgs<T> &a, int bx, int m, P
     int lo = L + 1, hi = -1;
 #pragma unroll
     for (int j = 0; j < NR; ++j) {
-        const int pr = bx * (LEG_THREADS * NR) + j * LEG_THREADS + threadIdx.x;
+        const int pr = bx * (LEG_THREADS * NR) + (threadIdx.x & ~31) * NR + j * 32 + (threadIdx.x & 31);
         S.pr[j] = pr;
         S.a1[j] = S.a2[j] = S.b1[j] = S.b2[j] = T(0);
         S.u[j] = T(1);
@@ -753,24 +757,13 @@ int launch_analysis_v(Plan *p, const typename VT<T>::C *G, int nmaps, const T *b
     return SHTG_OK;
 }
 
-// variant tables (one per precision translation unit)
-typedef int (*SynthFn32)(Plan *, const float2 *, int, int, const float *, float2 *, cudaStream_t);
-typedef int (*SynthFn64)(Plan *, const double2 *, int, int, const double *, double2 *, cudaStream_t);
-typedef int (*AnaFn32)(Plan *, const float2 *, int, const float *, float2 *, int, cudaStream_t, int);
-typedef int (*AnaFn64)(Plan *, const double2 *, int, const double *, double2 *, int, cudaStream_t, int);
-struct Variants32 {
-    int n[4];                // synth0, synth2, ana0, ana2
-    SynthFn32 syn[2][8];
-    AnaFn32 ana[2][8];
-    int shape[4][8][2];      // (NR, NM) per variant, for reporting
-};
-struct Variants64 {
-    int n[4];
-    SynthFn64 syn[2][8];
-    AnaFn64 ana[2][8];
-    int shape[4][8][2];
-};
-const Variants32 &variants32();
-const Variants64 &variants64();
+// FP32 shapes (legendre32.cu): the number of candidates for this many maps,
+// and the launch of candidate v
+int leg_synth32_count(int spin, int nmaps);
+int leg_synth32_shape(Plan *p, int spin, int v, const float2 *alm, int rs, int nmaps, const float *beam, float2 *F,
+                      cudaStream_t st);
+int leg_analysis32_count(int spin, int nmaps);
+int leg_analysis32_shape(Plan *p, int spin, int v, const float2 *G, int nmaps, const float *beam, float2 *alm, int rs,
+                         cudaStream_t st, int vjp);
 
 }  // namespace shtg
