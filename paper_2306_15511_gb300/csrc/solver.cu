@@ -15,6 +15,7 @@
 //
 // Inner products use <a, c> = sum_l [a_l0 c_l0 + 2 Re sum_{m>0} conj(a_lm) c_lm],
 // the metric in which Y^T is the transpose of Y and A is symmetric.
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -292,10 +293,23 @@ __global__ void k_row_sums(const double *__restrict__ part, int nb, double *__re
     }
 }
 
+// sum of the RB partials of realization b, by one whole warp in a fixed order
+// (every lane gets it).  One thread adding them in sequence took 8 us a slot,
+// a quarter of a small solve's iteration.
 __device__ __forceinline__ double sum_part(const double *part, int b, int nslot, int slot) {
+    const double *v = part + ((int64_t)b * nslot + slot) * RB;
     double s = 0.0;
-    for (int k = 0; k < RB; ++k) s += part[((int64_t)b * nslot + slot) * RB + k];
+#pragma unroll
+    for (int k = 0; k < RB / 32; ++k) s += v[k * 32 + (threadIdx.x & 31)];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
+}
+
+// alpha = <r, z> / <p, A p> of an active realization; 0 for a converged one or
+// where the curvature is not positive (scal_beta_one then records that)
+__device__ __forceinline__ double pcg_alpha(const double *s, const double pq) {
+    return (s[S_ACTIVE] != 0.0 && pq > 0.0 && isfinite(pq)) ? s[S_RZ] / pq : 0.0;
 }
 
 // apply the preconditioner inverse block to (r_T, r_E, r_B) at alm index i
@@ -318,23 +332,34 @@ __device__ __forceinline__ void apply_minv(const T *minv, int64_t nalm, int64_t 
 }
 
 // INIT: z = M^-1 r and partial (rz, rr).  Otherwise x += alpha p, r -= alpha q,
-// then the same.
-template <typename T, bool INIT>
+// then the same, with alpha formed by every block from the <p, A p> partials
+// (pqp), which no launch of its own has to sum.
+template <typename T, bool INIT, int NC>
 __device__ __forceinline__ void update_rows(typename HT<T>::C *__restrict__ x, typename HT<T>::C *__restrict__ r,
                                             typename HT<T>::C *__restrict__ z,
                                             const typename HT<T>::C *__restrict__ p,
                                             const typename HT<T>::C *__restrict__ q, const T *__restrict__ minv,
-                                            int nc, int64_t nalm, const int *__restrict__ mof,
-                                            const double *__restrict__ scal, double *__restrict__ part,
-                                            const int b, const int bx, const int nbx) {
+                                            int64_t nalm, const int *__restrict__ mof,
+                                            const double *__restrict__ scal, const double *__restrict__ pqp,
+                                            double *__restrict__ part, const int b, const int bx, const int nbx) {
     typedef typename HT<T>::C C;
     __shared__ double sm[RT / 32];
-    const int64_t off = (int64_t)b * nc * nalm;
-    const T alpha = INIT ? T(0) : (T)scal[b * 16 + S_ALPHA];
+    const int64_t off = (int64_t)b * NC * nalm;
+    T alpha = T(0);
+    if (!INIT) {
+        if (threadIdx.x < 32) {
+            const double pq = sum_part(pqp, b, 1, 0);
+            if (threadIdx.x == 0) sm[0] = pcg_alpha(scal + b * 16, pq);
+        }
+        __syncthreads();
+        alpha = (T)sm[0];
+        __syncthreads();
+    }
     double srz = 0.0, srr = 0.0;
     for (int64_t i = bx * (int64_t)blockDim.x + threadIdx.x; i < nalm; i += (int64_t)nbx * blockDim.x) {
         C rv[3], zv[3];
-        for (int k = 0; k < nc; ++k) {
+        #pragma unroll
+        for (int k = 0; k < NC; ++k) {
             const int64_t e = off + k * nalm + i;
             C rr = r[e];
             if (!INIT) {
@@ -349,10 +374,11 @@ __device__ __forceinline__ void update_rows(typename HT<T>::C *__restrict__ x, t
             }
             rv[k] = rr;
         }
-        apply_minv<T, C>(minv + (int64_t)b * 4 * nalm, nalm, i, nc, rv, zv);
+        apply_minv<T, C>(minv + (int64_t)b * 4 * nalm, nalm, i, NC, rv, zv);
         const double w = mof[i] ? 2.0 : 1.0;
         typename DotAcc<C>::t a1 = 0, a2 = 0;
-        for (int k = 0; k < nc; ++k) {
+        #pragma unroll
+        for (int k = 0; k < NC; ++k) {
             z[off + k * nalm + i] = zv[k];
             a1 = DotAcc<C>::add(a1, rv[k], zv[k]);
             a2 = DotAcc<C>::add(a2, rv[k], rv[k]);
@@ -372,16 +398,23 @@ __global__ void k_update(typename HT<T>::C *__restrict__ x, typename HT<T>::C *_
                          typename HT<T>::C *__restrict__ z, const typename HT<T>::C *__restrict__ p,
                          const typename HT<T>::C *__restrict__ q, const T *__restrict__ minv,
                          int nc, int64_t nalm, const int *__restrict__ mof,
-                         const double *__restrict__ scal, double *__restrict__ part) {
-    update_rows<T, INIT>(x, r, z, p, q, minv, nc, nalm, mof, scal, part, blockIdx.y, blockIdx.x, gridDim.x);
+                         const double *__restrict__ scal, const double *__restrict__ pqp, double *__restrict__ part) {
+    if (nc == 1)
+        update_rows<T, INIT, 1>(x, r, z, p, q, minv, nalm, mof, scal, pqp, part, blockIdx.y, blockIdx.x, gridDim.x);
+    else
+        update_rows<T, INIT, 3>(x, r, z, p, q, minv, nalm, mof, scal, pqp, part, blockIdx.y, blockIdx.x, gridDim.x);
 }
 
-// The scalar kernels run one block; thread t serves realizations t, t +
-// blockDim.x, ... (a plan holds up to 4096).
+// The scalar kernels run one warp per realization, SCAL_T threads a block.
+#define SCAL_T 256
+static dim3 scal_grid(int nb) { return dim3((unsigned)((nb + SCAL_T / 32 - 1) / (SCAL_T / 32))); }
+__device__ __forceinline__ int scal_row() { return blockIdx.x * (SCAL_T / 32) + (threadIdx.x >> 5); }
 __global__ void k_scal_init(const double *__restrict__ part, double *__restrict__ scal, int nb,
                             double tol2) {
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-        const double rz = sum_part(part, b, 2, 0), rr = sum_part(part, b, 2, 1);
+    const int b = scal_row();
+    if (b >= nb) return;
+    const double rz = sum_part(part, b, 2, 0), rr = sum_part(part, b, 2, 1);
+    if ((threadIdx.x & 31) == 0) {
         double *s = scal + b * 16;
         s[S_RZ] = rz;
         s[S_RR] = rr;
@@ -400,31 +433,19 @@ __global__ void k_scal_init(const double *__restrict__ part, double *__restrict_
 // preconditioner close to the exact inverse) ends the stage instead of
 // failing it, and the FP64 residual replacement judges convergence.  The
 // FP64 PCG passes 0 (any non-positive curvature is a failure).
-__device__ __forceinline__ void scal_alpha_one(const double *__restrict__ part, double *__restrict__ scal,
-                                               const int b, const double floor2) {
-    double *s = scal + b * 16;
-    const double pq = sum_part(part, b, 1, 0);
-    s[S_PQ] = pq;
-    double alpha = 0.0;
-    if (s[S_ACTIVE] != 0.0) {
-        if (pq > 0.0 && isfinite(pq)) {
-            alpha = s[S_RZ] / pq;
-        } else {
-            s[S_ACTIVE] = 0.0;
-            if (isfinite(pq) && s[S_RR] <= floor2 * s[S_BB]) s[S_RESTART] = 1.0;   // next stage: p = z
-            else s[S_BAD] = 1.0;
-        }
-    }
-    s[S_ALPHA] = alpha;
-}
-__global__ void k_scal_alpha(const double *__restrict__ part, double *__restrict__ scal, int nb, double floor2) {
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) scal_alpha_one(part, scal, b, floor2);
-}
-
-__device__ __forceinline__ void scal_beta_one(const double *__restrict__ part, double *__restrict__ scal,
-                                              const int b) {
-    double *s = scal + b * 16;
+__device__ __forceinline__ void scal_beta_one(const double *__restrict__ pqp, const double *__restrict__ part,
+                                              double *__restrict__ scal, const int b, const double floor2) {
+    const double pq = sum_part(pqp, b, 1, 0);
     const double rz = sum_part(part, b, 2, 0), rr = sum_part(part, b, 2, 1);
+    if ((threadIdx.x & 31) != 0) return;
+    double *s = scal + b * 16;
+    s[S_PQ] = pq;
+    s[S_ALPHA] = pcg_alpha(s, pq);
+    if (s[S_ACTIVE] != 0.0 && !(pq > 0.0 && isfinite(pq))) {
+        s[S_ACTIVE] = 0.0;
+        if (isfinite(pq) && s[S_RR] <= floor2 * s[S_BB]) s[S_RESTART] = 1.0;   // next stage: p = z
+        else s[S_BAD] = 1.0;
+    }
     double beta = 0.0;
     if (s[S_ACTIVE] != 0.0) {
         s[S_ITERS] += 1.0;
@@ -440,8 +461,10 @@ __device__ __forceinline__ void scal_beta_one(const double *__restrict__ part, d
     }
     s[S_BETA] = beta;
 }
-__global__ void k_scal_beta(const double *__restrict__ part, double *__restrict__ scal, int nb) {
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) scal_beta_one(part, scal, b);
+__global__ void k_scal_beta(const double *__restrict__ pqp, const double *__restrict__ part,
+                            double *__restrict__ scal, int nb, double floor2) {
+    const int b = scal_row();
+    if (b < nb) scal_beta_one(pqp, part, scal, b, floor2);
 }
 
 template <typename C>
@@ -474,7 +497,7 @@ struct VecGrp {
     float2 *x, *r, *z, *p, *q;
     const float *minv, *sinv, *isc;
     const int *lof, *mof;
-    double *scal, *part;
+    double *scal, *part, *pqp;
     const int *active;   // device flag: 0 = the group is skipped
     int64_t nalm;
     int nc, nb, lmax1;
@@ -495,25 +518,25 @@ __global__ void k_prior_add_grp(const __grid_constant__ VecGroups G) {
     const int g = vgroup(G, blockIdx.y);
     const VecGrp &v = G.v[g];
     if (*v.active == 0) return;
-    prior_add_rows<float, true>(v.p, v.q, v.nc, v.nalm, v.lmax1, v.lof, v.sinv, v.isc, v.mof, v.part,
+    prior_add_rows<float, true>(v.p, v.q, v.nc, v.nalm, v.lmax1, v.lof, v.sinv, v.isc, v.mof, v.pqp,
                                 blockIdx.y - G.firstb[g], blockIdx.x, gridDim.x);
-}
-__global__ void k_scal_alpha_grp(const __grid_constant__ VecGroups G, double floor2) {
-    const VecGrp &v = G.v[blockIdx.x];
-    if (*v.active == 0) return;
-    for (int b = threadIdx.x; b < v.nb; b += blockDim.x) scal_alpha_one(v.part, v.scal, b, floor2);
 }
 __global__ void k_update_grp(const __grid_constant__ VecGroups G) {
     const int g = vgroup(G, blockIdx.y);
     const VecGrp &v = G.v[g];
     if (*v.active == 0) return;
-    update_rows<float, false>(v.x, v.r, v.z, v.p, v.q, v.minv, v.nc, v.nalm, v.mof, v.scal, v.part,
-                              blockIdx.y - G.firstb[g], blockIdx.x, gridDim.x);
+    if (v.nc == 1)
+        update_rows<float, false, 1>(v.x, v.r, v.z, v.p, v.q, v.minv, v.nalm, v.mof, v.scal, v.pqp, v.part,
+                                     blockIdx.y - G.firstb[g], blockIdx.x, gridDim.x);
+    else
+        update_rows<float, false, 3>(v.x, v.r, v.z, v.p, v.q, v.minv, v.nalm, v.mof, v.scal, v.pqp, v.part,
+                                     blockIdx.y - G.firstb[g], blockIdx.x, gridDim.x);
 }
-__global__ void k_scal_beta_grp(const __grid_constant__ VecGroups G) {
-    const VecGrp &v = G.v[blockIdx.x];
+__global__ void k_scal_beta_grp(const __grid_constant__ VecGroups G, double floor2) {
+    const VecGrp &v = G.v[blockIdx.y];
     if (*v.active == 0) return;
-    for (int b = threadIdx.x; b < v.nb; b += blockDim.x) scal_beta_one(v.part, v.scal, b);
+    const int b = scal_row();
+    if (b < v.nb) scal_beta_one(v.pqp, v.part, v.scal, b, floor2);
 }
 __global__ void k_pupdate_grp(const __grid_constant__ VecGroups G) {
     const int g = vgroup(G, blockIdx.y);
@@ -573,9 +596,11 @@ __global__ void k_scale_vec(float2 *__restrict__ v, int64_t per, const double *_
 // after a residual replacement: new rz, rr from the partials; tol2 per realization
 __global__ void k_scal_reliable(const double *__restrict__ part, double *__restrict__ scal, int nb,
                                 const double *__restrict__ tol2) {
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+    const int b = scal_row();
+    if (b >= nb) return;
+    const double rz = sum_part(part, b, 2, 0), rr = sum_part(part, b, 2, 1);
+    if ((threadIdx.x & 31) == 0) {
         double *s = scal + b * 16;
-        const double rz = sum_part(part, b, 2, 0), rr = sum_part(part, b, 2, 1);
         s[S_RZ] = rz;
         s[S_RR] = rr;
         s[S_BB] = 1.0;                       // the FP32 residual is normalized to 1
@@ -601,19 +626,28 @@ __global__ void k_restart_dir(float2 *__restrict__ p, const float2 *__restrict__
 }
 
 // ------------------------------------------------------------ log-posterior
-// per-l sums of the prior term: lsum[l] += w_m |a_lm|^2 / C_l (active l)
-__global__ void k_prior_lsum(const float2 *__restrict__ a, int64_t nalm, const int *__restrict__ lof,
-                             const int *__restrict__ mof, const float *__restrict__ icl,
+// per-l sums of the prior term: lsum[l] += sum_m w_m |a_lm|^2 / C_l (active
+// l).  Thread = one l (consecutive threads read consecutive alm of one m),
+// block row = PL_M orders m; one atomic addition per thread (an atomic per
+// coefficient on l_max + 1 addresses took 20 us at l_max 1024).
+#define PL_M 64
+__global__ void k_prior_lsum(const float2 *__restrict__ a, int lmax, const float *__restrict__ icl,
                              double *__restrict__ lsum) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nalm;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int l = lof[i];
-        const float c = icl[l];
-        if (c == 0.f) continue;
-        const double w = mof[i] ? 2.0 : 1.0;
-        const float2 v = a[i];
-        atomicAdd(&lsum[l], w * ((double)v.x * v.x + (double)v.y * v.y) * (double)c);
+    const int l = blockIdx.x * blockDim.x + threadIdx.x;
+    const int m0 = blockIdx.y * PL_M;
+    if (l > lmax || m0 > l) return;
+    const double c = (double)icl[l];
+    if (c == 0.0) return;
+    double s = 0.0;
+    const int m1 = min(m0 + PL_M - 1, l);
+#pragma unroll 4
+    for (int m = m0; m <= m1; ++m) {
+        const float2 v = a[(int64_t)m * (2 * lmax + 1 - m) / 2 + l];
+        const double x = (double)v.x, y = (double)v.y;
+        const double q = fma(x, x, y * y);
+        s += m ? 2.0 * q : q;
     }
+    atomicAdd(&lsum[l], s * c);
 }
 // res = d - m (in place in m); chi2 partial = sum ninv res^2; m <- ninv res
 __global__ void k_resid_pix(const float *__restrict__ d, const float *__restrict__ ninv,
@@ -804,6 +838,9 @@ struct IterGraph {
     ~IterGraph() { release(); }
 };
 
+// the <p, A p> partials, behind the two slots of the update kernel's (<r, z>, <r, r>)
+static double *pq_part(Plan *p) { return p->d_part + 2 * (int64_t)p->max_batch * SHTG_RED_BLOCKS; }
+
 struct Solve {
     Plan *p;
     cudaStream_t st;
@@ -889,7 +926,7 @@ static int matvec(Solve &s, const typename HT<T>::C *x, typename HT<T>::C *y, bo
     prof_begin(p, K_VEC, s.st);
     if (dot)   // y's final values and <x, y> partials (slot 0) in one pass
         k_prior_add<T, true><<<s.rgrid, RT, 0, s.st>>>(x, y, s.nc, s.nalm, p->lmax + 1, p->d_lofidx,
-                                                       Vec<T>::sinv(p), Vec<T>::isc(p), p->d_mofidx, p->d_part);
+                                                       Vec<T>::sinv(p), Vec<T>::isc(p), p->d_mofidx, pq_part(p));
     else
         k_prior_add<T, false><<<dim3(grid_1d(s.nalm).x, s.nb), RT, 0, s.st>>>(
             x, y, s.nc, s.nalm, p->lmax + 1, p->d_lofidx, Vec<T>::sinv(p), Vec<T>::isc(p), nullptr, nullptr);
@@ -919,14 +956,14 @@ static int pcg_iteration(Solve &s, typename HT<T>::C *x, typename HT<T>::C *r, t
     Plan *p = s.p;
     SHTG_TRY(matvec<T>(s, pv, q, true));   // q = A p and the partials of <p, q>
     prof_begin(p, K_VEC, s.st);
-    // FP32 recursion: below 1e-3 of the stage's start a breakdown ends the stage
-    k_scal_alpha<<<1, 1024, 0, s.st>>>(p->d_part, p->d_scal, s.nb, sizeof(T) == 4 ? 1e-6 : 0.0);
     k_update<T, false><<<s.rgrid, RT, 0, s.st>>>(x, r, z, pv, q, minv, s.nc, s.nalm, p->d_mofidx,
-                                                 p->d_scal, p->d_part);
+                                                 p->d_scal, pq_part(p), p->d_part);
     SHTG_TRY(precond_fix<T>(s, r, z));
-    k_scal_beta<<<1, 1024, 0, s.st>>>(p->d_part, p->d_scal, s.nb);
+    // FP32 recursion: below 1e-3 of the stage's start a breakdown ends the stage
+    k_scal_beta<<<scal_grid(s.nb), SCAL_T, 0, s.st>>>(pq_part(p), p->d_part, p->d_scal, s.nb,
+                                                      sizeof(T) == 4 ? 1e-6 : 0.0);
     k_pupdate<C><<<dim3(grid_1d(s.per).x, s.nb), RT, 0, s.st>>>(pv, z, s.nc, s.nalm, p->d_scal);
-    prof_end(p, s.st, 4);
+    prof_end(p, s.st, 3);
     SHTG_CHECK_LAUNCH("pcg iteration");
     return SHTG_OK;
 }
@@ -989,10 +1026,10 @@ static int pcg(Solve &s, const typename HT<T>::C *b, typename HT<T>::C *x, doubl
     SHTG_CUDA(cudaMemsetAsync(x, 0, vb, s.st));
     SHTG_CUDA(cudaMemcpyAsync(r, b, vb, cudaMemcpyDeviceToDevice, s.st));
     k_update<T, true><<<s.rgrid, RT, 0, s.st>>>(nullptr, r, z, nullptr, nullptr, minv, s.nc, s.nalm,
-                                                p->d_mofidx, p->d_scal, p->d_part);
+                                                p->d_mofidx, p->d_scal, nullptr, p->d_part);
     SHTG_CHECK_LAUNCH("k_update init");
     SHTG_TRY(precond_fix<T>(s, r, z));
-    k_scal_init<<<1, 1024, 0, s.st>>>(p->d_part, p->d_scal, s.nb, tol * tol);
+    k_scal_init<<<scal_grid(s.nb), SCAL_T, 0, s.st>>>(p->d_part, p->d_scal, s.nb, tol * tol);
     p->prof.launches += 2;
     SHTG_CHECK_LAUNCH("k_scal_init");
     SHTG_CUDA(cudaMemcpyAsync(pv, z, vb, cudaMemcpyDeviceToDevice, s.st));
@@ -1268,10 +1305,10 @@ static int mixed_solve(Solve &s, const shtg_cg_opts &opt, const std::vector<doub
         if (first) SHTG_CUDA(cudaMemsetAsync(x32, 0, vb32, st));
         else k_scale_vec<<<s.vgrid, RT, 0, st>>>(p32, s.per, d_sc + 2 * nb);
         k_update<float, true><<<s.rgrid, RT, 0, st>>>(nullptr, r32, z32, nullptr, nullptr, minv, s.nc,
-                                                     s.nalm, p->d_mofidx, p->d_scal, p->d_part);
+                                                     s.nalm, p->d_mofidx, p->d_scal, nullptr, p->d_part);
         SHTG_TRY(precond_fix<float>(s, r32, z32));
         if (!first) k_restart_dir<<<s.vgrid, RT, 0, st>>>(p32, z32, s.per, p->d_scal);
-        k_scal_reliable<<<1, 1024, 0, st>>>(p->d_part, p->d_scal, nb, d_sc + nb);
+        k_scal_reliable<<<scal_grid(nb), SCAL_T, 0, st>>>(p->d_part, p->d_scal, nb, d_sc + nb);
         p->prof.launches += first ? 3 : 5;
         SHTG_CHECK_LAUNCH("reliable update");
         // the search direction is kept (rescaled to the new normalization); only
@@ -1358,7 +1395,7 @@ int precond_apply(Plan *p, const shtg_problem *pr, const shtg_cg_opts *o, const 
         const int64_t n2 = 2 * s.nvec;
         k_to_float<<<grid_1d(n2), RT, 0, st>>>(reinterpret_cast<const double *>(R), reinterpret_cast<float *>(r32), n2);
         k_update<float, true><<<s.rgrid, RT, 0, st>>>(nullptr, r32, z32, nullptr, nullptr, p->d_minv32, s.nc, s.nalm,
-                                                      p->d_mofidx, p->d_scal, p->d_part);
+                                                      p->d_mofidx, p->d_scal, nullptr, p->d_part);
         p->prof.launches += 2;
         SHTG_CHECK_LAUNCH("k_update");
         SHTG_TRY(precond_fix<float>(s, r32, z32));
@@ -1369,7 +1406,7 @@ int precond_apply(Plan *p, const shtg_problem *pr, const shtg_cg_opts *o, const 
         return SHTG_OK;
     }
     k_update<double, true><<<s.rgrid, RT, 0, st>>>(nullptr, R, Z, nullptr, nullptr, p->d_minv64, s.nc, s.nalm,
-                                                   p->d_mofidx, p->d_scal, p->d_part);
+                                                   p->d_mofidx, p->d_scal, nullptr, p->d_part);
     SHTG_CHECK_LAUNCH("k_update");
     p->prof.launches += 1;
     if (s.pc == SHTG_PRECOND_LOWL)
@@ -1653,15 +1690,15 @@ static int pcg_iteration_grp(GroupIter &G, cudaStream_t st) {
     prof_begin(acct, K_VEC, st);
     const dim3 rows(RB, G.nbtot);
     k_prior_add_grp<<<rows, RT, 0, st>>>(G.V);
-    k_scal_alpha_grp<<<G.ng, 1024, 0, st>>>(G.V, 1e-6);
     k_update_grp<<<rows, RT, 0, st>>>(G.V);
     if (G.pc == SHTG_PRECOND_AZIM)
         SHTG_TRY(az_apply_grp(G.ng, ps, reinterpret_cast<const float *const *>(G.r32.data()),
                               reinterpret_cast<float *const *>(G.z32.data()), G.nb.data(), G.per.data(),
                               G.part.data(), act, st));
-    k_scal_beta_grp<<<G.ng, 1024, 0, st>>>(G.V);
+    const int maxnb = *std::max_element(G.nb.begin(), G.nb.end());
+    k_scal_beta_grp<<<dim3(scal_grid(maxnb).x, G.ng), SCAL_T, 0, st>>>(G.V, 1e-6);
     k_pupdate_grp<<<rows, RT, 0, st>>>(G.V);
-    prof_end(acct, st, 5);
+    prof_end(acct, st, 4);
     SHTG_CHECK_LAUNCH("grouped pcg iteration");
     return SHTG_OK;
 }
@@ -1758,6 +1795,7 @@ static int mixed_solve_grp(int ng, Plan *const *ps, std::vector<CgCall> &c, cuda
         v.mof = p->d_mofidx;
         v.scal = p->d_scal;
         v.part = p->d_part;
+        v.pqp = pq_part(p);
         v.active = p->d_flag + 1;
         v.nalm = s.nalm;
         v.nc = s.nc;
@@ -1836,12 +1874,12 @@ static int mixed_solve_grp(int ng, Plan *const *ps, std::vector<CgCall> &c, cuda
             if (q.first) SHTG_CUDA(cudaMemsetAsync(x32, 0, vb32, st));
             else k_scale_vec<<<s.vgrid, RT, 0, st>>>(p32, s.per, q.d_sc + 2 * nb);
             k_update<float, true><<<s.rgrid, RT, 0, st>>>(nullptr, r32, z32, nullptr, nullptr, p->d_minv32, s.nc,
-                                                         s.nalm, p->d_mofidx, p->d_scal, p->d_part);
+                                                         s.nalm, p->d_mofidx, p->d_scal, nullptr, p->d_part);
             if (G.pc == SHTG_PRECOND_AZIM)
                 SHTG_TRY(az_apply<float>(p, reinterpret_cast<const float *>(r32), reinterpret_cast<float *>(z32), nb,
                                          s.per, p->d_part, st, false));
             if (!q.first) k_restart_dir<<<s.vgrid, RT, 0, st>>>(p32, z32, s.per, p->d_scal);
-            k_scal_reliable<<<1, 1024, 0, st>>>(p->d_part, p->d_scal, nb, q.d_sc + nb);
+            k_scal_reliable<<<scal_grid(nb), SCAL_T, 0, st>>>(p->d_part, p->d_scal, nb, q.d_sc + nb);
             p->prof.launches += q.first ? 3 : 5;
             SHTG_CHECK_LAUNCH("reliable update");
             if (q.first) SHTG_CUDA(cudaMemcpyAsync(p32, z32, vb32, cudaMemcpyDeviceToDevice, st));
@@ -2024,7 +2062,10 @@ int logpost_grad(Plan *p, const double *cl, const double *bl, const float *alm, 
     const float2 *a = reinterpret_cast<const float2 *>(alm);
     SHTG_TRY(leg_synth<float>(p, 0, a, 1, 1, beam, p->d_phase32, st));
     SHTG_TRY(ring_synth<float>(p, p->d_phase32, 1, p->d_map32, st));
-    k_resid_pix<<<RB, RT, 0, st>>>(d, ninv, p->d_map32, p->npix, p->d_part);
+    // 4 RB blocks (the partial buffer's size with one realization): the FP64
+    // products bound the kernel, and RB blocks of eight warps filled half of
+    // the SMs' schedulers
+    k_resid_pix<<<4 * RB, RT, 0, st>>>(d, ninv, p->d_map32, p->npix, p->d_part);
     SHTG_CHECK_LAUNCH("k_resid_pix");
     if (grad) {
         float2 *g = reinterpret_cast<float2 *>(grad);
@@ -2035,10 +2076,10 @@ int logpost_grad(Plan *p, const double *cl, const double *bl, const float *alm, 
         SHTG_CHECK_LAUNCH("k_grad_prior");
     }
     SHTG_CUDA(cudaMemsetAsync(p->d_lsum, 0, sizeof(double) * L1, st));
-    k_prior_lsum<<<grid_1d(p->nalm), RT, 0, st>>>(a, p->nalm, p->d_lofidx, p->d_mofidx, d_icl, p->d_lsum);
+    k_prior_lsum<<<dim3((L1 + 127) / 128, (L1 + PL_M - 1) / PL_M), 128, 0, st>>>(a, p->lmax, d_icl, p->d_lsum);
     SHTG_CHECK_LAUNCH("k_prior_lsum");
-    std::vector<double> part(RB), ls(L1);
-    SHTG_CUDA(cudaMemcpyAsync(part.data(), p->d_part, sizeof(double) * RB, cudaMemcpyDeviceToHost, st));
+    std::vector<double> part(4 * RB), ls(L1);
+    SHTG_CUDA(cudaMemcpyAsync(part.data(), p->d_part, sizeof(double) * part.size(), cudaMemcpyDeviceToHost, st));
     SHTG_CUDA(cudaMemcpyAsync(ls.data(), p->d_lsum, sizeof(double) * L1, cudaMemcpyDeviceToHost, st));
     SHTG_CUDA(cudaStreamSynchronize(st));
     double chi2 = 0.0, prior = 0.0;
