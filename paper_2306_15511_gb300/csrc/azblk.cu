@@ -44,8 +44,7 @@ namespace {
 
 constexpr int GT = 32;      // Gram tile and pair chunk
 constexpr int AZT = 256;    // threads of the ring-sum kernel
-constexpr int AZF = 1024;   // threads of the factor kernels (one CTA per m: the largest block alone
-                            // bounds the launch, so its rank-1 updates need every warp of the SM)
+constexpr int AZF = 512;    // threads of the factor kernels (one CTA per m)
 
 __host__ __device__ __forceinline__ int64_t tri(int64_t i) { return i * (i + 1) / 2; }
 
@@ -233,100 +232,230 @@ __global__ void k_az_assemble(int lb, int ncb, const int64_t *__restrict__ goff,
                               double *__restrict__ H) {
     const int m = blockIdx.y;
     const int k = lb + 1 - m, n = ncb * k;
-    const int64_t ne = tri(n);
     const double *Gm = G + goff[m];
     double *Hm = H + hoff[m];
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne; e += (int64_t)gridDim.x * blockDim.x) {
-        // packed (i, j), j <= i
-        int i = (int)((sqrt(8.0 * (double)e + 1.0) - 1.0) / 2.0);
-        while (tri(i) > e) --i;
-        while (tri(i + 1) <= e) ++i;
-        const int j = (int)(e - tri(i));
-        const int ci = i / k, cj = j / k, ii = i % k, jj = j % k;
-        const int li = m + ii, lj = m + jj;
-        const bool ai = ltab[5 * lmax1 + li] > 0.0, aj = ltab[5 * lmax1 + lj] > 0.0;
-        double v;
-        if (!ai || !aj) {
-            v = i == j ? 1.0 : 0.0;
-        } else {
-            v = 0.0;
-            if (ci == cj) v = ltab[li] * ltab[lj] * Gm[(int64_t)ci * tri(k) + tri(ii) + jj];
-            if (li == lj) {
-                const int row = (ci == 0 && cj == 0) ? 1 : (ci == 1 && cj == 1) ? 3 : 2;   // TT, EE, TE
-                v += ltab[row * lmax1 + li] * isc;
+    // one warp per row i
+    const int nw = gridDim.x * (blockDim.x >> 5);
+    for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += nw) {
+        const int ci = i / k, ii = i % k, li = m + ii;
+        const bool ai = ltab[5 * lmax1 + li] > 0.0;
+        for (int j = threadIdx.x & 31; j <= i; j += 32) {
+            const int cj = j / k, jj = j % k, lj = m + jj;
+            double v;
+            if (!ai || !(ltab[5 * lmax1 + lj] > 0.0)) {
+                v = i == j ? 1.0 : 0.0;
+            } else {
+                v = 0.0;
+                if (ci == cj) v = ltab[li] * ltab[lj] * Gm[(int64_t)ci * tri(k) + tri(ii) + jj];
+                if (li == lj) {
+                    const int row = (ci == 0 && cj == 0) ? 1 : (ci == 1 && cj == 1) ? 3 : 2;   // TT, EE, TE
+                    v += ltab[row * lmax1 + li] * isc;
+                }
             }
+            Hm[tri(i) + j] = v;
         }
-        Hm[e] = v;
     }
 }
 
-// One CTA per m: Cholesky H = R R^T in place (packed lower, right-looking;
-// column j of the trailing update staged in shared memory).  flag bit 1: a
-// pivot was not positive.
+// Blocked factor kernels, one CTA per m (the largest block alone keeps an SM
+// busy: n^3 / 6 multiply-adds at two per clock, 2.5 ms for n = 384; that is
+// what bounds the launch).  Blocks of FB = 32 columns; the CTA's AZG groups of
+// 128 threads (four warps, one per scheduler) work on 32 x 32 tiles staged in
+// shared memory, 2 x 4 entries per thread.  The unblocked forms before them
+// went over the whole trailing triangle in L2 for every column: n = 384 (l_b
+// 383, 384 values of m) 4.8 ms the Cholesky, 10.9 ms the inverse; now 3.5 and
+// 4.6.
+constexpr int FB = 32, AZG = AZF / 128;
+constexpr size_t AZ_FACTOR_SMEM = sizeof(double) * FB * (FB + 1) * (2 + 2 * AZG);
+
+__device__ __forceinline__ void az_group_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory"); }
+
+// acc[a][b] += sum_t P[2 ty + a][t] Q[t or 4 tx + b][...]: rows 2 ty + a,
+// columns 4 tx + b of P Q^T (QT: Q holds the columns as rows) or P Q
+template <bool QT>
+__device__ __forceinline__ void az_tile_fma(const double (*P)[FB + 1], const double (*Q)[FB + 1], int ty, int tx,
+                                            double (&acc)[2][4]) {
+#pragma unroll 4
+    for (int t = 0; t < FB; ++t) {
+        double q[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) q[b] = QT ? Q[4 * tx + b][t] : Q[t][4 * tx + b];
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const double pv = P[2 * ty + a][t];
+#pragma unroll
+            for (int b = 0; b < 4; ++b) acc[a][b] = fma(pv, q[b], acc[a][b]);
+        }
+    }
+}
+
+// One CTA per m: Cholesky H = R R^T in place (packed lower, right-looking):
+// per block column the 32 x 32 diagonal block by one warp, the panel below it
+// by forward substitution (one thread per row), then the trailing update
+// A_IK -= P_I P_K^T tile by tile.  flag bit 1: a pivot was not positive.
 __global__ void __launch_bounds__(AZF) k_az_chol(int lb, int ncb, const int64_t *__restrict__ hoff, double *H,
                                                  int *__restrict__ flag) {
     extern __shared__ __align__(16) unsigned char az_raw[];
-    double *col = reinterpret_cast<double *>(az_raw);
-    __shared__ double s_d;
+    typedef double(*Tile)[FB + 1];
+    Tile sD = reinterpret_cast<Tile>(az_raw);
+    double *sInv = reinterpret_cast<double *>(az_raw) + FB * (FB + 1);   // 1 / diagonal
+    const int grp = threadIdx.x >> 7, gt = threadIdx.x & 127;
+    Tile sP = sD + (2 + 2 * grp) * FB, sQ = sP + FB;
+    const int ty = gt >> 3, tx = gt & 7;
     const int m = blockIdx.x;
     const int n = ncb * (lb + 1 - m);
     double *A = H + hoff[m];
-    for (int j = 0; j < n; ++j) {
-        if (threadIdx.x == 0) {
-            const double d = A[tri(j) + j];
-            if (!(d > 0.0)) atomicOr(flag, 1);
-            s_d = d > 0.0 ? sqrt(d) : 1.0;
-            A[tri(j) + j] = s_d;
+    for (int j0 = 0; j0 < n; j0 += FB) {
+        const int nb = min(FB, n - j0);
+        for (int e = threadIdx.x; e < FB * FB; e += AZF) {
+            const int r = e / FB, c = e % FB;
+            sD[r][c] = (r < nb && c <= r) ? A[tri(j0 + r) + j0 + c] : (r == c ? 1.0 : 0.0);
         }
         __syncthreads();
-        const double id = 1.0 / s_d;
-        for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) {
-            const double v = A[tri(i) + j] * id;
-            A[tri(i) + j] = v;
-            col[i] = v;
+        if (threadIdx.x < 32) {   // lane = row
+            const int lane = threadIdx.x;
+            for (int c = 0; c < FB; ++c) {
+                const double d = sD[c][c];
+                if (!(d > 0.0) && lane == 0) atomicOr(flag, 1);
+                const double sd = d > 0.0 ? sqrt(d) : 1.0, id = 1.0 / sd;
+                const double v = sD[lane][c] * id;
+                __syncwarp();
+                if (lane > c) sD[lane][c] = v;
+                if (lane == c) {
+                    sD[c][c] = sd;
+                    sInv[c] = id;
+                }
+                __syncwarp();
+                for (int k = c + 1; k <= lane; ++k) sD[lane][k] = fma(-v, sD[k][c], sD[lane][k]);
+                __syncwarp();
+            }
         }
         __syncthreads();
-        // A_ik -= R_ij R_kj for j < k <= i: one warp per row, lanes over k
-        // (unrolled, so that each lane has several independent loads in flight)
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        for (int i = j + 1 + warp; i < n; i += blockDim.x >> 5) {
-            const double rij = col[i];
-            double *row = A + tri(i);
-#pragma unroll 4
-            for (int kk = j + 1 + lane; kk <= i; kk += 32) row[kk] = fma(-rij, col[kk], row[kk]);
+        for (int e = threadIdx.x; e < FB * FB; e += AZF) {
+            const int r = e / FB, c = e % FB;
+            if (r < nb && c <= r) A[tri(j0 + r) + j0 + c] = sD[r][c];
+        }
+        const int i1 = j0 + FB;
+        if (i1 >= n) break;
+        for (int i = i1 + threadIdx.x; i < n; i += AZF) {
+            double *row = A + tri(i) + j0;
+            double x[FB];
+#pragma unroll
+            for (int c = 0; c < FB; ++c) x[c] = row[c];
+#pragma unroll
+            for (int c = 0; c < FB; ++c) {
+#pragma unroll
+                for (int t = 0; t < c; ++t) x[c] = fma(-x[t], sD[c][t], x[c]);
+                x[c] *= sInv[c];
+                asm volatile("" ::: "memory");   // keeps the compiler from loading all of sD at once (it spills)
+            }
+#pragma unroll
+            for (int c = 0; c < FB; ++c) row[c] = x[c];
+        }
+        __syncthreads();
+        const int nrb = (n - i1 + FB - 1) / FB, ntile = nrb * (nrb + 1) / 2;
+        int lastI = -1;
+        for (int t = grp; t < ntile; t += AZG) {
+            int I = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+            while ((I + 1) * (I + 2) / 2 <= t) ++I;
+            while (I * (I + 1) / 2 > t) --I;
+            const int K = t - I * (I + 1) / 2;
+            const int ib = i1 + I * FB, kb = i1 + K * FB;
+            for (int e = gt; e < FB * FB; e += 128) {
+                const int r = e / FB, c = e % FB;
+                if (I != lastI) sP[r][c] = ib + r < n ? A[tri(ib + r) + j0 + c] : 0.0;
+                sQ[r][c] = kb + r < n ? A[tri(kb + r) + j0 + c] : 0.0;
+            }
+            lastI = I;
+            az_group_sync(grp);
+            double acc[2][4] = {};
+            az_tile_fma<true>(sP, sQ, ty, tx, acc);
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                const int i = ib + 2 * ty + a;
+                if (i >= n) continue;
+                double *row = A + tri(i) + kb + 4 * tx;
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    if (kb + 4 * tx + b <= i) row[b] -= acc[a][b];
+            }
+            az_group_sync(grp);   // the tiles are consumed
         }
         __syncthreads();
     }
 }
 
-// One CTA per m: R <- R^-1 in place (packed lower), column by column from
-// the last: X_jj = 1 / R_jj, X_kj = -X_jj sum_{j < t <= k} X_kt R_tj for
-// k > j (the trailing block already inverted; column j of R staged in
-// shared memory, one warp per row k).
-__global__ void __launch_bounds__(AZF) k_az_trinv(int lb, int ncb, const int64_t *__restrict__ hoff, double *H) {
+// One CTA per m: R <- X = R^-1 in place (packed lower), by block columns from
+// the last: X_jj = R_jj^-1 (one warp), X_Ij = -(sum_{j < K <= I} X_IK R_Kj)
+// X_jj for the row blocks I below.  The panel R_Kj is copied to scr (the
+// block's full square, written by the next kernel only) because its rows are
+// overwritten while other groups still read it.
+__global__ void __launch_bounds__(AZF) k_az_trinv(int lb, int ncb, const int64_t *__restrict__ hoff,
+                                                  const int64_t *__restrict__ moff, double *H, double *scr) {
     extern __shared__ __align__(16) unsigned char az_raw[];
-    double *col = reinterpret_cast<double *>(az_raw);
-    __shared__ double s_d;
+    typedef double(*Tile)[FB + 1];
+    Tile sD = reinterpret_cast<Tile>(az_raw), sX = sD + FB;
+    const int grp = threadIdx.x >> 7, gt = threadIdx.x & 127;
+    Tile sP = sD + (2 + 2 * grp) * FB, sQ = sP + FB;
+    const int ty = gt >> 3, tx = gt & 7;
     const int m = blockIdx.x;
     const int n = ncb * (lb + 1 - m);
-    double *A = H + hoff[m];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int j = n - 1; j >= 0; --j) {
-        if (threadIdx.x == 0) {
-            s_d = 1.0 / A[tri(j) + j];
-            A[tri(j) + j] = s_d;
+    double *A = H + hoff[m], *S = scr + moff[m];
+    const int nblk = (n + FB - 1) / FB;
+    for (int jb = nblk - 1; jb >= 0; --jb) {
+        const int j0 = jb * FB, nb = min(FB, n - j0), i1 = j0 + FB;
+        for (int e = threadIdx.x; e < FB * FB; e += AZF) {
+            const int r = e / FB, c = e % FB;
+            sD[r][c] = (r < nb && c <= r) ? A[tri(j0 + r) + j0 + c] : (r == c ? 1.0 : 0.0);
         }
-        for (int t = j + 1 + threadIdx.x; t < n; t += blockDim.x) col[t] = A[tri(t) + j];
+        for (int64_t e = threadIdx.x; e < (int64_t)(n - i1) * FB; e += AZF) {
+            const int i = i1 + (int)(e / FB), c = (int)(e % FB);
+            S[e] = A[tri(i) + j0 + c];
+        }
         __syncthreads();
-        const double d = s_d;
-        for (int k = j + 1 + warp; k < n; k += blockDim.x >> 5) {
-            const double *row = A + tri(k);
-            double s = 0.0;
-#pragma unroll 4
-            for (int t = j + 1 + lane; t <= k; t += 32) s = fma(row[t], col[t], s);
+        if (threadIdx.x < 32) {   // lane = column c of X_jj, rows in order
+            const int c = threadIdx.x;
+            for (int r = 0; r < FB; ++r) {
+                double v = r == c ? 1.0 : 0.0;
+                for (int t = 0; t < r; ++t) v = fma(-sD[r][t], sX[t][c], v);
+                sX[r][c] = v / sD[r][r];
+            }
+        }
+        __syncthreads();
+        const int nrb = i1 < n ? (n - i1 + FB - 1) / FB : 0;
+        for (int I = nrb - 1 - grp; I >= 0; I -= AZG) {
+            const int ib = i1 + I * FB;
+            double acc[2][4] = {};
+            for (int K = 0; K <= I; ++K) {
+                const int kb = i1 + K * FB;
+                for (int e = gt; e < FB * FB; e += 128) {
+                    const int r = e / FB, c = e % FB;
+                    sP[r][c] = (ib + r < n && kb + c <= ib + r) ? A[tri(ib + r) + kb + c] : 0.0;
+                    sQ[r][c] = kb + r < n ? S[(int64_t)(kb + r - i1) * FB + c] : 0.0;
+                }
+                az_group_sync(grp);
+                az_tile_fma<false>(sP, sQ, ty, tx, acc);
+                az_group_sync(grp);
+            }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) A[tri(k) + j] = -d * s;
+            for (int a = 0; a < 2; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) sP[2 * ty + a][4 * tx + b] = acc[a][b];
+            az_group_sync(grp);
+            double out[2][4] = {};
+            az_tile_fma<false>(sP, sX, ty, tx, out);
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                const int i = ib + 2 * ty + a;
+                if (i >= n) continue;
+#pragma unroll
+                for (int b = 0; b < 4; ++b) A[tri(i) + j0 + 4 * tx + b] = -out[a][b];
+            }
+            az_group_sync(grp);
+        }
+        for (int e = threadIdx.x; e < FB * FB; e += AZF) {
+            const int r = e / FB, c = e % FB;
+            if (r < nb && c <= r) A[tri(j0 + r) + j0 + c] = sX[r][c];
         }
         __syncthreads();
     }
@@ -407,29 +536,32 @@ __global__ void k_az_gather(int lb, int ncb, int lmax, int nb, const int64_t *__
     az_gather_cta<T, TF>(lb, ncb, lmax, nb, xoff, r, nalm, per, Xg, blockIdx.x, blockIdx.y);
 }
 
-// z <- M^-1 r on the block rows, as a tall-skinny product Z = M X per m
-// (X: the staged right-hand sides, up to 16 per pass): grid.x = m, grid.y =
-// tile of MR = 128 rows; 128 threads, thread t computes rows 4 (t / 4) ..
-// + 3 for right-hand sides 4 (t % 4) .. + 3.  The columns run in steps of KT:
-// the step's 128 x KT piece of M is loaded into registers (one row per
-// thread, the next step's loads in flight during this step's products) and
-// stored transposed in shared memory, so each k reads four rows and four
-// right-hand sides with two 16-byte loads.  q = 2 b + part (part 0 real, 1
-// imaginary; m = 0 real only).  slot[((b (lb + 1) + m) ntile + tile) 2 +
-// part] = the change of sum w r z of system b's part on these rows (every
-// slot of an existing tile is written by every application; the others stay
-// zero).
-constexpr int MR = 128, KT = 32;
-template <typename T, typename TF>
+// z <- M^-1 r on the block rows, as a tall-skinny product Z = M X per m (X:
+// the staged right-hand sides, up to QB per pass): grid.x = m, grid.y = tile
+// of MR = 128 rows; 8 warps, each over one eighth of the columns, each lane
+// for 4 rows and QB right-hand sides.  M is symmetric and read by columns, so
+// a warp's loads are contiguous and independent of one another, and no
+// barrier stands in the loop; the warps' sums are added in a fixed order.
+// (The form before read a row per thread in steps of 32 columns with two
+// barriers each and summed the change of <r, z> with 112 FP64 instructions
+// per thread: 203 us for the 75 MB of blocks of l_b 383 with 4 realizations,
+// which stay in L2; now 91 us.)  q = 2 b + part (part 0 real, 1 imaginary;
+// m = 0 real only).  slot[((b (lb + 1) + m) ntile + tile) 2 + part] = the
+// change of sum w r z of system b's part on these rows (every slot of an
+// existing tile is written by every application; the others stay zero).
+constexpr int MR = 128, AZM = 256, KC = 512;   // rows per tile, threads, columns staged at a time
+template <typename TF, int QB> constexpr int az_mapply_smem() { return (int)sizeof(TF) * KC * QB; }
+template <typename T, typename TF, int QB>
 __device__ __forceinline__ void az_mapply_cta(int lb, int ncb, int lmax, int nb, int ntile,
                                               const int64_t *__restrict__ moff, const TF *__restrict__ M,
                                               const int64_t *__restrict__ xoff, const TF *__restrict__ Xg,
-                                              const T *__restrict__ r, T *__restrict__ z, int64_t nalm,
-                                              int64_t per, double *__restrict__ slot, const int m,
-                                              const int tile) {
-    __shared__ __align__(16) TF As[KT][MR];
-    __shared__ __align__(16) TF Xs[KT][16];
-    __shared__ double sred[16][33];
+                                              const T *r, T *z, int64_t nalm, int64_t per,
+                                              double *__restrict__ slot, const int m, const int tile) {
+    extern __shared__ __align__(16) unsigned char az_raw[];
+    TF(*Xs)[QB] = reinterpret_cast<TF(*)[QB]>(az_raw);          // [KC][QB] in the product,
+    TF(*red)[MR][QB] = reinterpret_cast<TF(*)[MR][QB]>(az_raw); // [4][MR][QB] after it (KC = 4 MR)
+    static_assert(KC == 4 * MR, "the reduction buffer takes the staged columns' place");
+    __shared__ double sds[AZM / 32][QB];
     const int k = lb + 1 - m, n = ncb * k;
     const int i0 = tile * MR;
     if (i0 >= n) return;
@@ -438,100 +570,111 @@ __device__ __forceinline__ void az_mapply_cta(int lb, int ncb, int lmax, int nb,
     const int nq = nb * nparts;
     const int64_t base = (int64_t)m * (2 * lmax + 1 - m) / 2 + m;   // alm index of l = m
     const double wm = m ? 2.0 : 1.0;
-    const int tid = threadIdx.x, rg = tid >> 2, qg = tid & 3;
-    // this thread's row of the staged piece of M
-    const int ri = min(i0 + tid, n - 1);
-    const TF *mrow = Mm + (int64_t)ri * n;
-    const bool rlive = i0 + tid < n;
-    for (int q0 = 0; q0 < nq; q0 += 16) {
-        const int qn = min(16, nq - q0);
-        TF acc[4][4];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const TF *mc[4];   // this lane's rows i0 + lane + 32 a (clamped: rows beyond n are dropped below)
+#pragma unroll
+    for (int a = 0; a < 4; ++a) mc[a] = Mm + min(i0 + lane + 32 * a, n - 1);
+    for (int q0 = 0; q0 < nq; q0 += QB) {
+        const int qn = min(QB, nq - q0);
+        TF acc[4][QB];
 #pragma unroll
         for (int a = 0; a < 4; ++a)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[a][c] = TF(0);
-        TF nxt[KT];
-        auto load_piece = [&](int j0) {
-#pragma unroll
-            for (int kk = 0; kk < KT; ++kk) nxt[kk] = (rlive && j0 + kk < n) ? mrow[j0 + kk] : TF(0);
-        };
-        load_piece(0);
-        for (int j0 = 0; j0 < n; j0 += KT) {
+            for (int c = 0; c < QB; ++c) acc[a][c] = TF(0);
+        for (int k0 = 0; k0 < n; k0 += KC) {
+            const int kn = min(KC, n - k0);
             __syncthreads();
-#pragma unroll
-            for (int kk = 0; kk < KT; ++kk) As[kk][tid] = nxt[kk];
-            for (int e = tid; e < KT * 16; e += 128) {
-                const int kk = e / 16, q = e % 16;
-                Xs[kk][q] = (j0 + kk < n && q < qn) ? Xg[xoff[m] + (int64_t)(q0 + q) * n + j0 + kk] : TF(0);
+            for (int e = tid; e < kn * QB; e += AZM) {
+                const int j = e % kn, q = e / kn;
+                Xs[j][q] = q < qn ? Xg[xoff[m] + (int64_t)(q0 + q) * n + k0 + j] : TF(0);
             }
             __syncthreads();
-            if (j0 + KT < n) load_piece(j0 + KT);
+            const int per_w = (kn + 7) / 8, j1 = min(kn, (warp + 1) * per_w);
+#pragma unroll 4
+            for (int j = warp * per_w; j < j1; ++j) {
+                const int64_t o = (int64_t)(k0 + j) * n;
+                TF mv[4];
 #pragma unroll
-            for (int kk = 0; kk < KT; ++kk) {
-                TF a4[4], x4[4];
+                for (int a = 0; a < 4; ++a) mv[a] = mc[a][o];
 #pragma unroll
-                for (int a = 0; a < 4; ++a) a4[a] = As[kk][4 * rg + a];
+                for (int c = 0; c < QB; ++c) {
+                    const TF x = Xs[j][c];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) x4[c] = Xs[kk][4 * qg + c];
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[a][c] = fma(a4[a], x4[c], acc[a][c]);
+                    for (int a = 0; a < 4; ++a) acc[a][c] = fma(mv[a], x, acc[a][c]);
+                }
             }
         }
-        // write z and this thread's change of w r z per right-hand side
-        double ds[4] = {0.0, 0.0, 0.0, 0.0};
+        __syncthreads();
+        if (warp >= 4) {
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const int i = i0 + 4 * rg + a;
-            if (i >= n) continue;
-            const int c = i / k, ll = i % k;
+            for (int a = 0; a < 4; ++a)
 #pragma unroll
-            for (int cq = 0; cq < 4; ++cq) {
-                const int q = 4 * qg + cq;
-                if (q >= qn) continue;
-                const int gq = q0 + q, b = gq / nparts, part = gq % nparts;
-                const int64_t el = 2 * ((int64_t)b * per + (int64_t)c * nalm + base + ll) + part;
-                const double rv = (double)r[el], zo = (double)z[el];
-                ds[cq] += wm * rv * ((double)acc[a][cq] - zo);
-                z[el] = (T)acc[a][cq];
+                for (int c = 0; c < QB; ++c) red[warp - 4][lane + 32 * a][c] = acc[a][c];
+        }
+        __syncthreads();
+        if (warp < 4) {
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int c = 0; c < QB; ++c) red[warp][lane + 32 * a][c] += acc[a][c];
+        }
+        __syncthreads();
+        // z and the change of w r z: thread = right-hand side tid % QB, rows tid / QB + ...
+        const int q = tid % QB;
+        double ds = 0.0;
+        if (q < qn) {
+            const int gq = q0 + q, b = gq / nparts, part = gq % nparts;
+#pragma unroll 2
+            for (int row = tid / QB; row < MR; row += AZM / QB) {
+                const int i = i0 + row;
+                if (i >= n) break;
+                const TF zn = (red[0][row][q] + red[1][row][q]) + (red[2][row][q] + red[3][row][q]);
+                const int c = i >= k ? 1 : 0;   // T, then E
+                const int64_t el = 2 * ((int64_t)b * per + (int64_t)c * nalm + base + (i - c * k)) + part;
+                ds = ::fma((double)r[el], (double)zn - (double)z[el], ds);
+                z[el] = (T)zn;
             }
         }
 #pragma unroll
-        for (int cq = 0; cq < 4; ++cq) sred[4 * qg + cq][rg] = ds[cq];
+        for (int o = 16; o >= QB; o >>= 1) ds += __shfl_xor_sync(0xffffffffu, ds, o);
+        if (lane < QB) sds[warp][lane] = ds;
         __syncthreads();
         if (tid < qn) {
             const int gq = q0 + tid, b = gq / nparts, part = gq % nparts;
-            double s = 0.0;
-            for (int g = 0; g < 32; ++g) s += sred[tid][g];
-            slot[(((int64_t)b * (lb + 1) + m) * ntile + tile) * 2 + part] = s;
+            double t = 0.0;
+#pragma unroll
+            for (int w = 0; w < AZM / 32; ++w) t += sds[w][tid];
+            slot[(((int64_t)b * (lb + 1) + m) * ntile + tile) * 2 + part] = wm * t;
         }
         __syncthreads();
     }
 }
-template <typename T, typename TF>
-__global__ void __launch_bounds__(128) k_az_mapply(int lb, int ncb, int lmax, int nb, int ntile,
-                                                   const int64_t *__restrict__ moff, const TF *__restrict__ M,
-                                                   const int64_t *__restrict__ xoff, const TF *__restrict__ Xg,
-                                                   const T *__restrict__ r, T *__restrict__ z, int64_t nalm,
-                                                   int64_t per, double *__restrict__ slot) {
-    az_mapply_cta<T, TF>(lb, ncb, lmax, nb, ntile, moff, M, xoff, Xg, r, z, nalm, per, slot, blockIdx.x,
-                         blockIdx.y);
+template <typename T, typename TF, int QB>
+__global__ void __launch_bounds__(AZM, 2) k_az_mapply(int lb, int ncb, int lmax, int nb, int ntile,
+                                                      const int64_t *__restrict__ moff, const TF *__restrict__ M,
+                                                      const int64_t *__restrict__ xoff, const TF *__restrict__ Xg,
+                                                      const T *r, T *z, int64_t nalm, int64_t per,
+                                                      double *__restrict__ slot) {
+    az_mapply_cta<T, TF, QB>(lb, ncb, lmax, nb, ntile, moff, M, xoff, Xg, r, z, nalm, per, slot, blockIdx.x,
+                             blockIdx.y);
 }
 
 // per system b: the sum of its slots in a fixed order (each thread a fixed
-// strided subset, then the threads in order), added to its first rz partial
+// strided subset, then a fixed tree), added to its first rz partial
 __device__ __forceinline__ void az_addpart_cta(int nslot, const double *__restrict__ slot,
                                                double *__restrict__ part, int rb, const int b) {
-    __shared__ double sm[256];
+    __shared__ double sm[8];
     const double *s = slot + (int64_t)b * nslot;
     double t = 0.0;
     for (int e = threadIdx.x; e < nslot; e += 256) t += s[e];
-    sm[threadIdx.x] = t;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = t;
     __syncthreads();
     if (threadIdx.x == 0) {
         double u = 0.0;
-        for (int w = 0; w < 256; ++w) u += sm[w];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) u += sm[w];
         part[((int64_t)b * 2 + 0) * rb + 0] += u;
     }
 }
@@ -573,13 +716,13 @@ __global__ void k_az_gather_grp(const __grid_constant__ AzGroups G) {
     az_gather_cta<float, float>(a.lb, a.ncb, a.lmax, a.nb, a.xoff, a.r, a.nalm, a.per, a.Xg, li % (a.lb + 1),
                                 li / (a.lb + 1));
 }
-__global__ void __launch_bounds__(128) k_az_mapply_grp(const __grid_constant__ AzGroups G) {
+__global__ void __launch_bounds__(AZM, 2) k_az_mapply_grp(const __grid_constant__ AzGroups G) {
     const int g = az_group(G, blockIdx.x);
     const AzGrp &a = G.a[g];
     if (*a.active == 0) return;
     const int li = blockIdx.x - G.first[g];
-    az_mapply_cta<float, float>(a.lb, a.ncb, a.lmax, a.nb, a.ntile, a.moff, a.M, a.xoff, a.Xg, a.r, a.z, a.nalm,
-                                a.per, a.slot, li % (a.lb + 1), li / (a.lb + 1));
+    az_mapply_cta<float, float, 16>(a.lb, a.ncb, a.lmax, a.nb, a.ntile, a.moff, a.M, a.xoff, a.Xg, a.r, a.z, a.nalm,
+                                    a.per, a.slot, li % (a.lb + 1), li / (a.lb + 1));
 }
 __global__ void k_az_addpart_grp(const __grid_constant__ AzGroups G) {
     const int g = az_group(G, blockIdx.x);
@@ -748,14 +891,11 @@ int az_setup(Plan *p, int lb, int nc, double isc, cudaStream_t st) {
     k_az_assemble<<<dim3(64, lb + 1), 256, 0, st>>>(lb, ncb, q.goff, q.hoff, q.G, p->d_ltab64, L1, isc, q.H);
     SHTG_CHECK_LAUNCH("k_az_assemble");
     SHTG_CUDA(cudaMemsetAsync(q.flag, 0, sizeof(int), st));
-    const size_t csm = sizeof(double) * (size_t)ncb * (lb + 1);
-    if (csm > 48 * 1024) {
-        SHTG_CUDA(allow_max_smem(k_az_chol));
-        SHTG_CUDA(allow_max_smem(k_az_trinv));
-    }
-    k_az_chol<<<lb + 1, AZF, csm, st>>>(lb, ncb, q.hoff, q.H, q.flag);
+    SHTG_CUDA(cudaFuncSetAttribute(k_az_chol, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AZ_FACTOR_SMEM));
+    SHTG_CUDA(cudaFuncSetAttribute(k_az_trinv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AZ_FACTOR_SMEM));
+    k_az_chol<<<lb + 1, AZF, AZ_FACTOR_SMEM, st>>>(lb, ncb, q.hoff, q.H, q.flag);
     SHTG_CHECK_LAUNCH("k_az_chol");
-    k_az_trinv<<<lb + 1, AZF, csm, st>>>(lb, ncb, q.hoff, q.H);
+    k_az_trinv<<<lb + 1, AZF, AZ_FACTOR_SMEM, st>>>(lb, ncb, q.hoff, q.moff, q.H, q.M64);
     SHTG_CHECK_LAUNCH("k_az_trinv");
     const int nt = (ncb * (lb + 1) + GT - 1) / GT;
     k_az_minv<<<dim3(nt * (nt + 1) / 2, lb + 1), 256, 0, st>>>(lb, ncb, q.hoff, q.moff, q.H, q.M64, q.M32);
@@ -780,8 +920,18 @@ static int az_apply_t(Plan *p, const T *r, T *z, int nb, int64_t per, double *pa
     const TF *M = sizeof(TF) == 4 ? reinterpret_cast<const TF *>(q.M32) : reinterpret_cast<const TF *>(q.M64);
     TF *Xg = reinterpret_cast<TF *>(q.Xg);
     k_az_gather<T, TF><<<dim3(q.lb + 1, 2 * nb), 256, 0, st>>>(q.lb, q.ncb, p->lmax, nb, q.xoff, r, p->nalm, per, Xg);
-    k_az_mapply<T, TF><<<dim3(q.lb + 1, q.ntile), 128, 0, st>>>(q.lb, q.ncb, p->lmax, nb, q.ntile, q.moff, M, q.xoff,
-                                                                Xg, r, z, p->nalm, per, q.slot);
+    const dim3 grid(q.lb + 1, q.ntile);
+    if constexpr (sizeof(TF) == 4) {
+        // more than four realizations (eight right-hand sides): sixteen per
+        // pass, so the blocks are read half as often; FP64 sums keep eight
+        // (registers)
+        if (nb > 4)
+            k_az_mapply<T, TF, 16><<<grid, AZM, (az_mapply_smem<TF, 16>()), st>>>(
+                q.lb, q.ncb, p->lmax, nb, q.ntile, q.moff, M, q.xoff, Xg, r, z, p->nalm, per, q.slot);
+    }
+    if (sizeof(TF) == 8 || nb <= 4)
+        k_az_mapply<T, TF, 8><<<grid, AZM, (az_mapply_smem<TF, 8>()), st>>>(
+            q.lb, q.ncb, p->lmax, nb, q.ntile, q.moff, M, q.xoff, Xg, r, z, p->nalm, per, q.slot);
     k_az_addpart<<<nb, 256, 0, st>>>((q.lb + 1) * q.ntile * 2, q.slot, part, SHTG_RED_BLOCKS);
     p->prof.launches += 3;
     SHTG_CHECK_LAUNCH("k_az_mapply");
@@ -843,7 +993,7 @@ int az_apply_grp(int ng, Plan *const *ps, const float *const *r, float *const *z
         G[k].first[ng] = (int)tot[k];
     }
     k_az_gather_grp<<<(unsigned)tot[0], 256, 0, st>>>(G[0]);
-    k_az_mapply_grp<<<(unsigned)tot[1], 128, 0, st>>>(G[1]);
+    k_az_mapply_grp<<<(unsigned)tot[1], AZM, (az_mapply_smem<float, 16>()), st>>>(G[1]);
     k_az_addpart_grp<<<(unsigned)tot[2], 256, 0, st>>>(G[2]);
     ps[0]->prof.launches += 3;
     SHTG_CHECK_LAUNCH("k_az_mapply_grp");
