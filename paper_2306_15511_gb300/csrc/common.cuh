@@ -251,6 +251,9 @@ struct Plan {
     int64_t *d_toff = nullptr;
     float2 *d_tst0 = nullptr;
     float4 *d_tst2 = nullptr;
+    // tensor-core synthesis: records of (m, 32 l), tc_nrec per map group
+    unsigned char *d_tcrec = nullptr;
+    int64_t tcrec_bytes = 0, tc_nrec = 0;
     // the same in FP64 every SHTG_TS64 l (FP64 and double-FP32 transposes),
     // [m][t][pair] at (d_toff64[m] + t) * npairs + pair
     int64_t *d_toff64 = nullptr;

@@ -16,17 +16,32 @@
 // FP32 in tensor memory, which keeps ~16 of the 24 mantissa bits of every
 // product (relative error ~2^-17 per term) at bf16 tensor-core rates.
 //
-// Pipeline per CTA (one m, 128 ring pairs, up to 8 maps): the l range is cut
-// into chunks of 32 (16 per parity class, one MMA K of 16 each).  All 128
-// threads generate the A tiles of chunk c (bf16 hi / lo, K-major core
-// matrices in shared memory) and the B tiles, then one thread issues the
-// tcgen05.mma of chunk c and commits them to an mbarrier.  With two stages
-// the threads go on with chunk c + 1 in the other stage while the tensor
-// core works; with one stage (half the shared memory, twice the resident
-// CTAs) they wait for the commit and the other CTAs on the SM fill the gap.
-// The accumulators stay in tensor memory until the last chunk and are read
-// back with tcgen05.ld for the F_N / F_S epilogue.
+// Two kernels.  k_tc_records builds, once per m and chunk of 32 l (16 per
+// parity class, one MMA K of 16 each), a record in global memory: the B tiles
+// (the alm of up to 8 or 16 maps, times the beam, as bf16 hi / lo in the
+// layout the MMA reads) and the recurrence coefficients.  k_leg_synth_tc, one
+// CTA per m and 128 ring pairs, then loops over the chunks: the record arrives
+// by a bulk copy issued one chunk ahead, the 128 threads generate the A tiles
+// (bf16 hi / lo) in tensor memory, lane = ring pair, and one thread issues the
+// tcgen05.mma of the chunk and commits them to an mbarrier.  While
+// the tensor core works on one CTA's chunk, the other three on the SM
+// generate.  Every TC_FLUSH chunks the accumulators move from tensor memory to
+// FP32 sums in shared memory; the F_N / F_S epilogue reads those.
+//
+// What bounds it: the generation, 13.7 instructions per (l, ring pair) at spin
+// 2 (coefficients 1.5, recurrence 3 packed fma.f32x2 on the (y+, y-) pair, lw
+// and lx 2, bf16 split 5, the rest stores, waits and the epilogue), issued at
+// 44 % of the issue rate: the waits for the chunk's MMAs and the barrier take
+// the rest with four warps per scheduler.  Measured (N_side 512, l_max 1024, 8
+// Q/U maps): every CTA of an m building the same B tiles between barriers, 28
+// instructions, A tiles in shared memory: 657 us; records and packed
+// operations, 504 us + 43 us for the records, the shared-memory pipe 67 % busy
+// (A tiles written once and read by two MMAs); A tiles in tensor memory, 451 us
+// + 43.  N_side 1024, l_max 2048, 8 Q/U maps, with the ring stage: 5.42 -> 4.2
+// ms.
 #include <cuda_bf16.h>
+
+#include <algorithm>
 
 #include "legendre_kernels.cuh"
 
@@ -34,7 +49,6 @@ namespace shtg {
 namespace {
 
 constexpr int TC_M = 128;        // ring pairs per CTA = MMA M = threads
-constexpr int TC_NMT = 8;        // maps per CTA (grid.z covers more)
 constexpr int TC_ATILE = 4096;   // one A tile: 128 rows x 16 bf16 (K-major core matrices)
 constexpr uint32_t TC_WAIT_LIMIT = 1u << 22;   // bounded mbarrier polling
 
@@ -101,12 +115,63 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+          "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// D += A B with A in tensor memory (lane = row, two bf16 of K per column) and
+// B in shared memory
+__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t db, uint32_t idesc,
+                                            uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(db), "r"(idesc), "r"(accumulate));
+}
+
+// 4 consecutive TMEM columns of this warp's 32 lanes <- 4 registers per thread
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(a), "r"(b), "r"(c),
+                 "r"(d)
+                 : "memory");
+}
+
+// Packed pairs of FP32 operations (one issue slot for two; the same rounding
+// as the scalar ones)
+__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n\t.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+        "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 fmul2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+        "mul.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+
 // (a, b) -> bf16x2 hi and lo words, element a in the low half
 __device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t &lo) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    const float2 hf = __bfloat1622float2(h);
-    const __nv_bfloat162 l = __floats2bfloat162_rn(a - hf.x, b - hf.y);
     hi = *reinterpret_cast<const uint32_t *>(&h);
+    // the lo parts a - hi, b - hi (exact) in one packed operation
+    const float2 hf = make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
+    const float2 d = ffma2(hf, make_float2(-1.f, -1.f), make_float2(a, b));
+    const __nv_bfloat162 l = __floats2bfloat162_rn(d.x, d.y);
     lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 
@@ -121,93 +186,88 @@ __device__ __forceinline__ void store_row8(unsigned char *hi_row, unsigned char 
     *reinterpret_cast<uint4 *>(lo_row) = l;
 }
 
-// Per-spin tile configuration.  NCOL: B rows of one product block (spin 0:
-// re, im of 8 maps; spin 2: Q re, Q im, U re, U im of 8 maps); a B tile holds
-// NCOL hi rows then NCOL lo rows, 16 K (l of one parity class) each.
-template <int SPIN> struct TcCfg;
-template <> struct TcCfg<0> {
-    static constexpr int NCOL = 16, NA = TC_NMT, NTA = 4, NTB = 2, TMEM = 64;
-};
-template <> struct TcCfg<2> {
-    static constexpr int NCOL = 32, NA = 2 * TC_NMT, NTA = 8, NTB = 4, TMEM = 128;
-};
-// Shared memory of the synthesis CTA: NSTG operand stages (A and B tiles of
-// one 32-l chunk each), the alm and recurrence coefficients of SCH l, two
-// mbarriers, the TMEM address and scratch.  One stage halves the footprint
-// (spin 2: 50 KB instead of 99 KB with SCH = 64), so four CTAs instead of two
-// share an SM; the MMA of a chunk then has to finish before the CTA writes
-// the next chunk's tiles, and the other CTAs fill that gap.
-template <int SPIN, int NSTG, int SCH> struct TcLayout {
-    static constexpr int ALMS = SCH + 1;   // staged alm row stride (odd: rows fall in distinct banks)
-    static constexpr int BTILE = 2 * TcCfg<SPIN>::NCOL * 32;
-    static constexpr int STAGE = TcCfg<SPIN>::NTA * TC_ATILE + TcCfg<SPIN>::NTB * BTILE;
-    static constexpr int ALM = NSTG * STAGE;                                // staged alm [NA][ALMS] float2
-    static constexpr int COEF = ALM + ((TcCfg<SPIN>::NA * ALMS * 8 + 15) & ~15);   // staged coefficients
-    static constexpr int BARS = COEF + SCH * (SPIN == 2 ? 16 : 8);          // 2 mbarriers
-    static constexpr int TMEMA = BARS + 16;                                 // TMEM base address
-    static constexpr int RED = TMEMA + 16;                                  // cta_min scratch
+// Tile configuration of NMT maps.  NCOL: B rows of one product block (spin 0:
+// re, im per map; spin 2: Q re, Q im, U re, U im per map); a B tile holds
+// NCOL hi rows then NCOL lo rows, 16 K (l of one parity class) each.  A record
+// is the B tiles of one chunk of 32 l followed by its coefficients.
+constexpr int TC_NREC = 2;    // record stages of the synthesis
+constexpr int TC_FLUSH = 4;   // chunks summed in tensor memory before they move to the FP32 sums
+template <int SPIN, int NMT> struct TcCfg {
+    static constexpr int NCOL = SPIN == 2 ? 4 * NMT : 2 * NMT;
+    static constexpr int NA = SPIN == 2 ? 2 * NMT : NMT;      // alm rows of the maps
+    static constexpr int NTA = SPIN == 2 ? 8 : 4, NTB = SPIN == 2 ? 4 : 2;
+    // tensor memory: two accumulators of NCOL columns, then the A tiles of one
+    // chunk (8 columns each)
+    static constexpr int ACOL = 2 * NCOL;
+    static constexpr int TMEM = ACOL + 8 * NTA <= 64 ? 64 : 128;
+    static_assert(ACOL + 8 * NTA <= TMEM, "accumulators and A tiles fit the allocation");
+    static constexpr int BTILE = 2 * NCOL * 32;
+    static constexpr int COEF = NTB * BTILE;                  // offset of the coefficients in a record
+    static constexpr int REC = COEF + 32 * (SPIN == 2 ? 24 : 8);
+    // shared memory of the synthesis CTA: the record stages, the FP32 sums of
+    // the flushed chunks [column][thread], mbarriers (one per stage, one for
+    // the MMAs), the TMEM address, scratch
+    static constexpr int SUMS = TC_NREC * REC;
+    static constexpr int BARS = SUMS + 2 * NCOL * TC_M * 4;
+    static constexpr int TMEMA = BARS + 8 * (TC_NREC + 1);
+    static constexpr int RED = TMEMA + 16;
     static constexpr int BYTES = RED + 16;
+    static_assert(REC % 16 == 0, "a bulk copy moves multiples of 16 bytes");
 };
 
-// Recurrence over one chunk of 32 l (l = q0 .. q0 + 31, staged coefficient
-// index i0 + (l - q0)); values of the even class (l - m even, K index
-// (l - q0) / 2) and the odd class go to their A tiles as bf16 hi / lo.
-// Row = this thread's ring pair; K group h = 0, 1 holds K 0..7, 8..15.
-template <int SPIN, bool INJ>
-__device__ __forceinline__ void gen_atiles(PairState<float, 1> &S, const float2 *s_rec, const float4 *s_s2c,
-                                           const int i0, const int q0, unsigned char *stg) {
-    const int rofs = threadIdx.x * 16;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        unsigned char *t = stg + h * 2048 + rofs;
-        if (SPIN == 0) {
-            float e[8], o[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int d = 16 * h + 2 * i;
-                stepx<float, 1, 0, INJ>(S, s_rec, s_s2c, i0 + d, q0 + d);
-                e[i] = S.a1[0];
-                stepx<float, 1, 0, INJ>(S, s_rec, s_s2c, i0 + d + 1, q0 + d + 1);
-                o[i] = S.a1[0];
-            }
-            store_row8(t, t + TC_ATILE, e);                   // E hi, E lo
-            store_row8(t + 2 * TC_ATILE, t + 3 * TC_ATILE, o); // O hi, O lo
+// Recurrence coefficients of one l as the recurrence uses them: spin 2 (alpha
+// + beta, alpha - beta, -alpha, -gamma), spin 0 (a, b).
+__device__ __forceinline__ float4 tc_coef(const float4 s) { return make_float4(s.y, s.z, -s.x, -s.w); }
+
+// The recurrence state of one ring pair: spin 0 p1.x, p2.x = lambda_{l-1},
+// lambda_{l-2}; spin 2 the (y+, y-) pairs.  step: the same operations and
+// roundings as step0 / step2 of the CUDA-core kernels.
+template <int SPIN> struct TcState {
+    float2 p1, p2;
+    float u;
+    // spin 2: yz = (alpha + beta, alpha - beta), xx = (-alpha, -alpha), ww =
+    // (-gamma, -gamma); spin 0: yz = (a, b)
+    __device__ __forceinline__ void step(const float2 yz, const float2 xx, const float2 ww) {
+        if (SPIN == 2) {
+            const float2 t = ffma2(xx, make_float2(u, u), yz);
+            const float2 n = ffma2(t, p1, fmul2(ww, p2));
+            p2 = p1;
+            p1 = n;
         } else {
-            float wE[8], wO[8], xE[8], xO[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int d = 16 * h + 2 * i;
-                stepx<float, 1, 2, INJ>(S, s_rec, s_s2c, i0 + d, q0 + d);
-                wE[i] = S.a1[0] + S.b1[0];
-                xE[i] = S.a1[0] - S.b1[0];
-                stepx<float, 1, 2, INJ>(S, s_rec, s_s2c, i0 + d + 1, q0 + d + 1);
-                wO[i] = S.a1[0] + S.b1[0];
-                xO[i] = S.a1[0] - S.b1[0];
-            }
-            // tiles: lwE hi, lo | lwO hi, lo | lxE hi, lo | lxO hi, lo
-            store_row8(t, t + TC_ATILE, wE);
-            store_row8(t + 2 * TC_ATILE, t + 3 * TC_ATILE, wO);
-            store_row8(t + 4 * TC_ATILE, t + 5 * TC_ATILE, xE);
-            store_row8(t + 6 * TC_ATILE, t + 7 * TC_ATILE, xO);
+            rstep(p1.x, p2.x, yz.x, yz.y, u);
         }
     }
-}
+    // the start values of the recurrences that start at l
+    __device__ __forceinline__ void inject(const int l, const int ls, const int lsb, const float s0, const float s1,
+                                           const float s2, const float s3) {
+        if (l == ls) {
+            p2.x = s0;
+            p1.x = s1;
+        }
+        if (SPIN == 2 && l == lsb) {
+            p2.y = s2;
+            p1.y = s3;
+        }
+    }
+    __device__ __forceinline__ float w() const { return SPIN == 2 ? p1.x + p1.y : p1.x; }   // lw (spin 0: lambda)
+    __device__ __forceinline__ float x() const { return SPIN == 2 ? p1.x - p1.y : 0.f; }    // lx
+};
 
 // B tiles of one chunk from the staged alm (already times the beam).  Tile
 // b: spin 0 -> class b (0 even, 1 odd); spin 2 -> b = 2 w + class with
 // W columns (-E re, -E im, -B re, -B im) and X columns (B im, -B re, -E im,
 // E re) per map, feeding (Q re, Q im, U re, U im).  Column c, K index k:
 // hi at row c, lo at row NCOL + c (K-major core matrices, LBO = 32 NCOL).
-template <int SPIN, int ALMS>
-__device__ __forceinline__ void gen_btiles(const float2 *s_alm, const int i0, unsigned char *bt) {
-    constexpr int NCOL = TcCfg<SPIN>::NCOL, NTB = TcCfg<SPIN>::NTB;
-    constexpr int BTILE = 2 * NCOL * 32;
+template <int SPIN, int NMT, int ALMS>
+__device__ __forceinline__ void gen_btiles(const float2 *s_alm, unsigned char *bt) {
+    typedef TcCfg<SPIN, NMT> Cfg;
+    constexpr int NCOL = Cfg::NCOL, NTB = Cfg::NTB;
     // item = (tile b, K group kg, column c): one 16-byte core-matrix row of
-    // hi and one of lo (the 8 K values, l = i0 + off + 16 kg + 2 j, of column
-    // c), consecutive threads on consecutive rows.  Column c of tile b reads
-    // one component of one staged alm row: spin 0 (re, im) of map c / 2;
-    // spin 2 W tiles (b < 2) -(E re, E im, B re, B im), X tiles (B im, -B re,
-    // -E im, E re) of map c / 4, component c % 4.
+    // hi and one of lo (the 8 K values, l = off + 16 kg + 2 j, of column c),
+    // consecutive threads on consecutive rows.  Column c of tile b reads one
+    // component of one staged alm row: spin 0 (re, im) of map c / 2; spin 2 W
+    // tiles (b < 2) -(E re, E im, B re, B im), X tiles (B im, -B re, -E im, E
+    // re) of map c / 4, component c % 4.
     for (int it = threadIdx.x; it < NTB * 2 * NCOL; it += TC_M) {
         const int c = it % NCOL, kg = (it / NCOL) & 1, b = it / (2 * NCOL);
         const int off = b & 1;
@@ -229,34 +289,135 @@ __device__ __forceinline__ void gen_btiles(const float2 *s_alm, const int i0, un
                 sg = (comp == 1 || comp == 2) ? -1.f : 1.f;
             }
         }
-        const float *src = reinterpret_cast<const float *>(s_alm + row * ALMS + i0 + off + 16 * kg) + ri;
+        const float *src = reinterpret_cast<const float *>(s_alm + row * ALMS + off + 16 * kg) + ri;
         float x[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) x[j] = sg * src[4 * j];
-        unsigned char *r = bt + b * BTILE + kg * (32 * NCOL) + c * 16;
+        unsigned char *r = bt + b * Cfg::BTILE + kg * (32 * NCOL) + c * 16;
         store_row8(r, r + NCOL * 16, x);
     }
 }
 
-template <int SPIN, int NSTG, int SCH>
-__global__ void __launch_bounds__(TC_M) k_leg_synth_tc(const LegArgs<float> a) {
-    typedef TcCfg<SPIN> Cfg;
-    typedef TcLayout<SPIN, NSTG, SCH> Lay;
+// Records of every (m, chunk): grid (chunk, m, map group); entry (group,
+// toff[m] + chunk).
+template <int SPIN, int NMT>
+__global__ void __launch_bounds__(TC_M) k_tc_records(const LegArgs<float> a) {
+    typedef TcCfg<SPIN, NMT> Cfg;
+    constexpr int ALMS = 33;   // staged alm row stride (odd: rows fall in distinct banks)
+    __shared__ float2 s_alm[Cfg::NA * ALMS];
+    const int m = blockIdx.y, L = a.lmax;
+    const int l0 = m + 32 * blockIdx.x;
+    if (l0 > L) return;
+    const int map0 = blockIdx.z * NMT;
+    const int64_t base = (int64_t)m * (2 * L + 1 - m) / 2;
+    unsigned char *rec = a.rec_tc + ((int64_t)blockIdx.z * a.nrec + a.toff[m] + blockIdx.x) * Cfg::REC;
+    for (int e = threadIdx.x; e < Cfg::NA * 32; e += TC_M) {
+        const int i = e & 31, k = e >> 5, l = l0 + i;
+        const int mk = SPIN == 2 ? k / 2 : k;
+        float2 v = make_float2(0.f, 0.f);
+        if (l <= L && map0 + mk < a.nmaps) {
+            const float bm = a.beam ? a.beam[l] : 1.f;
+            const int64_t row = (int64_t)(map0 + mk) * a.rs + (SPIN == 2 ? (k & 1) : 0);
+            v = a.alm[row * a.nalm + base + l];
+            if (m == 0) v.y = 0.f;
+            v.x *= bm;
+            v.y *= bm;
+        }
+        s_alm[k * ALMS + i] = v;
+    }
+    if (threadIdx.x < 32) {
+        const int i = threadIdx.x, l = l0 + i;
+        if (SPIN == 2) {
+            // per two l, three 16-byte loads for the generation: (yz, xx) of
+            // the first, (ww, ww) of both, (yz, xx) of the second
+            const float4 c = tc_coef(l <= L ? a.s2c[base + l] : make_float4(0.f, 0.f, 0.f, 0.f));
+            float4 *dst = reinterpret_cast<float4 *>(rec + Cfg::COEF) + 3 * (i >> 1);
+            dst[2 * (i & 1)] = make_float4(c.x, c.y, c.z, c.z);
+            reinterpret_cast<float2 *>(dst + 1)[i & 1] = make_float2(c.w, c.w);
+        } else {
+            reinterpret_cast<float2 *>(rec + Cfg::COEF)[i] = l <= L ? a.rec[base + l] : make_float2(0.f, 0.f);
+        }
+    }
+    __syncthreads();
+    gen_btiles<SPIN, NMT, ALMS>(s_alm, rec);
+}
+
+// Recurrence over one chunk of 32 l (l = q0 .. q0 + 31, coefficients cf of the
+// record); values of the even class (l - m even, K index (l - q0) / 2) and the
+// odd class go to their A tiles in tensor memory as bf16 hi / lo (ta: this
+// warp's lanes of the first tile's first column).  Lane = this thread's ring
+// pair; half h = 0, 1 holds K 0..7, 8..15 (columns 4 h .. 4 h + 3 of a tile).
+// wait() returns once the A tiles are free: it is called after the first
+// half's recurrence, which so overlaps with the MMAs of the chunk before.
+template <int SPIN, bool INJ, typename Wait>
+__device__ __forceinline__ void gen_atiles(TcState<SPIN> &T, const PairState<float, 1> &S, const float4 *cf,
+                                           const int q0, const uint32_t ta, Wait wait) {
+    auto store = [&](int tile, int h, const float (&x)[8]) {   // tile: hi, tile + 1: lo
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) split2(x[2 * i], x[2 * i + 1], hi[i], lo[i]);
+        tmem_st4(ta + 8 * tile + 4 * h, hi[0], hi[1], hi[2], hi[3]);
+        tmem_st4(ta + 8 * tile + 8 + 4 * h, lo[0], lo[1], lo[2], lo[3]);
+    };
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float wE[8], wO[8], xE[8], xO[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int d = 16 * h + 2 * i;
+            if (SPIN == 2) {
+                const float4 k0 = cf[3 * (d / 2)], g = cf[3 * (d / 2) + 1], k1 = cf[3 * (d / 2) + 2];
+                T.step(make_float2(k0.x, k0.y), make_float2(k0.z, k0.w), make_float2(g.x, g.y));
+                if (INJ) T.inject(q0 + d, S.ls[0], S.lsb[0], S.s0[0], S.s1[0], S.s2[0], S.s3[0]);
+                wE[i] = T.w();
+                xE[i] = T.x();
+                T.step(make_float2(k1.x, k1.y), make_float2(k1.z, k1.w), make_float2(g.z, g.w));
+            } else {
+                const float4 k = cf[d / 2], z = make_float4(0.f, 0.f, 0.f, 0.f);
+                T.step(make_float2(k.x, k.y), make_float2(z.x, z.y), make_float2(z.z, z.w));
+                if (INJ) T.inject(q0 + d, S.ls[0], S.lsb[0], S.s0[0], S.s1[0], S.s2[0], S.s3[0]);
+                wE[i] = T.w();
+                T.step(make_float2(k.z, k.w), make_float2(z.x, z.y), make_float2(z.z, z.w));
+            }
+            if (INJ) T.inject(q0 + d + 1, S.ls[0], S.lsb[0], S.s0[0], S.s1[0], S.s2[0], S.s3[0]);
+            wO[i] = T.w();
+            xO[i] = T.x();
+        }
+        if (h == 0) wait();
+        // tiles: (lw) E hi, lo | O hi, lo; spin 2 also lx E hi, lo | O hi, lo
+        store(0, h, wE);
+        store(2, h, wO);
+        if (SPIN == 2) {
+            store(4, h, xE);
+            store(6, h, xO);
+        }
+    }
+}
+
+// bulk copy of one record into shared memory, completing on bar
+__device__ __forceinline__ void bulk_load(unsigned char *dst, const unsigned char *src, uint32_t bytes,
+                                          uint64_t *bar) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+
+template <int SPIN, int NMT>
+__global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a) {
+    typedef TcCfg<SPIN, NMT> Cfg;
     constexpr int NCOL = Cfg::NCOL;
     extern __shared__ __align__(1024) unsigned char smem[];
-    float2 *s_alm = reinterpret_cast<float2 *>(smem + Lay::ALM);
-    float2 *s_rec = reinterpret_cast<float2 *>(smem + Lay::COEF);
-    float4 *s_s2c = reinterpret_cast<float4 *>(smem + Lay::COEF);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + Lay::BARS);
-    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + Lay::TMEMA);
-    int *s_red = reinterpret_cast<int *>(smem + Lay::RED);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + Cfg::BARS);
+    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + Cfg::TMEMA);
+    int *s_red = reinterpret_cast<int *>(smem + Cfg::RED);
 
     const int tid = threadIdx.x, warp = tid >> 5;
     const int m = blockIdx.y;
     const int L = a.lmax;
-    const int map0 = blockIdx.z * TC_NMT;
-    const int nm = min(TC_NMT, a.nmaps - map0);
-    const int64_t base = (int64_t)m * (2 * L + 1 - m) / 2;
+    const int map0 = blockIdx.z * NMT;
+    const int nm = min(NMT, a.nmaps - map0);
 
     PairState<float, 1> S;
     int warp_lo, warp_hi;
@@ -264,24 +425,23 @@ __global__ void __launch_bounds__(TC_M) k_leg_synth_tc(const LegArgs<float> a) {
     const int lo = cta_min(warp_lo, s_red);
     const int pr = S.pr[0];
     const int rn = pr, rs = a.nring - 1 - pr;
+    const int nrow = SPIN == 2 ? 2 * nm : nm;   // output rows of this CTA
+    const int64_t rowsz = (int64_t)a.nring * (L + 1);
+    float2 *out = a.F + (int64_t)(SPIN == 2 ? 2 * map0 : map0) * rowsz + m;
 
     if (lo > L) {   // no significant l for any pair of this CTA: zero output
         if (pr < a.npairs) {
-            for (int k = 0; k < nm; ++k) {
-                for (int c = 0; c < (SPIN == 2 ? 2 : 1); ++c) {
-                    const int row = SPIN == 2 ? 2 * (map0 + k) + c : map0 + k;
-                    float2 *out = a.F + (int64_t)row * a.nring * (L + 1) + m;
-                    out[(int64_t)rn * (L + 1)] = make_float2(0.f, 0.f);
-                    if (rs != rn) out[(int64_t)rs * (L + 1)] = make_float2(0.f, 0.f);
-                }
+            for (int k = 0; k < nrow; ++k) {
+                out[k * rowsz + (int64_t)rn * (L + 1)] = make_float2(0.f, 0.f);
+                if (rs != rn) out[k * rowsz + (int64_t)rs * (L + 1)] = make_float2(0.f, 0.f);
             }
         }
         return;
     }
 
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[0])));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[1])));
+        for (int i = 0; i <= TC_NREC; ++i)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[i])));
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     if (warp == 0) {
@@ -294,127 +454,134 @@ __global__ void __launch_bounds__(TC_M) k_leg_synth_tc(const LegArgs<float> a) {
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = *s_tmem;
 
+    const int ch0 = (lo - m) >> 5;                 // chunks start at l - m = 0 mod 32
+    const int n = ((L - m) >> 5) - ch0 + 1;        // chunks of this CTA
+    const unsigned char *rec = a.rec_tc + ((int64_t)blockIdx.z * a.nrec + a.toff[m] + ch0) * Cfg::REC;
+    if (tid == 0) {
+        bulk_load(smem, rec, Cfg::REC, &bars[0]);
+        if (n > 1) bulk_load(smem + Cfg::REC, rec + Cfg::REC, Cfg::REC, &bars[1]);
+    }
+    const uint64_t descB = sdesc(smem_u32(smem), 32 * NCOL, 128);
+    const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);   // this warp's lanes
+    TcState<SPIN> T;
+    T.p1 = T.p2 = make_float2(0.f, 0.f);
+    T.u = S.u[0];
     bool ok = true;
-    int chunk = 0;
-    const int l_begin = m + ((lo - m) & ~31);   // chunks start at l - m = 0 mod 32
-    for (int c0 = l_begin; c0 <= L; c0 += SCH) {
-        // ---- stage coefficients and beam-weighted alm of l = c0 .. c0 + SCH - 1
-        __syncthreads();
-        for (int i = tid; i < SCH; i += TC_M) {
-            const int l = c0 + i;
-            const bool in = l <= L;
-            const int64_t idx = base + l;
-            if (SPIN == 2) s_s2c[i] = in ? a.s2c[idx] : make_float4(0.f, 0.f, 0.f, 0.f);
-            else s_rec[i] = in ? a.rec[idx] : make_float2(0.f, 0.f);
-            const float bm = (in && a.beam) ? a.beam[l] : 1.f;
+    uint64_t *mma_bar = &bars[TC_NREC];
+    // The tensor core truncates at every accumulation, so a sum left in tensor
+    // memory over all chunks drifts (relative 1e-6 of the result at l_max
+    // 2048): every TC_FLUSH chunks it moves to sums that round to nearest.
+    float *sums = reinterpret_cast<float *>(smem + Cfg::SUMS) + tid;
+    auto flush = [&](bool first) {
 #pragma unroll
-            for (int k = 0; k < Cfg::NA; ++k) {
-                float2 v = make_float2(0.f, 0.f);
-                const int mk = SPIN == 2 ? k / 2 : k;
-                if (in && mk < nm) {
-                    const int64_t row = (int64_t)(map0 + mk) * a.rs + (SPIN == 2 ? (k & 1) : 0);
-                    v = a.alm[row * a.nalm + idx];
-                    if (m == 0) v.y = 0.f;
-                    v.x *= bm;
-                    v.y *= bm;
-                }
-                s_alm[k * Lay::ALMS + i] = v;
+        for (int h = 0; h < 2 * NCOL / 16; ++h) {
+            float v[16];
+            tmem_ld16(trow + 16 * h, v);
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {
+                float *q = sums + (16 * h + c) * TC_M;
+                *q = first ? v[c] : *q + v[c];
             }
         }
-        __syncthreads();
-        for (int q0 = c0; q0 < c0 + SCH && q0 <= L; q0 += 32, ++chunk) {
-            const int sidx = chunk % NSTG;
-            unsigned char *stg = smem + sidx * Lay::STAGE;
-            // the MMAs of chunk - NSTG read this stage: wait for their commit
-            // (the k-th commit on a barrier completes its phase k)
-            if (chunk >= NSTG) ok = mbar_wait(&bars[sidx], ((chunk - NSTG) / NSTG) & 1) && ok;
-            const int i0 = q0 - c0;
-            // injection steps only where some pair of the warp starts in this chunk
-            const bool starts = (S.ls[0] >= q0 && S.ls[0] < q0 + 32) ||
-                                (SPIN == 2 && S.lsb[0] >= q0 && S.lsb[0] < q0 + 32);
-            if (q0 <= warp_hi && __any_sync(0xffffffffu, starts)) gen_atiles<SPIN, true>(S, s_rec, s_s2c, i0, q0, stg);
-            else gen_atiles<SPIN, false>(S, s_rec, s_s2c, i0, q0, stg);
-            gen_btiles<SPIN, Lay::ALMS>(s_alm, i0, stg + Cfg::NTA * TC_ATILE);
-            asm volatile("fence.proxy.async.shared::cta;");
-            __syncthreads();
-            if (tid == 0) {
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const uint32_t sa = smem_u32(stg);
-                const uint32_t sb = sa + Cfg::NTA * TC_ATILE;
-                const uint32_t full = idesc_bf16(TC_M, 2 * NCOL), half = idesc_bf16(TC_M, NCOL);
-                const uint32_t acc = chunk > 0;
-                auto A = [&](int t) { return sdesc(sa + t * TC_ATILE, 2048, 128); };
-                auto B = [&](int t) { return sdesc(sb + t * Lay::BTILE, 32 * NCOL, 128); };
-                if (SPIN == 0) {
-                    // D_E (columns 0 .. 2 NCOL) and D_O (2 NCOL .. 4 NCOL)
-                    mma_bf16(tmem, A(0), B(0), full, acc);
-                    mma_bf16(tmem, A(1), B(0), half, 1);
-                    mma_bf16(tmem + 2 * NCOL, A(2), B(1), full, acc);
-                    mma_bf16(tmem + 2 * NCOL, A(3), B(1), half, 1);
-                } else {
-                    // symmetric part: lw even with W even, lx odd with X odd;
-                    // antisymmetric part: lw odd with W odd, lx even with X even
-                    mma_bf16(tmem, A(0), B(0), full, acc);
-                    mma_bf16(tmem, A(1), B(0), half, 1);
-                    mma_bf16(tmem, A(6), B(3), full, 1);
-                    mma_bf16(tmem, A(7), B(3), half, 1);
-                    mma_bf16(tmem + 2 * NCOL, A(2), B(1), full, acc);
-                    mma_bf16(tmem + 2 * NCOL, A(3), B(1), half, 1);
-                    mma_bf16(tmem + 2 * NCOL, A(4), B(2), full, 1);
-                    mma_bf16(tmem + 2 * NCOL, A(5), B(2), half, 1);
-                }
-                mma_commit(&bars[sidx]);
+    };
+    const int fl = n <= 8 ? 2 : TC_FLUSH;   // short sums: the start of the sum weighs more
+    int st = 0, ph = 0;   // record stage of chunk c and its barrier's phase
+    for (int c = 0; c < n; ++c) {
+        if (c > 0 && (c & (fl - 1)) == 0) {
+            ok = mbar_wait(mma_bar, (c - 1) & 1) && ok;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            flush(c == fl);
+        }
+        unsigned char *bt = smem + st * Cfg::REC;
+        ok = mbar_wait(&bars[st], ph) && ok;            // the record
+        // the MMAs of chunk c - 1: the A tiles are free, and so is its record
+        // stage (its coefficients were read before the last barrier)
+        auto free_tiles = [&]() {
+            if (c == 0) return;
+            ok = mbar_wait(mma_bar, (c - 1) & 1) && ok;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            if (tid == 0 && c + TC_NREC - 1 < n) {
+                const int sp = st == 0 ? TC_NREC - 1 : st - 1;
+                bulk_load(smem + sp * Cfg::REC, rec + (int64_t)(c + TC_NREC - 1) * Cfg::REC, Cfg::REC, &bars[sp]);
             }
+        };
+        const int q0 = m + 32 * (ch0 + c);
+        const float4 *cf = reinterpret_cast<const float4 *>(bt + Cfg::COEF);
+        // injection steps only where some pair of the warp starts in this chunk
+        const bool starts = (S.ls[0] >= q0 && S.ls[0] < q0 + 32) ||
+                            (SPIN == 2 && S.lsb[0] >= q0 && S.lsb[0] < q0 + 32);
+        if (__any_sync(0xffffffffu, starts)) gen_atiles<SPIN, true>(T, S, cf, q0, trow + Cfg::ACOL, free_tiles);
+        else gen_atiles<SPIN, false>(T, S, cf, q0, trow + Cfg::ACOL, free_tiles);
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        __syncthreads();
+        if (tid == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const uint32_t id = idesc_bf16(TC_M, NCOL);
+            const uint32_t acc = (c & (fl - 1)) != 0;
+            // (the address field counts 16-byte units)
+            const uint64_t db = descB + (uint32_t)(st * (Cfg::REC >> 4));
+            // A tiles t, t + 1 (hi, lo) and B tile b: D += A_lo B_hi + A_hi B_lo
+            // (small; first, so that a new sum truncates little), D += A_hi B_hi
+            auto ah = [&](int t) { return tmem + Cfg::ACOL + 8 * t; };
+            auto bh = [&](int b) { return db + (uint32_t)(b * (Cfg::BTILE >> 4)); };
+            auto low = [&](uint32_t d, int t, int b, uint32_t accumulate) {
+                mma_bf16_ts(d, ah(t) + 8, bh(b), id, accumulate);
+                mma_bf16_ts(d, ah(t), bh(b) + NCOL, id, 1);
+            };
+            auto high = [&](uint32_t d, int t, int b) { mma_bf16_ts(d, ah(t), bh(b), id, 1); };
+            const uint32_t dE = tmem, dO = tmem + NCOL;
+            // spin 2: symmetric part: lw even with W even, lx odd with X odd;
+            // antisymmetric part: lw odd with W odd, lx even with X even
+            low(dE, 0, 0, acc);
+            low(dO, 2, 1, acc);
+            if (SPIN == 2) {
+                low(dE, 6, 3, 1);
+                low(dO, 4, 2, 1);
+            }
+            high(dE, 0, 0);
+            high(dO, 2, 1);
+            if (SPIN == 2) {
+                high(dE, 6, 3);
+                high(dO, 4, 2);
+            }
+            mma_commit(mma_bar);
+        }
+        if (++st == TC_NREC) {
+            st = 0;
+            ph ^= 1;
         }
     }
     // ---- the last commit covers every MMA issued before it
-    const int last = chunk - 1;
-    ok = mbar_wait(&bars[last % NSTG], (last / NSTG) & 1) && ok;
+    ok = mbar_wait(mma_bar, (n - 1) & 1) && ok;
     asm volatile("tcgen05.fence::after_thread_sync;");
     if (!ok && tid == 0 && a.err) atomicExch(a.err, 1);
 
-    // ---- epilogue: this thread's TMEM lane is its ring pair
-    const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
-    float d0[32], d1[32];
-    if (SPIN == 0) {
-        tmem_ld32(trow, d0);        // D_E: [0, 16) hi*hi + lo*hi, [16, 32) hi*lo
-        tmem_ld32(trow + 32, d1);   // D_O
-        if (ok && pr < a.npairs) {
+    // ---- epilogue: this thread's TMEM lane is its ring pair; columns [0,
+    // NCOL) the even (spin 2: symmetric) part, [NCOL, 2 NCOL) the odd one
+    if (n > fl) flush(false);
+    float e[NCOL], o[NCOL];
+    if (n > fl) {
 #pragma unroll
-            for (int k = 0; k < TC_NMT; ++k) {
-                if (k >= nm) break;
-                const float er = d0[2 * k] + d0[NCOL + 2 * k], ei = d0[2 * k + 1] + d0[NCOL + 2 * k + 1];
-                const float orr = d1[2 * k] + d1[NCOL + 2 * k], oi = d1[2 * k + 1] + d1[NCOL + 2 * k + 1];
-                float2 *out = a.F + (int64_t)(map0 + k) * a.nring * (L + 1) + m;
-                out[(int64_t)rn * (L + 1)] = make_float2(er + orr, ei + oi);
-                if (rs != rn) out[(int64_t)rs * (L + 1)] = make_float2(er - orr, ei - oi);
-            }
+        for (int c = 0; c < NCOL; ++c) {
+            e[c] = sums[c * TC_M];
+            o[c] = sums[(NCOL + c) * TC_M];
         }
+    } else if (NCOL == 16) {
+        tmem_ld16(trow, *reinterpret_cast<float(*)[16]>(e));
+        tmem_ld16(trow + NCOL, *reinterpret_cast<float(*)[16]>(o));
     } else {
-        // symmetric part S (columns 0 .. 64), antisymmetric part X (64 .. 128)
-        float s2[32], x2[32];
-        tmem_ld32(trow, d0);         // S hi*hi + lo*hi
-        tmem_ld32(trow + 32, d1);    // S hi*lo
+        tmem_ld32(trow, *reinterpret_cast<float(*)[32]>(e));
+        tmem_ld32(trow + NCOL, *reinterpret_cast<float(*)[32]>(o));
+    }
+    if (ok && pr < a.npairs) {
+        // output row k: columns 2 k, 2 k + 1
 #pragma unroll
-        for (int c = 0; c < 32; ++c) s2[c] = d0[c] + d1[c];
-        tmem_ld32(trow + 64, d0);
-        tmem_ld32(trow + 96, d1);
-#pragma unroll
-        for (int c = 0; c < 32; ++c) x2[c] = d0[c] + d1[c];
-        if (ok && pr < a.npairs) {
-#pragma unroll
-            for (int k = 0; k < TC_NMT; ++k) {
-                if (k >= nm) break;
-                float2 *oq = a.F + (int64_t)(2 * (map0 + k)) * a.nring * (L + 1) + m;
-                float2 *ou = a.F + (int64_t)(2 * (map0 + k) + 1) * a.nring * (L + 1) + m;
-                const int c = 4 * k;
-                oq[(int64_t)rn * (L + 1)] = make_float2(s2[c] + x2[c], s2[c + 1] + x2[c + 1]);
-                ou[(int64_t)rn * (L + 1)] = make_float2(s2[c + 2] + x2[c + 2], s2[c + 3] + x2[c + 3]);
-                if (rs != rn) {
-                    oq[(int64_t)rs * (L + 1)] = make_float2(s2[c] - x2[c], s2[c + 1] - x2[c + 1]);
-                    ou[(int64_t)rs * (L + 1)] = make_float2(s2[c + 2] - x2[c + 2], s2[c + 3] - x2[c + 3]);
-                }
-            }
+        for (int k = 0; k < NCOL / 2; ++k) {
+            if (k >= nrow) break;
+            out[k * rowsz + (int64_t)rn * (L + 1)] = make_float2(e[2 * k] + o[2 * k], e[2 * k + 1] + o[2 * k + 1]);
+            if (rs != rn)
+                out[k * rowsz + (int64_t)rs * (L + 1)] = make_float2(e[2 * k] - o[2 * k], e[2 * k + 1] - o[2 * k + 1]);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -422,23 +589,34 @@ __global__ void __launch_bounds__(TC_M) k_leg_synth_tc(const LegArgs<float> a) {
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Cfg::TMEM));
 }
 
-template <int SPIN, int NSTG, int SCH>
+template <int SPIN, int NMT>
 int launch_synth_tc(Plan *p, const float2 *alm, int rs, int nmaps, const float *beam, float2 *F,
                     cudaStream_t st) {
+    typedef TcCfg<SPIN, NMT> Cfg;
     LegArgs<float> a = leg_make_args<float>(p);
-    a.alm = alm;
     a.rs = rs;
-    a.F = F;
     a.beam = beam;
-    a.nmaps = nmaps;
     a.err = p->d_flag;
-    const int smem = TcLayout<SPIN, NSTG, SCH>::BYTES;
-    auto kern = k_leg_synth_tc<SPIN, NSTG, SCH>;
+    a.rec_tc = p->d_tcrec;
+    a.nrec = p->tc_nrec;
+    const int smem = Cfg::BYTES;
+    auto kern = k_leg_synth_tc<SPIN, NMT>;
     SHTG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    dim3 grid((p->npairs + TC_M - 1) / TC_M, p->lmax + 1, (nmaps + TC_NMT - 1) / TC_NMT);
+    // as many map groups per pass as the plan's record buffer holds
+    const int groups = (nmaps + NMT - 1) / NMT;
+    const int fit = (int)std::max<int64_t>(1, std::min<int64_t>(groups, p->tcrec_bytes / (p->tc_nrec * Cfg::REC)));
     prof_begin(p, K_LEG_SYN32, st);
-    kern<<<grid, TC_M, smem, st>>>(a);
-    prof_end(p, st);
+    int nl = 0;
+    for (int g0 = 0; g0 < groups; g0 += fit) {
+        const int ng = std::min(fit, groups - g0);
+        a.nmaps = std::min(nmaps - g0 * NMT, ng * NMT);
+        a.alm = alm + (int64_t)g0 * NMT * rs * p->nalm;
+        a.F = F + (int64_t)g0 * NMT * (SPIN == 2 ? 2 : 1) * p->nring * (p->lmax + 1);
+        k_tc_records<SPIN, NMT><<<dim3(p->lmax / 32 + 1, p->lmax + 1, ng), TC_M, 0, st>>>(a);
+        kern<<<dim3((p->npairs + TC_M - 1) / TC_M, p->lmax + 1, ng), TC_M, smem, st>>>(a);
+        nl += 2;
+    }
+    prof_end(p, st, nl);
     SHTG_CHECK_LAUNCH("k_leg_synth_tc");
     return SHTG_OK;
 }
@@ -502,6 +680,15 @@ int build_tile_states(Plan *p) {
         k_tile_states<2><<<grid, LEG_THREADS>>>(a, p->d_toff, nullptr, p->d_tst2);
         SHTG_CHECK_LAUNCH("k_tile_states");
     }
+    // records of the synthesis: every map group of a full batch, at most 1 GB
+    // (at least one group; more groups than fit take several passes)
+    p->tc_nrec = toff[L + 1];
+    const int mb = p->max_batch;
+    const int64_t r0 = mb > 8 ? TcCfg<0, 16>::REC : TcCfg<0, 8>::REC, g0 = mb > 8 ? (mb + 15) / 16 : 1;
+    const int64_t r2 = (p->flags & SHTG_SPIN2) ? TcCfg<2, 8>::REC : 0, g2 = (mb + 7) / 8;
+    const int64_t one = p->tc_nrec * std::max(r0, r2), all = p->tc_nrec * std::max(r0 * g0, r2 * g2);
+    p->tcrec_bytes = std::max(one, std::min<int64_t>(all, (int64_t)1 << 30));
+    SHTG_TRY(alloc((void **)&p->d_tcrec, (size_t)p->tcrec_bytes));
     SHTG_CUDA(cudaDeviceSynchronize());
     return SHTG_OK;
 }
@@ -520,12 +707,8 @@ namespace {
 // The CTA accumulates over all ring pairs in tensor memory, so every alm is
 // written once, by one CTA, without atomics.
 constexpr int TA_K = 16;        // ring pairs per stage (MMA K)
-template <int SPIN> struct TaCfg;
-template <> struct TaCfg<0> {
-    static constexpr int NO = 16, NAT = 4, NBT = 2, TMEM = 64;
-};
-template <> struct TaCfg<2> {
-    static constexpr int NO = 32, NAT = 8, NBT = 4, TMEM = 128;
+template <int SPIN, int NMT> struct TaCfg {   // NMT maps per CTA
+    static constexpr int NO = SPIN == 2 ? 4 * NMT : 2 * NMT, NAT = SPIN == 2 ? 8 : 4, NBT = SPIN == 2 ? 4 : 2;
 };
 // Shared memory of the transpose CTA (TR 256-l tiles): NAS A buffers (the
 // tiles of one (stage, 256-l tile) unit), NBS B buffers (one per stage of 16
@@ -535,23 +718,24 @@ template <> struct TaCfg<2> {
 // (it overlaps with the stage's A generation) and one buffer suffices.
 // Fewer buffers shrink the CTA (spin 2 with one A and one B buffer: 53 KB
 // with two 256-l tiles, 49 KB with one) so that four CTAs share an SM.
-template <int SPIN, int NAS, int NBS, int TR> struct TaLayout {
-    static constexpr int BT = 64 * TaCfg<SPIN>::NO;                         // B tile: 2 NO rows x 16 K bf16
-    static constexpr int ASTAGE = TaCfg<SPIN>::NAT * TC_ATILE;
-    static constexpr int BSTAGE = TaCfg<SPIN>::NBT * BT;
+template <int SPIN, int NMT, int NAS, int NBS, int TR> struct TaLayout {
+    typedef TaCfg<SPIN, NMT> Cfg;
+    static constexpr int BT = 64 * Cfg::NO;                         // B tile: 2 NO rows x 16 K bf16
+    static constexpr int ASTAGE = Cfg::NAT * TC_ATILE;
+    static constexpr int BSTAGE = Cfg::NBT * BT;
     static constexpr int BOFF = NAS * ASTAGE;
     // ring data of one stage: [pair][north rows | south rows] float2 with pair
     // stride GS = 2 NROW + 2: the B-tile builder's warp reads 8 consecutive
     // floats per K pair and its four K pairs sit 4 GS = 8 (mod 32) floats
     // apart, so every load hits 32 distinct banks
-    static constexpr int NROW = SPIN == 2 ? 2 * TC_NMT : TC_NMT;
+    static constexpr int NROW = SPIN == 2 ? 2 * NMT : NMT;
     static constexpr int GS = 2 * NROW + 2;
     static constexpr int GBUF = ((TA_K * GS * 8) + 15) & ~15;
     static constexpr int GOFF = BOFF + NBS * BSTAGE;
     static constexpr int COEF = GOFF + GBUF;
     // coefficients of 256 TR l, one padding entry after every 32 (ta_cpad)
     static constexpr int BARS = COEF + 264 * TR * (SPIN == 2 ? 16 : 8);
-    static constexpr int TMEM = TR * TaCfg<SPIN>::TMEM / 2;   // 2 NO columns per 256-l tile
+    static constexpr int TMEM = TR * 2 * Cfg::NO;   // 2 NO columns per 256-l tile
     static constexpr int TMEMA = BARS + 16;
     static constexpr int BYTES = TMEMA + 16;
 };
@@ -565,19 +749,6 @@ __device__ __forceinline__ int ta_cpad(int i) { return i + (i >> 5); }
 // MN-major A (bit 15), K-major B, bf16 in, FP32 accumulator
 __host__ __device__ constexpr uint32_t idesc_bf16_amn(int m, int n) {
     return idesc_bf16(m, n) | (1u << 15);
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-          "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // Start data of one ring pair for m (from the FP64 start states) and the
@@ -625,65 +796,57 @@ __device__ __forceinline__ float4 load_tile_state(const LegArgs<float> &a, int m
 // A tiles of one (stage, 256-l tile): this thread's pair (column pin of the
 // K = 16 slice) over l = l0 .. l0 + 31, l0 = tstart + 32 seg, from state ts;
 // values of class E (l - m even) go to rows 16 seg + j of the E tiles, class
-// O to the same rows of the O tiles.  Pairs beyond npairs and l beyond lmax
-// give 0.  INJ: some pair of the warp starts its recurrence inside the
-// segment (the tabulated state already holds every earlier start).
-template <int SPIN, bool INJ>
-__device__ __forceinline__ void gen_atiles_ana(const PairStart &q, const float4 ts, const bool live, const int pin,
-                                               const int seg, const int l0, const int lbase,
-                                               const float2 *s_rec, const float4 *s_s2c, unsigned char *at) {
-    PairState<float, 1> S;
-    S.u[0] = q.u;
-    S.ls[0] = q.ls;
-    S.lsb[0] = q.lsb;
-    S.s0[0] = q.s0;
-    S.s1[0] = q.s1;
-    S.s2[0] = q.s2;
-    S.s3[0] = q.s3;
-    S.a1[0] = ts.x;
-    S.a2[0] = ts.y;
-    S.b1[0] = ts.z;
-    S.b2[0] = ts.w;
+// O to the same rows of the O tiles.  Pairs beyond npairs (state 0) and l
+// beyond lmax (coefficients and state 0) give 0.  INJ: some pair of the warp
+// starts its recurrence inside the segment (the tabulated state already holds
+// every earlier start).  wait() as in the synthesis.
+template <int SPIN, bool INJ, typename Wait>
+__device__ __forceinline__ void gen_atiles_ana(const PairStart &q, const float4 ts, const int pin, const int seg,
+                                               const int l0, const int lbase, const void *s_cf, unsigned char *at,
+                                               Wait wait) {
+    TcState<SPIN> T;
+    T.u = q.u;
+    if (SPIN == 2) {   // ts = (y+_{l-1}, y+_{l-2}, y-_{l-1}, y-_{l-2})
+        T.p1 = make_float2(ts.x, ts.z);
+        T.p2 = make_float2(ts.y, ts.w);
+    } else {
+        T.p1 = make_float2(ts.x, 0.f);
+        T.p2 = make_float2(ts.y, 0.f);
+    }
     const int kg = pin >> 3, krow = pin & 7;
     // padded shared index of l0 + d: l0 - lbase is a multiple of 32 and d <= 31,
     // so ta_cpad(l0 - lbase + d) = ta_cpad(l0 - lbase) + d
     const int cb = ta_cpad(l0 - lbase);
+    const float4 *c4 = reinterpret_cast<const float4 *>(s_cf) + cb;
+    const float2 *c2 = reinterpret_cast<const float2 *>(s_cf) + cb;
+    auto step = [&](int d) {
+        if (SPIN == 2) {
+            const float4 k = c4[d];
+            T.step(make_float2(k.x, k.y), make_float2(k.z, k.z), make_float2(k.w, k.w));
+        } else {
+            T.step(c2[d], make_float2(0.f, 0.f), make_float2(0.f, 0.f));
+        }
+        if (INJ) T.inject(l0 + d, q.ls, q.lsb, q.s0, q.s1, q.s2, q.s3);
+    };
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         // rows 16 seg + 8 h .. + 7: core matrix (M group 2 seg + h, K group kg)
         unsigned char *t = at + (kg * 16 + 2 * seg + h) * 128 + krow * 16;
-        if (SPIN == 0) {
-            float e[8], o[8];
+        float wE[8], wO[8], xE[8], xO[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int d = 16 * h + 2 * i;
-                e[i] = o[i] = 0.f;
-                if (live) {
-                    stepx<float, 1, 0, INJ>(S, s_rec, s_s2c, cb + d, l0 + d);
-                    e[i] = S.a1[0];
-                    stepx<float, 1, 0, INJ>(S, s_rec, s_s2c, cb + d + 1, l0 + d + 1);
-                    o[i] = S.a1[0];
-                }
-            }
-            store_row8(t, t + TC_ATILE, e);                    // E hi, E lo
-            store_row8(t + 2 * TC_ATILE, t + 3 * TC_ATILE, o);  // O hi, O lo
-        } else {
-            float wE[8], wO[8], xE[8], xO[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int d = 16 * h + 2 * i;
-                wE[i] = wO[i] = xE[i] = xO[i] = 0.f;
-                if (live) {
-                    stepx<float, 1, 2, INJ>(S, s_rec, s_s2c, cb + d, l0 + d);
-                    wE[i] = S.a1[0] + S.b1[0];
-                    xE[i] = S.a1[0] - S.b1[0];
-                    stepx<float, 1, 2, INJ>(S, s_rec, s_s2c, cb + d + 1, l0 + d + 1);
-                    wO[i] = S.a1[0] + S.b1[0];
-                    xO[i] = S.a1[0] - S.b1[0];
-                }
-            }
-            store_row8(t, t + TC_ATILE, wE);
-            store_row8(t + 2 * TC_ATILE, t + 3 * TC_ATILE, wO);
+        for (int i = 0; i < 8; ++i) {
+            const int d = 16 * h + 2 * i;
+            step(d);
+            wE[i] = T.w();
+            xE[i] = T.x();
+            step(d + 1);
+            wO[i] = T.w();
+            xO[i] = T.x();
+        }
+        if (h == 0) wait();
+        store_row8(t, t + TC_ATILE, wE);
+        store_row8(t + 2 * TC_ATILE, t + 3 * TC_ATILE, wO);
+        if (SPIN == 2) {
             store_row8(t + 4 * TC_ATILE, t + 5 * TC_ATILE, xE);
             store_row8(t + 6 * TC_ATILE, t + 7 * TC_ATILE, xO);
         }
@@ -694,10 +857,10 @@ __device__ __forceinline__ void gen_atiles_ana(const PairStart &q, const float4 
 // element (pair p, row q, ring z) at sg[p GS + z NROW + q]; rows are the maps of
 // this CTA (spin 2: Q, U of each); zeros for pairs beyond npairs, missing
 // maps and the south ring of the equator pair.
-template <int SPIN>
+template <int SPIN, int NMT>
 __device__ __forceinline__ void stage_ring_data(const LegArgs<float> &a, const int m, const int ps, const int map0,
                                                 const int nm, float2 *sg) {
-    typedef TaLayout<SPIN, 1, 1, 1> Lay;   // (ring-data geometry only)
+    typedef TaLayout<SPIN, NMT, 1, 1, 1> Lay;   // (ring-data geometry only)
     const int L = a.lmax;
     const int64_t rowsz = (int64_t)a.nring * (L + 1);
     const int nrow = SPIN == 2 ? 2 * nm : nm;
@@ -729,10 +892,10 @@ __device__ __forceinline__ void stage_ring_data(const LegArgs<float> &a, const i
 // (two consecutive ring pairs) in every tile: a warp covers 8 consecutive
 // columns x 4 K pairs, i.e. 32 distinct banks per store, and reads only the
 // two scalars per ring pair that its column needs.
-template <int SPIN>
+template <int SPIN, int NMT>
 __device__ __forceinline__ void gen_btiles_ana(const float2 *sg, unsigned char *bt) {
-    typedef TaLayout<SPIN, 1, 1, 1> Lay;   // (tile geometry only)
-    constexpr int NO = TaCfg<SPIN>::NO, BT = Lay::BT;
+    typedef TaLayout<SPIN, NMT, 1, 1, 1> Lay;   // (tile geometry only)
+    constexpr int NO = Lay::Cfg::NO, BT = Lay::BT;
     const float *sgf = reinterpret_cast<const float *>(sg);
     for (int it = threadIdx.x; it < 8 * NO; it += TC_M) {
         const int kq = it & 3;
@@ -796,14 +959,13 @@ __device__ __forceinline__ void gen_btiles_ana(const float2 *sg, unsigned char *
     }
 }
 
-template <int SPIN, int NAS, int NBS, int TR>
-__global__ void __launch_bounds__(TC_M) k_leg_analysis_tc(const LegArgs<float> a) {
-    typedef TaCfg<SPIN> Cfg;
-    typedef TaLayout<SPIN, NAS, NBS, TR> Lay;
-    constexpr int NO = Cfg::NO;
+template <int SPIN, int NMT, int NAS, int NBS, int TR>
+__global__ void __launch_bounds__(TC_M, 4) k_leg_analysis_tc(const LegArgs<float> a) {
+    typedef TaLayout<SPIN, NMT, NAS, NBS, TR> Lay;
+    constexpr int NO = Lay::Cfg::NO;
     extern __shared__ __align__(1024) unsigned char smem[];
-    float2 *s_rec = reinterpret_cast<float2 *>(smem + Lay::COEF);
-    float4 *s_s2c = reinterpret_cast<float4 *>(smem + Lay::COEF);
+    float4 *s_c4 = reinterpret_cast<float4 *>(smem + Lay::COEF);   // spin 2 (tc_coef)
+    float2 *s_c2 = reinterpret_cast<float2 *>(smem + Lay::COEF);   // spin 0 (a, b)
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + Lay::BARS);
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + Lay::TMEMA);
 
@@ -814,15 +976,15 @@ __global__ void __launch_bounds__(TC_M) k_leg_analysis_tc(const LegArgs<float> a
     if (lbase > L) return;
     const int ntile = min(TR, (L - lbase) / 256 + 1);
     const int lend = min(L, lbase + 256 * TR - 1);
-    const int map0 = blockIdx.z * TC_NMT;
-    const int nm = min(TC_NMT, a.nmaps - map0);
+    const int map0 = blockIdx.z * NMT;
+    const int nm = min(NMT, a.nmaps - map0);
     const int64_t base = (int64_t)m * (2 * L + 1 - m) / 2;
 
     for (int i = tid; i < 256 * TR; i += TC_M) {
         const int l = lbase + i;
         const bool in = l <= L;
-        if (SPIN == 2) s_s2c[ta_cpad(i)] = in ? a.s2c[base + l] : make_float4(0.f, 0.f, 0.f, 0.f);
-        else s_rec[ta_cpad(i)] = in ? a.rec[base + l] : make_float2(0.f, 0.f);
+        if (SPIN == 2) s_c4[ta_cpad(i)] = tc_coef(in ? a.s2c[base + l] : make_float4(0.f, 0.f, 0.f, 0.f));
+        else s_c2[ta_cpad(i)] = in ? a.rec[base + l] : make_float2(0.f, 0.f);
     }
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[0])));
@@ -872,6 +1034,7 @@ __global__ void __launch_bounds__(TC_M) k_leg_analysis_tc(const LegArgs<float> a
     const int nps = (a.npairs + TA_K - 1) / TA_K;
     const int nst = s0 < nps ? nps - s0 : 0;
 
+    const uint64_t descA = sdesc(smem_u32(smem), 2048, 128), descB = sdesc(smem_u32(smem + Lay::BOFF), 32 * NO, 128);
     bool ok = true;
     int unit = 0, waited = -1;
     int last_unit[NBS];            // last unit that read each B buffer
@@ -880,7 +1043,7 @@ __global__ void __launch_bounds__(TC_M) k_leg_analysis_tc(const LegArgs<float> a
     PairStart pst{}, pnext{};
     float4 tcur = make_float4(0.f, 0.f, 0.f, 0.f);
     if (nst > 0) {
-        stage_ring_data<SPIN>(a, m, s0, map0, nm, sgb);
+        stage_ring_data<SPIN, NMT>(a, m, s0, map0, nm, sgb);
         pst = load_pair_start<SPIN>(a, m, s0 * TA_K + pin);
         tcur = load_tile_state<SPIN>(a, m, s0 * TA_K + pin, lbase + 32 * seg);
     }
@@ -900,40 +1063,43 @@ __global__ void __launch_bounds__(TC_M) k_leg_analysis_tc(const LegArgs<float> a
             ok = mbar_wait(&bars[u % NAS], (u / NAS) & 1) && ok;
             waited = u;
         }
-        gen_btiles_ana<SPIN>(sgb, bt);
+        gen_btiles_ana<SPIN, NMT>(sgb, bt);
         for (int r = 0; r < ntile; ++r) {
             const int asel = unit % NAS;
             unsigned char *at = smem + asel * Lay::ASTAGE;
-            if (unit >= NAS && unit - NAS > waited) {   // the unit NAS back read this A buffer
-                ok = mbar_wait(&bars[asel], ((unit - NAS) / NAS) & 1) && ok;
-                waited = unit - NAS;
-            }
+            auto free_tiles = [&]() {   // the unit NAS back read this A buffer
+                if (unit >= NAS && unit - NAS > waited) {
+                    ok = mbar_wait(&bars[asel], ((unit - NAS) / NAS) & 1) && ok;
+                    waited = unit - NAS;
+                }
+            };
             const int tstart = lbase + 256 * r;
             const int l0 = tstart + 32 * seg;
             // state of the next unit: (this stage, next tile) or (next stage, first tile)
             float4 tnext = make_float4(0.f, 0.f, 0.f, 0.f);
             if (r + 1 < ntile) tnext = load_tile_state<SPIN>(a, m, pr, l0 + 256);
             else if (more) tnext = load_tile_state<SPIN>(a, m, pr + TA_K, lbase + 32 * seg);
-            const bool live = pr < a.npairs && l0 <= L;
             const bool starts = (pst.ls >= l0 && pst.ls < l0 + 32) || (SPIN == 2 && pst.lsb >= l0 && pst.lsb < l0 + 32);
-            if (__any_sync(0xffffffffu, live && starts))
-                gen_atiles_ana<SPIN, true>(pst, tcur, live, pin, seg, l0, lbase, s_rec, s_s2c, at);
+            if (__any_sync(0xffffffffu, starts && l0 <= L))
+                gen_atiles_ana<SPIN, true>(pst, tcur, pin, seg, l0, lbase, s_c4, at, free_tiles);
             else
-                gen_atiles_ana<SPIN, false>(pst, tcur, live, pin, seg, l0, lbase, s_rec, s_s2c, at);
+                gen_atiles_ana<SPIN, false>(pst, tcur, pin, seg, l0, lbase, s_c4, at, free_tiles);
             tcur = tnext;
             asm volatile("fence.proxy.async.shared::cta;");
             __syncthreads();
             // every thread has built this stage's B tiles: the ring-data buffer
             // takes the next stage's copy, in flight during the stage's units
-            if (r == 0 && more) stage_ring_data<SPIN>(a, m, ps + 1, map0, nm, sgb);
+            if (r == 0 && more) stage_ring_data<SPIN, NMT>(a, m, ps + 1, map0, nm, sgb);
             if (tid == 0) {
                 asm volatile("tcgen05.fence::after_thread_sync;");
-                const uint32_t sa = smem_u32(at), sb = smem_u32(bt);
                 const uint32_t id = idesc_bf16_amn(TC_M, NO);
                 const uint32_t acc = si > 0;
-                auto A = [&](int t) { return sdesc(sa + t * TC_ATILE, 2048, 128); };
-                auto Bh = [&](int t) { return sdesc(sb + t * Lay::BT, 32 * NO, 128); };
-                auto Bl = [&](int t) { return sdesc(sb + t * Lay::BT + (NO / 8) * 128, 32 * NO, 128); };
+                // (the address field counts 16-byte units)
+                const uint64_t da = descA + (uint32_t)(asel * (Lay::ASTAGE >> 4));
+                const uint64_t db = descB + (uint32_t)(bsel * (Lay::BSTAGE >> 4));
+                auto A = [&](int t) { return da + (uint32_t)(t * (TC_ATILE >> 4)); };
+                auto Bh = [&](int t) { return db + (uint32_t)(t * (Lay::BT >> 4)); };
+                auto Bl = [&](int t) { return db + (uint32_t)((t * Lay::BT + (NO / 8) * 128) >> 4); };
                 const uint32_t dE = tmem + r * 2 * NO, dO = dE + NO;
                 if (SPIN == 0) {
                     mma_bf16(dE, A(0), Bh(0), id, acc);
@@ -976,12 +1142,12 @@ __global__ void __launch_bounds__(TC_M) k_leg_analysis_tc(const LegArgs<float> a
         for (int cls = 0; cls < 2; ++cls) {
             const int l = tstart + 2 * tid + cls;
             float d[NO];
-            if (SPIN == 0) tmem_ld16(trow + r * 2 * NO + cls * NO, *reinterpret_cast<float(*)[16]>(d));
+            if (NO == 16) tmem_ld16(trow + r * 2 * NO + cls * NO, *reinterpret_cast<float(*)[16]>(d));
             else tmem_ld32(trow + r * 2 * NO + cls * NO, *reinterpret_cast<float(*)[32]>(d));
             if (!ok || l > L) continue;
             const float bm = (a.beam ? a.beam[l] : 1.f) * ((a.vjp && m > 0) ? 2.f : 1.f);
 #pragma unroll
-            for (int k = 0; k < TC_NMT; ++k) {
+            for (int k = 0; k < NMT; ++k) {
                 if (k >= nm) break;
 #pragma unroll
                 for (int c = 0; c < (SPIN == 2 ? 2 : 1); ++c) {
@@ -1003,7 +1169,7 @@ __global__ void __launch_bounds__(TC_M) k_leg_analysis_tc(const LegArgs<float> a
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Lay::TMEM));
 }
 
-template <int SPIN, int NAS, int NBS, int TR>
+template <int SPIN, int NMT, int NAS, int NBS, int TR>
 int launch_analysis_tc(Plan *p, const float2 *G, int nmaps, const float *beam, float2 *alm, int rs,
                        cudaStream_t st, int vjp) {
     LegArgs<float> a = leg_make_args<float>(p);
@@ -1018,10 +1184,10 @@ int launch_analysis_tc(Plan *p, const float2 *G, int nmaps, const float *beam, f
         set_error("tensor-core transpose: the plan has no recurrence tile states");
         return SHTG_ERR_ARG;
     }
-    const int smem = TaLayout<SPIN, NAS, NBS, TR>::BYTES;
-    auto kern = k_leg_analysis_tc<SPIN, NAS, NBS, TR>;
+    const int smem = TaLayout<SPIN, NMT, NAS, NBS, TR>::BYTES;
+    auto kern = k_leg_analysis_tc<SPIN, NMT, NAS, NBS, TR>;
     SHTG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    dim3 grid((p->lmax + 256 * TR) / (256 * TR), p->lmax + 1, (nmaps + TC_NMT - 1) / TC_NMT);
+    dim3 grid((p->lmax + 256 * TR) / (256 * TR), p->lmax + 1, (nmaps + NMT - 1) / NMT);
     prof_begin(p, K_LEG_ANA32, st);
     kern<<<grid, TC_M, smem, st>>>(a);
     prof_end(p, st);
@@ -1030,45 +1196,39 @@ int launch_analysis_tc(Plan *p, const float2 *G, int nmaps, const float *beam, f
 }
 }  // namespace
 
-// Shapes tried by the autotuner (key kind 2): synthesis (stages, staged l)
-// = (1, 64) [four CTAs per SM at spin 2], (2, 128), (1, 128); transpose
-// (A buffers, B buffers, 256-l tiles) = (1, 1, 2) [three CTAs per SM; the
-// fastest at N_side 1024, l_max 2048, 8 maps], (1, 2, 2), (2, 2, 2),
-// (1, 1, 1) [four CTAs per SM], (1, 2, 1), (2, 2, 1).
-// Every shape sums the same products in the same order, so the choice does
-// not change a bit of the result.
+// Synthesis: 8 maps per CTA, or 16 at spin 0 when the call has more than 8
+// (the recurrence is then generated once for all of them).
 int leg_synth_tc(Plan *p, int spin, const float2 *alm, int rs, int nmaps, const float *beam, float2 *F,
                  cudaStream_t st) {
-    return tune(p, 2, spin == 2 ? 1 : 0, nmaps, 3, st, [&](int v) {
-        if (spin == 2) {
-            if (v == 1) return launch_synth_tc<2, 2, 128>(p, alm, rs, nmaps, beam, F, st);
-            if (v == 2) return launch_synth_tc<2, 1, 128>(p, alm, rs, nmaps, beam, F, st);
-            return launch_synth_tc<2, 1, 64>(p, alm, rs, nmaps, beam, F, st);
-        }
-        if (v == 1) return launch_synth_tc<0, 2, 128>(p, alm, rs, nmaps, beam, F, st);
-        if (v == 2) return launch_synth_tc<0, 1, 128>(p, alm, rs, nmaps, beam, F, st);
-        return launch_synth_tc<0, 1, 64>(p, alm, rs, nmaps, beam, F, st);
-    });
+    if (spin == 2) return launch_synth_tc<2, 8>(p, alm, rs, nmaps, beam, F, st);
+    if (nmaps > 8) return launch_synth_tc<0, 16>(p, alm, rs, nmaps, beam, F, st);
+    return launch_synth_tc<0, 8>(p, alm, rs, nmaps, beam, F, st);
 }
 
-template <int SPIN>
+// Transpose: maps per CTA likewise; shapes tried by the autotuner (key kind
+// 2), (A buffers, B buffers, 256-l tiles) = (1, 1, 2) [the fastest at N_side
+// 1024, l_max 2048, 8 maps], (1, 2, 2), (2, 2, 2), (1, 1, 1), (1, 2, 1), (2,
+// 2, 1).  Every shape sums the same products in the same order, so the choice
+// does not change a bit of the result.
+template <int SPIN, int NMT>
 static int analysis_tc_shape(int v, Plan *p, const float2 *G, int nmaps, const float *beam, float2 *alm, int rs,
                              cudaStream_t st, int vjp) {
     switch (v) {
-        case 1: return launch_analysis_tc<SPIN, 1, 2, 2>(p, G, nmaps, beam, alm, rs, st, vjp);
-        case 2: return launch_analysis_tc<SPIN, 2, 2, 2>(p, G, nmaps, beam, alm, rs, st, vjp);
-        case 3: return launch_analysis_tc<SPIN, 1, 1, 1>(p, G, nmaps, beam, alm, rs, st, vjp);
-        case 4: return launch_analysis_tc<SPIN, 1, 2, 1>(p, G, nmaps, beam, alm, rs, st, vjp);
-        case 5: return launch_analysis_tc<SPIN, 2, 2, 1>(p, G, nmaps, beam, alm, rs, st, vjp);
-        default: return launch_analysis_tc<SPIN, 1, 1, 2>(p, G, nmaps, beam, alm, rs, st, vjp);
+        case 1: return launch_analysis_tc<SPIN, NMT, 1, 2, 2>(p, G, nmaps, beam, alm, rs, st, vjp);
+        case 2: return launch_analysis_tc<SPIN, NMT, 2, 2, 2>(p, G, nmaps, beam, alm, rs, st, vjp);
+        case 3: return launch_analysis_tc<SPIN, NMT, 1, 1, 1>(p, G, nmaps, beam, alm, rs, st, vjp);
+        case 4: return launch_analysis_tc<SPIN, NMT, 1, 2, 1>(p, G, nmaps, beam, alm, rs, st, vjp);
+        case 5: return launch_analysis_tc<SPIN, NMT, 2, 2, 1>(p, G, nmaps, beam, alm, rs, st, vjp);
+        default: return launch_analysis_tc<SPIN, NMT, 1, 1, 2>(p, G, nmaps, beam, alm, rs, st, vjp);
     }
 }
 
 int leg_analysis_tc(Plan *p, int spin, const float2 *G, int nmaps, const float *beam, float2 *alm, int rs,
                     cudaStream_t st, int vjp) {
     return tune(p, 2, spin == 2 ? 3 : 2, nmaps, 6, st, [&](int v) {
-        if (spin == 2) return analysis_tc_shape<2>(v, p, G, nmaps, beam, alm, rs, st, vjp);
-        return analysis_tc_shape<0>(v, p, G, nmaps, beam, alm, rs, st, vjp);
+        if (spin == 2) return analysis_tc_shape<2, 8>(v, p, G, nmaps, beam, alm, rs, st, vjp);
+        if (nmaps > 8) return analysis_tc_shape<0, 16>(v, p, G, nmaps, beam, alm, rs, st, vjp);
+        return analysis_tc_shape<0, 8>(v, p, G, nmaps, beam, alm, rs, st, vjp);
     });
 }
 
