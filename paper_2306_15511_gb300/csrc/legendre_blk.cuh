@@ -28,8 +28,11 @@
 // Measured (FP64; before: the best of the 8-map form and the warp-reduction
 // kernels that this replaces): N_side 300, l_max 500, 3 maps, spin 0 / 2:
 // 2.87 / 7.3 -> 1.65 / 5.5 ms; N_side 512, l_max 1024, 8 maps: 28.4 / 115 ->
-// 15.1 / 56 ms.  Double-FP32, N_side 512, l_max 1024, 4 maps, spin 2: 15.8 ->
-// 11.1 ms.
+// 15.1 / 56 ms.  The ring data as 16-byte (re, im) operands, signs and the
+// lw / lx exchange folded in when they are staged: N_side 128, l_max 256, 2
+// T+E+B maps, both transposes and both syntheses in FP64 1.93 -> 1.81 ms.
+// Double-FP32, N_side 512, l_max 1024, 4 maps, spin 2: 15.8 -> 11.1 ms, and
+// 9.2 ms with packed arithmetic (df2.cuh).
 #pragma once
 
 #include <string>
@@ -48,17 +51,23 @@ static_assert(SHTG_TS64 == 32, "a warp restarts its 32-l segment from a tabulate
 // (legendre64.cu)
 int leg_maps_per_pass(int spin, int nmaps, const int *nms, int n);
 
-// Ar: the arithmetic.  V value, Acc running sum, C2 / C4 staged coefficients,
-// State recurrence state of one pair (the fields of PairState).
+// Ar: the arithmetic.  V value, Acc two running sums (re, im), Op one ring-data
+// operand (re, im) in registers and OPB its bytes in shared memory, C2 / C4
+// staged coefficients, State<SPIN> recurrence state of one pair.
+//
+// Ring-data operands of a (ring pair, map, class c): spin 0 one, the class's
+// set G_c; spin 2 four, those of the lw terms -Q_c, -U_c (the class's set) and
+// of the lx terms (U_im, -U_re), (-Q_im, Q_re) of the other class's set:
+//   E^ = -lw G_Q - i lx G_U,  B^ = i lx G_Q - lw G_U.
 template <class Ar, int SPIN, int NMT> struct BlkLayout {
     typedef typename Ar::V V;
     static constexpr int NV = SPIN == 2 ? 2 : 1;   // value tiles: lambda, or (lw, lx)
     static constexpr int NO = SPIN == 2 ? 4 : 2;   // outputs per map
-    static constexpr int GS = SPIN == 2 ? 9 : 5;   // map stride of the ring-data sets (odd)
+    static constexpr int NOP = SPIN == 2 ? 4 : 1;  // ring-data operands per (pair, map, class)
     static constexpr int COEF = SPIN == 2 ? sizeof(typename Ar::C4) : sizeof(typename Ar::C2);
     static constexpr int LAM = 0;
-    static constexpr int GSET = LAM + NV * B_LR * B_LS * (int)sizeof(V);
-    static constexpr int CO = (GSET + B_KP * NMT * GS * (int)sizeof(V) + 31) & ~31;
+    static constexpr int GSET = (LAM + NV * B_LR * B_LS * (int)sizeof(V) + 15) & ~15;
+    static constexpr int CO = (GSET + B_KP * NOP * NMT * 2 * Ar::OPB + 31) & ~31;
     static constexpr int RED = CO + B_LR * COEF;
     static constexpr int BYTES = RED + 16;
 };
@@ -67,10 +76,10 @@ template <class Ar, int SPIN, int NMT>
 __global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double> a) {
     typedef BlkLayout<Ar, SPIN, NMT> Ly;
     typedef typename Ar::V V;
-    constexpr int NO = Ly::NO, GS = Ly::GS, NJ = NMT, RG = 64 / NJ;
+    constexpr int NO = Ly::NO, NOP = Ly::NOP, NJ = NMT, RG = 64 / NJ;
     extern __shared__ __align__(32) unsigned char smem[];
     V *lam = reinterpret_cast<V *>(smem + Ly::LAM);      // [NV][B_LR][B_LS]
-    V *gset = reinterpret_cast<V *>(smem + Ly::GSET);    // [B_KP][NMT][GS]
+    unsigned char *gset = smem + Ly::GSET;               // [B_KP][NOP][NMT][class] operands
     typename Ar::C2 *s_rec = reinterpret_cast<typename Ar::C2 *>(smem + Ly::CO);
     typename Ar::C4 *s_s2c = reinterpret_cast<typename Ar::C4 *>(smem + Ly::CO);
     int *s_first = reinterpret_cast<int *>(smem + Ly::RED);
@@ -117,11 +126,11 @@ __global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double>
 
     // this thread's outputs: map k, class c, rows i = c + 2 (rg + RG j)
     const int k = tid & (NMT - 1), c = (tid / NMT) & 1, rg = tid / (2 * NMT);
-    typename Ar::Acc acc[NJ][NO];
+    typename Ar::Acc acc[NJ][NO / 2];
 #pragma unroll
     for (int j = 0; j < NJ; ++j)
 #pragma unroll
-        for (int q = 0; q < NO; ++q) Ar::zero(acc[j][q]);
+        for (int q = 0; q < NO / 2; ++q) Ar::zero(acc[j][q]);
 
     // this warp's rows of block j: WR consecutive ones from row0 + 2 RG j
     constexpr int WR = 32 / NMT;
@@ -136,23 +145,14 @@ __global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double>
             const int pp = tid & 31, seg = tid >> 5;
             const int pr = s * B_KP + pp;
             const int l0 = lbase + 32 * seg;
-            typename Ar::State S;
+            typename Ar::template State<SPIN> S;
             Ar::template load<SPIN>(a, m, pr, S);
             const bool live = pr < a.npairs && l0 <= L;
             first_l = __reduce_min_sync(0xffffffffu, SPIN == 2 ? min(S.ls[0], S.lsb[0]) : S.ls[0]);
             if (live) {
                 const int64_t e = (a.toff64[m] + (l0 - m) / SHTG_TS64) * a.npairs + pr;
-                if (SPIN == 2) {
-                    const double4_32a t4 = a.tst64_2[e];
-                    S.a1[0] = Ar::from(t4.x);
-                    S.a2[0] = Ar::from(t4.y);
-                    S.b1[0] = Ar::from(t4.z);
-                    S.b2[0] = Ar::from(t4.w);
-                } else {
-                    const double2 t2 = a.tst64_0[e];
-                    S.a1[0] = Ar::from(t2.x);
-                    S.a2[0] = Ar::from(t2.y);
-                }
+                if constexpr (SPIN == 2) Ar::restart(S, a.tst64_2[e]);
+                else Ar::restart(S, a.tst64_0[e]);
             }
             // injection steps only if some pair of the warp starts in this segment
             const bool inj = __any_sync(0xffffffffu, live && ((S.ls[0] >= l0 && S.ls[0] < l0 + 32) ||
@@ -161,12 +161,10 @@ __global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double>
                 for (int i = 32 * seg; i < 32 * seg + 32; ++i) {
                     if (inj) Ar::template step<SPIN, true>(S, s_rec, s_s2c, i, lbase + i);
                     else Ar::template step<SPIN, false>(S, s_rec, s_s2c, i, lbase + i);
-                    if (SPIN == 2) {
-                        lam[i * B_LS + pp] = live ? Ar::add(S.a1[0], S.b1[0]) : Ar::from(0.0);
-                        lam[B_LR * B_LS + i * B_LS + pp] = live ? Ar::sub(S.a1[0], S.b1[0]) : Ar::from(0.0);
-                    } else {
-                        lam[i * B_LS + pp] = live ? S.a1[0] : Ar::from(0.0);
-                    }
+                    V v[2];
+                    Ar::template values<SPIN>(S, v);
+                    lam[i * B_LS + pp] = live ? v[0] : Ar::from(0.0);
+                    if (SPIN == 2) lam[B_LR * B_LS + i * B_LS + pp] = live ? v[1] : Ar::from(0.0);
                 }
             } else {   // beyond l_max or before every start
                 for (int i = 32 * seg; i < 32 * seg + 32; ++i) {
@@ -179,7 +177,6 @@ __global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double>
         for (int it = tid; it < B_KP * NMT; it += B_NT) {
             const int pp = it / NMT, kk = it % NMT;
             const int pr = s * B_KP + pp;
-            V *g = gset + (pp * NMT + kk) * GS;
             double2 z[4] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0),
                             make_double2(0.0, 0.0)};
             if (pr < a.npairs && kk < nm) {
@@ -194,11 +191,20 @@ __global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double>
                     z[2 * cc + 1] = make_double2(gn.x - gs.x, gn.y - gs.y);   // odd set
                 }
             }
-            // spin 0: [E re, E im, O re, O im]; spin 2: [QE re, QE im, QO re, QO im, UE re, UE im, UO re, UO im]
+            // z: spin 0 G_E, G_O; spin 2 Q_E, Q_O, U_E, U_O
 #pragma unroll
-            for (int q = 0; q < (SPIN == 2 ? 4 : 2); ++q) {
-                g[2 * q] = Ar::from(z[q].x);
-                g[2 * q + 1] = Ar::from(z[q].y);
+            for (int cl = 0; cl < 2; ++cl) {
+                unsigned char *g = gset + ((pp * NOP * NMT + kk) * 2 + cl) * Ar::OPB;
+                constexpr int OS = NMT * 2 * Ar::OPB;   // stride of the operands
+                if (SPIN == 0) {
+                    Ar::put(g, z[cl].x, z[cl].y);
+                } else {
+                    const double2 xq = z[1 - cl], xu = z[3 - cl];
+                    Ar::put(g, -z[cl].x, -z[cl].y);
+                    Ar::put(g + OS, -z[2 + cl].x, -z[2 + cl].y);
+                    Ar::put(g + 2 * OS, xu.y, -xu.x);
+                    Ar::put(g + 3 * OS, -xq.y, xq.x);
+                }
             }
         }
         __syncthreads();
@@ -212,43 +218,29 @@ __global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double>
         }
 #pragma unroll 2
         for (int p = 0; p < B_KP; ++p) {
-            const V *g = gset + (p * NMT + k) * GS;
-            if (SPIN == 0) {
-                const V gre = g[2 * c], gim = g[2 * c + 1];
+            typename Ar::Op g[NOP];
 #pragma unroll
-                for (int j = 0; j < NJ; ++j) {
-                    if (!on[j]) continue;   // warp-uniform
-                    const V lv = lam[(c + 2 * (rg + RG * j)) * B_LS + p];
-                    Ar::fma(acc[j][0], lv, gre);
-                    Ar::fma(acc[j][1], lv, gim);
-                }
-            } else {
-                // lw terms take the row's set, lx terms the other one:
-                //   E^ = -lw G_Q - i lx G_U,  B^ = i lx G_Q - lw G_U
-                const V qr = g[2 * c], qi = g[2 * c + 1], ur = g[4 + 2 * c], ui = g[4 + 2 * c + 1];
-                const V xqr = g[2 * (1 - c)], xqi = g[2 * (1 - c) + 1], xur = g[4 + 2 * (1 - c)],
-                        xui = g[4 + 2 * (1 - c) + 1];
+            for (int o = 0; o < NOP; ++o) g[o] = Ar::get(gset + (((p * NOP + o) * NMT + k) * 2 + c) * Ar::OPB);
 #pragma unroll
-                for (int j = 0; j < NJ; ++j) {
-                    if (!on[j]) continue;
-                    const int i = c + 2 * (rg + RG * j);
-                    const V lw = lam[i * B_LS + p], lx = lam[B_LR * B_LS + i * B_LS + p];
-                    const V nlw = Ar::neg(lw), nlx = Ar::neg(lx);
-                    Ar::fma(acc[j][0], lx, xui);
-                    Ar::fma(acc[j][0], nlw, qr);
-                    Ar::fma(acc[j][1], nlx, xur);
-                    Ar::fma(acc[j][1], nlw, qi);
-                    Ar::fma(acc[j][2], nlx, xqi);
-                    Ar::fma(acc[j][2], nlw, ur);
-                    Ar::fma(acc[j][3], lx, xqr);
-                    Ar::fma(acc[j][3], nlw, ui);
+            for (int j = 0; j < NJ; ++j) {
+                if (!on[j]) continue;   // warp-uniform
+                const int i = c + 2 * (rg + RG * j);
+                const V lw = lam[i * B_LS + p];
+                if (SPIN == 0) {
+                    Ar::fma(acc[j][0], lw, g[0]);
+                } else {
+                    const V lx = lam[B_LR * B_LS + i * B_LS + p];
+                    Ar::fma(acc[j][0], lx, g[NOP / 2]);
+                    Ar::fma(acc[j][0], lw, g[0]);
+                    Ar::fma(acc[j][NO / 2 - 1], lx, g[NOP - 1]);
+                    Ar::fma(acc[j][NO / 2 - 1], lw, g[NOP / 2 - 1]);
                 }
             }
         }
 #pragma unroll
         for (int j = 0; j < NJ; ++j)
 #pragma unroll
-            for (int q = 0; q < NO; ++q) Ar::norm(acc[j][q]);   // 64 terms at most since the last
+            for (int q = 0; q < NO / 2; ++q) Ar::norm(acc[j][q]);   // 64 terms at most since the last
     }
     // ---- epilogue: every alm of this CTA's l range written once
     if (k >= nm) return;
@@ -261,7 +253,8 @@ __global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double>
         for (int cc = 0; cc < NO / 2; ++cc) {
             const int64_t row = (int64_t)(map0 + k) * a.rs + cc;
             double2 *dst = const_cast<double2 *>(a.alm) + row * a.nalm + base + l;
-            *dst = make_double2(Ar::to(acc[j][2 * cc]) * bm, m == 0 ? 0.0 : Ar::to(acc[j][2 * cc + 1]) * bm);
+            const double2 v = Ar::to(acc[j][cc]);
+            *dst = make_double2(v.x * bm, m == 0 ? 0.0 : v.y * bm);
         }
     }
 }

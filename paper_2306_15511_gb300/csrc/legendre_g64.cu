@@ -13,22 +13,43 @@ namespace {
 
 struct ArF64 {
     typedef double V;
-    typedef double Acc;
+    typedef double2 Acc;
+    typedef double2 Op;
     typedef double2 C2;
     typedef double4_32a C4;
-    typedef PairState<double, 1> State;
+    template <int SPIN> using State = PairState<double, 1>;
+    static constexpr int OPB = sizeof(double2);
     static __device__ __forceinline__ V from(double x) { return x; }
     static __device__ __forceinline__ C2 c2(double2 v) { return v; }
     static __device__ __forceinline__ C4 c4(double4_32a v) { return v; }
-    static __device__ __forceinline__ V add(V x, V y) { return x + y; }
-    static __device__ __forceinline__ V sub(V x, V y) { return x - y; }
-    static __device__ __forceinline__ V neg(V x) { return -x; }
-    static __device__ __forceinline__ void zero(Acc &s) { s = 0.0; }
-    static __device__ __forceinline__ void fma(Acc &s, V x, V y) { s = ::fma(x, y, s); }
+    static __device__ __forceinline__ void put(unsigned char *p, double re, double im) {
+        *reinterpret_cast<double2 *>(p) = make_double2(re, im);
+    }
+    static __device__ __forceinline__ Op get(const unsigned char *p) { return *reinterpret_cast<const double2 *>(p); }
+    static __device__ __forceinline__ void zero(Acc &s) { s = make_double2(0.0, 0.0); }
+    static __device__ __forceinline__ void fma(Acc &s, V x, const Op &y) {
+        s.x = ::fma(x, y.x, s.x);
+        s.y = ::fma(x, y.y, s.y);
+    }
     static __device__ __forceinline__ void norm(Acc &) {}
-    static __device__ __forceinline__ double to(const Acc &s) { return s; }
+    static __device__ __forceinline__ double2 to(const Acc &s) { return s; }
+    static __device__ __forceinline__ void restart(State<2> &S, double2 t) {
+        S.a1[0] = t.x;
+        S.a2[0] = t.y;
+    }
+    static __device__ __forceinline__ void restart(State<2> &S, double4_32a t) {
+        S.a1[0] = t.x;
+        S.a2[0] = t.y;
+        S.b1[0] = t.z;
+        S.b2[0] = t.w;
+    }
+    // lambda, or (lw, lx)
+    template <int SPIN> static __device__ __forceinline__ void values(const State<SPIN> &S, V (&v)[2]) {
+        v[0] = SPIN == 2 ? S.a1[0] + S.b1[0] : S.a1[0];
+        v[1] = SPIN == 2 ? S.a1[0] - S.b1[0] : 0.0;
+    }
     template <int SPIN>
-    static __device__ __forceinline__ void load(const LegArgs<double> &a, int m, int pr, State &S) {
+    static __device__ __forceinline__ void load(const LegArgs<double> &a, int m, int pr, State<SPIN> &S) {
         S.a1[0] = S.a2[0] = S.b1[0] = S.b2[0] = 0.0;
         S.u[0] = 1.0;
         S.ls[0] = S.lsb[0] = a.lmax + 1;
@@ -53,7 +74,7 @@ struct ArF64 {
         }
     }
     template <int SPIN, bool INJ>
-    static __device__ __forceinline__ void step(State &S, const C2 *s_rec, const C4 *s_s2c, int i, int l) {
+    static __device__ __forceinline__ void step(State<SPIN> &S, const C2 *s_rec, const C4 *s_s2c, int i, int l) {
         stepx<double, 1, SPIN, INJ>(S, s_rec, s_s2c, i, l);
     }
 };
