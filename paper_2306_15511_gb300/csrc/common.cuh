@@ -252,8 +252,9 @@ struct Plan {
     float2 *d_tst0 = nullptr;
     float4 *d_tst2 = nullptr;
     // tensor-core synthesis: records of (m, 32 l), tc_nrec per map group
-    unsigned char *d_tcrec = nullptr;
-    int64_t tcrec_bytes = 0, tc_nrec = 0;
+    // (spin 0 and spin 2 apart: their launches may run at the same time)
+    unsigned char *d_tcrec[2] = {nullptr, nullptr};
+    int64_t tcrec_bytes[2] = {0, 0}, tc_nrec = 0;
     // the same in FP64 every SHTG_TS64 l (FP64 and double-FP32 transposes),
     // [m][t][pair] at (d_toff64[m] + t) * npairs + pair
     int64_t *d_toff64 = nullptr;
@@ -381,6 +382,9 @@ int leg_synth_df(Plan *p, int spin, const double2 *alm, int rs, int nmaps, const
                  cudaStream_t st);
 int leg_analysis_df(Plan *p, int spin, const double2 *G, int nmaps, const double *beam, double2 *alm, int rs,
                     cudaStream_t st, int vjp);
+// whether the autotuned launch of this kind (0 FP64, 1 FP32, 2 tensor cores;
+// family 0 / 1 synthesis, 2 / 3 transpose of spin 0 / 2) has its shape
+bool leg_tuned(const Plan *p, int kind, int family, int nmaps);
 
 // ringfft.cu
 // pass twiddles of every transform length (FP32: up to 1024), and where each starts

@@ -64,6 +64,10 @@ int leg_analysis<double>(Plan *p, int spin, const double2 *G, int nmaps, const d
     return leg_analysis_g64(p, spin, G, nmaps, beam, alm, rs, st, vjp);
 }
 
+bool leg_tuned(const Plan *p, int kind, int family, int nmaps) {
+    return p->tuned.count(tune_key(kind, family, nmaps)) != 0;
+}
+
 // ------------------------------------------------------- grouped launches
 // FP32 Legendre sums on the CUDA cores over several plans in one launch (the
 // chains of several geometries), each group with the shape of variant 0 of

@@ -69,9 +69,12 @@ inline bool tuning_log() {
     return on == 1;
 }
 
+inline long long tune_key(int key_prec, int family, int nmaps) {
+    return ((long long)key_prec * 16 + family) * 65536 + nmaps;
+}
 template <typename Run>
 int tune(Plan *p, int key_prec, int family, int nmaps, int nvar, cudaStream_t st, Run run) {
-    const long long key = ((long long)key_prec * 16 + family) * 65536 + nmaps;
+    const long long key = tune_key(key_prec, family, nmaps);
     auto it = p->tuned.find(key);
     if (it != p->tuned.end()) return run(it->second);
     if (tuning_force() >= 0) {

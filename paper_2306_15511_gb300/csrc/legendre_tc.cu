@@ -597,14 +597,14 @@ int launch_synth_tc(Plan *p, const float2 *alm, int rs, int nmaps, const float *
     a.rs = rs;
     a.beam = beam;
     a.err = p->d_flag;
-    a.rec_tc = p->d_tcrec;
+    a.rec_tc = p->d_tcrec[SPIN / 2];
     a.nrec = p->tc_nrec;
     const int smem = Cfg::BYTES;
     auto kern = k_leg_synth_tc<SPIN, NMT>;
     SHTG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     // as many map groups per pass as the plan's record buffer holds
     const int groups = (nmaps + NMT - 1) / NMT;
-    const int fit = (int)std::max<int64_t>(1, std::min<int64_t>(groups, p->tcrec_bytes / (p->tc_nrec * Cfg::REC)));
+    const int fit = (int)std::max<int64_t>(1, std::min<int64_t>(groups, p->tcrec_bytes[SPIN / 2] / (p->tc_nrec * Cfg::REC)));
     prof_begin(p, K_LEG_SYN32, st);
     int nl = 0;
     for (int g0 = 0; g0 < groups; g0 += fit) {
@@ -686,9 +686,11 @@ int build_tile_states(Plan *p) {
     const int mb = p->max_batch;
     const int64_t r0 = mb > 8 ? TcCfg<0, 16>::REC : TcCfg<0, 8>::REC, g0 = mb > 8 ? (mb + 15) / 16 : 1;
     const int64_t r2 = (p->flags & SHTG_SPIN2) ? TcCfg<2, 8>::REC : 0, g2 = (mb + 7) / 8;
-    const int64_t one = p->tc_nrec * std::max(r0, r2), all = p->tc_nrec * std::max(r0 * g0, r2 * g2);
-    p->tcrec_bytes = std::max(one, std::min<int64_t>(all, (int64_t)1 << 30));
-    SHTG_TRY(alloc((void **)&p->d_tcrec, (size_t)p->tcrec_bytes));
+    const int64_t cap = (int64_t)1 << 30;
+    p->tcrec_bytes[0] = p->tc_nrec * std::max(r0, std::min(r0 * g0, cap / p->tc_nrec));
+    p->tcrec_bytes[1] = p->tc_nrec * std::max(r2, std::min(r2 * g2, cap / p->tc_nrec));
+    SHTG_TRY(alloc((void **)&p->d_tcrec[0], (size_t)p->tcrec_bytes[0]));
+    if (r2 > 0) SHTG_TRY(alloc((void **)&p->d_tcrec[1], (size_t)p->tcrec_bytes[1]));
     SHTG_CUDA(cudaDeviceSynchronize());
     return SHTG_OK;
 }

@@ -772,7 +772,7 @@ void plan_free(Plan *p) {
                     p->d_minv32, p->d_diagT, p->d_diagP, p->d_wpairT, p->d_wpairP,
                     p->d_ltab64, p->d_ltab32, p->d_scal, p->d_part, p->d_lsum, p->d_stage,
                     p->d_ls2_64, p->d_st2_64, p->d_ls2_32, p->d_st2_32, p->d_ring_groups, p->d_flag,
-                    p->d_toff, p->d_tcrec, p->d_tst0, p->d_tst2, p->d_isc64, p->d_rsc64, p->d_isc32,
+                    p->d_toff, p->d_tcrec[0], p->d_tcrec[1], p->d_tst0, p->d_tst2, p->d_isc64, p->d_rsc64, p->d_isc32,
                     p->d_toff64, p->d_tst64_0, p->d_tst64_2, p->d_rph64, p->d_rph32, p->d_twr64, p->d_twr32,
                     p->d_tw32, p->d_twf32, p->d_jtab, p->d_blk, p->d_blklam, p->d_blkw, p->d_blkoff,
                     p->d_blkflag};

@@ -910,6 +910,42 @@ static int op_analysis(Solve &s, int spin, const float2 *G, const float *beam, f
     return leg_analysis<float>(s.p, spin, G, s.nb, beam, y, rs, s.st);
 }
 
+// The Legendre stage of T+E+B problems: spin 2 on the solve's stream, spin 0
+// beside it on one of the ring stage's side streams (idle here), joined before
+// the call returns.  The two launches touch different rows, and either alone
+// leaves SMs idle in its last wave: N_side 128, l_max 256: an FP64 operator
+// application of 2 realizations 1.81 -> 1.66 ms, a mixed solve of 4 with tensor
+// cores 11.3 -> 10.5 ms.  One after the other while a shape is still being tuned
+// (its candidates are timed) and while profiling.
+template <typename Op>
+static int both_spins(Solve &s, bool tuned, Op op) {
+    Plan *p = s.p;
+    if (s.nc != 3) return op(0);
+    if (!tuned || p->prof.on) {
+        SHTG_TRY(op(0));
+        return op(2);
+    }
+    const cudaStream_t main = s.st;
+    SHTG_CUDA(cudaEventRecord(p->ring_fork, main));
+    SHTG_CUDA(cudaStreamWaitEvent(p->ring_side[0], p->ring_fork, 0));
+    int rc = op(2);
+    s.st = p->ring_side[0];
+    if (rc == SHTG_OK) rc = op(0);
+    s.st = main;
+    // joined also after an error: nothing of this call runs on past it
+    const cudaError_t e = cudaEventRecord(p->ring_join[0], p->ring_side[0]);
+    if (e == cudaSuccess) cudaStreamWaitEvent(main, p->ring_join[0], 0);
+    if (rc == SHTG_OK && e != cudaSuccess) return cuda_fail(e, "cudaEventRecord", __FILE__, __LINE__);
+    return rc;
+}
+// whether both launches of the operator's synthesis / transpose are tuned
+// (FP64 arithmetic and the tensor-core synthesis have nothing to tune)
+template <typename T> static bool op_tuned(const Solve &s, bool transpose) {
+    if (sizeof(T) == 8 || (s.tc && !transpose)) return true;
+    const int kind = s.tc ? 2 : 1, f = transpose ? 2 : 0;
+    return leg_tuned(s.p, kind, f, s.nb) && leg_tuned(s.p, kind, f + 1, s.nb);
+}
+
 // y = A x = S^-1 x + B Y^T N^-1 Y B x for all realizations
 template <typename T>
 static int matvec(Solve &s, const typename HT<T>::C *x, typename HT<T>::C *y, bool dot = false) {
@@ -918,11 +954,14 @@ static int matvec(Solve &s, const typename HT<T>::C *x, typename HT<T>::C *y, bo
     C *F = Vec<T>::phase(p);
     const T *beam = Vec<T>::beam(p);
     const int64_t rowsz = (int64_t)(p->lmax + 1) * p->nring;
-    SHTG_TRY(op_synth(s, 0, x, s.nc, beam, F));
-    if (s.nc == 3) SHTG_TRY(op_synth(s, 2, x + s.nalm, 3, beam, F + s.nb * rowsz));
+    SHTG_TRY(both_spins(s, op_tuned<T>(s, false), [&](int spin) {
+        return spin == 0 ? op_synth(s, 0, x, s.nc, beam, F) : op_synth(s, 2, x + s.nalm, 3, beam, F + s.nb * rowsz);
+    }));
     SHTG_TRY(ring_fused<T>(p, F, s.nb * s.nc, s.nb, Vec<T>::ninv(p), s.st));
-    SHTG_TRY(op_analysis(s, 0, F, beam, y, s.nc));
-    if (s.nc == 3) SHTG_TRY(op_analysis(s, 2, F + s.nb * rowsz, beam, y + s.nalm, 3));
+    SHTG_TRY(both_spins(s, op_tuned<T>(s, true), [&](int spin) {
+        return spin == 0 ? op_analysis(s, 0, F, beam, y, s.nc)
+                         : op_analysis(s, 2, F + s.nb * rowsz, beam, y + s.nalm, 3);
+    }));
     prof_begin(p, K_VEC, s.st);
     if (dot)   // y's final values and <x, y> partials (slot 0) in one pass
         k_prior_add<T, true><<<s.rgrid, RT, 0, s.st>>>(x, y, s.nc, s.nalm, p->lmax + 1, p->d_lofidx,
@@ -1548,8 +1587,10 @@ static int cg_begin(Plan *p, const shtg_problem *pr, const double *alm_out, cons
     {
         const int64_t rowsz = (int64_t)(p->lmax + 1) * p->nring;
         SHTG_TRY(ring_analysis<double>(p, p->d_map64, nb * nc, 0, p->d_phase64, st));
-        SHTG_TRY(op_analysis(s, 0, p->d_phase64, p->d_ltab64, B, nc));
-        if (nc == 3) SHTG_TRY(op_analysis(s, 2, p->d_phase64 + nb * rowsz, p->d_ltab64, B + p->nalm, 3));
+        SHTG_TRY(both_spins(s, true, [&](int spin) {
+            return spin == 0 ? op_analysis(s, 0, p->d_phase64, p->d_ltab64, B, nc)
+                             : op_analysis(s, 2, p->d_phase64 + nb * rowsz, p->d_ltab64, B + p->nalm, 3);
+        }));
         const double2 *w1 = reinterpret_cast<const double2 *>(pr->w1);
         const size_t w1n = (size_t)nr * nc * p->nalm;
         if (host) {
