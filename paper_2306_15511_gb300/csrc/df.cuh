@@ -14,6 +14,9 @@
 //   two_prod     p + e = a * b exactly, via FMA (Dekker 1971 with a fused
 //                multiply-add in place of his splitting)
 #pragma once
+#include <cstdint>
+#include <cstring>
+
 #include <cuda_runtime.h>
 
 // host and device: the kernels use these on the GPU, and a CPU test checks
@@ -54,15 +57,37 @@ SHTG_DF_FN float two_prod(float a, float b, float &e) {
     return p;
 }
 
-// nearest df of a double (three FP64-pipe operations: used only when data
-// are staged, never per multiply-add)
+// nearest df of a double in integer operations: the float conversions and the
+// difference of the direct form are three instructions of the narrow FP64 pipe,
+// which then were a quarter of the FP64-accurate transpose's time.  hi: the
+// mantissa rounded to 24 bits (half up; the carry runs on into the exponent);
+// lo: the 29 bits below, as a signed integer, times their unit.  Zero, and
+// exponents where hi or the unit of lo leaves FP32's normal range: apart.
 SHTG_DF_FN df df_from(double x) {
 #ifdef __CUDA_ARCH__
-    const float h = __double2float_rn(x);
-    return df_make(h, __double2float_rn(x - (double)h));
+    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
 #else
-    const float h = (float)x;   // round to nearest, the host default
-    return df_make(h, (float)(x - (double)h));
+    uint64_t b;
+    std::memcpy(&b, &x, 8);
+    const unsigned h = (unsigned)(b >> 32), l = (unsigned)b;
+#endif
+    const unsigned ex = (h >> 20) & 0x7ffu, sign = h & 0x80000000u;
+    if (ex - 949u > 200u) {   // |x| outside [2^-74, 2^127)
+        if ((h << 1 | l) == 0u) return df_zero();
+        const float f = (float)x;   // round to nearest
+        return df_make(f, (float)(x - (double)f));
+    }
+    const unsigned l2 = l + 0x10000000u, h2 = h + (l2 < l ? 1u : 0u);
+    const unsigned hb = (((h2 << 3) | (l2 >> 29)) + 0x40000000u) | sign;   // exponent bias 1023 -> 127 (mod 2^32)
+    const unsigned ub = ((ex - 948u) << 23) | sign;                        // the sign times 2^(e - 52)
+    const int rem = (int)(l2 & 0x1fffffffu) - 0x10000000;
+#ifdef __CUDA_ARCH__
+    return df_make(__uint_as_float(hb), __int2float_rn(rem) * __uint_as_float(ub));
+#else
+    float hi, u;
+    std::memcpy(&hi, &hb, 4);
+    std::memcpy(&u, &ub, 4);
+    return df_make(hi, (float)rem * u);
 #endif
 }
 SHTG_DF_FN double df_to(df a) { return (double)a.hi + (double)a.lo; }

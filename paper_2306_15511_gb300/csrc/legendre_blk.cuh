@@ -31,8 +31,9 @@
 // 15.1 / 56 ms.  The ring data as 16-byte (re, im) operands, signs and the
 // lw / lx exchange folded in when they are staged: N_side 128, l_max 256, 2
 // T+E+B maps, both transposes and both syntheses in FP64 1.93 -> 1.81 ms.
-// Double-FP32, N_side 512, l_max 1024, 4 maps, spin 2: 15.8 -> 11.1 ms, and
-// 9.2 ms with packed arithmetic (df2.cuh).
+// Double-FP32, N_side 512, l_max 1024, 4 maps, spin 2: 15.8 -> 11.1 ms, 9.2 ms
+// with packed arithmetic (df2.cuh), 7.1 ms with the value tile in two halves
+// and integer conversions (df.cuh).
 #pragma once
 
 #include <string>
@@ -61,24 +62,73 @@ int leg_maps_per_pass(int spin, int nmaps, const int *nms, int n);
 //   E^ = -lw G_Q - i lx G_U,  B^ = i lx G_Q - lw G_U.
 template <class Ar, int SPIN, int NMT> struct BlkLayout {
     typedef typename Ar::V V;
+    // Parts of a segment generated at a time.  Two (double-FP32): the value tile
+    // takes 34 instead of 68 KB at spin 2, and four CTAs share an SM instead of
+    // two, so one's generation and staging run beside another's contraction (the
+    // FP32 pipe was 56 % busy).  One map: a half would leave threads without rows.
+    // FP64: its pipe is the bound with two CTAs as well.
+    static constexpr int HV = Ar::HALVES && NMT > 1 ? 2 : 1;   // parts of a segment generated at a time
+    static constexpr int TR = B_LR / HV;                       // rows of the value tile
     static constexpr int NV = SPIN == 2 ? 2 : 1;   // value tiles: lambda, or (lw, lx)
     static constexpr int NO = SPIN == 2 ? 4 : 2;   // outputs per map
     static constexpr int NOP = SPIN == 2 ? 4 : 1;  // ring-data operands per (pair, map, class)
     static constexpr int COEF = SPIN == 2 ? sizeof(typename Ar::C4) : sizeof(typename Ar::C2);
     static constexpr int LAM = 0;
-    static constexpr int GSET = (LAM + NV * B_LR * B_LS * (int)sizeof(V) + 15) & ~15;
+    static constexpr int GSET = (LAM + NV * TR * B_LS * (int)sizeof(V) + 15) & ~15;
     static constexpr int CO = (GSET + B_KP * NOP * NMT * 2 * Ar::OPB + 31) & ~31;
     static constexpr int RED = CO + B_LR * COEF;
     static constexpr int BYTES = RED + 16;
 };
+
+// Ring-data operands of stage s (32 ring pairs) for NMT maps
+template <class Ar, int SPIN, int NMT>
+__device__ __forceinline__ void stage_ops(const LegArgs<double> &a, int m, int s, int map0, int nm,
+                                          unsigned char *gset) {
+    constexpr int NOP = BlkLayout<Ar, SPIN, NMT>::NOP;
+    constexpr int OS = NMT * 2 * Ar::OPB;   // stride of the operands
+    const int64_t rowsz = (int64_t)a.nring * (a.lmax + 1);
+    for (int it = threadIdx.x; it < B_KP * NMT; it += B_NT) {
+        const int pp = it / NMT, kk = it % NMT;
+        const int pr = s * B_KP + pp;
+        // z: spin 0 G_E, G_O; spin 2 Q_E, Q_O, U_E, U_O
+        double2 z[4] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0),
+                        make_double2(0.0, 0.0)};
+        if (pr < a.npairs && kk < nm) {
+            const int rn = pr, rs = a.nring - 1 - pr;
+#pragma unroll
+            for (int cc = 0; cc < (SPIN == 2 ? 2 : 1); ++cc) {
+                const int64_t row = SPIN == 2 ? 2 * (map0 + kk) + cc : map0 + kk;
+                const double2 *gr = a.F + row * rowsz + m;
+                const double2 gn = gr[(int64_t)rn * (a.lmax + 1)];
+                const double2 gs = rs != rn ? gr[(int64_t)rs * (a.lmax + 1)] : make_double2(0.0, 0.0);
+                z[2 * cc] = make_double2(gn.x + gs.x, gn.y + gs.y);       // even set
+                z[2 * cc + 1] = make_double2(gn.x - gs.x, gn.y - gs.y);   // odd set
+            }
+        }
+#pragma unroll
+        for (int cl = 0; cl < 2; ++cl) {
+            unsigned char *g = gset + ((pp * NOP * NMT + kk) * 2 + cl) * Ar::OPB;
+            if (SPIN == 0) {
+                Ar::put(g, z[cl].x, z[cl].y);
+            } else {
+                const double2 xq = z[1 - cl], xu = z[3 - cl];
+                Ar::put(g, -z[cl].x, -z[cl].y);
+                Ar::put(g + OS, -z[2 + cl].x, -z[2 + cl].y);
+                Ar::put(g + 2 * OS, xu.y, -xu.x);
+                Ar::put(g + 3 * OS, -xq.y, xq.x);
+            }
+        }
+    }
+}
 
 template <class Ar, int SPIN, int NMT>
 __global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double> a) {
     typedef BlkLayout<Ar, SPIN, NMT> Ly;
     typedef typename Ar::V V;
     constexpr int NO = Ly::NO, NOP = Ly::NOP, NJ = NMT, RG = 64 / NJ;
+    constexpr int HV = Ly::HV, TR = Ly::TR, SR = 32 / HV, NJH = NJ / HV;
     extern __shared__ __align__(32) unsigned char smem[];
-    V *lam = reinterpret_cast<V *>(smem + Ly::LAM);      // [NV][B_LR][B_LS]
+    V *lam = reinterpret_cast<V *>(smem + Ly::LAM);      // [NV][TR][B_LS]
     unsigned char *gset = smem + Ly::GSET;               // [B_KP][NOP][NMT][class] operands
     typename Ar::C2 *s_rec = reinterpret_cast<typename Ar::C2 *>(smem + Ly::CO);
     typename Ar::C4 *s_s2c = reinterpret_cast<typename Ar::C4 *>(smem + Ly::CO);
@@ -93,7 +143,6 @@ __global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double>
     const int map0 = blockIdx.z * NMT;
     const int nm = min(NMT, a.nmaps - map0);
     const int64_t base = (int64_t)m * (2 * L + 1 - m) / 2;
-    const int64_t rowsz = (int64_t)a.nring * (L + 1);
 
     for (int i = tid; i < B_LR; i += B_NT) {
         const int l = lbase + i;
@@ -124,7 +173,9 @@ __global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double>
     const int s0 = *s_first / B_KP;
     const int nps = (a.npairs + B_KP - 1) / B_KP;
 
-    // this thread's outputs: map k, class c, rows i = c + 2 (rg + RG j)
+    // this thread's outputs: map k, class c, in part h of the segments the tile
+    // rows c + 2 (rg + RG j), j < NJH; tile row r is row lrow(h, r)
+    auto lrow = [](int h, int r) { return HV == 1 ? r : 32 * (r / SR) + SR * h + r % SR; };
     const int k = tid & (NMT - 1), c = (tid / NMT) & 1, rg = tid / (2 * NMT);
     typename Ar::Acc acc[NJ][NO / 2];
 #pragma unroll
@@ -132,108 +183,80 @@ __global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double>
 #pragma unroll
         for (int q = 0; q < NO / 2; ++q) Ar::zero(acc[j][q]);
 
-    // this warp's rows of block j: WR consecutive ones from row0 + 2 RG j
+    // this warp's tile rows of block j: WR consecutive ones from row0 + 2 RG j
     constexpr int WR = 32 / NMT;
     const int row0 = 2 * ((tid & ~31) / (2 * NMT));
     for (int s = s0; s < nps; ++s) {
-        __syncthreads();   // the previous stage's tiles are consumed
-        int first_l;       // no pair of the stage has a significant value below this l
-        {
-            // ---- recurrences of the stage's 32 ring pairs: warp w runs rows
-            // 32 w .. 32 w + 31 of pair s * 32 + lane from the FP64 state
-            // tabulated at l0 = lbase + 32 w
-            const int pp = tid & 31, seg = tid >> 5;
-            const int pr = s * B_KP + pp;
-            const int l0 = lbase + 32 * seg;
-            typename Ar::template State<SPIN> S;
-            Ar::template load<SPIN>(a, m, pr, S);
-            const bool live = pr < a.npairs && l0 <= L;
-            first_l = __reduce_min_sync(0xffffffffu, SPIN == 2 ? min(S.ls[0], S.lsb[0]) : S.ls[0]);
-            if (live) {
-                const int64_t e = (a.toff64[m] + (l0 - m) / SHTG_TS64) * a.npairs + pr;
-                if constexpr (SPIN == 2) Ar::restart(S, a.tst64_2[e]);
-                else Ar::restart(S, a.tst64_0[e]);
-            }
-            // injection steps only if some pair of the warp starts in this segment
-            const bool inj = __any_sync(0xffffffffu, live && ((S.ls[0] >= l0 && S.ls[0] < l0 + 32) ||
-                                                              (SPIN == 2 && S.lsb[0] >= l0 && S.lsb[0] < l0 + 32)));
-            if (__any_sync(0xffffffffu, live) && l0 + 31 >= first_l) {
-                for (int i = 32 * seg; i < 32 * seg + 32; ++i) {
+        // ---- recurrences of the stage's 32 ring pairs: warp w runs rows
+        // 32 w .. 32 w + 31 of pair s * 32 + lane from the FP64 state
+        // tabulated at l0 = lbase + 32 w
+        const int pp = tid & 31, seg = tid >> 5;
+        const int pr = s * B_KP + pp;
+        const int l0 = lbase + 32 * seg;
+        typename Ar::template State<SPIN> S;
+        Ar::template load<SPIN>(a, m, pr, S);
+        const bool live = pr < a.npairs && l0 <= L;
+        // no pair of the stage has a significant value below this l
+        const int first_l = __reduce_min_sync(0xffffffffu, SPIN == 2 ? min(S.ls[0], S.lsb[0]) : S.ls[0]);
+        if (live) {
+            const int64_t e = (a.toff64[m] + (l0 - m) / SHTG_TS64) * a.npairs + pr;
+            if constexpr (SPIN == 2) Ar::restart(S, a.tst64_2[e]);
+            else Ar::restart(S, a.tst64_0[e]);
+        }
+        // injection steps only if some pair of the warp starts in this segment
+        const bool inj = __any_sync(0xffffffffu, live && ((S.ls[0] >= l0 && S.ls[0] < l0 + 32) ||
+                                                          (SPIN == 2 && S.lsb[0] >= l0 && S.lsb[0] < l0 + 32)));
+        const bool gen = __any_sync(0xffffffffu, live) && l0 + 31 >= first_l;
+#pragma unroll
+        for (int h = 0; h < HV; ++h) {
+            __syncthreads();   // the previous part's (stage's) tiles are consumed
+            if (gen) {
+                for (int r = SR * seg; r < SR * seg + SR; ++r) {
+                    const int i = lrow(h, r);
                     if (inj) Ar::template step<SPIN, true>(S, s_rec, s_s2c, i, lbase + i);
                     else Ar::template step<SPIN, false>(S, s_rec, s_s2c, i, lbase + i);
                     V v[2];
                     Ar::template values<SPIN>(S, v);
-                    lam[i * B_LS + pp] = live ? v[0] : Ar::from(0.0);
-                    if (SPIN == 2) lam[B_LR * B_LS + i * B_LS + pp] = live ? v[1] : Ar::from(0.0);
+                    lam[r * B_LS + pp] = live ? v[0] : Ar::from(0.0);
+                    if (SPIN == 2) lam[(TR + r) * B_LS + pp] = live ? v[1] : Ar::from(0.0);
                 }
             } else {   // beyond l_max or before every start
-                for (int i = 32 * seg; i < 32 * seg + 32; ++i) {
-                    lam[i * B_LS + pp] = Ar::from(0.0);
-                    if (SPIN == 2) lam[B_LR * B_LS + i * B_LS + pp] = Ar::from(0.0);
+                for (int r = SR * seg; r < SR * seg + SR; ++r) {
+                    lam[r * B_LS + pp] = Ar::from(0.0);
+                    if (SPIN == 2) lam[(TR + r) * B_LS + pp] = Ar::from(0.0);
                 }
             }
-        }
-        // ---- ring data of the stage: per (pair, map) the even / odd sets
-        for (int it = tid; it < B_KP * NMT; it += B_NT) {
-            const int pp = it / NMT, kk = it % NMT;
-            const int pr = s * B_KP + pp;
-            double2 z[4] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0),
-                            make_double2(0.0, 0.0)};
-            if (pr < a.npairs && kk < nm) {
-                const int rn = pr, rs = a.nring - 1 - pr;
+            // ---- ring data of the stage: per (pair, map, class) the operands
+            if (h == 0) stage_ops<Ar, SPIN, NMT>(a, m, s, map0, nm, gset);
+            __syncthreads();
+            // ---- contraction over the stage's ring pairs; row blocks beyond
+            // l_max or before every start of the stage (exact zeros) are left out
+            bool on[NJH];
 #pragma unroll
-                for (int cc = 0; cc < (SPIN == 2 ? 2 : 1); ++cc) {
-                    const int64_t row = SPIN == 2 ? 2 * (map0 + kk) + cc : map0 + kk;
-                    const double2 *gr = a.F + row * rowsz + m;
-                    const double2 gn = gr[(int64_t)rn * (L + 1)];
-                    const double2 gs = rs != rn ? gr[(int64_t)rs * (L + 1)] : make_double2(0.0, 0.0);
-                    z[2 * cc] = make_double2(gn.x + gs.x, gn.y + gs.y);       // even set
-                    z[2 * cc + 1] = make_double2(gn.x - gs.x, gn.y - gs.y);   // odd set
-                }
+            for (int j = 0; j < NJH; ++j) {
+                const int l = lbase + lrow(h, row0 + 2 * RG * j);
+                on[j] = l <= L && l + WR > first_l;
             }
-            // z: spin 0 G_E, G_O; spin 2 Q_E, Q_O, U_E, U_O
-#pragma unroll
-            for (int cl = 0; cl < 2; ++cl) {
-                unsigned char *g = gset + ((pp * NOP * NMT + kk) * 2 + cl) * Ar::OPB;
-                constexpr int OS = NMT * 2 * Ar::OPB;   // stride of the operands
-                if (SPIN == 0) {
-                    Ar::put(g, z[cl].x, z[cl].y);
-                } else {
-                    const double2 xq = z[1 - cl], xu = z[3 - cl];
-                    Ar::put(g, -z[cl].x, -z[cl].y);
-                    Ar::put(g + OS, -z[2 + cl].x, -z[2 + cl].y);
-                    Ar::put(g + 2 * OS, xu.y, -xu.x);
-                    Ar::put(g + 3 * OS, -xq.y, xq.x);
-                }
-            }
-        }
-        __syncthreads();
-        // ---- contraction over the stage's ring pairs; row blocks beyond l_max
-        // or before every start of the stage (exact zeros) are left out
-        bool on[NJ];
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-            const int l = lbase + row0 + 2 * RG * j;
-            on[j] = l <= L && l + WR > first_l;
-        }
 #pragma unroll 2
-        for (int p = 0; p < B_KP; ++p) {
-            typename Ar::Op g[NOP];
+            for (int p = 0; p < B_KP; ++p) {
+                typename Ar::Op g[NOP];
 #pragma unroll
-            for (int o = 0; o < NOP; ++o) g[o] = Ar::get(gset + (((p * NOP + o) * NMT + k) * 2 + c) * Ar::OPB);
+                for (int o = 0; o < NOP; ++o) g[o] = Ar::get(gset + (((p * NOP + o) * NMT + k) * 2 + c) * Ar::OPB);
 #pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-                if (!on[j]) continue;   // warp-uniform
-                const int i = c + 2 * (rg + RG * j);
-                const V lw = lam[i * B_LS + p];
-                if (SPIN == 0) {
-                    Ar::fma(acc[j][0], lw, g[0]);
-                } else {
-                    const V lx = lam[B_LR * B_LS + i * B_LS + p];
-                    Ar::fma(acc[j][0], lx, g[NOP / 2]);
-                    Ar::fma(acc[j][0], lw, g[0]);
-                    Ar::fma(acc[j][NO / 2 - 1], lx, g[NOP - 1]);
-                    Ar::fma(acc[j][NO / 2 - 1], lw, g[NOP / 2 - 1]);
+                for (int j = 0; j < NJH; ++j) {
+                    if (!on[j]) continue;   // warp-uniform
+                    const int r = c + 2 * (rg + RG * j);
+                    typename Ar::Acc *ac = acc[h * NJH + j];
+                    const V lw = lam[r * B_LS + p];
+                    if (SPIN == 0) {
+                        Ar::fma(ac[0], lw, g[0]);
+                    } else {
+                        const V lx = lam[(TR + r) * B_LS + p];
+                        Ar::fma(ac[0], lx, g[NOP / 2]);
+                        Ar::fma(ac[0], lw, g[0]);
+                        Ar::fma(ac[NO / 2 - 1], lx, g[NOP - 1]);
+                        Ar::fma(ac[NO / 2 - 1], lw, g[NOP / 2 - 1]);
+                    }
                 }
             }
         }
@@ -246,7 +269,7 @@ __global__ void __launch_bounds__(B_NT) k_leg_analysis_blk(const LegArgs<double>
     if (k >= nm) return;
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
-        const int l = lbase + c + 2 * (rg + RG * j);
+        const int l = lbase + lrow(j / NJH, c + 2 * (rg + RG * (j % NJH)));
         if (l > L) continue;
         const double bm = (a.beam ? a.beam[l] : 1.0) * ((a.vjp && m > 0) ? 2.0 : 1.0);
 #pragma unroll

@@ -18,6 +18,7 @@ struct ArF64 {
     typedef double2 C2;
     typedef double4_32a C4;
     template <int SPIN> using State = PairState<double, 1>;
+    static constexpr bool HALVES = false;
     static constexpr int OPB = sizeof(double2);
     static __device__ __forceinline__ V from(double x) { return x; }
     static __device__ __forceinline__ C2 c2(double2 v) { return v; }

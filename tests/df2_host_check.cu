@@ -1,6 +1,8 @@
 // Host driver for the packed double-FP32 functions of csrc/df2.cuh (built and
 // run by tests/test_df2_host.py on the CPU; no GPU): counts the results whose
-// halves differ in any bit from the scalar functions of csrc/df.cuh.
+// halves differ in any bit from the scalar functions of csrc/df.cuh, and those
+// of df_from that differ in value from the float conversions.
+#include <cmath>
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
@@ -54,6 +56,26 @@ int main() {
         }
         acc += differs(s2, df_make(s[0].hi, s[0].lo), df_make(s[1].hi, s[1].lo));
     }
+    // df_from against the conversions it stands for, at both ends of its range
+    // of exponents and beyond, ties, zeros and infinity
+    int from = 0;
+    auto check = [&](double x) {
+        const df a = df_from(x);
+        const float hi = (float)x, lo = (float)(x - (double)hi);
+        const double sa = (double)a.hi + (double)a.lo, sb = (double)hi + (double)lo;
+        from += !(sa == sb || (sa != sa && sb != sb)) || std::fabs(a.lo) > std::fabs(std::nextafter(hi, INFINITY) - hi) / 2;
+    };
+    for (int e = -200; e <= 130; ++e)
+        for (int i = 0; i < 100; ++i) {
+            const double x = ldexp(draw(false), e);
+            check(x);
+            check((double)(float)x * (1.0 + ldexp(1.0, -24)));   // halfway between floats
+            check(ldexp(x < 0 ? -2.0 : 2.0, e) * (1.0 - ldexp(1.0, -30)));
+        }
+    check(0.0);
+    check(-0.0);
+    check(INFINITY);
+    std::printf("from %d ", from);
     std::printf("add %d sub %d mul %d fma %d\n", add, sub, mul, acc);
     return 0;
 }
