@@ -251,8 +251,9 @@ struct Plan {
     int64_t *d_toff = nullptr;
     float2 *d_tst0 = nullptr;
     float4 *d_tst2 = nullptr;
-    // tensor-core synthesis: records of (m, 32 l), tc_nrec per map group
-    // (spin 0 and spin 2 apart: their launches may run at the same time)
+    // records of the tensor-core synthesis, (m, 32 l), tc_nrec per map group,
+    // and of the transpose, (m, 16 ring pairs) (spin 0 and spin 2 apart: their
+    // launches may run at the same time)
     unsigned char *d_tcrec[2] = {nullptr, nullptr};
     int64_t tcrec_bytes[2] = {0, 0}, tc_nrec = 0;
     // the same in FP64 every SHTG_TS64 l (FP64 and double-FP32 transposes),

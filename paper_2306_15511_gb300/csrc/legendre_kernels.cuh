@@ -141,8 +141,9 @@ template <typename T> struct LegArgs {
     const int64_t *toff;  // tensor-core transpose: recurrence states every 32 l (FP32 plans)
     const float2 *tst0;
     const float4 *tst2;
-    unsigned char *rec_tc;    // tensor-core synthesis: records of every (m, 32 l), nrec per map group
-    int64_t nrec;
+    unsigned char *rec_tc;    // tensor-core synthesis: records of every (m, 32 l), nrec per map group; transpose:
+    int64_t nrec;             // records of every (m, 16 ring pairs) of m0 <= m < m0 + mcnt
+    int m0, mcnt;
     const int64_t *toff64;    // FP64 recurrence states every SHTG_TS64 l (FP64 and double-FP32 transposes)
     const double2 *tst64_0;
     const double4_32a *tst64_2;

@@ -650,6 +650,8 @@ __global__ void __launch_bounds__(LEG_THREADS) k_tile_states(const LegArgs<float
 
 }  // namespace
 
+static int alloc_records(Plan *p);
+
 int build_tile_states(Plan *p) {
     const int L = p->lmax;
     std::vector<int64_t> toff(L + 2);
@@ -680,17 +682,8 @@ int build_tile_states(Plan *p) {
         k_tile_states<2><<<grid, LEG_THREADS>>>(a, p->d_toff, nullptr, p->d_tst2);
         SHTG_CHECK_LAUNCH("k_tile_states");
     }
-    // records of the synthesis: every map group of a full batch, at most 1 GB
-    // (at least one group; more groups than fit take several passes)
     p->tc_nrec = toff[L + 1];
-    const int mb = p->max_batch;
-    const int64_t r0 = mb > 8 ? TcCfg<0, 16>::REC : TcCfg<0, 8>::REC, g0 = mb > 8 ? (mb + 15) / 16 : 1;
-    const int64_t r2 = (p->flags & SHTG_SPIN2) ? TcCfg<2, 8>::REC : 0, g2 = (mb + 7) / 8;
-    const int64_t cap = (int64_t)1 << 30;
-    p->tcrec_bytes[0] = p->tc_nrec * std::max(r0, std::min(r0 * g0, cap / p->tc_nrec));
-    p->tcrec_bytes[1] = p->tc_nrec * std::max(r2, std::min(r2 * g2, cap / p->tc_nrec));
-    SHTG_TRY(alloc((void **)&p->d_tcrec[0], (size_t)p->tcrec_bytes[0]));
-    if (r2 > 0) SHTG_TRY(alloc((void **)&p->d_tcrec[1], (size_t)p->tcrec_bytes[1]));
+    SHTG_TRY(alloc_records(p));
     SHTG_CUDA(cudaDeviceSynchronize());
     return SHTG_OK;
 }
@@ -698,49 +691,64 @@ int build_tile_states(Plan *p) {
 namespace {
 
 // ===================================================== transpose (Y^T)
-// c_lm = sum_r lambda_lm(theta_r) G_r(m) for one m and a range of 512 l:
-// rows = l (two 128-row tiles per 256 l: l - m even, l - m odd), K = ring
-// pairs in stages of 16, columns = (map, output) with the north / south
-// combination G_N + G_S (rows with the parity of lambda) or G_N - G_S
-// folded into the B tiles.  A tiles hold the recurrence values l-major
+// c_lm = sum_r lambda_lm(theta_r) G_r(m) for one m and a range of 256 l:
+// rows = l (two 128-row tiles: l - m even, l - m odd), K = ring pairs in
+// stages of 16, columns = (map, output) with the north / south combination
+// G_N + G_S (rows with the parity of lambda) or G_N - G_S folded into the B
+// tiles.  k_ta_records writes the B tiles of every (m, stage) as records in
+// global memory, eight m at a time; k_leg_analysis_tc fetches them by bulk
+// copies, one stage ahead.  A tiles hold the recurrence values l-major
 // (MN-major core matrices: 8 pairs x 8 consecutive rows of one class), which
 // is how a thread produces them: thread (pair p, segment s) runs the FP32
 // recurrence of pair p over 32 l from the tabulated state at l = m + 32 t.
 // The CTA accumulates over all ring pairs in tensor memory, so every alm is
 // written once, by one CTA, without atomics.
+//
+// What bounds it: the shared-memory / L1 data path, which the MMAs' operand
+// reads share.  Before the records every CTA copied its ring data with 8-byte
+// cp.async (neighbouring m lie side by side in memory, so each took a line of
+// its own) and built the same B tiles: about 1100 wavefronts per stage and 256
+// l at spin 2, and the MMAs read 12 A tiles of 4 KB (384 wavefronts).  Now the
+// products with hi and lo of B are one MMA of twice the columns into separate
+// sums, so each of the 8 A tiles is read once.  Measured (N_side 1024, l_max
+// 2048, 8 Q/U maps, with the ring stage): 7.18 -> 5.20 ms.  Spin 0 (8 maps) has
+// half the shared and tensor memory, and 71 registers let six CTAs share an SM:
+// N_side 512, l_max 1024, 4 maps, 0.38 -> 0.28 ms.
 constexpr int TA_K = 16;        // ring pairs per stage (MMA K)
 template <int SPIN, int NMT> struct TaCfg {   // NMT maps per CTA
     static constexpr int NO = SPIN == 2 ? 4 * NMT : 2 * NMT, NAT = SPIN == 2 ? 8 : 4, NBT = SPIN == 2 ? 4 : 2;
 };
-// Shared memory of the transpose CTA (TR 256-l tiles): NAS A buffers (the
-// tiles of one (stage, 256-l tile) unit), NBS B buffers (one per stage of 16
-// pairs), the ring data of one stage, the coefficients of 256 TR l, two
-// mbarriers and the TMEM address.  The ring data are consumed when the
-// stage's B tiles are built, so the next stage's copy is issued right after
-// (it overlaps with the stage's A generation) and one buffer suffices.
-// Fewer buffers shrink the CTA (spin 2 with one A and one B buffer: 53 KB
-// with two 256-l tiles, 49 KB with one) so that four CTAs share an SM.
-template <int SPIN, int NMT, int NAS, int NBS, int TR> struct TaLayout {
+// Staged ring data of one (m, stage): [pair][north rows | south rows] float2
+// with pair stride GS = 2 NROW + 2: the builder's warp reads 8 consecutive
+// floats per K pair and its four K pairs sit 4 GS = 8 (mod 32) floats apart,
+// so every load hits 32 distinct banks.
+template <int SPIN, int NMT> struct TaRing {
+    static constexpr int NROW = SPIN == 2 ? 2 * NMT : NMT;
+    static constexpr int GS = 2 * NROW + 2;
+    static constexpr int SG = TA_K * GS + 4;   // stride of the m
+};
+// Shared memory of the transpose CTA: NAS A buffers (the tiles of one stage),
+// NAS + 1 B buffers, without records (REC false) the ring data of one stage,
+// the coefficients of 256 l, the mbarriers (NAS of the
+// MMAs, NAS + 1 of the records) and the TMEM address.  With one A buffer (53 KB
+// at spin 2) four CTAs share an SM, and each waits for its own MMAs while the
+// others generate.
+template <int SPIN, int NMT, int NAS, bool REC> struct TaLayout {
     typedef TaCfg<SPIN, NMT> Cfg;
     static constexpr int BT = 64 * Cfg::NO;                         // B tile: 2 NO rows x 16 K bf16
     static constexpr int ASTAGE = Cfg::NAT * TC_ATILE;
-    static constexpr int BSTAGE = Cfg::NBT * BT;
+    static constexpr int BSTAGE = Cfg::NBT * BT;                    // one record
+    static constexpr int NBS = NAS + 1;
     static constexpr int BOFF = NAS * ASTAGE;
-    // ring data of one stage: [pair][north rows | south rows] float2 with pair
-    // stride GS = 2 NROW + 2: the B-tile builder's warp reads 8 consecutive
-    // floats per K pair and its four K pairs sit 4 GS = 8 (mod 32) floats
-    // apart, so every load hits 32 distinct banks
-    static constexpr int NROW = SPIN == 2 ? 2 * NMT : NMT;
-    static constexpr int GS = 2 * NROW + 2;
-    static constexpr int GBUF = ((TA_K * GS * 8) + 15) & ~15;
     static constexpr int GOFF = BOFF + NBS * BSTAGE;
-    static constexpr int COEF = GOFF + GBUF;
-    // coefficients of 256 TR l, one padding entry after every 32 (ta_cpad)
-    static constexpr int BARS = COEF + 264 * TR * (SPIN == 2 ? 16 : 8);
-    static constexpr int TMEM = TR * 2 * Cfg::NO;   // 2 NO columns per 256-l tile
-    static constexpr int TMEMA = BARS + 16;
+    static constexpr int COEF = GOFF + (REC ? 0 : ((TA_K * TaRing<SPIN, NMT>::GS * 8) + 15) & ~15);
+    // coefficients of 256 l, one padding entry after every 32 (ta_cpad)
+    static constexpr int BARS = COEF + 264 * (SPIN == 2 ? 16 : 8);
+    static constexpr int TMEM = 4 * Cfg::NO;   // two classes, products with B hi and with B lo
+    static constexpr int TMEMA = BARS + 48;
     static constexpr int BYTES = TMEMA + 16;
 };
+constexpr int TA_MB = 8;   // m per CTA of the records: 64-byte runs of the ring data
 
 // Shared index of the recurrence coefficients of l = lbase + i in the
 // transpose: one padding entry after every 32, so the two 32-l segments that
@@ -862,7 +870,7 @@ __device__ __forceinline__ void gen_atiles_ana(const PairStart &q, const float4 
 template <int SPIN, int NMT>
 __device__ __forceinline__ void stage_ring_data(const LegArgs<float> &a, const int m, const int ps, const int map0,
                                                 const int nm, float2 *sg) {
-    typedef TaLayout<SPIN, NMT, 1, 1, 1> Lay;   // (ring-data geometry only)
+    typedef TaRing<SPIN, NMT> Lay;
     const int L = a.lmax;
     const int64_t rowsz = (int64_t)a.nring * (L + 1);
     const int nrow = SPIN == 2 ? 2 * nm : nm;
@@ -896,8 +904,8 @@ __device__ __forceinline__ void stage_ring_data(const LegArgs<float> &a, const i
 // two scalars per ring pair that its column needs.
 template <int SPIN, int NMT>
 __device__ __forceinline__ void gen_btiles_ana(const float2 *sg, unsigned char *bt) {
-    typedef TaLayout<SPIN, NMT, 1, 1, 1> Lay;   // (tile geometry only)
-    constexpr int NO = Lay::Cfg::NO, BT = Lay::BT;
+    typedef TaRing<SPIN, NMT> Lay;
+    constexpr int NO = TaCfg<SPIN, NMT>::NO, BT = 64 * NO;
     const float *sgf = reinterpret_cast<const float *>(sg);
     for (int it = threadIdx.x; it < 8 * NO; it += TC_M) {
         const int kq = it & 3;
@@ -961,36 +969,65 @@ __device__ __forceinline__ void gen_btiles_ana(const float2 *sg, unsigned char *
     }
 }
 
-template <int SPIN, int NMT, int NAS, int NBS, int TR>
-__global__ void __launch_bounds__(TC_M, 4) k_leg_analysis_tc(const LegArgs<float> a) {
-    typedef TaLayout<SPIN, NMT, NAS, NBS, TR> Lay;
-    constexpr int NO = Lay::Cfg::NO;
+// Records of stage blockIdx.x for m = a.m0 + 8 blockIdx.y .. + 7 (below a.m0 +
+// a.mcnt) and map group blockIdx.z: entry ((group mcnt + m - m0) stages + stage).
+template <int SPIN, int NMT>
+__global__ void __launch_bounds__(TC_M) k_ta_records(const LegArgs<float> a) {
+    typedef TaRing<SPIN, NMT> Ring;
+    constexpr int BSTAGE = TaLayout<SPIN, NMT, 1, true>::BSTAGE;
+    __shared__ float2 sg[TA_MB * Ring::SG];
+    const int L = a.lmax, ps = blockIdx.x;
+    const int i0 = TA_MB * blockIdx.y, ni = min(TA_MB, a.mcnt - i0);
+    const int map0 = blockIdx.z * NMT;
+    const int nrow = (SPIN == 2 ? 2 : 1) * min(NMT, a.nmaps - map0);
+    const float2 *src = a.F + (int64_t)(SPIN == 2 ? 2 * map0 : map0) * a.nring * (L + 1) + a.m0 + i0;
+    // rows are the maps of the group (spin 2: Q, U of each); zeros for pairs
+    // beyond npairs, missing maps and the south ring of the equator pair
+#pragma unroll 8
+    for (int it = threadIdx.x; it < TA_K * 2 * Ring::NROW * TA_MB; it += TC_M) {
+        const int mi = it & (TA_MB - 1), q = (it / TA_MB) % Ring::NROW;
+        const int z = (it / (TA_MB * Ring::NROW)) & 1, pp = it / (2 * TA_MB * Ring::NROW);
+        const int rn = ps * TA_K + pp, rs = a.nring - 1 - rn;
+        float2 v = make_float2(0.f, 0.f);
+        if (mi < ni && rn < a.npairs && q < nrow && !(z && rs == rn))
+            v = src[((int64_t)q * a.nring + (z ? rs : rn)) * (L + 1) + mi];
+        sg[mi * Ring::SG + pp * Ring::GS + z * Ring::NROW + q] = v;
+    }
+    __syncthreads();
+    unsigned char *rec = a.rec_tc + (((int64_t)blockIdx.z * a.mcnt + i0) * gridDim.x + ps) * BSTAGE;
+    for (int mi = 0; mi < ni; ++mi)
+        gen_btiles_ana<SPIN, NMT>(sg + mi * Ring::SG, rec + (int64_t)mi * gridDim.x * BSTAGE);
+}
+
+template <int SPIN, int NMT, int NAS, bool REC>
+__global__ void __launch_bounds__(TC_M, (SPIN == 0 && NMT == 8 ? 6 : 4)) k_leg_analysis_tc(const LegArgs<float> a) {
+    typedef TaLayout<SPIN, NMT, NAS, REC> Lay;
+    constexpr int NO = Lay::Cfg::NO, NBS = Lay::NBS, BSTAGE = Lay::BSTAGE;
     extern __shared__ __align__(1024) unsigned char smem[];
     float4 *s_c4 = reinterpret_cast<float4 *>(smem + Lay::COEF);   // spin 2 (tc_coef)
     float2 *s_c2 = reinterpret_cast<float2 *>(smem + Lay::COEF);   // spin 0 (a, b)
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + Lay::BARS);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + Lay::BARS), *full = bars + NAS;
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + Lay::TMEMA);
 
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int m = blockIdx.y;
+    const int m = a.m0 + blockIdx.y;
     const int L = a.lmax;
-    const int lbase = m + blockIdx.x * (256 * TR);
+    const int lbase = m + blockIdx.x * 256;
     if (lbase > L) return;
-    const int ntile = min(TR, (L - lbase) / 256 + 1);
-    const int lend = min(L, lbase + 256 * TR - 1);
+    const int lend = min(L, lbase + 255);
     const int map0 = blockIdx.z * NMT;
     const int nm = min(NMT, a.nmaps - map0);
     const int64_t base = (int64_t)m * (2 * L + 1 - m) / 2;
 
-    for (int i = tid; i < 256 * TR; i += TC_M) {
+    for (int i = tid; i < 256; i += TC_M) {
         const int l = lbase + i;
         const bool in = l <= L;
         if (SPIN == 2) s_c4[ta_cpad(i)] = tc_coef(in ? a.s2c[base + l] : make_float4(0.f, 0.f, 0.f, 0.f));
         else s_c2[ta_cpad(i)] = in ? a.rec[base + l] : make_float2(0.f, 0.f);
     }
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[0])));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[1])));
+        for (int i = 0; i < NAS + NBS; ++i)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[i])));
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     if (warp == 0) {
@@ -1037,132 +1074,120 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_analysis_tc(const LegArgs<float
     const int nst = s0 < nps ? nps - s0 : 0;
 
     const uint64_t descA = sdesc(smem_u32(smem), 2048, 128), descB = sdesc(smem_u32(smem + Lay::BOFF), 32 * NO, 128);
+    const unsigned char *rec = a.rec_tc + (((int64_t)blockIdx.z * a.mcnt + blockIdx.y) * nps + s0) * BSTAGE;
     bool ok = true;
-    int unit = 0, waited = -1;
-    int last_unit[NBS];            // last unit that read each B buffer
-#pragma unroll
-    for (int i = 0; i < NBS; ++i) last_unit[i] = -1;
     PairStart pst{}, pnext{};
     float4 tcur = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int l0 = lbase + 32 * seg;
     if (nst > 0) {
-        stage_ring_data<SPIN, NMT>(a, m, s0, map0, nm, sgb);
+        if (!REC) stage_ring_data<SPIN, NMT>(a, m, s0, map0, nm, sgb);
+        else if (tid == 0) bulk_load(smem + Lay::BOFF, rec, BSTAGE, &full[0]);
         pst = load_pair_start<SPIN>(a, m, s0 * TA_K + pin);
-        tcur = load_tile_state<SPIN>(a, m, s0 * TA_K + pin, lbase + 32 * seg);
+        tcur = load_tile_state<SPIN>(a, m, s0 * TA_K + pin, l0);
     }
+    // Stage si commits its MMAs to barrier si % NAS, completing that barrier's
+    // phase si / NAS, and its record sits in B buffer si % NBS.
+    int bsel = 0, bph = 0;
     for (int si = 0; si < nst; ++si) {
-        const int ps = s0 + si;
-        const int pr = ps * TA_K + pin;
+        const int pr = (s0 + si) * TA_K + pin;
         const bool more = si + 1 < nst;
-        if (more) pnext = load_pair_start<SPIN>(a, m, pr + TA_K);   // in flight during this stage
-        asm volatile("cp.async.wait_group 0;" ::: "memory");          // this stage's ring data
-        __syncthreads();
-        // unit u commits to barrier u % NAS, completing its phase u / NAS; the
-        // commits complete in order, so waiting for u covers every unit before it
-        const int bsel = si % NBS;
-        unsigned char *bt = smem + Lay::BOFF + bsel * Lay::BSTAGE;
-        if (last_unit[bsel] > waited) {   // the stage NBS back read this B buffer
-            const int u = last_unit[bsel];
-            ok = mbar_wait(&bars[u % NAS], (u / NAS) & 1) && ok;
-            waited = u;
+        float4 tnext = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (more) {   // in flight during this stage
+            pnext = load_pair_start<SPIN>(a, m, pr + TA_K);
+            tnext = load_tile_state<SPIN>(a, m, pr + TA_K, l0);
         }
-        gen_btiles_ana<SPIN, NMT>(sgb, bt);
-        for (int r = 0; r < ntile; ++r) {
-            const int asel = unit % NAS;
-            unsigned char *at = smem + asel * Lay::ASTAGE;
-            auto free_tiles = [&]() {   // the unit NAS back read this A buffer
-                if (unit >= NAS && unit - NAS > waited) {
-                    ok = mbar_wait(&bars[asel], ((unit - NAS) / NAS) & 1) && ok;
-                    waited = unit - NAS;
-                }
-            };
-            const int tstart = lbase + 256 * r;
-            const int l0 = tstart + 32 * seg;
-            // state of the next unit: (this stage, next tile) or (next stage, first tile)
-            float4 tnext = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (r + 1 < ntile) tnext = load_tile_state<SPIN>(a, m, pr, l0 + 256);
-            else if (more) tnext = load_tile_state<SPIN>(a, m, pr + TA_K, lbase + 32 * seg);
-            const bool starts = (pst.ls >= l0 && pst.ls < l0 + 32) || (SPIN == 2 && pst.lsb >= l0 && pst.lsb < l0 + 32);
-            if (__any_sync(0xffffffffu, starts && l0 <= L))
-                gen_atiles_ana<SPIN, true>(pst, tcur, pin, seg, l0, lbase, s_c4, at, free_tiles);
-            else
-                gen_atiles_ana<SPIN, false>(pst, tcur, pin, seg, l0, lbase, s_c4, at, free_tiles);
-            tcur = tnext;
-            asm volatile("fence.proxy.async.shared::cta;");
+        if (!REC) {   // (this B buffer was read by stage si - NBS, waited for in stage si - 1)
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
             __syncthreads();
-            // every thread has built this stage's B tiles: the ring-data buffer
-            // takes the next stage's copy, in flight during the stage's units
-            if (r == 0 && more) stage_ring_data<SPIN, NMT>(a, m, ps + 1, map0, nm, sgb);
-            if (tid == 0) {
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const uint32_t id = idesc_bf16_amn(TC_M, NO);
-                const uint32_t acc = si > 0;
-                // (the address field counts 16-byte units)
-                const uint64_t da = descA + (uint32_t)(asel * (Lay::ASTAGE >> 4));
-                const uint64_t db = descB + (uint32_t)(bsel * (Lay::BSTAGE >> 4));
-                auto A = [&](int t) { return da + (uint32_t)(t * (TC_ATILE >> 4)); };
-                auto Bh = [&](int t) { return db + (uint32_t)(t * (Lay::BT >> 4)); };
-                auto Bl = [&](int t) { return db + (uint32_t)((t * Lay::BT + (NO / 8) * 128) >> 4); };
-                const uint32_t dE = tmem + r * 2 * NO, dO = dE + NO;
-                if (SPIN == 0) {
-                    mma_bf16(dE, A(0), Bh(0), id, acc);
-                    mma_bf16(dE, A(0), Bl(0), id, 1);
-                    mma_bf16(dE, A(1), Bh(0), id, 1);
-                    mma_bf16(dO, A(2), Bh(1), id, acc);
-                    mma_bf16(dO, A(2), Bl(1), id, 1);
-                    mma_bf16(dO, A(3), Bh(1), id, 1);
-                } else {
-                    mma_bf16(dE, A(0), Bh(0), id, acc);   // lw even rows, W from G_N + G_S
-                    mma_bf16(dE, A(0), Bl(0), id, 1);
-                    mma_bf16(dE, A(1), Bh(0), id, 1);
-                    mma_bf16(dE, A(4), Bh(2), id, 1);     // lx even rows, X from G_N - G_S
-                    mma_bf16(dE, A(4), Bl(2), id, 1);
-                    mma_bf16(dE, A(5), Bh(2), id, 1);
-                    mma_bf16(dO, A(2), Bh(1), id, acc);
-                    mma_bf16(dO, A(2), Bl(1), id, 1);
-                    mma_bf16(dO, A(3), Bh(1), id, 1);
-                    mma_bf16(dO, A(6), Bh(3), id, 1);
-                    mma_bf16(dO, A(6), Bl(3), id, 1);
-                    mma_bf16(dO, A(7), Bh(3), id, 1);
-                }
-                mma_commit(&bars[asel]);
-            }
-            last_unit[bsel] = unit;
-            ++unit;
+            gen_btiles_ana<SPIN, NMT>(sgb, smem + Lay::BOFF + bsel * BSTAGE);
         }
+        const int asel = si % NAS;
+        unsigned char *at = smem + asel * Lay::ASTAGE;
+        // the MMAs of stage si - NAS are done: its A buffer is free, and so is
+        // the B buffer that the next stage's record goes to
+        auto free_tiles = [&]() {
+            if (si >= NAS) ok = mbar_wait(&bars[asel], ((si - NAS) / NAS) & 1) && ok;
+            if (REC && tid == 0 && more) {
+                const int bn = bsel + 1 == NBS ? 0 : bsel + 1;
+                bulk_load(smem + Lay::BOFF + bn * BSTAGE, rec + (int64_t)(si + 1) * BSTAGE, BSTAGE, &full[bn]);
+            }
+        };
+        const bool starts = (pst.ls >= l0 && pst.ls < l0 + 32) || (SPIN == 2 && pst.lsb >= l0 && pst.lsb < l0 + 32);
+        if (__any_sync(0xffffffffu, starts && l0 <= L))
+            gen_atiles_ana<SPIN, true>(pst, tcur, pin, seg, l0, lbase, s_c4, at, free_tiles);
+        else
+            gen_atiles_ana<SPIN, false>(pst, tcur, pin, seg, l0, lbase, s_c4, at, free_tiles);
+        tcur = tnext;
         pst = pnext;
+        asm volatile("fence.proxy.async.shared::cta;");
+        __syncthreads();
+        // (the ring data are consumed: the next stage's copy runs beside this
+        // stage's MMAs and the next generation)
+        if (!REC && more) stage_ring_data<SPIN, NMT>(a, m, s0 + si + 1, map0, nm, sgb);
+        if (tid == 0) {
+            if (REC) ok = mbar_wait(&full[bsel], bph) && ok;   // the stage's record
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            // id2: hi and lo rows of B side by side (2 NO columns); id: hi only
+            const uint32_t id2 = idesc_bf16_amn(TC_M, 2 * NO), id = idesc_bf16_amn(TC_M, NO);
+            const uint32_t acc = si > 0;
+            // (the address field counts 16-byte units)
+            const uint64_t da = descA + (uint32_t)(asel * (Lay::ASTAGE >> 4));
+            const uint64_t db = descB + (uint32_t)(bsel * (BSTAGE >> 4));
+            auto A = [&](int t) { return da + (uint32_t)(t * (TC_ATILE >> 4)); };
+            auto B = [&](int t) { return db + (uint32_t)(t * (Lay::BT >> 4)); };
+            const uint32_t dE = tmem, dO = tmem + 2 * NO;
+            // A hi with B hi and B lo, A lo with B hi; spin 2: even rows lw with
+            // W from G_N + G_S, lx with X from G_N - G_S, odd rows the others
+            mma_bf16(dE, A(0), B(0), id2, acc);
+            mma_bf16(dE, A(1), B(0), id, 1);
+            mma_bf16(dO, A(2), B(1), id2, acc);
+            mma_bf16(dO, A(3), B(1), id, 1);
+            if (SPIN == 2) {
+                mma_bf16(dE, A(4), B(2), id2, 1);
+                mma_bf16(dE, A(5), B(2), id, 1);
+                mma_bf16(dO, A(6), B(3), id2, 1);
+                mma_bf16(dO, A(7), B(3), id, 1);
+            }
+            mma_commit(&bars[asel]);
+        }
+        if (++bsel == NBS) {
+            bsel = 0;
+            bph ^= 1;
+        }
     }
-    if (unit > 0 && unit - 1 > waited) ok = mbar_wait(&bars[(unit - 1) % NAS], ((unit - 1) / NAS) & 1) && ok;
+    if (nst > 0) ok = mbar_wait(&bars[(nst - 1) % NAS], ((nst - 1) / NAS) & 1) && ok;
     asm volatile("tcgen05.fence::after_thread_sync;");
+    ok = __syncthreads_and(ok);   // (the records' waits are one thread's)
     if (!ok && tid == 0 && a.err) atomicExch(a.err, 1);
 
-    // ---- epilogue: lane = row i, l = tstart + 2 i (E tile) and + 1 (O tile)
+    // ---- epilogue: lane = row i, l = lbase + 2 i (E tile) and + 1 (O tile)
 #pragma unroll
-    for (int r = 0; r < TR; ++r) {
-        if (r >= ntile) break;
-        const int tstart = lbase + 256 * r;
+    for (int cls = 0; cls < 2; ++cls) {
+        const int l = lbase + 2 * tid + cls;
+        float d[NO], e[NO];
+        if constexpr (NO == 16) {
+            tmem_ld16(trow + cls * 2 * NO, d);
+            tmem_ld16(trow + cls * 2 * NO + NO, e);
+        } else {
+            tmem_ld32(trow + cls * 2 * NO, d);
+            tmem_ld32(trow + cls * 2 * NO + NO, e);
+        }
+        if (!ok || l > L) continue;
+        const float bm = (a.beam ? a.beam[l] : 1.f) * ((a.vjp && m > 0) ? 2.f : 1.f);
 #pragma unroll
-        for (int cls = 0; cls < 2; ++cls) {
-            const int l = tstart + 2 * tid + cls;
-            float d[NO];
-            if (NO == 16) tmem_ld16(trow + r * 2 * NO + cls * NO, *reinterpret_cast<float(*)[16]>(d));
-            else tmem_ld32(trow + r * 2 * NO + cls * NO, *reinterpret_cast<float(*)[32]>(d));
-            if (!ok || l > L) continue;
-            const float bm = (a.beam ? a.beam[l] : 1.f) * ((a.vjp && m > 0) ? 2.f : 1.f);
+        for (int k = 0; k < NMT; ++k) {
+            if (k >= nm) break;
 #pragma unroll
-            for (int k = 0; k < NMT; ++k) {
-                if (k >= nm) break;
-#pragma unroll
-                for (int c = 0; c < (SPIN == 2 ? 2 : 1); ++c) {
-                    const int j = SPIN == 2 ? 4 * k + 2 * c : 2 * k;
-                    float re = 0.f, im = 0.f;
-                    if (nst > 0) {
-                        re = d[j] * bm;
-                        im = m == 0 ? 0.f : d[j + 1] * bm;
-                    }
-                    const int64_t row = (int64_t)(map0 + k) * a.rs + c;
-                    float2 *dst = const_cast<float2 *>(a.alm) + row * a.nalm + base + l;
-                    *dst = make_float2(re, im);
+            for (int c = 0; c < (SPIN == 2 ? 2 : 1); ++c) {
+                const int j = SPIN == 2 ? 4 * k + 2 * c : 2 * k;
+                float re = 0.f, im = 0.f;
+                if (nst > 0) {
+                    re = (d[j] + e[j]) * bm;
+                    im = m == 0 ? 0.f : (d[j + 1] + e[j + 1]) * bm;
                 }
+                const int64_t row = (int64_t)(map0 + k) * a.rs + c;
+                float2 *dst = const_cast<float2 *>(a.alm) + row * a.nalm + base + l;
+                *dst = make_float2(re, im);
             }
         }
     }
@@ -1171,30 +1196,52 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_analysis_tc(const LegArgs<float
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Lay::TMEM));
 }
 
-template <int SPIN, int NMT, int NAS, int NBS, int TR>
+template <int SPIN, int NMT, int NAS, bool REC>
 int launch_analysis_tc(Plan *p, const float2 *G, int nmaps, const float *beam, float2 *alm, int rs,
                        cudaStream_t st, int vjp) {
     LegArgs<float> a = leg_make_args<float>(p);
-    a.alm = alm;
+    typedef TaLayout<SPIN, NMT, NAS, REC> Lay;
     a.rs = rs;
     a.vjp = vjp;
-    a.F = const_cast<float2 *>(G);
     a.beam = beam;
-    a.nmaps = nmaps;
     a.err = p->d_flag;
+    a.rec_tc = p->d_tcrec[SPIN / 2];
     if (!a.toff || !a.tst0 || (SPIN == 2 && !a.tst2)) {
         set_error("tensor-core transpose: the plan has no recurrence tile states");
         return SHTG_ERR_ARG;
     }
-    const int smem = TaLayout<SPIN, NMT, NAS, NBS, TR>::BYTES;
-    auto kern = k_leg_analysis_tc<SPIN, NMT, NAS, NBS, TR>;
+    const int smem = Lay::BYTES;
+    auto kern = k_leg_analysis_tc<SPIN, NMT, NAS, REC>;
     SHTG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    dim3 grid((p->lmax + 256 * TR) / (256 * TR), p->lmax + 1, (nmaps + NMT - 1) / NMT);
+    // with records as many map groups, then as many m per pass as the plan's
+    // buffer holds (all of them up to its cap)
+    const int nps = (p->npairs + TA_K - 1) / TA_K, groups = (nmaps + NMT - 1) / NMT;
+    const int64_t per_m = (int64_t)nps * Lay::BSTAGE, bytes = p->tcrec_bytes[SPIN / 2];
+    const int gfit = REC ? (int)std::max<int64_t>(1, std::min<int64_t>(groups, bytes / per_m)) : groups;
+    const int mfit = REC ? (int)std::max<int64_t>(1, std::min<int64_t>(p->lmax + 1, bytes / (per_m * gfit))) : p->lmax + 1;
     prof_begin(p, K_LEG_ANA32, st);
-    kern<<<grid, TC_M, smem, st>>>(a);
-    prof_end(p, st);
+    int nl = 0;
+    for (int g0 = 0; g0 < groups; g0 += gfit) {
+        const int ng = std::min(gfit, groups - g0);
+        a.nmaps = std::min(nmaps - g0 * NMT, ng * NMT);
+        a.alm = alm + (int64_t)g0 * NMT * rs * p->nalm;
+        a.F = const_cast<float2 *>(G) + (int64_t)g0 * NMT * (SPIN == 2 ? 2 : 1) * p->nring * (p->lmax + 1);
+        for (a.m0 = 0; a.m0 <= p->lmax; a.m0 += mfit) {
+            a.mcnt = std::min(mfit, p->lmax + 1 - a.m0);
+            if (REC) k_ta_records<SPIN, NMT><<<dim3(nps, (a.mcnt + TA_MB - 1) / TA_MB, ng), TC_M, 0, st>>>(a);
+            kern<<<dim3((p->lmax - a.m0 + 256) / 256, a.mcnt, ng), TC_M, smem, st>>>(a);
+            nl += REC ? 2 : 1;
+        }
+    }
+    prof_end(p, st, nl);
     SHTG_CHECK_LAUNCH("k_leg_analysis_tc");
     return SHTG_OK;
+}
+
+// bytes of all records of the transpose for mb maps
+template <int SPIN, int NMT> int64_t ta_record_bytes(const Plan *p, int mb) {
+    const int64_t per_m = (int64_t)((p->npairs + TA_K - 1) / TA_K) * TaLayout<SPIN, NMT, 1, true>::BSTAGE;
+    return per_m * (p->lmax + 1) * ((mb + NMT - 1) / NMT);
 }
 }  // namespace
 
@@ -1207,31 +1254,66 @@ int leg_synth_tc(Plan *p, int spin, const float2 *alm, int rs, int nmaps, const 
     return launch_synth_tc<0, 8>(p, alm, rs, nmaps, beam, F, st);
 }
 
-// Transpose: maps per CTA likewise; shapes tried by the autotuner (key kind
-// 2), (A buffers, B buffers, 256-l tiles) = (1, 1, 2) [the fastest at N_side
-// 1024, l_max 2048, 8 maps], (1, 2, 2), (2, 2, 2), (1, 1, 1), (1, 2, 1), (2,
-// 2, 1).  Every shape sums the same products in the same order, so the choice
-// does not change a bit of the result.
+// Transpose: maps per CTA likewise; one or two A buffers, with records or with
+// the CTAs building their own B tiles (small grids, where the records' launch
+// costs more than it saves: N_side 64, l_max 128, 10 maps, spin 0, 23 against 16
+// us; N_side 512, l_max 1024, 4 maps, spin 2, 0.63 against 0.69 ms), tried by the autotuner (key kind 2).  All
+// sum the same products in the same order, so the choice does not change a bit of
+// the result.
 template <int SPIN, int NMT>
 static int analysis_tc_shape(int v, Plan *p, const float2 *G, int nmaps, const float *beam, float2 *alm, int rs,
                              cudaStream_t st, int vjp) {
     switch (v) {
-        case 1: return launch_analysis_tc<SPIN, NMT, 1, 2, 2>(p, G, nmaps, beam, alm, rs, st, vjp);
-        case 2: return launch_analysis_tc<SPIN, NMT, 2, 2, 2>(p, G, nmaps, beam, alm, rs, st, vjp);
-        case 3: return launch_analysis_tc<SPIN, NMT, 1, 1, 1>(p, G, nmaps, beam, alm, rs, st, vjp);
-        case 4: return launch_analysis_tc<SPIN, NMT, 1, 2, 1>(p, G, nmaps, beam, alm, rs, st, vjp);
-        case 5: return launch_analysis_tc<SPIN, NMT, 2, 2, 1>(p, G, nmaps, beam, alm, rs, st, vjp);
-        default: return launch_analysis_tc<SPIN, NMT, 1, 1, 2>(p, G, nmaps, beam, alm, rs, st, vjp);
+        case 1: return launch_analysis_tc<SPIN, NMT, 2, true>(p, G, nmaps, beam, alm, rs, st, vjp);
+        case 2: return launch_analysis_tc<SPIN, NMT, 1, false>(p, G, nmaps, beam, alm, rs, st, vjp);
+        case 3: return launch_analysis_tc<SPIN, NMT, 2, false>(p, G, nmaps, beam, alm, rs, st, vjp);
+        default: return launch_analysis_tc<SPIN, NMT, 1, true>(p, G, nmaps, beam, alm, rs, st, vjp);
     }
 }
 
 int leg_analysis_tc(Plan *p, int spin, const float2 *G, int nmaps, const float *beam, float2 *alm, int rs,
                     cudaStream_t st, int vjp) {
-    return tune(p, 2, spin == 2 ? 3 : 2, nmaps, 6, st, [&](int v) {
+    return tune(p, 2, spin == 2 ? 3 : 2, nmaps, 4, st, [&](int v) {
         if (spin == 2) return analysis_tc_shape<2, 8>(v, p, G, nmaps, beam, alm, rs, st, vjp);
         if (nmaps > 8) return analysis_tc_shape<0, 16>(v, p, G, nmaps, beam, alm, rs, st, vjp);
         return analysis_tc_shape<0, 8>(v, p, G, nmaps, beam, alm, rs, st, vjp);
     });
+}
+
+// The plan's record buffers, one per spin, which synthesis and transpose use in
+// turn: every record of a full batch, at most 1 GB for the synthesis and 4 GB
+// for the transpose (whose passes each end on a nearly empty wave), at least
+// one map group (synthesis) or one m (transpose); what does not fit takes
+// several passes.
+static int alloc_records(Plan *p) {
+    const int mb = p->max_batch;
+    const int64_t cap = (int64_t)1 << 30;
+    for (int k = 0; k < 2; ++k) {
+        if (k == 1 && !(p->flags & SHTG_SPIN2)) break;
+        const int64_t rec = k == 1 ? TcCfg<2, 8>::REC : mb > 8 ? TcCfg<0, 16>::REC : TcCfg<0, 8>::REC;
+        const int64_t groups = k == 0 && mb > 8 ? (mb + 15) / 16 : (mb + 7) / 8;
+        const int64_t ana = k == 1 ? ta_record_bytes<2, 8>(p, mb)
+                                   : mb > 8 ? ta_record_bytes<0, 16>(p, mb)
+                                            : ta_record_bytes<0, 8>(p, mb);
+        const int64_t least = std::max(p->tc_nrec * rec, ana / ((p->lmax + 1) * groups));
+        int64_t bytes = std::max(least, std::max(std::min(p->tc_nrec * rec * groups, cap), std::min(ana, 4 * cap)));
+        // on a device that is nearly full: a smaller buffer and more passes
+        cudaError_t e;
+        while ((e = cudaMalloc((void **)&p->d_tcrec[k], (size_t)bytes)) == cudaErrorMemoryAllocation && bytes > least) {
+            cudaGetLastError();
+            bytes = std::max(least, bytes / 2);
+        }
+        if (e != cudaSuccess) {
+            p->d_tcrec[k] = nullptr;
+            cudaGetLastError();
+            set_error(std::string("cudaMalloc of ") + std::to_string(bytes) +
+                      " bytes (tensor-core records) failed: " + cudaGetErrorString(e));
+            return SHTG_ERR_NOMEM;
+        }
+        p->tcrec_bytes[k] = bytes;
+        p->device_bytes += p->tcrec_bytes[k];
+    }
+    return SHTG_OK;
 }
 
 }  // namespace shtg
