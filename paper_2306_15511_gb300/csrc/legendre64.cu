@@ -3,6 +3,11 @@
 
 namespace shtg {
 
+// small grids (legendre_g64.cu)
+bool leg_synth_seg_fits(const Plan *p, int groups);
+int leg_synth_seg(Plan *p, int spin, int nm, const double2 *alm, int rs, int nmaps, const double *beam, double2 *F,
+                  cudaStream_t st);
+
 // Maps per pass: the FP64 pipe bounds this kernel (a warp instruction takes
 // 64 cycles of its scheduler's FP64 unit), and a pass over NM maps costs
 // R + W NM multiply-adds per (l, m, ring pair), whether or not all NM are
@@ -31,15 +36,18 @@ template <>
 int leg_synth<double>(Plan *p, int spin, const double2 *alm, int rs, int nmaps, const double *beam, double2 *F,
                       cudaStream_t st) {
     static const int nm0[] = {8, 6, 4, 3, 2, 1}, nm2[] = {4, 3, 2, 1};
+    const int nm = spin == 2 ? leg_maps_per_pass(2, nmaps, nm2, 4) : leg_maps_per_pass(0, nmaps, nm0, 6);
+    if ((spin == 0 || p->d_tst64_2) && leg_synth_seg_fits(p, (nmaps + nm - 1) / nm))
+        return leg_synth_seg(p, spin, nm, alm, rs, nmaps, beam, F, st);
     if (spin == 2) {
-        switch (leg_maps_per_pass(2, nmaps, nm2, 4)) {
+        switch (nm) {
             case 1: return launch_synth_v<double, 2, 1, 1>(p, alm, rs, nmaps, beam, F, st);
             case 2: return launch_synth_v<double, 2, 1, 2>(p, alm, rs, nmaps, beam, F, st);
             case 3: return launch_synth_v<double, 2, 1, 3>(p, alm, rs, nmaps, beam, F, st);
             default: return launch_synth_v<double, 2, 1, 4>(p, alm, rs, nmaps, beam, F, st);
         }
     }
-    switch (leg_maps_per_pass(0, nmaps, nm0, 6)) {
+    switch (nm) {
         case 1: return launch_synth_v<double, 0, 1, 1>(p, alm, rs, nmaps, beam, F, st);
         case 2: return launch_synth_v<double, 0, 1, 2>(p, alm, rs, nmaps, beam, F, st);
         case 3: return launch_synth_v<double, 0, 1, 3>(p, alm, rs, nmaps, beam, F, st);

@@ -298,7 +298,7 @@ struct ArDf {
     typedef dfc2 C2;
     typedef dfc4 C4;
     template <int SPIN> using State = DfPair<SPIN>;
-    static constexpr bool HALVES = true;
+    static constexpr bool HALVES = true, GROUPS = false;
     static constexpr int OPB = sizeof(df2);
     static __device__ __forceinline__ V from(double x) { return df_from(x); }
     static __device__ __forceinline__ C2 c2(double2 v) { return dfc2_from(v); }
