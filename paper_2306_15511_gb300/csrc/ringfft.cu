@@ -35,14 +35,19 @@ namespace shtg {
 // times as many threads, spread over all four schedulers.  Fused stage of one
 // map at N_side 32: 104 -> 30 us; of 12 T, Q, U maps at N_side 128, l_max 256:
 // 1009 -> 584 us; synthesis of 8 maps at N_side 512, M = 4096: 1.85 -> 1.71
-// ms (near the FP64 pipe).  FP32 lengths up to 1024: radix 8, 128 threads
-// (latency bound: one radix-16 butterfly a pass on 64 threads took longer);
-// the same 12 maps at N_side 128: 80 -> 50 us.  Launches of lengths up to
-// 1024 run one kernel for all their lengths with the threads of the longest.
-template <typename T> struct RingRadix { static constexpr int LR = sizeof(T) == 8 ? 2 : 3; };
+// ms (near the FP64 pipe).  FP64 lengths up to 256: radix 2, M / 2 threads: 8
+// FP64 instructions a pass on all four schedulers (radix 4: 28 on the first one
+// or two, and half as many passes): synthesis of one map at N_side 32, l_max 64,
+// with its Legendre sums 30 -> 27 us.  FP32 lengths up to 1024: radix 8, 128
+// threads (latency bound: one radix-16 butterfly a pass on 64 threads took
+// longer); the same 12 maps at N_side 128: 80 -> 50 us.  Launches of lengths up
+// to 1024 run one kernel for all their lengths with the threads of the longest.
+template <typename T> __host__ __device__ constexpr int ring_lr(int logm) {   // log2 of the radix
+    return sizeof(T) == 4 ? 3 : logm <= 8 ? 1 : 2;
+}
 template <typename T> __host__ __device__ constexpr int ring_nt(int logm) {
-    return logm <= 10 ? 1 << (10 - RingRadix<T>::LR)
-                      : (1 << (logm - RingRadix<T>::LR)) > 1024 ? 1024 : 1 << (logm - RingRadix<T>::LR);
+    return logm <= 10 ? 1 << (10 - ring_lr<T>(10))
+                      : (1 << (logm - ring_lr<T>(logm))) > 1024 ? 1024 : 1 << (logm - ring_lr<T>(logm));
 }
 // Which passes a launch runs: radix 4 / 8 as above (FP64; FP32 lengths up to
 // 1024 in the analysis and the fused stage), or FP32 radix 16 with M / 16
@@ -131,7 +136,7 @@ template <typename C> struct Dft<8, C> {
 // k / (R NS)}), does a radix-R DFT and writes output s to (j - k) R + k + s NS.
 //
 // Twiddles of the passes with NS > 1 come from a table rounded once from
-// FP64 (ring_twiddles): FP64 holds w, w^2, w^3 at k, NS + k, 2 NS + k; FP32
+// FP64 (ring_twiddles): FP64 holds w, w^2, w^3 (radix 2: w) at k, NS + k, 2 NS + k; FP32
 // holds w and w^4 and forms the others as products (at most three extra
 // roundings).  A warp's consecutive k read consecutive entries.
 //
@@ -158,6 +163,7 @@ __device__ __forceinline__ void fft_pass(C *buf, const C *__restrict__ tw) {
         const int j = threadIdx.x + b * NT;
         if (NB % NT == 0 || j < NB) {
             const int k = j & (NS - 1);
+            if constexpr (NS > 1 && R == 2) v[b][1] = cmul(v[b][1], tw[k]);
             if constexpr (NS > 1 && R == 4) {
                 v[b][1] = cmul(v[b][1], tw[k]);
                 v[b][2] = cmul(v[b][2], tw[NS + k]);
@@ -185,7 +191,7 @@ __device__ __forceinline__ void fft_pass(C *buf, const C *__restrict__ tw) {
 }
 // table entries of the passes of one length before the pass with this NS
 template <typename T> __host__ __device__ constexpr int ring_tw_off(int logm, int ns) {
-    constexpr int LR = RingRadix<T>::LR, PER = sizeof(T) == 8 ? 3 : 2;
+    const int LR = ring_lr<T>(logm), PER = sizeof(T) == 8 ? (1 << LR) - 1 : 2;
     int o = 0;
     for (int q = 1 << (logm % LR); q < ns; q <<= LR)
         if (q > 1) o += PER * q;
@@ -197,7 +203,7 @@ template <typename T> __host__ __device__ constexpr int ring_tw_len(int logm) {
 template <int LOGM, int NS, int NT, typename C>
 __device__ __forceinline__ void fft_passes(C *buf, const C *__restrict__ tw) {
     typedef decltype(buf[0].x + buf[0].x) T;
-    constexpr int LR = RingRadix<T>::LR;
+    constexpr int LR = ring_lr<T>(LOGM);
     if constexpr (NS < (1 << LOGM)) {
         fft_pass<(1 << LR), LOGM, NS, NT>(buf, tw + ring_tw_off<T>(LOGM, NS));
         fft_passes<LOGM, (NS << LR), NT>(buf, tw);
@@ -206,7 +212,7 @@ __device__ __forceinline__ void fft_passes(C *buf, const C *__restrict__ tw) {
 template <int LOGM, int NT, typename C>
 __device__ __forceinline__ void fft_fixed(C *buf, const C *__restrict__ tw) {
     typedef decltype(buf[0].x + buf[0].x) T;
-    constexpr int R0 = 1 << (LOGM % RingRadix<T>::LR);
+    constexpr int R0 = 1 << (LOGM % ring_lr<T>(LOGM));
     if constexpr (R0 > 1) fft_pass<R0, LOGM, 1, NT>(buf, tw);
     fft_passes<LOGM, R0, NT>(buf, tw);
 }
@@ -1001,8 +1007,8 @@ template <> RingArgs<double> ring_args<double>(Plan *p) {
 template <typename T, typename C>
 static void ring_twiddles_t(int logmax, std::vector<C> &t, int *off) {
     const double PI = 3.14159265358979323846;
-    constexpr int LR = RingRadix<T>::LR;
     for (int lg = 0; lg <= logmax; ++lg) {
+        const int LR = ring_lr<T>(lg);
         off[lg] = (int)t.size();
         for (int ns = 1 << (lg % LR); ns < (1 << lg); ns <<= LR) {
             if (ns == 1) continue;
