@@ -373,6 +373,9 @@ int check_device_flag(Plan *p, cudaStream_t st);
 int leg_analysis_tc(Plan *p, int spin, const float2 *G, int nmaps, const float *beam, float2 *alm, int rs,
                     cudaStream_t st, int vjp);
 int build_tile_states(Plan *p);
+// FP64 synthesis in the shape with the least work (not tuned)
+int leg_synth_g64(Plan *p, int spin, const double2 *alm, int rs, int nmaps, const double *beam, double2 *F,
+                  cudaStream_t st);
 // FP64 Legendre transpose as a register-blocked contraction; its FP64 tile states
 int leg_analysis_g64(Plan *p, int spin, const double2 *G, int nmaps, const double *beam, double2 *alm, int rs,
                      cudaStream_t st, int vjp);

@@ -58,12 +58,6 @@ int leg_analysis<float>(Plan *p, int spin, const float2 *G, int nmaps, const flo
     return tune(p, 1, spin == 2 ? 3 : 2, nmaps, leg_analysis32_count(spin, nmaps), st,
                 [&](int v) { return leg_analysis32_shape(p, spin, v, G, nmaps, beam, alm, rs, st, vjp); });
 }
-template <>
-int leg_analysis<double>(Plan *p, int spin, const double2 *G, int nmaps, const double *beam,
-                         double2 *alm, int rs, cudaStream_t st, int vjp) {
-    return leg_analysis_g64(p, spin, G, nmaps, beam, alm, rs, st, vjp);
-}
-
 bool leg_tuned(const Plan *p, int kind, int family, int nmaps) {
     return p->tuned.count(tune_key(kind, family, nmaps)) != 0;
 }

@@ -889,9 +889,13 @@ template <> struct Vec<float> {
 };
 
 // Legendre synthesis of the operator: FP64 (s.df: double-FP32), FP32 or
-// (s.tc) tensor-core FP32
+// (s.tc) tensor-core FP32.  FP64 sums of T+E+B problems take the shapes with the
+// least work: beside the other spin's launch (both_spins) a ragged last wave
+// costs nothing, and the shapes tuned alone were slower (N_side 128, l_max 256, 2
+// realizations, one application: 1.81 against 1.66 ms).
 static int op_synth(Solve &s, int spin, const double2 *x, int rs, const double *beam, double2 *F) {
     if (s.df) return leg_synth_df(s.p, spin, x, rs, s.nb, beam, F, s.st);
+    if (s.nc == 3) return leg_synth_g64(s.p, spin, x, rs, s.nb, beam, F, s.st);
     return leg_synth<double>(s.p, spin, x, rs, s.nb, beam, F, s.st);
 }
 static int op_synth(Solve &s, int spin, const float2 *x, int rs, const float *beam, float2 *F) {
@@ -903,6 +907,7 @@ static int op_synth(Solve &s, int spin, const float2 *x, int rs, const float *be
 // (s.tc) tensor-core FP32
 static int op_analysis(Solve &s, int spin, const double2 *G, const double *beam, double2 *y, int rs) {
     if (s.df) return leg_analysis_df(s.p, spin, G, s.nb, beam, y, rs, s.st, 0);
+    if (s.nc == 3) return leg_analysis_g64(s.p, spin, G, s.nb, beam, y, rs, s.st, 0);
     return leg_analysis<double>(s.p, spin, G, s.nb, beam, y, rs, s.st);
 }
 static int op_analysis(Solve &s, int spin, const float2 *G, const float *beam, float2 *y, int rs) {
@@ -938,8 +943,8 @@ static int both_spins(Solve &s, bool tuned, Op op) {
     if (rc == SHTG_OK && e != cudaSuccess) return cuda_fail(e, "cudaEventRecord", __FILE__, __LINE__);
     return rc;
 }
-// whether both launches of the operator's synthesis / transpose are tuned
-// (FP64 arithmetic and the tensor-core synthesis have nothing to tune)
+// whether both launches of the operator's synthesis / transpose are tuned (the
+// FP64-accurate sums and the tensor-core synthesis have nothing to tune here)
 template <typename T> static bool op_tuned(const Solve &s, bool transpose) {
     if (sizeof(T) == 8 || (s.tc && !transpose)) return true;
     const int kind = s.tc ? 2 : 1, f = transpose ? 2 : 0;
