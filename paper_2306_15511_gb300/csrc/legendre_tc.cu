@@ -298,48 +298,77 @@ __device__ __forceinline__ void gen_btiles(const float2 *s_alm, unsigned char *b
     }
 }
 
-// Records of every (m, chunk): grid (chunk, m, map group); entry (group,
-// toff[m] + chunk).
+// The record of the chunk of 32 l from l0 for the maps from map0 on, by the CTA's
+// threads: its inputs in registers (loaded a chunk ahead where a CTA builds one
+// after the other), then the record from them; s_alm: scratch for the alm,
+// TC_ALMS float2 per row
+constexpr int TC_ALMS = 33;   // (odd: rows fall in distinct banks)
+template <int SPIN, int NMT> struct RecIn {
+    static constexpr int N = TcCfg<SPIN, NMT>::NA * 32 / TC_M;
+    float2 v[N];
+    float4 c;   // threads below 32: coefficients of l0 + threadIdx.x
+};
 template <int SPIN, int NMT>
-__global__ void __launch_bounds__(TC_M) k_tc_records(const LegArgs<float> a) {
-    typedef TcCfg<SPIN, NMT> Cfg;
-    constexpr int ALMS = 33;   // staged alm row stride (odd: rows fall in distinct banks)
-    __shared__ float2 s_alm[Cfg::NA * ALMS];
-    const int m = blockIdx.y, L = a.lmax;
-    const int l0 = m + 32 * blockIdx.x;
-    if (l0 > L) return;
-    const int map0 = blockIdx.z * NMT;
+__device__ __forceinline__ void load_record(const LegArgs<float> &a, int m, int l0, int map0, RecIn<SPIN, NMT> &R) {
+    const int L = a.lmax;
     const int64_t base = (int64_t)m * (2 * L + 1 - m) / 2;
-    unsigned char *rec = a.rec_tc + ((int64_t)blockIdx.z * a.nrec + a.toff[m] + blockIdx.x) * Cfg::REC;
-    for (int e = threadIdx.x; e < Cfg::NA * 32; e += TC_M) {
-        const int i = e & 31, k = e >> 5, l = l0 + i;
-        const int mk = SPIN == 2 ? k / 2 : k;
+    const int i = threadIdx.x & 31, l = l0 + i;
+    const float bm = a.beam && l <= L ? a.beam[l] : 1.f;
+#pragma unroll
+    for (int e = 0; e < RecIn<SPIN, NMT>::N; ++e) {
+        const int k = (threadIdx.x + e * TC_M) >> 5, mk = SPIN == 2 ? k / 2 : k;
         float2 v = make_float2(0.f, 0.f);
         if (l <= L && map0 + mk < a.nmaps) {
-            const float bm = a.beam ? a.beam[l] : 1.f;
             const int64_t row = (int64_t)(map0 + mk) * a.rs + (SPIN == 2 ? (k & 1) : 0);
             v = a.alm[row * a.nalm + base + l];
             if (m == 0) v.y = 0.f;
             v.x *= bm;
             v.y *= bm;
         }
-        s_alm[k * ALMS + i] = v;
+        R.v[e] = v;
     }
+    R.c = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (threadIdx.x < 32 && l <= L) {
+        if (SPIN == 2) {
+            R.c = tc_coef(a.s2c[base + l]);
+        } else {
+            const float2 c = a.rec[base + l];
+            R.c = make_float4(c.x, c.y, 0.f, 0.f);
+        }
+    }
+}
+template <int SPIN, int NMT>
+__device__ __forceinline__ void store_record(const RecIn<SPIN, NMT> &R, float2 *s_alm, unsigned char *rec) {
+    typedef TcCfg<SPIN, NMT> Cfg;
+    const int i = threadIdx.x & 31;
+#pragma unroll
+    for (int e = 0; e < RecIn<SPIN, NMT>::N; ++e) s_alm[((threadIdx.x + e * TC_M) >> 5) * TC_ALMS + i] = R.v[e];
     if (threadIdx.x < 32) {
-        const int i = threadIdx.x, l = l0 + i;
         if (SPIN == 2) {
             // per two l, three 16-byte loads for the generation: (yz, xx) of
             // the first, (ww, ww) of both, (yz, xx) of the second
-            const float4 c = tc_coef(l <= L ? a.s2c[base + l] : make_float4(0.f, 0.f, 0.f, 0.f));
             float4 *dst = reinterpret_cast<float4 *>(rec + Cfg::COEF) + 3 * (i >> 1);
-            dst[2 * (i & 1)] = make_float4(c.x, c.y, c.z, c.z);
-            reinterpret_cast<float2 *>(dst + 1)[i & 1] = make_float2(c.w, c.w);
+            dst[2 * (i & 1)] = make_float4(R.c.x, R.c.y, R.c.z, R.c.z);
+            reinterpret_cast<float2 *>(dst + 1)[i & 1] = make_float2(R.c.w, R.c.w);
         } else {
-            reinterpret_cast<float2 *>(rec + Cfg::COEF)[i] = l <= L ? a.rec[base + l] : make_float2(0.f, 0.f);
+            reinterpret_cast<float2 *>(rec + Cfg::COEF)[i] = make_float2(R.c.x, R.c.y);
         }
     }
     __syncthreads();
-    gen_btiles<SPIN, NMT, ALMS>(s_alm, rec);
+    gen_btiles<SPIN, NMT, TC_ALMS>(s_alm, rec);
+}
+
+// Records of every (m, chunk): grid (chunk, m, map group); entry (group,
+// toff[m] + chunk).
+template <int SPIN, int NMT>
+__global__ void __launch_bounds__(TC_M) k_tc_records(const LegArgs<float> a) {
+    typedef TcCfg<SPIN, NMT> Cfg;
+    __shared__ float2 s_alm[Cfg::NA * TC_ALMS];
+    const int m = blockIdx.y, l0 = m + 32 * blockIdx.x;
+    if (l0 > a.lmax) return;
+    RecIn<SPIN, NMT> R;
+    load_record<SPIN, NMT>(a, m, l0, blockIdx.z * NMT, R);
+    store_record<SPIN, NMT>(R, s_alm, a.rec_tc + ((int64_t)blockIdx.z * a.nrec + a.toff[m] + blockIdx.x) * Cfg::REC);
 }
 
 // Recurrence over one chunk of 32 l (l = q0 .. q0 + 31, coefficients cf of the
@@ -404,7 +433,8 @@ __device__ __forceinline__ void bulk_load(unsigned char *dst, const unsigned cha
                  : "memory");
 }
 
-template <int SPIN, int NMT>
+// REC: the records are in global memory; otherwise the CTA builds each chunk's
+template <int SPIN, int NMT, bool REC>
 __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a) {
     typedef TcCfg<SPIN, NMT> Cfg;
     constexpr int NCOL = Cfg::NCOL;
@@ -457,7 +487,7 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
     const int ch0 = (lo - m) >> 5;                 // chunks start at l - m = 0 mod 32
     const int n = ((L - m) >> 5) - ch0 + 1;        // chunks of this CTA
     const unsigned char *rec = a.rec_tc + ((int64_t)blockIdx.z * a.nrec + a.toff[m] + ch0) * Cfg::REC;
-    if (tid == 0) {
+    if (REC && tid == 0) {
         bulk_load(smem, rec, Cfg::REC, &bars[0]);
         if (n > 1) bulk_load(smem + Cfg::REC, rec + Cfg::REC, Cfg::REC, &bars[1]);
     }
@@ -486,6 +516,8 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
     };
     const int fl = n <= 8 ? 2 : TC_FLUSH;   // short sums: the start of the sum weighs more
     int st = 0, ph = 0;   // record stage of chunk c and its barrier's phase
+    RecIn<SPIN, NMT> R;
+    if (!REC) load_record<SPIN, NMT>(a, m, m + 32 * ch0, map0, R);
     for (int c = 0; c < n; ++c) {
         if (c > 0 && (c & (fl - 1)) == 0) {
             ok = mbar_wait(mma_bar, (c - 1) & 1) && ok;
@@ -493,14 +525,20 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
             flush(c == fl);
         }
         unsigned char *bt = smem + st * Cfg::REC;
-        ok = mbar_wait(&bars[st], ph) && ok;            // the record
+        if (REC) {
+            ok = mbar_wait(&bars[st], ph) && ok;        // the record
+        } else {   // (chunk c - 2 used this stage; its MMAs were waited for in chunk c - 1)
+            store_record<SPIN, NMT>(R, reinterpret_cast<float2 *>(smem + Cfg::BYTES), bt);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            if (c + 1 < n) load_record<SPIN, NMT>(a, m, m + 32 * (ch0 + c + 1), map0, R);
+        }
         // the MMAs of chunk c - 1: the A tiles are free, and so is its record
         // stage (its coefficients were read before the last barrier)
         auto free_tiles = [&]() {
             if (c == 0) return;
             ok = mbar_wait(mma_bar, (c - 1) & 1) && ok;
             asm volatile("tcgen05.fence::after_thread_sync;");
-            if (tid == 0 && c + TC_NREC - 1 < n) {
+            if (REC && tid == 0 && c + TC_NREC - 1 < n) {
                 const int sp = st == 0 ? TC_NREC - 1 : st - 1;
                 bulk_load(smem + sp * Cfg::REC, rec + (int64_t)(c + TC_NREC - 1) * Cfg::REC, Cfg::REC, &bars[sp]);
             }
@@ -589,7 +627,7 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Cfg::TMEM));
 }
 
-template <int SPIN, int NMT>
+template <int SPIN, int NMT, bool REC>
 int launch_synth_tc(Plan *p, const float2 *alm, int rs, int nmaps, const float *beam, float2 *F,
                     cudaStream_t st) {
     typedef TcCfg<SPIN, NMT> Cfg;
@@ -599,12 +637,12 @@ int launch_synth_tc(Plan *p, const float2 *alm, int rs, int nmaps, const float *
     a.err = p->d_flag;
     a.rec_tc = p->d_tcrec[SPIN / 2];
     a.nrec = p->tc_nrec;
-    const int smem = Cfg::BYTES;
-    auto kern = k_leg_synth_tc<SPIN, NMT>;
+    const int smem = Cfg::BYTES + (REC ? 0 : Cfg::NA * TC_ALMS * (int)sizeof(float2));
+    auto kern = k_leg_synth_tc<SPIN, NMT, REC>;
     SHTG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     // as many map groups per pass as the plan's record buffer holds
     const int groups = (nmaps + NMT - 1) / NMT;
-    const int fit = (int)std::max<int64_t>(1, std::min<int64_t>(groups, p->tcrec_bytes[SPIN / 2] / (p->tc_nrec * Cfg::REC)));
+    const int fit = !REC ? groups : (int)std::max<int64_t>(1, std::min<int64_t>(groups, p->tcrec_bytes[SPIN / 2] / (p->tc_nrec * Cfg::REC)));
     prof_begin(p, K_LEG_SYN32, st);
     int nl = 0;
     for (int g0 = 0; g0 < groups; g0 += fit) {
@@ -612,9 +650,9 @@ int launch_synth_tc(Plan *p, const float2 *alm, int rs, int nmaps, const float *
         a.nmaps = std::min(nmaps - g0 * NMT, ng * NMT);
         a.alm = alm + (int64_t)g0 * NMT * rs * p->nalm;
         a.F = F + (int64_t)g0 * NMT * (SPIN == 2 ? 2 : 1) * p->nring * (p->lmax + 1);
-        k_tc_records<SPIN, NMT><<<dim3(p->lmax / 32 + 1, p->lmax + 1, ng), TC_M, 0, st>>>(a);
+        if (REC) k_tc_records<SPIN, NMT><<<dim3(p->lmax / 32 + 1, p->lmax + 1, ng), TC_M, 0, st>>>(a);
         kern<<<dim3((p->npairs + TC_M - 1) / TC_M, p->lmax + 1, ng), TC_M, smem, st>>>(a);
-        nl += 2;
+        nl += REC ? 2 : 1;
     }
     prof_end(p, st, nl);
     SHTG_CHECK_LAUNCH("k_leg_synth_tc");
@@ -1245,13 +1283,24 @@ template <int SPIN, int NMT> int64_t ta_record_bytes(const Plan *p, int mb) {
 }
 }  // namespace
 
-// Synthesis: 8 maps per CTA, or 16 at spin 0 when the call has more than 8
-// (the recurrence is then generated once for all of them).
+// Synthesis: 8 maps per CTA, or 16 at spin 0 when the call has more than 8 (the
+// recurrence is then generated once for all of them), from records or (small
+// grids: N_side 24, l_max 60, 5 Q/U maps, one call with its host check 73 us from
+// records, 64 us without) with the CTAs building each chunk's themselves, tried by
+// the autotuner; both give the same bits.
+template <int SPIN, int NMT>
+static int synth_tc_shape(int v, Plan *p, const float2 *alm, int rs, int nmaps, const float *beam, float2 *F,
+                          cudaStream_t st) {
+    if (v == 1) return launch_synth_tc<SPIN, NMT, false>(p, alm, rs, nmaps, beam, F, st);
+    return launch_synth_tc<SPIN, NMT, true>(p, alm, rs, nmaps, beam, F, st);
+}
 int leg_synth_tc(Plan *p, int spin, const float2 *alm, int rs, int nmaps, const float *beam, float2 *F,
                  cudaStream_t st) {
-    if (spin == 2) return launch_synth_tc<2, 8>(p, alm, rs, nmaps, beam, F, st);
-    if (nmaps > 8) return launch_synth_tc<0, 16>(p, alm, rs, nmaps, beam, F, st);
-    return launch_synth_tc<0, 8>(p, alm, rs, nmaps, beam, F, st);
+    return tune(p, 2, spin == 2 ? 1 : 0, nmaps, 2, st, [&](int v) {
+        if (spin == 2) return synth_tc_shape<2, 8>(v, p, alm, rs, nmaps, beam, F, st);
+        if (nmaps > 8) return synth_tc_shape<0, 16>(v, p, alm, rs, nmaps, beam, F, st);
+        return synth_tc_shape<0, 8>(v, p, alm, rs, nmaps, beam, F, st);
+    });
 }
 
 // Transpose: maps per CTA likewise; one or two A buffers, with records or with

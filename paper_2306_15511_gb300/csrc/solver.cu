@@ -944,9 +944,9 @@ static int both_spins(Solve &s, bool tuned, Op op) {
     return rc;
 }
 // whether both launches of the operator's synthesis / transpose are tuned (the
-// FP64-accurate sums and the tensor-core synthesis have nothing to tune here)
+// FP64-accurate sums have nothing to tune here)
 template <typename T> static bool op_tuned(const Solve &s, bool transpose) {
-    if (sizeof(T) == 8 || (s.tc && !transpose)) return true;
+    if (sizeof(T) == 8) return true;
     const int kind = s.tc ? 2 : 1, f = transpose ? 2 : 0;
     return leg_tuned(s.p, kind, f, s.nb) && leg_tuned(s.p, kind, f + 1, s.nb);
 }
