@@ -1285,9 +1285,9 @@ template <int SPIN, int NMT> int64_t ta_record_bytes(const Plan *p, int mb) {
 
 // Synthesis: 8 maps per CTA, or 16 at spin 0 when the call has more than 8 (the
 // recurrence is then generated once for all of them), from records or (small
-// grids: N_side 24, l_max 60, 5 Q/U maps, one call with its host check 73 us from
-// records, 64 us without) with the CTAs building each chunk's themselves, tried by
-// the autotuner; both give the same bits.
+// grids: N_side 24, l_max 60, 5 Q/U maps, 13 us from records, 10 us without;
+// N_side 200, l_max 390, 8 Q/U maps, 68 against 83 us) with the CTAs building each
+// chunk's themselves, tried by the autotuner; both give the same bits.
 template <int SPIN, int NMT>
 static int synth_tc_shape(int v, Plan *p, const float2 *alm, int rs, int nmaps, const float *beam, float2 *F,
                           cudaStream_t st) {
