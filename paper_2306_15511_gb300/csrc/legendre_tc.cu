@@ -76,13 +76,19 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t da, uint64_t 
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(da), "l"(db), "r"(idesc), "r"(accumulate));
+        "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
+        : "memory");
 }
 
 __device__ __forceinline__ void mma_commit(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-        smem_u32(bar)));
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+                 : "memory");
 }
+
+// Every statement below that orders memory (waits, fences, commits, the MMAs and
+// the tensor-memory accesses) clobbers "memory": the compiler then keeps plain
+// loads and stores of shared memory on their side of it.  A tcgen05.ld and its
+// wait are one statement, since the registers hold nothing before the wait.
 
 // Wait (bounded) for the completion of the mbarrier phase with the given
 // parity; false if the limit ran out.
@@ -93,7 +99,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
             "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}\n"
             : "=r"(done)
-            : "r"(smem_u32(bar)), "r"(parity));
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
     }
     return done != 0;
 }
@@ -103,14 +110,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     uint32_t r[32];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
           "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
           "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
           "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;");
+        : "r"(taddr)
+        : "memory");
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
@@ -118,12 +126,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
           "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;");
+        : "r"(taddr)
+        : "memory");
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
@@ -135,7 +144,8 @@ __device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, ui
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(db), "r"(idesc), "r"(accumulate));
+        "r"(a_tmem), "l"(db), "r"(idesc), "r"(accumulate)
+        : "memory");
 }
 
 // 4 consecutive TMEM columns of this warp's 32 lanes <- 4 registers per thread
@@ -471,17 +481,17 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
 
     if (tid == 0) {
         for (int i = 0; i <= TC_NREC; ++i)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[i])));
-        asm volatile("fence.mbarrier_init.release.cluster;");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[i])) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)),
-                     "r"(Cfg::TMEM));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+                     "r"(Cfg::TMEM) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *s_tmem;
 
     const int ch0 = (lo - m) >> 5;                 // chunks start at l - m = 0 mod 32
@@ -521,7 +531,7 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
     for (int c = 0; c < n; ++c) {
         if (c > 0 && (c & (fl - 1)) == 0) {
             ok = mbar_wait(mma_bar, (c - 1) & 1) && ok;
-            asm volatile("tcgen05.fence::after_thread_sync;");
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             flush(c == fl);
         }
         unsigned char *bt = smem + st * Cfg::REC;
@@ -537,7 +547,7 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
         auto free_tiles = [&]() {
             if (c == 0) return;
             ok = mbar_wait(mma_bar, (c - 1) & 1) && ok;
-            asm volatile("tcgen05.fence::after_thread_sync;");
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (REC && tid == 0 && c + TC_NREC - 1 < n) {
                 const int sp = st == 0 ? TC_NREC - 1 : st - 1;
                 bulk_load(smem + sp * Cfg::REC, rec + (int64_t)(c + TC_NREC - 1) * Cfg::REC, Cfg::REC, &bars[sp]);
@@ -551,10 +561,10 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
         if (__any_sync(0xffffffffu, starts)) gen_atiles<SPIN, true>(T, S, cf, q0, trow + Cfg::ACOL, free_tiles);
         else gen_atiles<SPIN, false>(T, S, cf, q0, trow + Cfg::ACOL, free_tiles);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;");
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t id = idesc_bf16(TC_M, NCOL);
             const uint32_t acc = (c & (fl - 1)) != 0;
             // (the address field counts 16-byte units)
@@ -592,7 +602,7 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
     }
     // ---- the last commit covers every MMA issued before it
     ok = mbar_wait(mma_bar, (n - 1) & 1) && ok;
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (!ok && tid == 0 && a.err) atomicExch(a.err, 1);
 
     // ---- epilogue: this thread's TMEM lane is its ring pair; columns [0,
@@ -622,9 +632,10 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
                 out[k * rowsz + (int64_t)rs * (L + 1)] = make_float2(e[2 * k] - o[2 * k], e[2 * k + 1] - o[2 * k + 1]);
         }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Cfg::TMEM));
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Cfg::TMEM) : "memory");
 }
 
 template <int SPIN, int NMT, bool REC>
@@ -1065,17 +1076,17 @@ __global__ void __launch_bounds__(TC_M, (SPIN == 0 && NMT == 8 ? 6 : 4)) k_leg_a
     }
     if (tid == 0) {
         for (int i = 0; i < NAS + NBS; ++i)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[i])));
-        asm volatile("fence.mbarrier_init.release.cluster;");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[i])) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)),
-                     "r"(Lay::TMEM));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+                     "r"(Lay::TMEM) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *s_tmem;
 
     const int pin = tid & (TA_K - 1), seg = tid >> 4;
@@ -1157,14 +1168,14 @@ __global__ void __launch_bounds__(TC_M, (SPIN == 0 && NMT == 8 ? 6 : 4)) k_leg_a
             gen_atiles_ana<SPIN, false>(pst, tcur, pin, seg, l0, lbase, s_c4, at, free_tiles);
         tcur = tnext;
         pst = pnext;
-        asm volatile("fence.proxy.async.shared::cta;");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
         // (the ring data are consumed: the next stage's copy runs beside this
         // stage's MMAs and the next generation)
         if (!REC && more) stage_ring_data<SPIN, NMT>(a, m, s0 + si + 1, map0, nm, sgb);
         if (tid == 0) {
             if (REC) ok = mbar_wait(&full[bsel], bph) && ok;   // the stage's record
-            asm volatile("tcgen05.fence::after_thread_sync;");
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             // id2: hi and lo rows of B side by side (2 NO columns); id: hi only
             const uint32_t id2 = idesc_bf16_amn(TC_M, 2 * NO), id = idesc_bf16_amn(TC_M, NO);
             const uint32_t acc = si > 0;
@@ -1194,7 +1205,7 @@ __global__ void __launch_bounds__(TC_M, (SPIN == 0 && NMT == 8 ? 6 : 4)) k_leg_a
         }
     }
     if (nst > 0) ok = mbar_wait(&bars[(nst - 1) % NAS], ((nst - 1) / NAS) & 1) && ok;
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     ok = __syncthreads_and(ok);   // (the records' waits are one thread's)
     if (!ok && tid == 0 && a.err) atomicExch(a.err, 1);
 
@@ -1229,9 +1240,10 @@ __global__ void __launch_bounds__(TC_M, (SPIN == 0 && NMT == 8 ? 6 : 4)) k_leg_a
             }
         }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Lay::TMEM));
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Lay::TMEM) : "memory");
 }
 
 template <int SPIN, int NMT, int NAS, bool REC>
