@@ -126,7 +126,8 @@ typedef struct shtg_plan shtg_plan;
 typedef struct {
     int geom, nside, nring, lmax, max_batch, flags;
     int64_t npix, nalm;
-    int64_t device_bytes;            /* device memory owned by the plan */
+    int64_t device_bytes;            /* device memory owned by the plan now (the first SHTG_TC32 transform
+                                        of a spin adds an operand buffer) */
 } shtg_plan_info;
 
 /* Create a plan: ring geometry, FP64 start states of the Legendre recurrence

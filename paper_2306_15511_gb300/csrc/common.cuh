@@ -253,9 +253,11 @@ struct Plan {
     float4 *d_tst2 = nullptr;
     // records of the tensor-core synthesis, (m, 32 l), tc_nrec per map group,
     // and of the transpose, (m, 16 ring pairs) (spin 0 and spin 2 apart: their
-    // launches may run at the same time)
+    // launches may run at the same time); optional, reserved by the first
+    // tensor-core call of the spin
     unsigned char *d_tcrec[2] = {nullptr, nullptr};
     int64_t tcrec_bytes[2] = {0, 0}, tc_nrec = 0;
+    bool tcrec_tried[2] = {false, false};
     // the same in FP64 every SHTG_TS64 l (FP64 and double-FP32 transposes),
     // [m][t][pair] at (d_toff64[m] + t) * npairs + pair
     int64_t *d_toff64 = nullptr;

@@ -42,6 +42,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cstdlib>
 
 #include "legendre_kernels.cuh"
 
@@ -699,8 +700,6 @@ __global__ void __launch_bounds__(LEG_THREADS) k_tile_states(const LegArgs<float
 
 }  // namespace
 
-static int alloc_records(Plan *p);
-
 int build_tile_states(Plan *p) {
     const int L = p->lmax;
     std::vector<int64_t> toff(L + 2);
@@ -732,7 +731,6 @@ int build_tile_states(Plan *p) {
         SHTG_CHECK_LAUNCH("k_tile_states");
     }
     p->tc_nrec = toff[L + 1];
-    SHTG_TRY(alloc_records(p));
     SHTG_CUDA(cudaDeviceSynchronize());
     return SHTG_OK;
 }
@@ -1295,6 +1293,53 @@ template <int SPIN, int NMT> int64_t ta_record_bytes(const Plan *p, int mb) {
 }
 }  // namespace
 
+// The plan's record buffers, one per spin, which synthesis and transpose use in
+// turn: every record of a full batch, at most 1 GB for the synthesis and 4 GB
+// for the transpose (whose passes each end on a nearly empty wave), and no more
+// than an eighth of the device's free memory; what does not fit takes several
+// passes.  The buffer is optional: it is reserved by the plan's first
+// tensor-core call at this spin, after everything that the plan cannot do
+// without, and where it does not hold one map group (synthesis) and one m
+// (transpose), the CTAs build their own operands.  Returns whether the plan has
+// it.  The calls that come here are host-synchronous (the wait flag) or captured
+// in the solver's relaxed mode; the allocation runs in that mode too, so that a
+// capture of another thread stands.
+static bool reserve_records(Plan *p, int spin) {
+    const int k = spin / 2;
+    if (p->tcrec_tried[k]) return p->d_tcrec[k] != nullptr;
+    p->tcrec_tried[k] = true;
+    const int mb = p->max_batch;
+    const int64_t cap = (int64_t)1 << 30;
+    const int64_t rec = k == 1 ? TcCfg<2, 8>::REC : mb > 8 ? TcCfg<0, 16>::REC : TcCfg<0, 8>::REC;
+    const int64_t groups = k == 0 && mb > 8 ? (mb + 15) / 16 : (mb + 7) / 8;
+    const int64_t ana = k == 1 ? ta_record_bytes<2, 8>(p, mb)
+                               : mb > 8 ? ta_record_bytes<0, 16>(p, mb)
+                                        : ta_record_bytes<0, 8>(p, mb);
+    const int64_t least = std::max(p->tc_nrec * rec, ana / ((p->lmax + 1) * groups));
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    size_t avail = 0, total = 0;
+    const bool known = cudaMemGetInfo(&avail, &total) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    int64_t room = known ? (int64_t)(avail / 8) : 0;
+    // SHTG_TC_RECORD_BYTES: this many bytes in place of the eighth (for tests of
+    // several passes and of a plan without the buffer)
+    if (const char *e = getenv("SHTG_TC_RECORD_BYTES")) room = atoll(e);
+    int64_t bytes = std::max(least, std::max(std::min(p->tc_nrec * rec * groups, cap), std::min(ana, 4 * cap)));
+    bytes = std::min(bytes, room);
+    for (; bytes >= least; bytes /= 2) {
+        if (cudaMalloc((void **)&p->d_tcrec[k], (size_t)bytes) == cudaSuccess) {
+            p->tcrec_bytes[k] = bytes;
+            p->device_bytes += bytes;
+            break;
+        }
+        p->d_tcrec[k] = nullptr;
+        cudaGetLastError();
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return p->d_tcrec[k] != nullptr;
+}
+
 // Synthesis: 8 maps per CTA, or 16 at spin 0 when the call has more than 8 (the
 // recurrence is then generated once for all of them), from records or (small
 // grids: N_side 24, l_max 60, 5 Q/U maps, 13 us from records, 10 us without;
@@ -1308,7 +1353,9 @@ static int synth_tc_shape(int v, Plan *p, const float2 *alm, int rs, int nmaps, 
 }
 int leg_synth_tc(Plan *p, int spin, const float2 *alm, int rs, int nmaps, const float *beam, float2 *F,
                  cudaStream_t st) {
-    return tune(p, 2, spin == 2 ? 1 : 0, nmaps, 2, st, [&](int v) {
+    const int v0 = reserve_records(p, spin) ? 0 : 1;   // the first shape that the plan can run
+    return tune(p, 2, spin == 2 ? 1 : 0, nmaps, 2 - v0, st, [&](int w) {
+        const int v = v0 + w;
         if (spin == 2) return synth_tc_shape<2, 8>(v, p, alm, rs, nmaps, beam, F, st);
         if (nmaps > 8) return synth_tc_shape<0, 16>(v, p, alm, rs, nmaps, beam, F, st);
         return synth_tc_shape<0, 8>(v, p, alm, rs, nmaps, beam, F, st);
@@ -1334,47 +1381,13 @@ static int analysis_tc_shape(int v, Plan *p, const float2 *G, int nmaps, const f
 
 int leg_analysis_tc(Plan *p, int spin, const float2 *G, int nmaps, const float *beam, float2 *alm, int rs,
                     cudaStream_t st, int vjp) {
-    return tune(p, 2, spin == 2 ? 3 : 2, nmaps, 4, st, [&](int v) {
+    const int v0 = reserve_records(p, spin) ? 0 : 2;
+    return tune(p, 2, spin == 2 ? 3 : 2, nmaps, 4 - v0, st, [&](int w) {
+        const int v = v0 + w;
         if (spin == 2) return analysis_tc_shape<2, 8>(v, p, G, nmaps, beam, alm, rs, st, vjp);
         if (nmaps > 8) return analysis_tc_shape<0, 16>(v, p, G, nmaps, beam, alm, rs, st, vjp);
         return analysis_tc_shape<0, 8>(v, p, G, nmaps, beam, alm, rs, st, vjp);
     });
-}
-
-// The plan's record buffers, one per spin, which synthesis and transpose use in
-// turn: every record of a full batch, at most 1 GB for the synthesis and 4 GB
-// for the transpose (whose passes each end on a nearly empty wave), at least
-// one map group (synthesis) or one m (transpose); what does not fit takes
-// several passes.
-static int alloc_records(Plan *p) {
-    const int mb = p->max_batch;
-    const int64_t cap = (int64_t)1 << 30;
-    for (int k = 0; k < 2; ++k) {
-        if (k == 1 && !(p->flags & SHTG_SPIN2)) break;
-        const int64_t rec = k == 1 ? TcCfg<2, 8>::REC : mb > 8 ? TcCfg<0, 16>::REC : TcCfg<0, 8>::REC;
-        const int64_t groups = k == 0 && mb > 8 ? (mb + 15) / 16 : (mb + 7) / 8;
-        const int64_t ana = k == 1 ? ta_record_bytes<2, 8>(p, mb)
-                                   : mb > 8 ? ta_record_bytes<0, 16>(p, mb)
-                                            : ta_record_bytes<0, 8>(p, mb);
-        const int64_t least = std::max(p->tc_nrec * rec, ana / ((p->lmax + 1) * groups));
-        int64_t bytes = std::max(least, std::max(std::min(p->tc_nrec * rec * groups, cap), std::min(ana, 4 * cap)));
-        // on a device that is nearly full: a smaller buffer and more passes
-        cudaError_t e;
-        while ((e = cudaMalloc((void **)&p->d_tcrec[k], (size_t)bytes)) == cudaErrorMemoryAllocation && bytes > least) {
-            cudaGetLastError();
-            bytes = std::max(least, bytes / 2);
-        }
-        if (e != cudaSuccess) {
-            p->d_tcrec[k] = nullptr;
-            cudaGetLastError();
-            set_error(std::string("cudaMalloc of ") + std::to_string(bytes) +
-                      " bytes (tensor-core records) failed: " + cudaGetErrorString(e));
-            return SHTG_ERR_NOMEM;
-        }
-        p->tcrec_bytes[k] = bytes;
-        p->device_bytes += p->tcrec_bytes[k];
-    }
-    return SHTG_OK;
 }
 
 }  // namespace shtg
