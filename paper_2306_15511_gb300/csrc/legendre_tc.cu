@@ -201,7 +201,7 @@ __device__ __forceinline__ void store_row8(unsigned char *hi_row, unsigned char 
 // re, im per map; spin 2: Q re, Q im, U re, U im per map); a B tile holds
 // NCOL hi rows then NCOL lo rows, 16 K (l of one parity class) each.  A record
 // is the B tiles of one chunk of 32 l followed by its coefficients.
-constexpr int TC_NREC = 2;    // record stages of the synthesis
+constexpr int TC_NREC = 2;    // record stages of the synthesis (chunk c uses stage c % 2)
 constexpr int TC_FLUSH = 4;   // chunks summed in tensor memory before they move to the FP32 sums
 template <int SPIN, int NMT> struct TcCfg {
     static constexpr int NCOL = SPIN == 2 ? 4 * NMT : 2 * NMT;
@@ -311,9 +311,8 @@ __device__ __forceinline__ void gen_btiles(const float2 *s_alm, unsigned char *b
 
 // The record of the chunk of 32 l from l0 for the maps from map0 on, by the CTA's
 // threads: its inputs in registers (loaded a chunk ahead where a CTA builds one
-// after the other), then the record from them; s_alm: scratch for the alm,
-// TC_ALMS float2 per row
-constexpr int TC_ALMS = 33;   // (odd: rows fall in distinct banks)
+// after the other), then the coefficients and the B tiles from them
+constexpr int TC_ALMS = 33;   // float2 per staged alm row (odd: rows fall in distinct banks)
 template <int SPIN, int NMT> struct RecIn {
     static constexpr int N = TcCfg<SPIN, NMT>::NA * 32 / TC_M;
     float2 v[N];
@@ -349,24 +348,50 @@ __device__ __forceinline__ void load_record(const LegArgs<float> &a, int m, int 
     }
 }
 template <int SPIN, int NMT>
-__device__ __forceinline__ void store_record(const RecIn<SPIN, NMT> &R, float2 *s_alm, unsigned char *rec) {
+__device__ __forceinline__ void store_coefs(const RecIn<SPIN, NMT> &R, unsigned char *rec) {
+    const int i = threadIdx.x;
+    if (i >= 32) return;
+    if (SPIN == 2) {
+        // per two l, three 16-byte loads for the generation: (yz, xx) of
+        // the first, (ww, ww) of both, (yz, xx) of the second
+        float4 *dst = reinterpret_cast<float4 *>(rec + TcCfg<SPIN, NMT>::COEF) + 3 * (i >> 1);
+        dst[2 * (i & 1)] = make_float4(R.c.x, R.c.y, R.c.z, R.c.z);
+        reinterpret_cast<float2 *>(dst + 1)[i & 1] = make_float2(R.c.w, R.c.w);
+    } else {
+        reinterpret_cast<float2 *>(rec + TcCfg<SPIN, NMT>::COEF)[i] = make_float2(R.c.x, R.c.y);
+    }
+}
+// B tiles straight from the registers (the words of gen_btiles): a warp holds one
+// alm row, lane i the l of class i & 1 and K index i / 2, so lanes i and i ^ 2
+// exchange one component and each stores the 4-byte words (two K) of the other:
+// lanes with bit 1 clear re, the others im.
+template <int SPIN, int NMT>
+__device__ __forceinline__ void store_btiles(const RecIn<SPIN, NMT> &R, unsigned char *bt) {
     typedef TcCfg<SPIN, NMT> Cfg;
-    const int i = threadIdx.x & 31;
+    constexpr int NCOL = Cfg::NCOL, LO = NCOL * 16;   // offset of the lo rows
+    const int i = threadIdx.x & 31, im = (i >> 1) & 1;
+    unsigned char *t = bt + (i & 1) * Cfg::BTILE + (i >> 4) * (32 * NCOL) + ((i >> 2) & 3) * 4;
 #pragma unroll
-    for (int e = 0; e < RecIn<SPIN, NMT>::N; ++e) s_alm[((threadIdx.x + e * TC_M) >> 5) * TC_ALMS + i] = R.v[e];
-    if (threadIdx.x < 32) {
-        if (SPIN == 2) {
-            // per two l, three 16-byte loads for the generation: (yz, xx) of
-            // the first, (ww, ww) of both, (yz, xx) of the second
-            float4 *dst = reinterpret_cast<float4 *>(rec + Cfg::COEF) + 3 * (i >> 1);
-            dst[2 * (i & 1)] = make_float4(R.c.x, R.c.y, R.c.z, R.c.z);
-            reinterpret_cast<float2 *>(dst + 1)[i & 1] = make_float2(R.c.w, R.c.w);
+    for (int e = 0; e < RecIn<SPIN, NMT>::N; ++e) {
+        const int k = (threadIdx.x + e * TC_M) >> 5;
+        const float2 v = R.v[e];
+        const float o = __shfl_xor_sync(0xffffffffu, im ? v.x : v.y, 2);
+        uint32_t hi, lo;
+        split2(im ? o : v.x, im ? v.y : o, hi, lo);
+        auto put = [&](int tile, int c, uint32_t sign) {   // class pair of tiles, column, sign of both words
+            unsigned char *q = t + tile * Cfg::BTILE + c * 16;
+            *reinterpret_cast<uint32_t *>(q) = hi ^ sign;
+            *reinterpret_cast<uint32_t *>(q + LO) = lo ^ sign;
+        };
+        if (SPIN == 0) {
+            put(0, 2 * k + im, 0u);
         } else {
-            reinterpret_cast<float2 *>(rec + Cfg::COEF)[i] = make_float2(R.c.x, R.c.y);
+            // row k = (map, E or B); W -(E re, E im, B re, B im), X (B im, -B re, -E im, E re)
+            const int c0 = 4 * (k >> 1), B = k & 1;
+            put(0, c0 + 2 * B + im, 0x80008000u);
+            put(2, c0 + (B ? 1 - im : 3 - im), B == im ? 0u : 0x80008000u);
         }
     }
-    __syncthreads();
-    gen_btiles<SPIN, NMT, TC_ALMS>(s_alm, rec);
 }
 
 // Records of every (m, chunk): grid (chunk, m, map group); entry (group,
@@ -379,7 +404,13 @@ __global__ void __launch_bounds__(TC_M) k_tc_records(const LegArgs<float> a) {
     if (l0 > a.lmax) return;
     RecIn<SPIN, NMT> R;
     load_record<SPIN, NMT>(a, m, l0, blockIdx.z * NMT, R);
-    store_record<SPIN, NMT>(R, s_alm, a.rec_tc + ((int64_t)blockIdx.z * a.nrec + a.toff[m] + blockIdx.x) * Cfg::REC);
+    unsigned char *rec = a.rec_tc + ((int64_t)blockIdx.z * a.nrec + a.toff[m] + blockIdx.x) * Cfg::REC;
+#pragma unroll
+    for (int e = 0; e < RecIn<SPIN, NMT>::N; ++e)
+        s_alm[((threadIdx.x + e * TC_M) >> 5) * TC_ALMS + (threadIdx.x & 31)] = R.v[e];
+    store_coefs<SPIN, NMT>(R, rec);
+    __syncthreads();
+    gen_btiles<SPIN, NMT, TC_ALMS>(s_alm, rec);   // (whole 16-byte rows: coalesced in global memory)
 }
 
 // Recurrence over one chunk of 32 l (l = q0 .. q0 + 31, coefficients cf of the
@@ -444,9 +475,18 @@ __device__ __forceinline__ void bulk_load(unsigned char *dst, const unsigned cha
                  : "memory");
 }
 
-// REC: the records are in global memory; otherwise the CTA builds each chunk's
+// REC: the records are in global memory; otherwise the CTA builds each chunk's (at
+// spin 2 three CTAs per SM: with 128 registers it spills, N_side 128, l_max 256, 4
+// Q/U maps 31.3 us, with 168 28.4).  Alone on an SM or nearly so, a CTA takes as
+// long as its serial chain per chunk.  So one barrier per chunk: the coefficients
+// of the next chunk are stored before it, the B tiles go from registers to their
+// places without a staging pass, and the sums move out of tensor memory after the
+// generation, when the MMAs they wait for are done.  With the staging pass, its
+// second barrier and a wait of its own for the move: N_side 48, l_max 100, 8 Q/U
+// maps 19.7 -> 18.0 us, N_side 64, l_max 150, 3 maps 20.4 -> 18.6 us (the form
+// before the records: 17.5 and 18.3 us).
 template <int SPIN, int NMT, bool REC>
-__global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a) {
+__global__ void __launch_bounds__(TC_M, (REC || SPIN == 0 ? 4 : 3)) k_leg_synth_tc(const LegArgs<float> a) {
     typedef TcCfg<SPIN, NMT> Cfg;
     constexpr int NCOL = Cfg::NCOL;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -480,6 +520,10 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
         return;
     }
 
+    const int ch0 = (lo - m) >> 5;                 // chunks start at l - m = 0 mod 32
+    const int n = ((L - m) >> 5) - ch0 + 1;        // chunks of this CTA
+    RecIn<SPIN, NMT> R;
+    if (!REC) load_record<SPIN, NMT>(a, m, m + 32 * ch0, map0, R);
     if (tid == 0) {
         for (int i = 0; i <= TC_NREC; ++i)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[i])) : "memory");
@@ -490,13 +534,12 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
                      "r"(Cfg::TMEM) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    if (!REC) store_coefs<SPIN, NMT>(R, smem);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *s_tmem;
 
-    const int ch0 = (lo - m) >> 5;                 // chunks start at l - m = 0 mod 32
-    const int n = ((L - m) >> 5) - ch0 + 1;        // chunks of this CTA
     const unsigned char *rec = a.rec_tc + ((int64_t)blockIdx.z * a.nrec + a.toff[m] + ch0) * Cfg::REC;
     if (REC && tid == 0) {
         bulk_load(smem, rec, Cfg::REC, &bars[0]);
@@ -527,19 +570,12 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
     };
     const int fl = n <= 8 ? 2 : TC_FLUSH;   // short sums: the start of the sum weighs more
     int st = 0, ph = 0;   // record stage of chunk c and its barrier's phase
-    RecIn<SPIN, NMT> R;
-    if (!REC) load_record<SPIN, NMT>(a, m, m + 32 * ch0, map0, R);
     for (int c = 0; c < n; ++c) {
-        if (c > 0 && (c & (fl - 1)) == 0) {
-            ok = mbar_wait(mma_bar, (c - 1) & 1) && ok;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            flush(c == fl);
-        }
         unsigned char *bt = smem + st * Cfg::REC;
         if (REC) {
             ok = mbar_wait(&bars[st], ph) && ok;        // the record
         } else {   // (chunk c - 2 used this stage; its MMAs were waited for in chunk c - 1)
-            store_record<SPIN, NMT>(R, reinterpret_cast<float2 *>(smem + Cfg::BYTES), bt);
+            store_btiles<SPIN, NMT>(R, bt);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             if (c + 1 < n) load_record<SPIN, NMT>(a, m, m + 32 * (ch0 + c + 1), map0, R);
         }
@@ -561,6 +597,10 @@ __global__ void __launch_bounds__(TC_M, 4) k_leg_synth_tc(const LegArgs<float> a
                             (SPIN == 2 && S.lsb[0] >= q0 && S.lsb[0] < q0 + 32);
         if (__any_sync(0xffffffffu, starts)) gen_atiles<SPIN, true>(T, S, cf, q0, trow + Cfg::ACOL, free_tiles);
         else gen_atiles<SPIN, false>(T, S, cf, q0, trow + Cfg::ACOL, free_tiles);
+        // (that stage's coefficients were read before the last barrier)
+        if (!REC && c + 1 < n) store_coefs<SPIN, NMT>(R, smem + (st ^ 1) * Cfg::REC);
+        // the sums up to chunk c - 1, whose MMAs free_tiles waited for
+        if (c > 0 && (c & (fl - 1)) == 0) flush(c == fl);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
@@ -649,7 +689,7 @@ int launch_synth_tc(Plan *p, const float2 *alm, int rs, int nmaps, const float *
     a.err = p->d_flag;
     a.rec_tc = p->d_tcrec[SPIN / 2];
     a.nrec = p->tc_nrec;
-    const int smem = Cfg::BYTES + (REC ? 0 : Cfg::NA * TC_ALMS * (int)sizeof(float2));
+    const int smem = Cfg::BYTES;
     auto kern = k_leg_synth_tc<SPIN, NMT, REC>;
     SHTG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     // as many map groups per pass as the plan's record buffer holds
@@ -1341,10 +1381,16 @@ static bool reserve_records(Plan *p, int spin) {
 }
 
 // Synthesis: 8 maps per CTA, or 16 at spin 0 when the call has more than 8 (the
-// recurrence is then generated once for all of them), from records or (small
-// grids: N_side 24, l_max 60, 5 Q/U maps, 13 us from records, 10 us without;
-// N_side 200, l_max 390, 8 Q/U maps, 68 against 83 us) with the CTAs building each
-// chunk's themselves, tried by the autotuner; both give the same bits.
+// recurrence is then generated once for all of them) and the CTAs of one map
+// group are more than the SMs (N_side 64, l_max 128, 10 maps, 129 CTAs: two
+// groups of 8 side by side 15.9 us, one of 16 17.0).  From records, or with the
+// CTAs building each chunk's themselves; both give the same bits.  Up to two
+// waves of CTAs the autotuner tries both (N_side 24, l_max 60, 5 Q/U maps: 15.8 us
+// from records, 13.1 without, in calls with the ring stage; N_side 128, l_max
+// 380, 1 Q/U map: 37.2 and 38.4).  Beyond, the records: each is read by more
+// than one CTA, and the alm come from further away between other calls than in
+// the tuner's runs (N_side 256, l_max 500, 8 Q/U maps: 125 and 117 us in the
+// tuner's runs, 130 and 140 in calls).
 template <int SPIN, int NMT>
 static int synth_tc_shape(int v, Plan *p, const float2 *alm, int rs, int nmaps, const float *beam, float2 *F,
                           cudaStream_t st) {
@@ -1353,11 +1399,14 @@ static int synth_tc_shape(int v, Plan *p, const float2 *alm, int rs, int nmaps, 
 }
 int leg_synth_tc(Plan *p, int spin, const float2 *alm, int rs, int nmaps, const float *beam, float2 *F,
                  cudaStream_t st) {
+    const int64_t ctas = (int64_t)((p->npairs + TC_M - 1) / TC_M) * (p->lmax + 1);   // of a map group
     const int v0 = reserve_records(p, spin) ? 0 : 1;   // the first shape that the plan can run
-    return tune(p, 2, spin == 2 ? 1 : 0, nmaps, 2 - v0, st, [&](int w) {
+    const int nv = v0 == 0 && ctas * ((nmaps + 7) / 8) > 8 * p->nsm ? 1 : 2 - v0;
+    return tune(p, 2, spin == 2 ? 1 : 0, nmaps, nv, st, [&](int w) {
         const int v = v0 + w;
         if (spin == 2) return synth_tc_shape<2, 8>(v, p, alm, rs, nmaps, beam, F, st);
-        if (nmaps > 8) return synth_tc_shape<0, 16>(v, p, alm, rs, nmaps, beam, F, st);
+        if (nmaps > 8 && ctas > p->nsm)
+            return synth_tc_shape<0, 16>(v, p, alm, rs, nmaps, beam, F, st);
         return synth_tc_shape<0, 8>(v, p, alm, rs, nmaps, beam, F, st);
     });
 }

@@ -16,10 +16,11 @@ import numpy as np
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-# (N_side, l_max, maps): map groups of 8 (spin 2) and 16 (spin 0); the second
-# grid's transpose records of one m are larger than its synthesis records of
-# a quarter of the m, so a small buffer splits the map groups there
-SIZES = [(32, 64, 40), (64, 16, 40), (24, 60, 5)]
+# (N_side, l_max, maps): map groups of 8 (spin 2, and spin 0 synthesis with fewer
+# CTAs than SMs) and 16 (spin 0); the second grid's transpose records of one m are
+# larger than its synthesis records of a quarter of the m, so a small buffer
+# splits the map groups there
+SIZES = [(32, 64, 40), (64, 16, 40), (24, 60, 5), (96, 160, 40)]
 
 
 def transforms(path):
@@ -60,7 +61,7 @@ def whole(tmp_path_factory):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("shape,room", [
-    (0, 1000000), (0, 200000), (0, 80000),   # several passes over m, over map groups
+    (0, 4000000), (0, 1000000), (0, 200000), (0, 80000),   # several passes over m, over map groups
     (1, 200000),                             # (two A buffers; synthesis without records)
     (0, 0), (1, 0),                          # no buffer
     (1, None), (2, None), (3, None),         # every shape that the tuner may choose
@@ -70,6 +71,27 @@ def test_every_buffer_and_shape_gives_the_same_bits(tmp_path, whole, shape, room
     assert got.keys() == whole.keys()
     for k in whole:
         assert np.array_equal(got[k], whole[k]), k
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nside,lmax", [(64, 128), (96, 160)])
+def test_map_groups_give_the_same_bits(nside, lmax):
+    """Spin 0 by groups of 8 or 16 maps (as the grid is small or large, or the
+    call has more than 8 maps) against 8 maps per call."""
+    torch = pytest.importorskip("torch")
+    from paper_2306_15511_gb300 import Plan
+    nb = 21
+    many = Plan(nside=nside, lmax=lmax, max_batch=nb)
+    few = Plan(nside=nside, lmax=lmax, max_batch=8)
+    m = torch.randn(nb, many.npix, device="cuda", generator=torch.Generator(device="cuda").manual_seed(lmax))
+    a = many.alm2map_adjoint(m, tensor_cores=True)
+    s = many.alm2map(a, tensor_cores=True)
+    for k in range(0, nb, 8):
+        ak = few.alm2map_adjoint(m[k:k + 8].contiguous(), tensor_cores=True)
+        assert torch.equal(ak, a[k:k + 8])
+        assert torch.equal(few.alm2map(ak, tensor_cores=True), s[k:k + 8])
+    many.close()
+    few.close()
 
 
 def device_bytes(plan):
