@@ -66,8 +66,10 @@ CLASS_SOURCES = {
     "leg_synth_fp32": ["legendre_tc.cu", "legendre_kernels.cuh", "legendre32.cu"],
     "leg_analysis_fp32": ["legendre_tc.cu", "legendre_kernels.cuh", "legendre32.cu"],
     "ring_fft_fp32": ["ringfft.cu"],
-    "leg_synth_fp64": ["legendre_df.cu", "df.cuh", "df2.cuh", "legendre_kernels.cuh", "legendre64.cu"],
-    "leg_analysis_fp64": ["legendre_df.cu", "df.cuh", "df2.cuh", "legendre_blk.cuh", "legendre_g64.cu"],
+    "leg_synth_fp64": ["legendre_df.cu", "df.cuh", "df2.cuh", "legendre_kernels.cuh", "legendre64.cu",
+                       "legendre_g64.cu"],
+    "leg_analysis_fp64": ["legendre_df.cu", "df.cuh", "df2.cuh", "legendre_blk.cuh", "legendre_kernels.cuh",
+                          "legendre64.cu", "legendre_g64.cu"],
     "ring_fft_fp64": ["ringfft.cu"],
 }
 

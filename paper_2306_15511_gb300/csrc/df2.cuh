@@ -1,7 +1,10 @@
 // Two double-FP32 values at a time (df.cuh) in packed FP32 instructions
-// (add / mul / fma.rn.f32x2): hi and lo hold the parts of both.  Every
-// operation rounds as its scalar form does, so the results are the same bit for
-// bit.  The FP32 pipe runs a packed instruction over two cycles, so its rate of
+// (add / mul / fma.rn.f32x2): hi and lo hold the parts of both.  Every packed
+// operation rounds as its scalar form does: on the host, without contraction,
+// the results are the same bit for bit (a CPU test).  In device code nvcc may
+// contract a product and a sum of the scalar functions into one FMA, never those
+// of the packed asm, so there the two differ in the last bits (2^-43 relative
+// in whole transforms; the error against FP64 is the same).  The FP32 pipe runs a packed instruction over two cycles, so its rate of
 // operations is that of scalar instructions; what falls by half are the issue
 // slots and the independent instructions a warp needs in flight.  Measured
 // (N_side 512, l_max 1024, 4 maps, spin 2): transpose 11.1 -> 9.2 ms, synthesis

@@ -31,7 +31,8 @@ int leg_maps_per_pass(int spin, int nmaps, const int *nms, int n) {
 // (N_side 512, l_max 1024, 8 maps: 12.8 against 13.7 ms at spin 0, 54.3
 // against 59.0 ms at spin 2; N_side 300, one map: 0.61 against 0.93 ms).
 // Before, at most four maps shared a recurrence and none of the shapes was
-// made for one or three maps (N_side 32, l_max 64, one map: 51 us, now 21).
+// made for one or three maps (N_side 32, l_max 64, one map: 51 us, with this
+// kernel 15.5; such small grids now take the segment kernel, 11.4).
 // At spin 2 and two or more maps the autotuner may take another shape: where the
 // grid is a wave and a bit, a shape with more or smaller CTAs can win (304
 // Gauss-Legendre rings, l_max 300, 4 maps: four maps per pass 1.31 ms with the

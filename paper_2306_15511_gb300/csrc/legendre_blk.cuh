@@ -26,7 +26,8 @@
 // - row blocks beyond l_max, or before the first significant l of the stage's
 //   pairs, are left out.
 // Measured (FP64; before: the best of the 8-map form and the warp-reduction
-// kernels that this replaces): N_side 300, l_max 500, 3 maps, spin 0 / 2:
+// kernels, which stay candidates of the spin-0 FP64 transpose, legendre64.cu):
+// N_side 300, l_max 500, 3 maps, spin 0 / 2:
 // 2.87 / 7.3 -> 1.65 / 5.5 ms; N_side 512, l_max 1024, 8 maps: 28.4 / 115 ->
 // 15.1 / 56 ms.  The ring data as 16-byte (re, im) operands, signs and the
 // lw / lx exchange folded in when they are staged: N_side 128, l_max 256, 2

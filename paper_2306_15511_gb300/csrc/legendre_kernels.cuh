@@ -38,9 +38,12 @@ namespace shtg {
 
 // ------------------------------------------------------------- autotuner
 // Key: (kernel kind, family, nmaps).  On the first call with a key every
-// candidate runs twice on the caller's buffers (all compute the same
-// result); the second run of each is timed with CUDA events on the stream
-// and the fastest is kept.  SHTG_TUNE=0 in the environment, or profiling,
+// candidate runs four times on the caller's buffers: once to warm up, then
+// three times timed with CUDA events on the stream; the candidate with the
+// shortest single run is kept.  All compute the same sums: the shapes of a
+// synthesis and of the tensor-core kernels give the same bits, those of the
+// CUDA-core transposes (whose order of summation differs) the same up to
+// rounding, so there the last bits may differ between two processes.  SHTG_TUNE=0 in the environment, or profiling,
 // keeps variant 0; SHTG_TUNE_LOG=1 prints every candidate's time to stderr.
 inline bool tuning_enabled() {
     static int on = -1;

@@ -254,10 +254,9 @@ __device__ __forceinline__ void fft_run(C *buf, const int buf_off, const int log
 // the whole transform of 8 Q/U maps at N_side 1024), and the synthesis of the
 // short ones, so that FP32 maps (and what is summed over them, such as the
 // log-posterior's value) keep their rounding.
-// butterflies per thread of the first radix-R pass of a launch with nt threads
-__host__ __device__ constexpr int ring_first_bpt(int R, int nt) {
-    return nt >= 512 ? (R == 2 ? 8 : 1) : nt == 256 ? 1 : nt == 128 ? (R == 2 ? 1 : 2) : (R == 8 ? 1 : 4);
-}
+// butterflies per thread of the first radix-R pass of a 64-thread launch (M <= 1024;
+// a radix-8 pass goes first at M = 8, 128 only)
+__host__ __device__ constexpr int ring_first_bpt(int R) { return R == 8 ? 1 : 4; }
 // v * e^{-2 pi i k / 16}; k is a compile-time constant after unrolling, so the
 // switch folds away
 template <typename C>
@@ -415,19 +414,20 @@ __device__ __forceinline__ void spass(C *buf, const int M, const int Ns, const T
 template <int NT, typename C>
 __device__ __forceinline__ void fft_stockham(C *buf, const int logM, const TwTab<C> tw,
                                           const C *__restrict__ post, const bool cj) {
-    // M <= 16 NT.  A radix-2, -4 or -8 pass (when log2 M is not a multiple of
-    // four) goes first, where it needs no twiddles (Ns = 1), with
-    // ring_first_bpt butterflies per thread (the plan checks that this covers
-    // M / R for every ring of the launch); the radix-16 passes follow with at
-    // most one butterfly per thread, the last of them applying post / cj.
+    static_assert(NT == 64, "ring_first_bpt");
+    // M <= 16 NT (the plan checks it).  A radix-2, -4 or -8 pass (when log2 M is
+    // not a multiple of four) goes first, where it needs no twiddles (Ns = 1),
+    // with ring_first_bpt butterflies per thread (M / R <= 256 for R = 2 and 4, 16
+    // for R = 8); the radix-16 passes follow with at most one butterfly per
+    // thread, the last of them applying post / cj.
     const int M = 1 << logM;
     int Ns = 1, rem = logM;
     const int r0 = logM & 3;
     if (r0 != 0) {
         const bool last = rem == r0;
-        if (r0 == 3) spass<8, ring_first_bpt(8, NT), NT, false>(buf, M, 1, tw, last ? post : nullptr, last && cj);
-        else if (r0 == 2) spass<4, ring_first_bpt(4, NT), NT, false>(buf, M, 1, tw, last ? post : nullptr, last && cj);
-        else spass<2, ring_first_bpt(2, NT), NT, false>(buf, M, 1, tw, last ? post : nullptr, last && cj);
+        if (r0 == 3) spass<8, ring_first_bpt(8), NT, false>(buf, M, 1, tw, last ? post : nullptr, last && cj);
+        else if (r0 == 2) spass<4, ring_first_bpt(4), NT, false>(buf, M, 1, tw, last ? post : nullptr, last && cj);
+        else spass<2, ring_first_bpt(2), NT, false>(buf, M, 1, tw, last ? post : nullptr, last && cj);
         Ns = 1 << r0;
         rem -= r0;
     }
